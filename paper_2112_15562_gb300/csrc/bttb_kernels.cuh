@@ -24,13 +24,15 @@ struct OpView {
     const cpx<R> *twy;   // W_Ny^k, k < Ny
     const cpx<R> *spec;  // [nz][Ny][ncol] layer spectra / (Nx Ny)
     cpx<R> *Z;           // [nz*ny][ncol]  row-pass output / adjoint column output
-    cpx<R> *Y;           // [Ny][ncol]     summed spectrum / residual spectrum
+    cpx<R> *Y;           // [slots][Ny][ncol]  layer groups' partial sums
+    int *cnt;            // [ncol]         arrivals of a column tile's layer groups, zero between launches
     cpx<R> *W;           // [max(sy, ...)][ncol]  inverse-column output / residual rows
     cpx<R> *V;           // fast path: residual-row spectra [ncol][256] (unused otherwise)
     int real_spec;       // fast path: spec holds the real, even spectrum of an even table for
                          // ky <= Ny/2 only, R[nz][ncol][even_spec_len(Ny)]
     int rbase;           // first layer of a column launch (per-layer launches of the recompute mode)
     int spec_r0;         // layer held at spec index 0 (0 when all layers are stored)
+    int split_half;      // 1: the row passes halve the split spectra; 0: the factor is in `spec`
     int tcol;            // 0: Z, W, V row-major ([line][ncol]); > 0: transposed, line iy of layer r and
                          // bin k at ((r * ncol + k) * tcol + iy) (the N_y = 1024 column kernels' layout)
 };
@@ -81,254 +83,11 @@ __device__ __forceinline__ void staged_loop(int total, Load load, Store store) {
         }
     }
 }
-constexpr int kStageU = 8;  // loads in flight per thread in the general kernels' staging loops
 // Batch of a row functor's staging loop: Pro::STAGE_U where the functor states it
 // (a functor whose fetch is long arithmetic keeps 1, so that its code is not
 // replicated), else 4.
 template <class F, class = void> struct StageU { static constexpr int value = 4; };
 template <class F> struct StageU<F, decltype((void)F::STAGE_U)> { static constexpr int value = F::STAGE_U; };
-
-// ---------------------------------------------------------------------------
-// Row pass, real -> half spectrum.  Pro::fetch(la, lb, hasb, j, a, b) supplies the
-// two real inputs of element j (< n_in); Pro::flush(scratch) runs once per block.
-template <typename R, class Pro>
-__global__ void __launch_bounds__(256) k_row_fwd(OpView<R> op, PairMap pm, int n_in, int P,
-                                                 cpx<R> *out0, cpx<R> *out1, Pro pro, const int *done) {
-    using C = cpx<R>;
-    if (stopped(done)) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = op.Nx, ncol = op.ncol;
-    C *buf0 = reinterpret_cast<C *>(smem_raw);
-    C *buf1 = buf0 + N * P;
-    C *tw = buf1 + N * P;
-    __shared__ double red[128];
-    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = op.twx[i];
-    pro.init();
-    const int q0 = blockIdx.x * P;
-    const int np = pm.npairs();
-    staged_loop<StageU<Pro>::value>(
-        n_in * P,
-        [&](int it) {
-            const int p = it % P, j = it / P, q = q0 + p;
-            R a = 0, b = 0;
-            if (q < np) {
-                int la, lb; bool hb;
-                pm.lines(q, la, lb, hb);
-                pro.fetch(la, lb, hb, j, a, b);
-            }
-            return mk<C>(a, b);
-        },
-        [&](int it, C z) { buf0[it] = z; });
-    __syncthreads();
-    C *X = fft_lines<R, false>(buf0, buf1, op.px, P, tw, n_in);
-    for (int it = threadIdx.x; it < ncol * P; it += blockDim.x) {
-        const int p = it % P, k = it / P, q = q0 + p;
-        if (q >= np) continue;
-        const C zk = X[k * P + p];
-        const C zm = X[((N - k) % N) * P + p];
-        int la, lb; bool hb;
-        pm.lines(q, la, lb, hb);
-        out0[pm.at(la, k, ncol, op.tcol)] = mk<C>(R(0.5) * (zk.x + zm.x), R(0.5) * (zk.y - zm.y));
-        if (hb) out1[pm.at(lb, k, ncol, op.tcol)] = mk<C>(R(0.5) * (zk.y + zm.y), R(-0.5) * (zk.x - zm.x));
-    }
-    pro.flush(red);
-}
-
-// ---------------------------------------------------------------------------
-// Row pass, half spectrum -> real, cropped to n_out.  Epi::store(la, lb, hasb, j, a, b).
-template <typename R, class Epi>
-__global__ void __launch_bounds__(256) k_row_inv(OpView<R> op, PairMap pm, int n_out, int P,
-                                                 const cpx<R> *in0, const cpx<R> *in1, Epi epi,
-                                                 const int *done) {
-    using C = cpx<R>;
-    if (stopped(done)) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = op.Nx, ncol = op.ncol;
-    C *buf0 = reinterpret_cast<C *>(smem_raw);
-    C *buf1 = buf0 + N * P;
-    C *tw = buf1 + N * P;
-    __shared__ double red[128];
-    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = op.twx[i];
-    epi.init();
-    const int q0 = blockIdx.x * P;
-    const int np = pm.npairs();
-    staged_loop<kStageU>(
-        N * P,
-        [&](int it) {
-            const int p = it % P, k = it / P, q = q0 + p;
-            C z = czero<C>();
-            if (q < np) {
-                int la, lb; bool hb;
-                pm.lines(q, la, lb, hb);
-                const bool lo = k < ncol;
-                const int kk = lo ? k : N - k;
-                C A = in0[pm.at(la, kk, ncol, op.tcol)];
-                C B = hb ? in1[pm.at(lb, kk, ncol, op.tcol)] : czero<C>();
-                if (kk == 0 || 2 * kk == N) { A.y = 0; B.y = 0; }
-                z = lo ? mk<C>(A.x - B.y, A.y + B.x) : mk<C>(A.x + B.y, B.x - A.y);
-            }
-            return z;
-        },
-        [&](int it, C z) { buf0[it] = z; });
-    __syncthreads();
-    C *X = fft_lines<R, true>(buf0, buf1, op.px, P, tw, N);
-    for (int it = threadIdx.x; it < n_out * P; it += blockDim.x) {
-        const int p = it % P, j = it / P, q = q0 + p;
-        if (q >= np) continue;
-        int la, lb; bool hb;
-        pm.lines(q, la, lb, hb);
-        const C z = X[j * P + p];
-        epi.store(la, lb, hb, j, z.x, z.y);
-    }
-    epi.flush(red);
-}
-
-// ---------------------------------------------------------------------------
-// Column pass of the forward product: for a tile of C columns and a group of
-// layers, Y += sum_r T^_r . FFT_y(Z_r).  Y must be zeroed before the launch.
-template <typename R>
-__global__ void __launch_bounds__(256) k_col_fwd_mac(OpView<R> op0, OpView<R> op1, int C, int L,
-                                                     const int *done) {
-    using Cx = cpx<R>;
-    if (stopped(done)) return;
-    const OpView<R> &op = blockIdx.z ? op1 : op0;
-    const int c0 = blockIdx.x * C;
-    const int r0 = op.rbase + blockIdx.y * L;
-    if (r0 >= op.nz || c0 >= op.ncol) return;
-    const int r1 = min(r0 + L, op.nz);
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int Ny = op.Ny, ny = op.ny, ncol = op.ncol;
-    Cx *buf0 = reinterpret_cast<Cx *>(smem_raw);
-    Cx *buf1 = buf0 + Ny * C;
-    Cx *acc = buf1 + Ny * C;
-    Cx *tw = acc + Ny * C;
-    for (int i = threadIdx.x; i < Ny; i += blockDim.x) tw[i] = op.twy[i];
-    for (int it = threadIdx.x; it < Ny * C; it += blockDim.x) acc[it] = czero<Cx>();
-    for (int r = r0; r < r1; ++r) {
-        const Cx *Zr = op.Z + (size_t)r * ny * ncol;
-        staged_loop<kStageU>(
-            ny * C,
-            [&](int it) {
-                const int c = it % C, iy = it / C;
-                return (c0 + c < ncol) ? Zr[(size_t)iy * ncol + c0 + c] : czero<Cx>();
-            },
-            [&](int it, Cx z) { buf0[it] = z; });
-        __syncthreads();
-        const Cx *X = fft_lines<R, false>(buf0, buf1, op.py, C, tw, ny);
-        const Cx *Tr = op.spec + (size_t)(r - op.spec_r0) * Ny * ncol;
-        staged_loop<kStageU>(
-            Ny * C,
-            [&](int it) {
-                const int c = it % C, ky = it / C;
-                return (c0 + c < ncol) ? Tr[(size_t)ky * ncol + c0 + c] : czero<Cx>();
-            },
-            [&](int it, Cx t) {
-                if (c0 + it % C < ncol) acc[it] = cadd(acc[it], cmul(X[it], t));
-            });
-        __syncthreads();
-    }
-    for (int it = threadIdx.x; it < Ny * C; it += blockDim.x) {
-        const int c = it % C, ky = it / C;
-        if (c0 + c < ncol) {
-            R *y = reinterpret_cast<R *>(op.Y + (size_t)ky * ncol + c0 + c);
-            atomicAdd(y, acc[it].x);
-            atomicAdd(y + 1, acc[it].y);
-        }
-    }
-}
-
-// Inverse column pass of the forward product: W[jy] = IFFT_y(Y)[jy], jy < sy.
-template <typename R>
-__global__ void __launch_bounds__(256) k_col_inv(OpView<R> op0, OpView<R> op1, int C, const int *done) {
-    using Cx = cpx<R>;
-    if (stopped(done)) return;
-    const OpView<R> &op = blockIdx.y ? op1 : op0;
-    const int c0 = blockIdx.x * C;
-    if (c0 >= op.ncol) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int Ny = op.Ny, ncol = op.ncol;
-    Cx *buf0 = reinterpret_cast<Cx *>(smem_raw);
-    Cx *buf1 = buf0 + Ny * C;
-    Cx *tw = buf1 + Ny * C;
-    for (int i = threadIdx.x; i < Ny; i += blockDim.x) tw[i] = op.twy[i];
-    staged_loop<kStageU>(
-        Ny * C,
-        [&](int it) {
-            const int c = it % C, ky = it / C;
-            return (c0 + c < ncol) ? op.Y[(size_t)ky * ncol + c0 + c] : czero<Cx>();
-        },
-        [&](int it, Cx z) { buf0[it] = z; });
-    __syncthreads();
-    const Cx *X = fft_lines<R, true>(buf0, buf1, op.py, C, tw, Ny);
-    for (int it = threadIdx.x; it < op.sy * C; it += blockDim.x) {
-        const int c = it % C, jy = it / C;
-        if (c0 + c < ncol) op.W[(size_t)jy * ncol + c0 + c] = X[it];
-    }
-}
-
-// Forward column pass of the residual (adjoint preparation): Y = FFT_y(W), W has
-// sy nonzero rows.
-template <typename R>
-__global__ void __launch_bounds__(256) k_col_fft(OpView<R> op0, OpView<R> op1, int C, const int *done) {
-    using Cx = cpx<R>;
-    if (stopped(done)) return;
-    const OpView<R> &op = blockIdx.y ? op1 : op0;
-    const int c0 = blockIdx.x * C;
-    if (c0 >= op.ncol) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int Ny = op.Ny, ncol = op.ncol;
-    Cx *buf0 = reinterpret_cast<Cx *>(smem_raw);
-    Cx *buf1 = buf0 + Ny * C;
-    Cx *tw = buf1 + Ny * C;
-    for (int i = threadIdx.x; i < Ny; i += blockDim.x) tw[i] = op.twy[i];
-    staged_loop<kStageU>(
-        op.sy * C,
-        [&](int it) {
-            const int c = it % C, iy = it / C;
-            return (c0 + c < ncol) ? op.W[(size_t)iy * ncol + c0 + c] : czero<Cx>();
-        },
-        [&](int it, Cx z) { buf0[it] = z; });
-    __syncthreads();
-    const Cx *X = fft_lines<R, false>(buf0, buf1, op.py, C, tw, op.sy);
-    for (int it = threadIdx.x; it < Ny * C; it += blockDim.x) {
-        const int c = it % C, ky = it / C;
-        if (c0 + c < ncol) op.Y[(size_t)ky * ncol + c0 + c] = X[it];
-    }
-}
-
-// Column pass of the adjoint product: for layer r, Z_r = IFFT_y(conj(T^_r) . Y),
-// rows iy < ny.
-template <typename R>
-__global__ void __launch_bounds__(256) k_col_adj(OpView<R> op0, OpView<R> op1, int C, const int *done) {
-    using Cx = cpx<R>;
-    if (stopped(done)) return;
-    const OpView<R> &op = blockIdx.z ? op1 : op0;
-    const int c0 = blockIdx.x * C;
-    const int r = op.rbase + blockIdx.y;
-    if (c0 >= op.ncol || r >= op.nz) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int Ny = op.Ny, ncol = op.ncol, ny = op.ny;
-    Cx *buf0 = reinterpret_cast<Cx *>(smem_raw);
-    Cx *buf1 = buf0 + Ny * C;
-    Cx *tw = buf1 + Ny * C;
-    for (int i = threadIdx.x; i < Ny; i += blockDim.x) tw[i] = op.twy[i];
-    const Cx *Tr = op.spec + (size_t)(r - op.spec_r0) * Ny * ncol;
-    staged_loop<kStageU>(
-        Ny * C,
-        [&](int it) {
-            const int c = it % C, ky = it / C;
-            return (c0 + c < ncol) ? cmulc(op.Y[(size_t)ky * ncol + c0 + c], Tr[(size_t)ky * ncol + c0 + c])
-                                   : czero<Cx>();
-        },
-        [&](int it, Cx z) { buf0[it] = z; });
-    __syncthreads();
-    const Cx *X = fft_lines<R, true>(buf0, buf1, op.py, C, tw, Ny);
-    Cx *Zr = op.Z + (size_t)r * ny * ncol;
-    for (int it = threadIdx.x; it < ny * C; it += blockDim.x) {
-        const int c = it % C, iy = it / C;
-        if (c0 + c < ncol) Zr[(size_t)iy * ncol + c0 + c] = X[it];
-    }
-}
 
 // ---------------------------------------------------------------------------
 // Plain functors.
@@ -431,5 +190,353 @@ template <typename R>
 __device__ __forceinline__ LoadPlain<R> field_functor(LoadPlain2<R> &p, int f) { return p.of(f); }
 template <typename R>
 __device__ __forceinline__ StorePlain<R> field_functor(StorePlain2<R> &p, int f) { return p.of(f); }
+
+// Launch shape of a row pass: P line pairs per CTA, element j of pair p at j * pitch + p
+// (odd pitch: the global accesses run along j, the butterflies along p, and neither
+// meets its own banks).
+struct RowShape {
+    int P, pitch;
+    unsigned mP;
+};
+
+// Launch shape of a column pass: a CTA takes C columns and G layers of them at a time
+// (B = C G interleaved lines, column fastest), L layers in all.
+struct ColShape {
+    int C, G, L;
+    int pitch;       // of the C G lines
+    int pitch1;      // of the C lines of the residual or summed spectrum
+    unsigned mB, mC;
+    int arrivals;    // layer groups of a column tile (1: the sum stays on chip)
+    int serial;      // 1: a launch per layer, which add to Y one after the other
+};
+
+template <typename C>
+__device__ __forceinline__ void load_twiddles(C *tw, const C *src, int N) {
+    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = src[i];
+}
+
+// In-place forward transform of P lines staged in buf0 (elements < valid): returns the
+// buffer that holds the result (buf0 or buf1).  Ends with a barrier.
+template <typename R, bool INV>
+__device__ __forceinline__ cpx<R> *fft_staged(const FftPlanDev &plan, const RowShape &rs, cpx<R> *buf0, cpx<R> *buf1,
+                                              const cpx<R> *tw, int valid, int need) {
+    using C = cpx<R>;
+    const int pitch = rs.pitch;
+    C *X = (plan.nst & 1) ? buf1 : buf0;  // the buffer that the last stage does not read
+    auto in = [&](int j, int p) { return j < valid ? buf0[j * pitch + p] : czero<C>(); };
+    auto out = [&](int n, int p, C x) { X[n * pitch + p] = x; };
+    fft_run<R, INV, !INV, INV>(plan, rs.P, rs.mP, pitch, buf1, buf0, tw, valid, need, in, out);
+    __syncthreads();
+    return X;
+}
+
+// The split of P transforms Z = FFT(a + i b) into the half spectra of their real lines:
+// A[k] = (Z[k] + conj Z[N-k]) / 2, B[k] = (Z[k] - conj Z[N-k]) / 2i.
+template <typename R>
+__device__ __forceinline__ void split_lines(const OpView<R> &op, const PairMap &pm, const RowShape &rs, int q0,
+                                            const cpx<R> *X, cpx<R> *out0, cpx<R> *out1) {
+    using C = cpx<R>;
+    const int N = op.Nx, ncol = op.ncol, np = pm.npairs();
+    const unsigned mcol = div_magic(ncol);
+    for (int it = threadIdx.x; it < ncol * rs.P; it += blockDim.x) {
+        int p, k;
+        if (op.tcol) { k = fast_div(it, rs.mP); p = it - k * rs.P; }  // consecutive lines are consecutive words
+        else { p = fast_div(it, mcol); k = it - p * ncol; }
+        const int q = q0 + p;
+        if (q >= np) continue;
+        const C zk = X[k * rs.pitch + p];
+        const C zm = X[(k ? N - k : 0) * rs.pitch + p];
+        int la, lb; bool hb;
+        pm.lines(q, la, lb, hb);
+        C A = mk<C>(zk.x + zm.x, zk.y - zm.y), B = mk<C>(zk.y + zm.y, zm.x - zk.x);
+        if (op.split_half) {
+            A = mk<C>(R(0.5) * A.x, R(0.5) * A.y);
+            B = mk<C>(R(0.5) * B.x, R(0.5) * B.y);
+        }
+        out0[pm.at(la, k, ncol, op.tcol)] = A;
+        if (hb) out1[pm.at(lb, k, ncol, op.tcol)] = B;
+    }
+}
+
+// The Hermitian-extended A + i B of P pairs of half spectra into buf (each read once).
+template <typename R>
+__device__ __forceinline__ void stage_spectra(const OpView<R> &op, const PairMap &pm, const RowShape &rs, int q0,
+                                              const cpx<R> *in0, const cpx<R> *in1, cpx<R> *buf) {
+    using C = cpx<R>;
+    struct Two { C a, b; };
+    const int N = op.Nx, ncol = op.ncol, np = pm.npairs();
+    const unsigned mcol = div_magic(ncol);
+    auto at = [&](int it, int &p, int &k) {
+        if (op.tcol) { k = fast_div(it, rs.mP); p = it - k * rs.P; }
+        else { p = fast_div(it, mcol); k = it - p * ncol; }
+    };
+    staged_loop<4>(
+        ncol * rs.P,
+        [&](int it) {
+            int p, k;
+            at(it, p, k);
+            Two t{czero<C>(), czero<C>()};
+            if (q0 + p < np) {
+                int la, lb; bool hb;
+                pm.lines(q0 + p, la, lb, hb);
+                t.a = in0[pm.at(la, k, ncol, op.tcol)];
+                if (hb) t.b = in1[pm.at(lb, k, ncol, op.tcol)];
+            }
+            return t;
+        },
+        [&](int it, Two t) {
+            int p, k;
+            at(it, p, k);
+            const bool self = k == 0 || 2 * k == N;
+            if (self) { t.a.y = 0; t.b.y = 0; }
+            buf[k * rs.pitch + p] = mk<C>(t.a.x - t.b.y, t.a.y + t.b.x);
+            if (!self) buf[(N - k) * rs.pitch + p] = mk<C>(t.a.x + t.b.y, t.b.x - t.a.y);
+        });
+}
+
+// ---------------------------------------------------------------------------
+// Row pass, real -> half spectrum.  Pro::fetch(la, lb, hasb, j, a, b) supplies the
+// two real inputs of element j (< n_in); Pro::flush(scratch) runs once per block.
+// grid y: the field of the pair calls (Pro2 functors).
+template <typename R, class Pro>
+__global__ void __launch_bounds__(256) k_row_fwd(OpView<R> op, PairMap pm, int n_in, RowShape rs,
+                                                 cpx<R> *out0, cpx<R> *out1, Pro pro, const int *done) {
+    using C = cpx<R>;
+    if (stopped(done)) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = op.Nx, P = rs.P;
+    C *buf0 = reinterpret_cast<C *>(smem_raw);
+    C *buf1 = buf0 + N * rs.pitch;
+    C *tw = buf1 + N * rs.pitch;
+    __shared__ double red[128];
+    load_twiddles(tw, op.twx, N);
+    pro.init();
+    const int field = blockIdx.y;
+    const int q0 = blockIdx.x * P;
+    const int np = pm.npairs();
+    const unsigned mn = div_magic(n_in);
+    staged_loop<StageU<Pro>::value>(
+        n_in * P,
+        [&](int it) {
+            const int p = fast_div(it, mn), j = it - p * n_in, q = q0 + p;
+            R a = 0, b = 0;
+            if (q < np) {
+                int la, lb; bool hb;
+                pm.lines(q, la, lb, hb);
+                field_functor(pro, field).fetch(la, lb, hb, j, a, b);
+            }
+            return mk<C>(a, b);
+        },
+        [&](int it, C z) {
+            const int p = fast_div(it, mn), j = it - p * n_in;
+            buf0[j * rs.pitch + p] = z;
+        });
+    __syncthreads();
+    const C *X = fft_staged<R, false>(op.px, rs, buf0, buf1, tw, n_in, N);
+    split_lines<R>(op, pm, rs, q0, X, field ? out1 : out0, pm.joint ? out1 : (field ? out1 : out0));
+    pro.flush(red);
+}
+
+// ---------------------------------------------------------------------------
+// Row pass, half spectrum -> real, cropped to n_out.  Epi::store(la, lb, hasb, j, a, b).
+template <typename R, class Epi>
+__global__ void __launch_bounds__(256) k_row_inv(OpView<R> op, PairMap pm, int n_out, RowShape rs,
+                                                 const cpx<R> *in0, const cpx<R> *in1, Epi epi,
+                                                 const int *done) {
+    using C = cpx<R>;
+    if (stopped(done)) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = op.Nx, P = rs.P;
+    C *buf0 = reinterpret_cast<C *>(smem_raw);
+    C *buf1 = buf0 + N * rs.pitch;
+    C *tw = buf1 + N * rs.pitch;
+    __shared__ double red[128];
+    load_twiddles(tw, op.twx, N);
+    epi.init();
+    const int field = blockIdx.y;
+    const int q0 = blockIdx.x * P;
+    const int np = pm.npairs();
+    stage_spectra<R>(op, pm, rs, q0, field ? in1 : in0, pm.joint ? in1 : (field ? in1 : in0), buf0);
+    __syncthreads();
+    const C *X = fft_staged<R, true>(op.px, rs, buf0, buf1, tw, N, n_out);
+    const unsigned mn = div_magic(n_out);
+    for (int it = threadIdx.x; it < n_out * P; it += blockDim.x) {
+        const int p = fast_div(it, mn), j = it - p * n_out, q = q0 + p;
+        if (q >= np) continue;
+        int la, lb; bool hb;
+        pm.lines(q, la, lb, hb);
+        const C z = X[j * rs.pitch + p];
+        field_functor(epi, field).store(la, lb, hb, j, z.x, z.y);
+    }
+    epi.flush(red);
+}
+
+// Data-line pass of the solver (joint lines): inverse rows of the cropped forward
+// product, the residual epilogue (epi.residual turns the two fields' data into W_d r~),
+// and the forward rows of the result for the adjoint's column pass.  out may be in: a
+// CTA reads its lines before it writes them.
+template <typename R, class Epi>
+__global__ void __launch_bounds__(256) k_row_resid(OpView<R> op, PairMap pm, int n_out, RowShape rs,
+                                                   const cpx<R> *in0, const cpx<R> *in1, cpx<R> *out0, cpx<R> *out1,
+                                                   Epi epi, const int *done) {
+    using C = cpx<R>;
+    if (stopped(done)) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = op.Nx, P = rs.P;
+    C *buf0 = reinterpret_cast<C *>(smem_raw);
+    C *buf1 = buf0 + N * rs.pitch;
+    C *tw = buf1 + N * rs.pitch;
+    __shared__ double red[128];
+    load_twiddles(tw, op.twx, N);
+    epi.init();
+    const int q0 = blockIdx.x * P;
+    const int np = pm.npairs();
+    stage_spectra<R>(op, pm, rs, q0, in0, in1, buf0);
+    __syncthreads();
+    C *X = fft_staged<R, true>(op.px, rs, buf0, buf1, tw, N, n_out);
+    const unsigned mn = div_magic(n_out);
+    for (int it = threadIdx.x; it < n_out * P; it += blockDim.x) {
+        const int p = fast_div(it, mn), j = it - p * n_out;
+        C z = X[j * rs.pitch + p];
+        if (q0 + p < np) epi.residual(q0 + p, j, z.x, z.y);
+        X[j * rs.pitch + p] = z;
+    }
+    __syncthreads();
+    const C *Y = fft_staged<R, false>(op.px, rs, X, X == buf0 ? buf1 : buf0, tw, n_out, N);
+    split_lines<R>(op, pm, rs, q0, Y, out0, out1);
+    epi.flush(red);
+}
+
+// ---------------------------------------------------------------------------
+// Column pass of the forward product: for a tile of C columns and a group of layers,
+// sum_r T^_r . FFT_y(Z_r); the last group of a tile to arrive takes the sum of all
+// groups (through Y) and writes W[jy] = IFFT_y(sum)[jy], jy < sy.  With one group the sum
+// never leaves the CTA.
+template <typename R>
+__global__ void __launch_bounds__(256) k_col_fwd(OpView<R> op0, OpView<R> op1, ColShape cs, const int *done) {
+    using Cx = cpx<R>;
+    if (stopped(done)) return;
+    const OpView<R> &op = blockIdx.z ? op1 : op0;
+    const int C = cs.C, G = cs.G, pitch = cs.pitch;
+    const int c0 = blockIdx.x * C;
+    const int r0 = op.rbase + blockIdx.y * cs.L;
+    if (r0 >= op.nz || c0 >= op.ncol) return;
+    const int r1 = min(r0 + cs.L, op.nz);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int last_in;
+    const int N = op.Ny, ny = op.ny, ncol = op.ncol;
+    const int cols = min(C, ncol - c0);
+    Cx *bufA = reinterpret_cast<Cx *>(smem_raw);
+    Cx *bufB = bufA + N * pitch;
+    Cx *acc = bufB + N * pitch;
+    Cx *tw = acc + N * pitch;
+    load_twiddles(tw, op.twy, N);
+    bool first = true;
+    for (int rg = r0; rg < r1; rg += G) {
+        auto in = [&](int j, int b) {
+            const int g = fast_div(b, cs.mC), c = b - g * C, r = rg + g;
+            return (j < ny && c < cols && r < r1) ? op.Z[((size_t)r * ny + j) * ncol + c0 + c] : czero<Cx>();
+        };
+        auto out = [&](int n, int b, Cx x) {
+            const int g = fast_div(b, cs.mC), c = b - g * C, r = rg + g;
+            Cx y = czero<Cx>();
+            if (c < cols && r < r1) y = cmul(x, __ldg(op.spec + ((size_t)(r - op.spec_r0) * N + n) * ncol + c0 + c));
+            Cx *a = acc + n * pitch + b;  // this thread's own entry in every layer group
+            *a = first ? y : cadd(*a, y);
+        };
+        fft_run<R, false, true, false>(op.py, C * G, cs.mB, pitch, bufA, bufB, tw, ny, N, in, out);
+        first = false;
+        if (!(op.py.nst & 1)) { Cx *t = bufA; bufA = bufB; bufB = t; }  // the last stage may still be reading bufA
+    }
+    __syncthreads();
+    auto tile_sum = [&](int k, int c) {
+        Cx y = acc[k * pitch + c];
+        for (int g = 1; g < G; ++g) y = cadd(y, acc[k * pitch + g * C + c]);
+        return y;
+    };
+    // Groups meet in Y in the order of the layers, so that a product repeats bit for bit:
+    // the groups of one launch in a slot each, summed by the last to arrive; the launches of
+    // the recompute mode (one layer each) add to slot 0 one after the other.
+    const size_t plane = (size_t)N * ncol;
+    Cx *Yt = op.Y + c0;
+    const int slots = cs.arrivals;
+    const bool before = cs.serial && r0 > 0;
+    if (cs.serial ? r1 < op.nz : slots > 1) {
+        Cx *Ys = Yt + (cs.serial ? 0 : blockIdx.y * plane);
+        for (int it = threadIdx.x; it < N * C; it += blockDim.x) {
+            const int k = fast_div(it, cs.mC), c = it - k * C;
+            if (c < cols) {
+                const Cx t = tile_sum(k, c);
+                Ys[(size_t)k * ncol + c] = before ? cadd(Ys[(size_t)k * ncol + c], t) : t;
+            }
+        }
+        if (cs.serial) return;
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last_in = atomicAdd(op.cnt + blockIdx.x, 1) == slots - 1;
+        __syncthreads();
+        if (!last_in) return;
+        __threadfence();
+        if (threadIdx.x == 0) op.cnt[blockIdx.x] = 0;
+    }
+    auto in = [&](int k, int c) {
+        if (c >= cols) return czero<Cx>();
+        const Cx *y = Yt + (size_t)k * ncol + c;
+        if (cs.serial) return before ? cadd(*y, tile_sum(k, c)) : tile_sum(k, c);
+        if (slots == 1) return tile_sum(k, c);
+        Cx t = __ldcg(y);
+        for (int s = 1; s < slots; ++s) t = cadd(t, __ldcg(y + s * plane));
+        return t;
+    };
+    auto out = [&](int n, int c, Cx x) {
+        if (n < op.sy && c < cols) op.W[(size_t)n * ncol + c0 + c] = x;
+    };
+    fft_run<R, true, false, true>(op.py, C, cs.mC, cs.pitch1, bufA, bufB, tw, N, op.sy, in, out);
+}
+
+// Column pass of the adjoint product: V^ = FFT_y(W) of a tile of C columns (W has sy
+// nonzero rows), kept on chip; then for each layer of the group
+// Z_r = IFFT_y(conj(T^_r) . V^), rows iy < ny.
+template <typename R>
+__global__ void __launch_bounds__(256) k_col_adj(OpView<R> op0, OpView<R> op1, ColShape cs, const int *done) {
+    using Cx = cpx<R>;
+    if (stopped(done)) return;
+    const OpView<R> &op = blockIdx.z ? op1 : op0;
+    const int C = cs.C, G = cs.G, pitch1 = cs.pitch1;
+    const int c0 = blockIdx.x * C;
+    const int r0 = op.rbase + blockIdx.y * cs.L;
+    if (c0 >= op.ncol || r0 >= op.nz) return;
+    const int r1 = min(r0 + cs.L, op.nz);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = op.Ny, ncol = op.ncol, ny = op.ny;
+    const int cols = min(C, ncol - c0);
+    Cx *bufA = reinterpret_cast<Cx *>(smem_raw);
+    Cx *bufB = bufA + N * cs.pitch;
+    Cx *vh = bufB + N * cs.pitch;
+    Cx *tw = vh + N * pitch1;
+    load_twiddles(tw, op.twy, N);
+    {
+        auto in = [&](int j, int c) {
+            return (j < op.sy && c < cols) ? op.W[(size_t)j * ncol + c0 + c] : czero<Cx>();
+        };
+        auto out = [&](int n, int c, Cx x) { vh[n * pitch1 + c] = x; };
+        fft_run<R, false, true, false>(op.py, C, cs.mC, pitch1, bufA, bufB, tw, op.sy, N, in, out);
+    }
+    __syncthreads();
+    for (int rg = r0; rg < r1; rg += G) {
+        auto in = [&](int k, int b) {
+            const int g = fast_div(b, cs.mC), c = b - g * C, r = rg + g;
+            return (c < cols && r < r1)
+                       ? cmulc(vh[k * pitch1 + c], __ldg(op.spec + ((size_t)(r - op.spec_r0) * N + k) * ncol + c0 + c))
+                       : czero<Cx>();
+        };
+        auto out = [&](int n, int b, Cx x) {
+            const int g = fast_div(b, cs.mC), c = b - g * C, r = rg + g;
+            if (n < ny && c < cols && r < r1) op.Z[((size_t)r * ny + n) * ncol + c0 + c] = x;
+        };
+        fft_run<R, true, false, true>(op.py, C * G, cs.mB, cs.pitch, bufA, bufB, tw, N, ny, in, out);
+        if (!(op.py.nst & 1)) { Cx *t = bufA; bufA = bufB; bufB = t; }  // the last stage may still be reading bufA
+    }
+}
 
 }  // namespace gj

@@ -1,0 +1,75 @@
+// Definitions of the general kernels' launches (general_launch.cuh).
+#pragma once
+#include "general_launch.cuh"
+
+namespace gj {
+
+template <typename R, class Pro> void gen_row_fwd_attr() { allow_max_smem(k_row_fwd<R, Pro>); }
+template <typename R, class Epi> void gen_row_inv_attr() { allow_max_smem(k_row_inv<R, Epi>); }
+template <typename R, class Epi> void gen_row_resid_attr() { allow_max_smem(k_row_resid<R, Epi>); }
+template <typename R> void gen_col_attr() {
+    allow_max_smem(k_col_fwd<R>);
+    allow_max_smem(k_col_adj<R>);
+}
+
+template <typename R, class Pro>
+void gen_row_fwd(const gj_op *o, const OpView<R> &v, const PairMap &pm, int n_in, cpx<R> *out0, cpx<R> *out1,
+                        const Pro &pro, const int *done, cudaStream_t st, int nf) {
+    const int np = pm.joint ? pm.nlines : (pm.nlines + 1) / 2;
+    const RowShape rs = row_shape(o, np * nf, sizeof(cpx<R>));
+    k_row_fwd<R, Pro><<<dim3((np + rs.P - 1) / rs.P, nf), gen_threads(o->px.mmax, rs.P),
+                        row_smem(o->Nx, rs.pitch, sizeof(cpx<R>)), st>>>(v, pm, n_in, rs, out0, out1, pro, done);
+}
+template <typename R, class Epi>
+void gen_row_inv(const gj_op *o, const OpView<R> &v, const PairMap &pm, int n_out, const cpx<R> *in0,
+                        const cpx<R> *in1, const Epi &epi, const int *done, cudaStream_t st, int nf) {
+    const int np = pm.joint ? pm.nlines : (pm.nlines + 1) / 2;
+    const RowShape rs = row_shape(o, np * nf, sizeof(cpx<R>));
+    k_row_inv<R, Epi><<<dim3((np + rs.P - 1) / rs.P, nf), gen_threads(o->px.mmax, rs.P),
+                        row_smem(o->Nx, rs.pitch, sizeof(cpx<R>)), st>>>(v, pm, n_out, rs, in0, in1, epi, done);
+}
+template <typename R, class Epi>
+void gen_row_resid(const gj_op *o, const OpView<R> &v, const PairMap &pm, int n_out, const cpx<R> *in0,
+                          const cpx<R> *in1, cpx<R> *out0, cpx<R> *out1, const Epi &epi, const int *done,
+                          cudaStream_t st) {
+    const RowShape rs = row_shape(o, pm.nlines, sizeof(cpx<R>));
+    k_row_resid<R, Epi><<<(pm.nlines + rs.P - 1) / rs.P, gen_threads(o->px.mmax, rs.P),
+                          row_smem(o->Nx, rs.pitch, sizeof(cpx<R>)), st>>>(v, pm, n_out, rs, in0, in1, out0, out1, epi,
+                                                                          done);
+}
+template <typename R>
+void gen_col_fwd(const gj_op *o, const OpView<R> &v0, const OpView<R> &v1, int nf, int layers, const int *done,
+                        cudaStream_t st) {
+    const ColShape s = col_shape(o, nf, layers, sizeof(cpx<R>), false);
+    k_col_fwd<R><<<dim3((o->ncol + s.C - 1) / s.C, (layers + s.L - 1) / s.L, nf), gen_threads(o->py.mmax, s.C * s.G),
+                   col_smem(o->Ny, s.pitch, s.pitch, sizeof(cpx<R>)), st>>>(v0, v1, s, done);
+}
+template <typename R>
+void gen_col_adj(const gj_op *o, const OpView<R> &v0, const OpView<R> &v1, int nf, int layers, const int *done,
+                        cudaStream_t st) {
+    const ColShape s = col_shape(o, nf, layers, sizeof(cpx<R>), true);
+    k_col_adj<R><<<dim3((o->ncol + s.C - 1) / s.C, (layers + s.L - 1) / s.L, nf), gen_threads(o->py.mmax, s.C * s.G),
+                   col_smem(o->Ny, s.pitch, s.pitch1, sizeof(cpx<R>)), st>>>(v0, v1, s, done);
+}
+
+}  // namespace gj
+
+// Explicit instantiations.
+#define GJ_ROW_FWD(R, PRO)                                                                                        \
+    template void gen_row_fwd_attr<R, PRO>();                                                                     \
+    template void gen_row_fwd<R, PRO>(const gj_op *, const OpView<R> &, const PairMap &, int, cpx<R> *, cpx<R> *, \
+                                      const PRO &, const int *, cudaStream_t, int);
+#define GJ_ROW_INV(R, EPI)                                                                                    \
+    template void gen_row_inv_attr<R, EPI>();                                                                 \
+    template void gen_row_inv<R, EPI>(const gj_op *, const OpView<R> &, const PairMap &, int, const cpx<R> *, \
+                                      const cpx<R> *, const EPI &, const int *, cudaStream_t, int);
+#define GJ_ROW_RESID(R, EPI)                                                                                    \
+    template void gen_row_resid_attr<R, EPI>();                                                                 \
+    template void gen_row_resid<R, EPI>(const gj_op *, const OpView<R> &, const PairMap &, int, const cpx<R> *, \
+                                        const cpx<R> *, cpx<R> *, cpx<R> *, const EPI &, const int *, cudaStream_t);
+#define GJ_COLS(R)                                                                                               \
+    template void gen_col_attr<R>();                                                                             \
+    template void gen_col_fwd<R>(const gj_op *, const OpView<R> &, const OpView<R> &, int, int, const int *,     \
+                                 cudaStream_t);                                                                  \
+    template void gen_col_adj<R>(const gj_op *, const OpView<R> &, const OpView<R> &, int, int, const int *,     \
+                                 cudaStream_t);

@@ -28,13 +28,15 @@ struct gj_op {
     size_t spec_bytes = 0, ws_bytes = 0;
     // launch shapes
     int P_row = 8, C_col = 8, L_grp = 4;
+    bool rows_tuned = false, cols_tuned = false, layers_tuned = false;  // set by gj_op_tune: use them as they are
     int radix_order = 0;
+    int gen_slots = 1;  // general kernels: layer groups that Y has room for
     // fast path (FP32, N_x = 512 and N_y = 512 or 256, at most N/2 prisms and stations
     // per direction): transposed spectra and intermediates, layer-sum partials and counters
     bool fast = false;
     bool real_spec = false;  // fast path: the table is even in both offsets, its spectrum is real
     void *P = nullptr;     // [ncol][slots][Ny] complex
-    int *cnt = nullptr;    // [ncol] arrival counters
+    int *cnt = nullptr;    // [ncol] arrival counters (every path)
     int *err = nullptr;    // device error word (bounded waits)
     void *twtab = nullptr; // the column kernels' twiddle table (FP32, TabTw or Tab1024 layout)
     // N_y = 1024 (FP32, at most 512 prisms and stations per column): warp-FFT column
@@ -57,10 +59,6 @@ bool plan_size(int N, FftPlanDev &plan, int order = 0);  // false if N has an un
 int  autotune_size(int minN);               // smallest 7-smooth N >= minN
 size_t elem_bytes(gj_precision p);           // bytes of one real value
 void make_twiddles(int N, std::vector<double> &re, std::vector<double> &im);
-
-// smem sizing helpers
-int pick_row_pairs(int Nx, size_t csize);
-int pick_col_tile(int Ny, size_t csize, int nbuf);
 
 template <typename R> struct OpView;
 template <typename R> OpView<R> view_of(const gj_op *op);

@@ -1,50 +1,60 @@
 // G m and G^T r of one field (Sec. 2.7.1): the C-ABI entry points and the launch
 // sequences shared with the solver.
 #include "fast_launch.cuh"
-#include "view.cuh"
+#include "general_launch.cuh"
 
 namespace gj {
 
+// General kernels, one field or both (b: the second operator, or NULL).
 template <typename R>
-static void launch_forward(const gj_op *o, const R *m, R *d, cudaStream_t st) {
-    OpView<R> v = view_of<R>(o);
-    const size_t cs = sizeof(cpx<R>);
-    // rows: m -> Z (pairs of consecutive (layer, row) lines)
-    PairMap pm{o->nz * o->ny, 0};
-    const int P = o->P_row;
-    const size_t rsm = row_smem(o->Nx, P, cs);
-    allow_max_smem(k_row_fwd<R, LoadPlain<R>>);
-    const int npr = (pm.nlines + 1) / 2;
-    k_row_fwd<R, LoadPlain<R>><<<(npr + P - 1) / P, 256, rsm, st>>>(v, pm, o->nx, P, v.Z, v.Z,
-                                                                    LoadPlain<R>{m, m, o->nx}, nullptr);
-    // columns with the layer spectra, summed over layers
-    cudaMemsetAsync(v.Y, 0, (size_t)o->Ny * o->ncol * cs, st);
-    const int C = o->C_col;
-    const int nt = (o->ncol + C - 1) / C;
-    const size_t msm = col_smem(o->Ny, C, 3, cs);
-    allow_max_smem(k_col_fwd_mac<R>);
-    if (o->recompute) {
+static void set_general_attributes() {
+    gen_row_fwd_attr<R, LoadPlain2<R>>();
+    gen_row_inv_attr<R, StorePlain2<R>>();
+    gen_col_attr<R>();
+}
+
+template <typename R>
+static void general_forward(const gj_op *a, const gj_op *b, const R *m0, const R *m1, R *d0, R *d1, cudaStream_t st) {
+    set_general_attributes<R>();
+    const int nf = b ? 2 : 1;
+    const OpView<R> v0 = view_of<R>(a), v1 = view_of<R>(b ? b : a);
+    // rows: pairs of consecutive (layer, row) lines of one field
+    gen_row_fwd<R>(a, v0, PairMap{a->nz * a->ny, 0, 0}, a->nx, v0.Z, v1.Z, LoadPlain2<R>{{m0, m1}, a->nx}, nullptr, st,
+                   nf);
+    if (a->recompute) {
         // one layer at a time: rebuild its spectrum, then add its column products
-        for (int r = 0; r < o->nz; ++r) {
-            recompute_layer(o, r, st);
-            OpView<R> vr = v;
+        for (int r = 0; r < a->nz; ++r) {
+            recompute_layer(a, r, st);
+            OpView<R> vr = v0;
             vr.rbase = r;
             vr.spec_r0 = r;
-            k_col_fwd_mac<R><<<dim3(nt, 1, 1), 256, msm, st>>>(vr, vr, C, 1, nullptr);
+            gen_col_fwd<R>(a, vr, vr, 1, 1, nullptr, st);
         }
     } else {
-        k_col_fwd_mac<R><<<dim3(nt, (o->nz + o->L_grp - 1) / o->L_grp, 1), 256, msm, st>>>(v, v, C, o->L_grp, nullptr);
+        gen_col_fwd<R>(a, v0, v1, nf, a->nz, nullptr, st);
     }
-    // inverse columns
-    const size_t ism = col_smem(o->Ny, C, 2, cs);
-    allow_max_smem(k_col_inv<R>);
-    k_col_inv<R><<<dim3(nt, 1), 256, ism, st>>>(v, v, C, nullptr);
-    // inverse rows, cropped to the stations
-    PairMap ps{o->sy, 0};
-    const int nps = (ps.nlines + 1) / 2;
-    allow_max_smem(k_row_inv<R, StorePlain<R>>);
-    k_row_inv<R, StorePlain<R>><<<(nps + P - 1) / P, 256, rsm, st>>>(v, ps, o->sx, P, v.W, v.W,
-                                                                     StorePlain<R>{d, d, o->sx}, nullptr);
+    gen_row_inv<R>(a, v0, PairMap{a->sy, 0, 0}, a->sx, v0.W, v1.W, StorePlain2<R>{{d0, d1}, a->sx}, nullptr, st, nf);
+}
+
+template <typename R>
+static void general_adjoint(const gj_op *a, const gj_op *b, const R *r0, const R *r1, R *g0, R *g1, cudaStream_t st) {
+    set_general_attributes<R>();
+    const int nf = b ? 2 : 1;
+    const OpView<R> v0 = view_of<R>(a), v1 = view_of<R>(b ? b : a);
+    gen_row_fwd<R>(a, v0, PairMap{a->sy, 0, 0}, a->sx, v0.W, v1.W, LoadPlain2<R>{{r0, r1}, a->sx}, nullptr, st, nf);
+    if (a->recompute) {
+        for (int r = 0; r < a->nz; ++r) {
+            recompute_layer(a, r, st);
+            OpView<R> vr = v0;
+            vr.rbase = r;
+            vr.spec_r0 = r;
+            gen_col_adj<R>(a, vr, vr, 1, 1, nullptr, st);
+        }
+    } else {
+        gen_col_adj<R>(a, v0, v1, nf, a->nz, nullptr, st);
+    }
+    gen_row_inv<R>(a, v0, PairMap{a->nz * a->ny, 0, 0}, a->nx, v0.Z, v1.Z, StorePlain2<R>{{g0, g1}, a->nx}, nullptr, st,
+                   nf);
 }
 
 // N_y = 1024 column kernels: the general row kernels write and read the transposed
@@ -53,11 +63,8 @@ static void launch_forward(const gj_op *o, const R *m, R *d, cudaStream_t st) {
 static void fast1024_forward(const gj_op *a, const gj_op *b, const float *m0, const float *m1, float *d0, float *d1,
                              cudaStream_t st) {
     using R = float;
-    const size_t cs = sizeof(cpx<R>);
-    const int P = a->P_row;
-    const size_t rsm = row_smem(a->Nx, P, cs);
-    allow_max_smem(k_row_fwd<R, LoadPlain<R>>);
-    allow_max_smem(k_row_inv<R, StorePlain<R>>);
+    gen_row_fwd_attr<R, LoadPlain2<R>>();
+    gen_row_inv_attr<R, StorePlain2<R>>();
     f1024::set_col_attr<R>();
     const bool rows1024 = a->Nx == 1024;  // warp-FFT rows as well
     if (rows1024) {
@@ -84,35 +91,30 @@ static void fast1024_forward(const gj_op *a, const gj_op *b, const float *m0, co
         const gj_op *o = ops[i];
         OpView<R> v = view_of<R>(o);
         PairMap pm{o->nz * o->ny, 0, o->ny};
-        const int npr = (pm.nlines + 1) / 2;
         const LoadPlain<R> lp{ms[i], ms[i], o->nx};
         if (rows1024)
             f1024::row_fwd<R>(v, pm, o->nx, v.Z, v.Z, o->twtab, lp, nullptr, st);
         else
-            k_row_fwd<R, LoadPlain<R>><<<(npr + P - 1) / P, 256, rsm, st>>>(v, pm, o->nx, P, v.Z, v.Z, lp, nullptr);
+            gen_row_fwd<R>(o, v, pm, o->nx, v.Z, v.Z, LoadPlain2<R>{{ms[i], ms[i]}, o->nx}, nullptr, st);
     }
     f1024::col_fwd<R>(f512::make_view2<R>(a, b), a->col_grid, nullptr, st);
     for (int i = 0; i < nf; ++i) {
         const gj_op *o = ops[i];
         OpView<R> v = view_of<R>(o);
         PairMap ps{o->sy, 0, o->sy};
-        const int nps = (ps.nlines + 1) / 2;
         const StorePlain<R> sp{ds[i], ds[i], o->sx};
         if (rows1024)
             f1024::row_inv<R>(v, ps, o->sx, v.W, v.W, o->twtab, sp, nullptr, st);
         else
-            k_row_inv<R, StorePlain<R>><<<(nps + P - 1) / P, 256, rsm, st>>>(v, ps, o->sx, P, v.W, v.W, sp, nullptr);
+            gen_row_inv<R>(o, v, ps, o->sx, v.W, v.W, StorePlain2<R>{{ds[i], ds[i]}, o->sx}, nullptr, st);
     }
 }
 
 static void fast1024_adjoint(const gj_op *a, const gj_op *b, const float *r0, const float *r1, float *g0, float *g1,
                              cudaStream_t st) {
     using R = float;
-    const size_t cs = sizeof(cpx<R>);
-    const int P = a->P_row;
-    const size_t rsm = row_smem(a->Nx, P, cs);
-    allow_max_smem(k_row_fwd<R, LoadPlain<R>>);
-    allow_max_smem(k_row_inv<R, StorePlain<R>>);
+    gen_row_fwd_attr<R, LoadPlain2<R>>();
+    gen_row_inv_attr<R, StorePlain2<R>>();
     f1024::set_col_attr<R>();
     const bool rows1024 = a->Nx == 1024;
     if (rows1024) {
@@ -139,61 +141,23 @@ static void fast1024_adjoint(const gj_op *a, const gj_op *b, const float *r0, co
         const gj_op *o = ops[i];
         OpView<R> v = view_of<R>(o);
         PairMap ps{o->sy, 0, o->sy};
-        const int nps = (ps.nlines + 1) / 2;
         const LoadPlain<R> lp{rs[i], rs[i], o->sx};
         if (rows1024)
             f1024::row_fwd<R>(v, ps, o->sx, v.V, v.V, o->twtab, lp, nullptr, st);
         else
-            k_row_fwd<R, LoadPlain<R>><<<(nps + P - 1) / P, 256, rsm, st>>>(v, ps, o->sx, P, v.V, v.V, lp, nullptr);
+            gen_row_fwd<R>(o, v, ps, o->sx, v.V, v.V, LoadPlain2<R>{{rs[i], rs[i]}, o->sx}, nullptr, st);
     }
     f1024::col_adj<R>(f512::make_view2<R>(a, b), a->col_grid, nullptr, st);
     for (int i = 0; i < nf; ++i) {
         const gj_op *o = ops[i];
         OpView<R> v = view_of<R>(o);
         PairMap pm{o->nz * o->ny, 0, o->ny};
-        const int npr = (pm.nlines + 1) / 2;
         const StorePlain<R> sp{gs[i], gs[i], o->nx};
         if (rows1024)
             f1024::row_inv<R>(v, pm, o->nx, v.Z, v.Z, o->twtab, sp, nullptr, st);
         else
-            k_row_inv<R, StorePlain<R>><<<(npr + P - 1) / P, 256, rsm, st>>>(v, pm, o->nx, P, v.Z, v.Z, sp, nullptr);
+            gen_row_inv<R>(o, v, pm, o->nx, v.Z, v.Z, StorePlain2<R>{{gs[i], gs[i]}, o->nx}, nullptr, st);
     }
-}
-
-template <typename R>
-static void launch_adjoint(const gj_op *o, const R *r, R *g, cudaStream_t st) {
-    OpView<R> v = view_of<R>(o);
-    const size_t cs = sizeof(cpx<R>);
-    const int P = o->P_row;
-    const size_t rsm = row_smem(o->Nx, P, cs);
-    // rows of the residual -> W
-    PairMap ps{o->sy, 0};
-    const int nps = (ps.nlines + 1) / 2;
-    allow_max_smem(k_row_fwd<R, LoadPlain<R>>);
-    k_row_fwd<R, LoadPlain<R>><<<(nps + P - 1) / P, 256, rsm, st>>>(v, ps, o->sx, P, v.W, v.W,
-                                                                    LoadPlain<R>{r, r, o->sx}, nullptr);
-    const int C = o->C_col;
-    const int nt = (o->ncol + C - 1) / C;
-    const size_t sm2 = col_smem(o->Ny, C, 2, cs);
-    allow_max_smem(k_col_fft<R>);
-    k_col_fft<R><<<dim3(nt, 1), 256, sm2, st>>>(v, v, C, nullptr);
-    allow_max_smem(k_col_adj<R>);
-    if (o->recompute) {
-        for (int r = 0; r < o->nz; ++r) {
-            recompute_layer(o, r, st);
-            OpView<R> vr = v;
-            vr.rbase = r;
-            vr.spec_r0 = r;
-            k_col_adj<R><<<dim3(nt, 1, 1), 256, sm2, st>>>(vr, vr, C, nullptr);
-        }
-    } else {
-        k_col_adj<R><<<dim3(nt, o->nz, 1), 256, sm2, st>>>(v, v, C, nullptr);
-    }
-    PairMap pm{o->nz * o->ny, 0};
-    const int npr = (pm.nlines + 1) / 2;
-    allow_max_smem(k_row_inv<R, StorePlain<R>>);
-    k_row_inv<R, StorePlain<R>><<<(npr + P - 1) / P, 256, rsm, st>>>(v, pm, o->nx, P, v.Z, v.Z,
-                                                                     StorePlain<R>{g, g, o->nx}, nullptr);
 }
 
 // 512 x 512 fast path: rows -> persistent layer-summed columns -> inverse rows
@@ -254,19 +218,23 @@ static void fast_adjoint_pair(const gj_op *a, const gj_op *b, const float *r0, c
     row_inv_t<float, true>(V, a->col_grid, a->nz, a->ny, a->nx, 0, StorePlain2<float>{{g0, g1}, a->nx}, nullptr, st);
 }
 
-// Two operators serve one joint launch when both are on the fast path with the same
-// grid (their workspaces stay separate; the launch uses the first one's error word).
+// Two operators serve one joint launch per pass when both are served by the same kernels
+// with the same grid, padded size and launch shapes (their workspaces stay separate; the
+// fast paths' launches use the first one's error word).  Operators that rebuild their
+// spectra run one after the other.
 static bool pair_eligible(const gj_op *a, const gj_op *b) {
-    return a != b && ((a->fast && b->fast) || (a->fast1024 && b->fast1024)) && a->sx == b->sx && a->sy == b->sy &&
-           a->nx == b->nx && a->ny == b->ny && a->nz == b->nz && a->Ny == b->Ny && a->Nx == b->Nx &&
-           a->P_row == b->P_row && a->col_grid == b->col_grid;
+    return a != b && a->fast == b->fast && a->fast1024 == b->fast1024 && a->prec == b->prec && !a->recompute &&
+           !b->recompute && a->sx == b->sx && a->sy == b->sy && a->nx == b->nx && a->ny == b->ny && a->nz == b->nz &&
+           a->Ny == b->Ny && a->Nx == b->Nx && a->P_row == b->P_row && a->C_col == b->C_col && a->L_grp == b->L_grp &&
+           a->radix_order == b->radix_order && a->rows_tuned == b->rows_tuned && a->cols_tuned == b->cols_tuned &&
+           a->layers_tuned == b->layers_tuned && a->col_grid == b->col_grid;
 }
 
 gj_status forward_enqueue(const gj_op *o, const void *m, void *d, cudaStream_t st) {
     if (o->fast) fast_forward(o, (const float *)m, (float *)d, st);
     else if (o->fast1024) fast1024_forward(o, nullptr, (const float *)m, nullptr, (float *)d, nullptr, st);
-    else if (o->prec == GJ_FP64) launch_forward<double>(o, (const double *)m, (double *)d, st);
-    else launch_forward<float>(o, (const float *)m, (float *)d, st);
+    else if (o->prec == GJ_FP64) general_forward<double>(o, nullptr, (const double *)m, nullptr, (double *)d, nullptr, st);
+    else general_forward<float>(o, nullptr, (const float *)m, nullptr, (float *)d, nullptr, st);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? GJ_OK : cuda_fail(e, "g_forward launch");
 }
@@ -274,8 +242,8 @@ gj_status forward_enqueue(const gj_op *o, const void *m, void *d, cudaStream_t s
 gj_status adjoint_enqueue(const gj_op *o, const void *r, void *g, cudaStream_t st) {
     if (o->fast) fast_adjoint(o, (const float *)r, (float *)g, st);
     else if (o->fast1024) fast1024_adjoint(o, nullptr, (const float *)r, nullptr, (float *)g, nullptr, st);
-    else if (o->prec == GJ_FP64) launch_adjoint<double>(o, (const double *)r, (double *)g, st);
-    else launch_adjoint<float>(o, (const float *)r, (float *)g, st);
+    else if (o->prec == GJ_FP64) general_adjoint<double>(o, nullptr, (const double *)r, nullptr, (double *)g, nullptr, st);
+    else general_adjoint<float>(o, nullptr, (const float *)r, nullptr, (float *)g, nullptr, st);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? GJ_OK : cuda_fail(e, "g_adjoint launch");
 }
@@ -353,8 +321,14 @@ extern "C" gj_status gj_g_forward_pair(const gj_op *const ops[2], const void *co
     if (gj::pair_eligible(ops[0], ops[1])) {
         if (ops[0]->fast1024)
             gj::fast1024_forward(ops[0], ops[1], (const float *)m[0], (const float *)m[1], (float *)d[0], (float *)d[1], st);
-        else
+        else if (ops[0]->fast)
             gj::fast_forward_pair(ops[0], ops[1], (const float *)m[0], (const float *)m[1], (float *)d[0], (float *)d[1], st);
+        else if (ops[0]->prec == GJ_FP64)
+            gj::general_forward<double>(ops[0], ops[1], (const double *)m[0], (const double *)m[1], (double *)d[0],
+                                    (double *)d[1], st);
+        else
+            gj::general_forward<float>(ops[0], ops[1], (const float *)m[0], (const float *)m[1], (float *)d[0],
+                                   (float *)d[1], st);
         cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? GJ_OK : gj::cuda_fail(e, "gj_g_forward_pair launch");
     }
@@ -372,8 +346,14 @@ extern "C" gj_status gj_g_adjoint_pair(const gj_op *const ops[2], const void *co
     if (gj::pair_eligible(ops[0], ops[1])) {
         if (ops[0]->fast1024)
             gj::fast1024_adjoint(ops[0], ops[1], (const float *)r[0], (const float *)r[1], (float *)g[0], (float *)g[1], st);
-        else
+        else if (ops[0]->fast)
             gj::fast_adjoint_pair(ops[0], ops[1], (const float *)r[0], (const float *)r[1], (float *)g[0], (float *)g[1], st);
+        else if (ops[0]->prec == GJ_FP64)
+            gj::general_adjoint<double>(ops[0], ops[1], (const double *)r[0], (const double *)r[1], (double *)g[0],
+                                    (double *)g[1], st);
+        else
+            gj::general_adjoint<float>(ops[0], ops[1], (const float *)r[0], (const float *)r[1], (float *)g[0],
+                                   (float *)g[1], st);
         cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? GJ_OK : gj::cuda_fail(e, "gj_g_adjoint_pair launch");
     }

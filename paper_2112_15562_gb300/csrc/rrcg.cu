@@ -23,531 +23,10 @@
 #include <vector>
 
 #include "fast_launch.cuh"
-#include "view.cuh"
+#include "general_launch.cuh"
+#include "rrcg_functors.cuh"
 
 namespace gj {
-
-struct SolverDev {
-    int k, done, status, pending_update;
-    int sat[2];
-    int kmax, stop_on_chi2, per_field;
-    int anchor;           // GJ_ANCHOR_*
-    int gspace;           // GJ_GRAMIAN_*
-    int p[2];
-    double eps2;
-    double alpha[2], q[2], alpha_min[2], lam[2], lo[2], hi[2];
-    double chi2_target[2];
-    double s[2], beta[2];
-    double ll_prev[2];
-    double phi_last[2], SG_last;
-    // accumulators, zeroed after use
-    double G[3];          // (m1,m1), (m2,m2), (m1,m2) of the current models
-    double phi[2];        // ||r~||^2
-    double ll[2];         // ||l||^2
-    double pl[2], pp[2];  // (p,l), ||p||^2
-    double qq[2];         // ||A~ p||^2
-    gj_rrcg_hist *hist;
-};
-
-template <typename R>
-struct FieldVecs {
-    R *m[2];
-    R *p[2];
-    R *l[2];
-    R *v[2];               // W_d r~ (s values)
-    const R *wd[2];        // 1 / sigma
-    const R *dobs[2];
-    const R *mapr[2];      // may be null
-    const R *wdep[2];      // nz values
-    const R *iwdep[2];     // 1 / wdep, nz values
-    const R *whard[2];     // may be null
-    R *mtp[2];             // W_{k-1} m_{k-1} (previous-model anchor only), else null
-};
-
-template <typename R> __device__ __forceinline__ R rsqrt_t(R x);
-template <> __device__ __forceinline__ float rsqrt_t<float>(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return rsqrt(x); }
-
-// Diagonal of W = W_depth W_hard W_L at cell c of layer r (Eq. W, Eq. WL).
-template <typename R>
-__device__ __forceinline__ R weight(const FieldVecs<R> &F, int i, int p, R eps2, int r, size_t c, R m) {
-    R w = F.wdep[i][r];
-    if (F.whard[i]) w *= F.whard[i][c];
-    if (p == 1) {
-        const R d = m - (F.mapr[i] ? F.mapr[i][c] : R(0));
-        w *= rsqrt_t<R>(sqrt(d * d + eps2));
-    }
-    return w;
-}
-
-// The L1 reweighting factor of Eq. WL and its reciprocal for p = 1 (1 for p = 2):
-// ((m - m_apr)^2 + eps^2)^(-1/4) and ((m - m_apr)^2 + eps^2)^(1/4).
-template <typename R>
-__device__ __forceinline__ void lp_factors(int p, R d, R eps2, R &wl, R &inv_wl) {
-    if (p == 1) {
-        const R q = sqrt(d * d + eps2);
-        wl = rsqrt_t<R>(q);
-        inv_wl = sqrt(q);
-    } else {
-        wl = R(1);
-        inv_wl = R(1);
-    }
-}
-// One hardware reciprocal square root (relative error about 1e-7; arguments below
-// FLT_MIN flush to zero).  Its arguments here are d^2 + eps^2 and (d^2 + eps^2)^-1/2.
-__device__ __forceinline__ float rsqrt_approx(float x) {
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-// FP32: two reciprocal square roots, u = q^-1/2, q^1/4 = u^-1/2, q^-1/4 = u q^1/4
-template <>
-__device__ __forceinline__ void lp_factors<float>(int p, float d, float eps2, float &wl, float &inv_wl) {
-    if (p == 1) {
-        const float u = rsqrt_approx(d * d + eps2);
-        inv_wl = rsqrt_approx(u);
-        wl = u * inv_wl;
-    } else {
-        wl = 1.0f;
-        inv_wl = 1.0f;
-    }
-}
-
-// Forward of m with the pending model update (RRCG:7-8 and the bounds) and the
-// Gramian sums of the updated models.
-template <typename R, bool OPT = true>
-struct ProModel {
-    FieldVecs<R> F;
-    SolverDev *S;
-    int nx, ny;
-    // per-thread
-    int upd, pw[2], gsp;
-    R s[2], lo[2], hi[2], eps2;
-    R acc[3];
-    __device__ void init() {
-        upd = S->pending_update;
-        gsp = S->gspace;
-        eps2 = (R)S->eps2;
-        for (int i = 0; i < 2; ++i) {
-            s[i] = (R)S->s[i]; lo[i] = (R)S->lo[i]; hi[i] = (R)S->hi[i]; pw[i] = S->p[i];
-        }
-        acc[0] = acc[1] = acc[2] = 0;
-    }
-    __device__ __forceinline__ void fetch(int la, int lb, bool, int j, R &a, R &b) {
-        const size_t c = (size_t)la * nx + j;
-        const int r = la / ny;
-        R mv[2], gv[2];
-        for (int i = 0; i < 2; ++i) {
-            R mi = F.m[i][c];
-            if (upd) {
-                const R w = weight(F, i, pw[i], eps2, r, c, mi);
-                if (OPT && F.mtp[i]) F.mtp[i][c] = w * mi;  // W_k m_k, the next anchor
-                mi = mi - s[i] * F.p[i][c] / w;
-                mi = fmin(fmax(mi, lo[i]), hi[i]);
-                F.m[i][c] = mi;
-            }
-            mv[i] = mi;
-            gv[i] = gsp ? weight(F, i, pw[i], eps2, r, c, mi) * mi : mi;  // Gramian space
-        }
-        acc[0] += gv[0] * gv[0];
-        acc[1] += gv[1] * gv[1];
-        acc[2] += gv[0] * gv[1];
-        a = mv[0];
-        b = mv[1];
-    }
-    // rows a line needs in every launch (m, p), staged ahead by the persistent row
-    // pass as pre[a][field][j]; the optional rows are read in place
-    static constexpr int NPRE = 2;
-    __device__ const R *pre_src(int a, int i) const { return a == 0 ? F.m[i] : (upd ? F.p[i] : nullptr); }
-    // batched form: every load of the K elements is issued before any store
-    template <int K, bool PRE = false>
-    __device__ __forceinline__ void fetch_batch(int la, int, bool, int j0, int stride, int n, R (&a)[K], R (&b)[K],
-                                                const R *pre = nullptr) {
-        const size_t c0 = (size_t)la * nx;
-        const int r = la / ny;
-        R mv[2][K], pv[2][K], wh[2][K], ma[2][K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            const bool ok = j < n;
-            const size_t c = c0 + j;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                mv[i][k] = ok ? (PRE ? pre[i * f512::H + j] : F.m[i][c]) : R(0);
-                pv[i][k] = (ok && upd) ? (PRE ? pre[(2 + i) * f512::H + j] : F.p[i][c]) : R(0);
-                wh[i][k] = (ok && OPT && F.whard[i]) ? F.whard[i][c] : R(1);
-                ma[i][k] = (ok && OPT && F.mapr[i]) ? F.mapr[i][c] : R(0);
-            }
-        }
-        R wd[2], iwd[2];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) { wd[i] = F.wdep[i][r]; iwd[i] = F.iwdep[i][r]; }
-        if (upd) {
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                const int j = j0 + k * stride;
-                if (j >= n) continue;
-                const size_t c = c0 + j;
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    R wl, iwl;
-                    lp_factors<R>(pw[i], mv[i][k] - ma[i][k], eps2, wl, iwl);
-                    R inv_w = iwl * iwd[i];
-                    if (OPT && F.whard[i]) inv_w /= wh[i][k];
-                    if (OPT && F.mtp[i]) F.mtp[i][c] = wd[i] * wh[i][k] * wl * mv[i][k];  // W_k m_k, the next anchor
-                    R mi = mv[i][k] - s[i] * pv[i][k] * inv_w;
-                    mi = fmin(fmax(mi, lo[i]), hi[i]);
-                    F.m[i][c] = mi;
-                    mv[i][k] = mi;
-                }
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            R gv[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                gv[i] = mv[i][k];
-                if (gsp) {  // the Gramian of the weighted models W(m) m
-                    R wl, iwl;
-                    lp_factors<R>(pw[i], mv[i][k] - ma[i][k], eps2, wl, iwl);
-                    gv[i] = wd[i] * wh[i][k] * wl * mv[i][k];
-                }
-            }
-            acc[0] += gv[0] * gv[0];
-            acc[1] += gv[1] * gv[1];
-            acc[2] += gv[0] * gv[1];
-            a[k] = mv[0][k];
-            b[k] = mv[1][k];
-        }
-    }
-    __device__ void flush(double *red) { block_accumulate<3>(acc, S->G, red); }
-};
-
-// Residual epilogue: r~ = W_d (A m - d), v = W_d r~, Phi partials (RRCG:1).
-template <typename R>
-struct EpiResidual {
-    FieldVecs<R> F;
-    SolverDev *S;
-    int sx;
-    R acc[2];
-    __device__ void init() { acc[0] = acc[1] = 0; }
-    __device__ __forceinline__ void store(int la, int, bool, int j, R a, R b) {
-        const size_t t = (size_t)la * sx + j;
-        const R y[2] = {a, b};
-        for (int i = 0; i < 2; ++i) {
-            const R w = F.wd[i][t];
-            const R rt = w * (y[i] - F.dobs[i][t]);
-            acc[i] += rt * rt;
-            F.v[i][t] = w * rt;
-        }
-    }
-    // fused form, in two steps so that the loads can be issued before the transform:
-    // resid_load fetches W_d and d; resid_apply takes y in a, b and returns v = W_d r~
-    template <int K>
-    __device__ __forceinline__ void resid_load(int la, int j0, int stride, int n, R (&w)[2][K], R (&d)[2][K]) const {
-        const size_t t0 = (size_t)la * sx;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            const bool ok = j < n;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                w[i][k] = ok ? F.wd[i][t0 + j] : R(0);
-                d[i][k] = ok ? F.dobs[i][t0 + j] : R(0);
-            }
-        }
-    }
-    template <int K>
-    __device__ __forceinline__ void resid_apply(int j0, int stride, int n, const R (&w)[2][K], const R (&d)[2][K],
-                                                R (&a)[K], R (&b)[K]) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            const bool ok = j < n;
-            const R r0 = w[0][k] * (a[k] - d[0][k]);
-            const R r1 = w[1][k] * (b[k] - d[1][k]);
-            if (ok) {
-                acc[0] += r0 * r0;
-                acc[1] += r1 * r1;
-            }
-            a[k] = ok ? w[0][k] * r0 : R(0);
-            b[k] = ok ? w[1][k] * r1 : R(0);
-        }
-    }
-    template <int K>
-    __device__ __forceinline__ void store_batch(int la, int, bool, int j0, int stride, int n, const R (&a)[K],
-                                                const R (&b)[K]) {
-        const size_t t0 = (size_t)la * sx;
-        R w[2][K], d[2][K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            const bool ok = j < n;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                w[i][k] = ok ? F.wd[i][t0 + j] : R(0);
-                d[i][k] = ok ? F.dobs[i][t0 + j] : R(0);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            if (j >= n) continue;
-            const R y[2] = {a[k], b[k]};
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const R rt = w[i][k] * (y[i] - d[i][k]);
-                acc[i] += rt * rt;
-                F.v[i][t0 + j] = w[i][k] * rt;
-            }
-        }
-    }
-    __device__ void flush(double *red) { block_accumulate<2>(acc, S->phi, red); }
-};
-
-template <typename R>
-struct LoadPair {
-    const R *x0;
-    const R *x1;
-    int pitch;
-    __device__ void init() {}
-    __device__ __forceinline__ void fetch(int la, int lb, bool, int j, R &a, R &b) const {
-        a = x0[(size_t)la * pitch + j];
-        b = x1[(size_t)lb * pitch + j];
-    }
-    template <int K>
-    __device__ __forceinline__ void fetch_batch(int la, int lb, bool, int j0, int stride, int n, R (&a)[K],
-                                                R (&b)[K]) const {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            a[k] = j < n ? x0[(size_t)la * pitch + j] : R(0);
-            b[k] = j < n ? x1[(size_t)lb * pitch + j] : R(0);
-        }
-    }
-    __device__ void flush(double *) {}
-};
-
-// Gradient epilogue (RRCG:2-4): l = W^-1 A^T v + alpha (W m - W m_apr) + lambda l_G.
-template <typename R, bool OPT = true>
-struct EpiGradient {
-    FieldVecs<R> F;
-    SolverDev *S;
-    int nx, ny;
-    R alpha[2], lam[2], eps2, g11, g22, g12;
-    int pw[2], gsp, prev;
-    R acc[2];
-    __device__ void init() {
-        for (int i = 0; i < 2; ++i) { alpha[i] = (R)S->alpha[i]; lam[i] = (R)S->lam[i]; pw[i] = S->p[i]; }
-        eps2 = (R)S->eps2;
-        g11 = (R)S->G[0]; g22 = (R)S->G[1]; g12 = (R)S->G[2];
-        gsp = S->gspace;
-        prev = S->anchor == GJ_ANCHOR_PREVIOUS && S->k > 0;  // W_{k-1} m_{k-1} exists from k = 1
-        acc[0] = acc[1] = 0;
-    }
-    __device__ __forceinline__ void store(int la, int, bool, int j, R a, R b) {
-        const size_t c = (size_t)la * nx + j;
-        const int r = la / ny;
-        const R mm[2] = {F.m[0][c], F.m[1][c]};
-        const R w[2] = {weight(F, 0, pw[0], eps2, r, c, mm[0]), weight(F, 1, pw[1], eps2, r, c, mm[1])};
-        // ascent directions in the chosen space (RRCG:2-3 or Eq. steepestascenta/b)
-        const R u0 = gsp ? w[0] * mm[0] : mm[0], u1 = gsp ? w[1] * mm[1] : mm[1];
-        const R lG[2] = {g22 * u0 - g12 * u1, g11 * u1 - g12 * u0};
-        const R g[2] = {a, b};
-        for (int i = 0; i < 2; ++i) {
-            const R ma = (OPT && F.mapr[i]) ? F.mapr[i][c] : R(0);
-            const R anchor = (OPT && prev) ? F.mtp[i][c] : w[i] * ma;
-            const R li = g[i] / w[i] + alpha[i] * (w[i] * mm[i] - anchor) + lam[i] * lG[i];
-            F.l[i][c] = li;
-            acc[i] += li * li;
-        }
-    }
-    static constexpr int NPRE = 1;  // m, staged ahead by the persistent row pass
-    __device__ const R *pre_src(int, int i) const { return F.m[i]; }
-    template <int K, bool PRE = false>
-    __device__ __forceinline__ void store_batch(int la, int, bool, int j0, int stride, int n, const R (&a)[K],
-                                                const R (&b)[K], const R *pre = nullptr) {
-        const size_t c0 = (size_t)la * nx;
-        const int r = la / ny;
-        R mv[2][K], wh[2][K], ma[2][K], an[2][K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            const bool ok = j < n;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                mv[i][k] = ok ? (PRE ? pre[i * f512::H + j] : F.m[i][c0 + j]) : R(0);
-                wh[i][k] = (ok && OPT && F.whard[i]) ? F.whard[i][c0 + j] : R(1);
-                ma[i][k] = (ok && OPT && F.mapr[i]) ? F.mapr[i][c0 + j] : R(0);
-                an[i][k] = (ok && OPT && prev) ? F.mtp[i][c0 + j] : R(0);
-            }
-        }
-        R wd[2], iwd[2];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) { wd[i] = F.wdep[i][r]; iwd[i] = F.iwdep[i][r]; }
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            if (j >= n) continue;
-            R w[2], inv_w[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                R wl, iwl;
-                lp_factors<R>(pw[i], mv[i][k] - ma[i][k], eps2, wl, iwl);
-                w[i] = wd[i] * wl;
-                inv_w[i] = iwl * iwd[i];
-                if (OPT && F.whard[i]) { w[i] *= wh[i][k]; inv_w[i] /= wh[i][k]; }
-            }
-            const R u0 = gsp ? w[0] * mv[0][k] : mv[0][k], u1 = gsp ? w[1] * mv[1][k] : mv[1][k];
-            const R lG[2] = {g22 * u0 - g12 * u1, g11 * u1 - g12 * u0};
-            const R g[2] = {a[k], b[k]};
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const R anchor = (OPT && prev) ? an[i][k] : w[i] * ma[i][k];
-                const R li = g[i] * inv_w[i] + alpha[i] * (w[i] * mv[i][k] - anchor) + lam[i] * lG[i];
-                F.l[i][c0 + j] = li;
-                acc[i] += li * li;
-            }
-        }
-    }
-    __device__ void flush(double *red) { block_accumulate<2>(acc, S->ll, red); }
-};
-
-// Search direction (RRCG:5) and the forward input W^-1 p.
-template <typename R, bool OPT = true>
-struct ProDirection {
-    FieldVecs<R> F;
-    SolverDev *S;
-    int nx, ny;
-    R beta[2], eps2;
-    int first, pw[2];
-    R acc[4];  // (p,l)_0, (p,l)_1, ||p||^2_0, ||p||^2_1
-    __device__ void init() {
-        first = S->k == 0;
-        eps2 = (R)S->eps2;
-        for (int i = 0; i < 2; ++i) pw[i] = S->p[i];
-        if (S->per_field) {
-            for (int i = 0; i < 2; ++i) beta[i] = S->ll_prev[i] > 0 ? (R)(S->ll[i] / S->ll_prev[i]) : R(0);
-        } else {
-            const double den = S->ll_prev[0] + S->ll_prev[1];
-            const R b = den > 0 ? (R)((S->ll[0] + S->ll[1]) / den) : R(0);
-            beta[0] = beta[1] = b;
-        }
-        acc[0] = acc[1] = acc[2] = acc[3] = 0;
-    }
-    __device__ __forceinline__ void fetch(int la, int, bool, int j, R &a, R &b) {
-        const size_t c = (size_t)la * nx + j;
-        const int r = la / ny;
-        R x[2];
-        for (int i = 0; i < 2; ++i) {
-            const R li = F.l[i][c];
-            const R pi = first ? li : li + beta[i] * F.p[i][c];
-            F.p[i][c] = pi;
-            acc[i] += pi * li;
-            acc[2 + i] += pi * pi;
-            x[i] = pi / weight(F, i, pw[i], eps2, r, c, F.m[i][c]);
-        }
-        a = x[0];
-        b = x[1];
-    }
-    static constexpr int NPRE = 3;  // l, p, m, staged ahead by the persistent row pass
-    __device__ const R *pre_src(int a, int i) const {
-        return a == 0 ? F.l[i] : (a == 1 ? (first ? nullptr : F.p[i]) : F.m[i]);
-    }
-    template <int K, bool PRE = false>
-    __device__ __forceinline__ void fetch_batch(int la, int, bool, int j0, int stride, int n, R (&a)[K], R (&b)[K],
-                                                const R *pre = nullptr) {
-        const size_t c0 = (size_t)la * nx;
-        const int r = la / ny;
-        R lv[2][K], pv[2][K], mv[2][K], wh[2][K], ma[2][K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            const bool ok = j < n;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                lv[i][k] = ok ? (PRE ? pre[i * f512::H + j] : F.l[i][c0 + j]) : R(0);
-                pv[i][k] = (ok && !first) ? (PRE ? pre[(2 + i) * f512::H + j] : F.p[i][c0 + j]) : R(0);
-                mv[i][k] = ok ? (PRE ? pre[(4 + i) * f512::H + j] : F.m[i][c0 + j]) : R(0);
-                wh[i][k] = (ok && OPT && F.whard[i]) ? F.whard[i][c0 + j] : R(1);
-                ma[i][k] = (ok && OPT && F.mapr[i]) ? F.mapr[i][c0 + j] : R(0);
-            }
-        }
-        R iwd[2];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) iwd[i] = F.iwdep[i][r];
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            const bool ok = j < n;
-            R x[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const R pi = first ? lv[i][k] : lv[i][k] + beta[i] * pv[i][k];
-                R wl, iwl;
-                lp_factors<R>(pw[i], mv[i][k] - ma[i][k], eps2, wl, iwl);
-                R inv_w = iwl * iwd[i];
-                if (OPT && F.whard[i]) inv_w /= wh[i][k];
-                if (ok) {
-                    F.p[i][c0 + j] = pi;
-                    acc[i] += pi * lv[i][k];
-                    acc[2 + i] += pi * pi;
-                }
-                x[i] = ok ? pi * inv_w : R(0);
-            }
-            a[k] = x[0];
-            b[k] = x[1];
-        }
-    }
-    __device__ void flush(double *red) {
-        // pl and pp are adjacent in SolverDev: one pass adds all four sums
-        static_assert(offsetof(SolverDev, pp) == offsetof(SolverDev, pl) + 2 * sizeof(double), "layout");
-        block_accumulate<4>(acc, S->pl, red);
-    }
-};
-
-// ||A~ p||^2 = ||W_d A (W^-1 p)||^2 partials (RRCG:6).
-template <typename R>
-struct EpiQNorm {
-    FieldVecs<R> F;
-    SolverDev *S;
-    int sx;
-    R acc[2];
-    __device__ void init() { acc[0] = acc[1] = 0; }
-    __device__ __forceinline__ void store(int la, int, bool, int j, R a, R b) {
-        const size_t t = (size_t)la * sx + j;
-        const R q0 = F.wd[0][t] * a, q1 = F.wd[1][t] * b;
-        acc[0] += q0 * q0;
-        acc[1] += q1 * q1;
-    }
-    // batched form (the 512 kernels): prefetch loads W_d of line la, elements
-    // lane + 32 k, before the transform; store_batch(j0 = lane or lane + 128) uses them
-    R wq[2][8];
-    __device__ __forceinline__ void prefetch(int la, int, bool, int lane, int n) {
-        const size_t t0 = (size_t)la * sx;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int j = lane + 32 * k;
-            wq[0][k] = j < n ? F.wd[0][t0 + j] : R(0);
-            wq[1][k] = j < n ? F.wd[1][t0 + j] : R(0);
-        }
-    }
-    template <int K>
-    __device__ __forceinline__ void store_batch(int, int, bool, int j0, int stride, int n, const R (&a)[K],
-                                                const R (&b)[K]) {
-        const int o = (j0 - (int)(threadIdx.x & 31)) / 32;  // 0 or 4
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            if (j >= n) continue;
-            const R q0 = wq[0][o + k] * a[k], q1 = wq[1][o + k] * b[k];
-            acc[0] += q0 * q0;
-            acc[1] += q1 * q1;
-        }
-    }
-    __device__ void flush(double *red) { block_accumulate<2>(acc, S->qq, red); }
-};
 
 // The one-thread scalar steps run on a shared-memory copy of the solver state: a
 // warp copies it in with one coalesced read (instead of a chain of dependent global
@@ -721,10 +200,7 @@ struct SolverLaunch {
     bool fast1024 = false;  // general row kernels (transposed intermediates) + N_y = 1024 column kernels
     bool rows1024 = false;  // fast1024 with N_x = 1024: the warp-FFT row kernels of fast1024.cuh
     FieldVecs<R> F;
-    int P, C, L;
     int grid;  // CTAs of the persistent fast-path launches
-    size_t rsm, msm, csm;
-    int n_rows_cells, n_rows_st;  // pairs in the cell / station row passes
 
     void setup() {  // views and launch shapes only (no CUDA calls: safe during capture)
         const gj_op *o = sv->op[0];
@@ -737,11 +213,6 @@ struct SolverLaunch {
             rows1024 = fast1024 && o->Nx == 1024;
             if (fast || fast1024) V2 = f512::make_view2<R>(sv->op[0], sv->op[1]);
         }
-        const size_t cs = sizeof(cpx<R>);
-        P = o->P_row; C = o->C_col; L = o->L_grp;
-        rsm = row_smem(o->Nx, P, cs);
-        msm = col_smem(o->Ny, C, 3, cs);
-        csm = col_smem(o->Ny, C, 2, cs);
         const int n = o->nx * o->ny * o->nz, s = o->sx * o->sy;
         R *b = static_cast<R *>(sv->buf);
         for (int i = 0; i < 2; ++i) {
@@ -795,16 +266,13 @@ struct SolverLaunch {
             f1024::set_row_inv_attr<R, EpiGradient<R>>();
             f1024::set_row_inv_attr<R, EpiQNorm<R>>();
         }
-        allow_max_smem(k_row_fwd<R, ProModel<R>>);
-        allow_max_smem(k_row_fwd<R, ProDirection<R>>);
-        allow_max_smem(k_row_fwd<R, LoadPair<R>>);
-        allow_max_smem(k_row_inv<R, EpiResidual<R>>);
-        allow_max_smem(k_row_inv<R, EpiGradient<R>>);
-        allow_max_smem(k_row_inv<R, EpiQNorm<R>>);
-        allow_max_smem(k_col_fwd_mac<R>);
-        allow_max_smem(k_col_inv<R>);
-        allow_max_smem(k_col_fft<R>);
-        allow_max_smem(k_col_adj<R>);
+        if constexpr (std::is_same_v<R, float>) if (rows1024) return;
+        gen_row_fwd_attr<R, ProModel<R>>();
+        gen_row_fwd_attr<R, ProDirection<R>>();
+        gen_row_resid_attr<R, EpiResidual<R>>();
+        gen_row_inv_attr<R, EpiGradient<R>>();
+        gen_row_inv_attr<R, EpiQNorm<R>>();
+        gen_col_attr<R>();
     }
 
     // Row passes of the general path over both fields (joint pair maps): the block FFT
@@ -816,7 +284,7 @@ struct SolverLaunch {
             f1024::row_fwd<R>(v0, pm, n_in, o0, o1, sv->op[0]->twtab, pro, done, st);
             return;
         }
-        k_row_fwd<R, Pro><<<(pm.nlines + P - 1) / P, 256, rsm, st>>>(v0, pm, n_in, P, o0, o1, pro, done);
+        gen_row_fwd<R>(sv->op[0], v0, pm, n_in, o0, o1, pro, done, st);
     }
     template <class Epi>
     void rows_inv(const PairMap &pm, int n_out, const cpx<R> *i0, const cpx<R> *i1, const Epi &epi, const int *done,
@@ -825,7 +293,7 @@ struct SolverLaunch {
             f1024::row_inv<R>(v0, pm, n_out, i0, i1, sv->op[0]->twtab, epi, done, st);
             return;
         }
-        k_row_inv<R, Epi><<<(pm.nlines + P - 1) / P, 256, rsm, st>>>(v0, pm, n_out, P, i0, i1, epi, done);
+        gen_row_inv<R>(sv->op[0], v0, pm, n_out, i0, i1, epi, done, st);
     }
 
     // Forward columns (Y = sum_r T^_r FFT_y(Z_r)) and inverse columns, both fields.
@@ -861,21 +329,16 @@ struct SolverLaunch {
             }
             return;
         }
-        const size_t cs = sizeof(cpx<R>);
-        cudaMemsetAsync(v0.Y, 0, (size_t)o->Ny * o->ncol * cs, st);
-        cudaMemsetAsync(v1.Y, 0, (size_t)o->Ny * o->ncol * cs, st);
-        const int nt = (o->ncol + C - 1) / C;
         ProfilePair pp{};
         if (sv->profile && !sv->capturing) {
             pp = take_pair(sv);
             cudaEventRecord(pp.a, st);
         }
-        k_col_fwd_mac<R><<<dim3(nt, (o->nz + L - 1) / L, 2), 256, msm, st>>>(v0, v1, C, L, &sv->S->done);
+        gen_col_fwd<R>(o, v0, v1, 2, o->nz, &sv->S->done, st);
         if (sv->profile && !sv->capturing) {
             cudaEventRecord(pp.b, st);
             sv->eager_pairs.push_back(pp);
         }
-        k_col_inv<R><<<dim3(nt, 2), 256, csm, st>>>(v0, v1, C, &sv->S->done);
     }
 
     void head(cudaStream_t st) {  // forward of (updated) m, residual, chi^2 scalars
@@ -903,7 +366,11 @@ struct SolverLaunch {
         forward_columns(st);
         PairMap ps{o->sy, 1, o->sy};
         EpiResidual<R> er{F, sv->S, o->sx};
-        rows_inv(ps, o->sx, v0.W, v1.W, er, done, st);
+        // residual, Phi and the residual rows' spectra for the adjoint, in one pass
+        if constexpr (std::is_same_v<R, float>)
+            if (rows1024) f1024::row_inv<R>(v0, ps, o->sx, v0.W, v1.W, o->twtab, er, done, st);
+        if (!rows1024)
+            gen_row_resid<R>(o, v0, ps, o->sx, v0.W, v1.W, fast1024 ? v0.V : v0.W, fast1024 ? v1.V : v1.W, er, done, st);
         k_scalars_after_residual<<<1, 32, 0, st>>>(sv->S);
     }
 
@@ -931,23 +398,15 @@ struct SolverLaunch {
             head(st);
             return;
         }
-        const int nt = (o->ncol + C - 1) / C;
         PairMap ps{o->sy, 1, o->sy};
         PairMap pc{o->nz * o->ny, 1, o->ny};
-        // adjoint: rows of v -> W, columns -> Y, per-layer conj-spectrum columns -> Z
-        // (N_y = 1024 column kernels: rows of v -> V, then one persistent column pass)
-        LoadPair<R> lv{F.v[0], F.v[1], o->sx};
-        bool cols1024 = false;
-        if constexpr (std::is_same_v<R, float>) cols1024 = fast1024;
-        if (cols1024) {
-            rows_fwd(ps, o->sx, v0.V, v1.V, lv, done, st);
-            if constexpr (std::is_same_v<R, float>) f1024::col_adj<R>(V2, grid, done, st);
-        } else {
-            k_row_fwd<R, LoadPair<R>><<<(ps.nlines + P - 1) / P, 256, rsm, st>>>(v0, ps, o->sx, P, v0.W, v1.W, lv,
-                                                                                done);
-            k_col_fft<R><<<dim3(nt, 2), 256, csm, st>>>(v0, v1, C, done);
-            k_col_adj<R><<<dim3(nt, o->nz, 2), 256, csm, st>>>(v0, v1, C, done);
+        // adjoint: the residual rows' spectra (head) -> per-layer conj-spectrum columns -> Z
+        if constexpr (std::is_same_v<R, float>) {
+            if (rows1024)
+                f1024::row_fwd<R>(v0, ps, o->sx, v0.V, v1.V, o->twtab, LoadPair<R>{F.v[0], F.v[1], o->sx}, done, st);
+            if (fast1024) f1024::col_adj<R>(V2, grid, done, st);
         }
+        if (!fast1024) gen_col_adj<R>(o, v0, v1, 2, o->nz, done, st);
         EpiGradient<R> eg{F, sv->S, o->nx, o->ny};
         rows_inv(pc, o->nx, v0.Z, v1.Z, eg, done, st);
         // direction and its forward product

@@ -10,7 +10,7 @@
 
 #include "fast1024.cuh"
 #include "fast512.cuh"
-#include "view.cuh"
+#include "general_launch.cuh"
 
 namespace gj {
 
@@ -203,75 +203,102 @@ struct LoadTable {
 
 // Column pass of the setup: spec[r] = FFT_y of the row-pass output of layer r.
 template <typename Rout>
-__global__ void __launch_bounds__(256) k_col_spec(OpView<double> op, const double2 *Zs, cpx<Rout> *spec, int C,
+__global__ void __launch_bounds__(256) k_col_spec(OpView<double> op, const double2 *Zs, cpx<Rout> *spec, ColShape cs,
                                                   int transposed, int real_only) {
     using Cx = double2;
-    const int c0 = blockIdx.x * C;
+    const int c0 = blockIdx.x * cs.C;
     const int r = blockIdx.y;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int Ny = op.Ny, ncol = op.ncol;
-    Cx *buf0 = reinterpret_cast<Cx *>(smem_raw);
-    Cx *buf1 = buf0 + Ny * C;
-    Cx *tw = buf1 + Ny * C;
-    for (int i = threadIdx.x; i < Ny; i += blockDim.x) tw[i] = op.twy[i];
+    const int cols = min(cs.C, ncol - c0);
+    Cx *bufA = reinterpret_cast<Cx *>(smem_raw);
+    Cx *bufB = bufA + Ny * cs.pitch;
+    Cx *tw = bufB + Ny * cs.pitch;
+    load_twiddles(tw, op.twy, Ny);
     const Cx *Zr = Zs + (size_t)r * Ny * ncol;
-    for (int it = threadIdx.x; it < Ny * C; it += blockDim.x) {
-        const int c = it % C, iy = it / C;
-        buf0[it] = (c0 + c < ncol) ? Zr[(size_t)iy * ncol + c0 + c] : make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-    const Cx *X = fft_lines<double, false>(buf0, buf1, op.py, C, tw, Ny);
     cpx<Rout> *Sr = spec + (size_t)r * Ny * ncol;
     const int ke = even_spec_len(Ny);
-    for (int it = threadIdx.x; it < Ny * C; it += blockDim.x) {
-        const int c = it % C, ky = it / C;
-        if (c0 + c < ncol) {
-            if (real_only) {
-                // the table is even in both offsets: the spectrum is real (its imaginary part
-                // is zero in exact arithmetic) and even in ky, so only ky <= Ny/2 is kept,
-                // as R[r][kx][ke] (fast path)
-                if (ky <= Ny / 2)
-                    reinterpret_cast<Rout *>(spec)[((size_t)r * ncol + c0 + c) * ke + ky] = (Rout)X[it].x;
-            } else {
-                const size_t at = transposed ? (size_t)(c0 + c) * Ny + ky : (size_t)ky * ncol + c0 + c;
-                Sr[at] = mk<cpx<Rout>>((Rout)X[it].x, (Rout)X[it].y);
-            }
+    auto in = [&](int j, int c) { return c < cols ? Zr[(size_t)j * ncol + c0 + c] : czero<Cx>(); };
+    auto out = [&](int ky, int c, Cx x) {
+        if (c >= cols) return;
+        if (real_only) {
+            // the table is even in both offsets: the spectrum is real (its imaginary part
+            // is zero in exact arithmetic) and even in ky, so only ky <= Ny/2 is kept,
+            // as R[r][kx][ke] (fast path)
+            if (ky <= Ny / 2) reinterpret_cast<Rout *>(spec)[((size_t)r * ncol + c0 + c) * ke + ky] = (Rout)x.x;
+        } else {
+            const size_t at = transposed ? (size_t)(c0 + c) * Ny + ky : (size_t)ky * ncol + c0 + c;
+            Sr[at] = mk<cpx<Rout>>((Rout)x.x, (Rout)x.y);
         }
-    }
+    };
+    fft_run<double, false, false, false>(op.py, cs.C, cs.mB, cs.pitch, bufA, bufB, tw, Ny, Ny, in, out);
 }
 
 // ---------------------------------------------------------------------------
 // Host helpers
 
-// Radix plan of an N-point transform.  order 0: the power-of-two part in radix 8
-// (one or two radix-4 stages for the rest), then the odd primes ascending; order 1:
-// the same stages in reverse; order 2: the power-of-two part in radix 4 (and one
+// Radix plan of an N-point transform.  order 0: the cheapest product of codelet radices
+// (by the codelets' operation counts, twiddles and a shared-memory round trip a stage),
+// with even radices first and last where there are any (the pruned stages halve those);
+// order 1: the same stages in reverse; order 2: the power-of-two part in radix 4 (and one
 // radix 2), then the odd primes.
+static void cheapest_radices(int n, int N, int most, double cost, std::vector<int> &cur, double &best,
+                             std::vector<int> &out) {
+    // real operations of the codelets, radix 0 to 17
+    static const double ops[kMaxRadix + 1] = {0,   0,   4,   14,  16,  40,  40,  84,  56,
+                                              104, 100, 220, 104, 312, 196, 250, 168, 544};
+    if (n == 1) {
+        if (cost < best) { best = cost; out = cur; }
+        return;
+    }
+    for (int r = std::min(n, most); r >= 2; --r) {
+        if (n % r) continue;
+        // butterflies, the round trip and the twiddles of one stage
+        const double c = (double)N / r * ops[r] + 14.0 * N + 300.0;
+        if (cost + c >= best) continue;
+        cur.push_back(r);
+        cheapest_radices(n / r, N, r, cost + c, cur, best, out);
+        cur.pop_back();
+    }
+}
+
 bool plan_size(int N, FftPlanDev &plan, int order) {
     if (N < 1 || N > 2048 || order < 0 || order > 2) return false;
     int n = N, e = 0;
     while (n % 2 == 0) { n /= 2; ++e; }
-    std::vector<int> rs;
+    std::vector<int> rs, odd;
+    for (int p : {3, 5, 7, 11, 13, 17})
+        while (n % p == 0) { n /= p; odd.push_back(p); }
+    if (n != 1) return false;
     if (order == 2) {
         rs.assign(e / 2, 4);
         if (e % 2) rs.push_back(2);
+        rs.insert(rs.end(), odd.begin(), odd.end());
     } else {
-        rs.assign(e / 3, 8);
-        if (e % 3 == 1) {
-            if (!rs.empty()) { rs.back() = 4; rs.push_back(4); } else rs.push_back(2);
-        } else if (e % 3 == 2) {
-            rs.push_back(4);
-        }
+        std::vector<int> cur;
+        double best = 1e300;
+        cheapest_radices(N, N, kMaxRadix, 0.0, cur, best, rs);  // descending
+        std::stable_sort(rs.begin(), rs.end(), [](int a, int b) { return a % 2 < b % 2; });
+        if (rs.size() > 2 && rs[1] % 2 == 0) std::swap(rs[1], rs.back());  // an even one last as well
+        if (order == 1) std::reverse(rs.begin(), rs.end());
     }
-    const int primes[] = {3, 5, 7, 11, 13, 17};
-    for (int p : primes)
-        while (n % p == 0) { n /= p; rs.push_back(p); }
-    if (n != 1) return false;
-    if (order == 1) std::reverse(rs.begin(), rs.end());
+    while (rs.size() < 2) rs.push_back(1);  // the transforms run at least two stages
     if ((int)rs.size() > kMaxStages) return false;
     plan.N = N;
     plan.nst = (int)rs.size();
-    for (int i = 0; i < kMaxStages; ++i) plan.radix[i] = i < plan.nst ? rs[i] : 1;
+    plan.mmax = 1;
+    int Ns = 1;
+    for (int i = 0; i < kMaxStages; ++i) {
+        const int r = i < plan.nst ? rs[i] : 1;
+        FftStage &st = plan.st[i];
+        st.rad = r;
+        st.M = N / r;
+        st.Ns = Ns;
+        st.tws = std::max(1, N / (Ns * r));
+        st.mNs = div_magic(Ns);
+        if (i < plan.nst && r > 1) plan.mmax = std::max(plan.mmax, st.M);
+        Ns *= r;
+    }
     return true;
 }
 
@@ -331,18 +358,6 @@ int fast_slots(int nfield, int ncol, int nz, long long warps) {
 
 bool fast1024_eligible(const gj_op *op) {
     return op->prec == GJ_FP32_MIXED && !op->fast && op->Ny == 1024 && op->ny <= 512 && op->sy <= 512;
-}
-
-int pick_row_pairs(int Nx, size_t cs) {
-    int P = 16;
-    while (P > 1 && row_smem(Nx, P, cs) > 96 * 1024) P >>= 1;
-    return P;
-}
-
-int pick_col_tile(int Ny, size_t cs, int nbuf) {
-    int C = 16;
-    while (C > 1 && col_smem(Ny, C, nbuf, cs) > 100 * 1024) C >>= 1;
-    return C;
 }
 
 static gj_status upload_twiddles(int N, gj_precision prec, void **out) {
@@ -462,7 +477,9 @@ static void build_layers(const gj_op *op, const gj_setup_scratch_impl &sc, int r
     L.dy = op->dy;
     L.zw = sc.zw + r0;
     MagCoef mc{};
-    double scale = 1.0 / ((double)op->Nx * (double)op->Ny);
+    // the row passes below, and those of the general kernels, leave out the half of the
+    // real-line split: it is part of the spectra (a power of two: nothing rounds)
+    double scale = (op->fast || op->fast1024 ? 0.5 : 0.25) / ((double)op->Nx * (double)op->Ny);
     const int magnetic = op->field == GJ_MAGNETIC;
     if (magnetic) {
         const double d2r = 3.14159265358979323846 / 180.0;
@@ -494,15 +511,20 @@ static void build_layers(const gj_op *op, const gj_setup_scratch_impl &sc, int r
     lt.magnetic = magnetic;
     lt.far32 = op->prec == GJ_FP32_MIXED ? 1 : 0;
     lt.mc = mc;
-    PairMap pm{count * op->Ny, 0};
-    const int P = pick_row_pairs(op->Nx, sizeof(double2));
+    PairMap pm{count * op->Ny, 0, 0};
     const int npairs = (pm.nlines + 1) / 2;
-    const size_t rsm = row_smem(op->Nx, P, sizeof(double2));
-    k_row_fwd<double, LoadTable><<<(npairs + P - 1) / P, 256, rsm, st>>>(v, pm, op->Nx, P, sc.Zs, sc.Zs, lt, nullptr);
-    const int C = pick_col_tile(op->Ny, sizeof(double2), 2);
-    const size_t csm = col_smem(op->Ny, C, 2, sizeof(double2));
-    dim3 g((op->ncol + C - 1) / C, count);
-    k_col_spec<Rout><<<g, 256, csm, st>>>(v, sc.Zs, spec, C, (op->fast || op->fast1024) ? 1 : 0, op->real_spec ? 1 : 0);
+    const RowShape rs = row_shape_of(op->px, pick_row_pairs(op->px, npairs, sizeof(double2)), sizeof(double2));
+    k_row_fwd<double, LoadTable><<<(npairs + rs.P - 1) / rs.P, gen_threads(op->px.mmax, rs.P),
+                                   row_smem(op->Nx, rs.pitch, sizeof(double2)), st>>>(v, pm, op->Nx, rs, sc.Zs, sc.Zs,
+                                                                                     lt, nullptr);
+    ColShape cs{};
+    cs.C = pick_col_tile(op->py, op->ncol, count, 1, sizeof(double2));
+    cs.G = 1;
+    cs.pitch = cs.C;
+    cs.mB = cs.mC = div_magic(cs.C);
+    k_col_spec<Rout><<<dim3((op->ncol + cs.C - 1) / cs.C, count), gen_threads(op->py.mmax, cs.C),
+                       col_smem(op->Ny, cs.pitch, 0, sizeof(double2)), st>>>(
+        v, sc.Zs, spec, cs, (op->fast || op->fast1024) ? 1 : 0, op->real_spec ? 1 : 0);
 }
 
 static void set_build_attributes() {
@@ -579,9 +601,6 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
     op->prec = prec;
     op->Nx = Nx; op->Ny = Ny; op->ncol = Nx / 2 + 1;
     const size_t cs = 2 * elem_bytes(prec);
-    op->P_row = pick_row_pairs(Nx, cs);
-    op->C_col = pick_col_tile(Ny, cs, 3);
-    op->L_grp = 4;
     op->recompute = (flags & GJ_SETUP_RECOMPUTE_SPECTRA) != 0;
     op->fast = !op->recompute && fast_eligible(op);
     if (op->fast) {
@@ -606,6 +625,15 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
         op->slots = std::max(fast_slots(1, op->ncol, G.nz, warps), fast_slots(2, op->ncol, G.nz, warps));
         op->real_spec = field == GJ_GRAVITY && G.sx == G.nx && G.sy == G.ny && G.off_x == 0 && G.off_y == 0;
     }
+    // the shapes of both fields' launches (single-field ones pick their own until tuned)
+    const int layers = op->recompute ? 1 : G.nz;
+    op->P_row = pick_row_pairs(op->px, (long long)G.nz * G.ny, cs);
+    if (op->fast1024) {  // transposed intermediates: runs of P lines
+        op->P_row = 16;
+        while (op->P_row > 1 && row_smem(Nx, odd_pitch(op->P_row), cs) > kGenSmem) op->P_row >>= 1;
+    }
+    op->C_col = pick_col_tile(op->py, op->ncol, layers, 2, cs);
+    op->L_grp = pick_layers(op->py, op->C_col, (op->ncol + op->C_col - 1) / op->C_col * 2, layers, cs);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     gj_status rc;
     cudaError_t e;
@@ -629,12 +657,24 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
     }
     if (!op->fast && !op->fast1024) {
         const size_t zb = (size_t)G.nz * G.ny * op->ncol * cs;
-        const size_t yb = (size_t)Ny * op->ncol * cs;
+        // partial layer sums (as many groups as a launch of one field or of both makes; a
+        // tuned L_grp makes no more) and arrival counters, which are zero between launches
+        for (int nf = 1; nf <= 2 && !op->recompute; ++nf) {
+            const int C = pick_col_tile(op->py, op->ncol, layers, nf, cs);
+            const int L = pick_layers(op->py, C, (op->ncol + C - 1) / C * nf, layers, cs);
+            op->gen_slots = std::max(op->gen_slots, (layers + L - 1) / L);
+        }
+        const size_t sb = (size_t)op->gen_slots * Ny * op->ncol * cs, yb = sb + op->ncol * sizeof(int);
         const size_t wb = (size_t)std::max(G.sy, 1) * op->ncol * cs;
         op->ws_bytes = zb + yb + wb;
         if ((e = cudaMalloc(&op->Z, zb)) != cudaSuccess) { rc = cuda_fail(e, "workspace"); goto fail; }
         if ((e = cudaMalloc(&op->Y, yb)) != cudaSuccess) { rc = cuda_fail(e, "workspace"); goto fail; }
         if ((e = cudaMalloc(&op->W, wb)) != cudaSuccess) { rc = cuda_fail(e, "workspace"); goto fail; }
+        if ((e = cudaMemsetAsync(op->Y, 0, yb, st)) != cudaSuccess || (e = cudaStreamSynchronize(st)) != cudaSuccess) {
+            rc = cuda_fail(e, "workspace");
+            goto fail;
+        }
+        op->cnt = reinterpret_cast<int *>(static_cast<char *>(op->Y) + sb);
     } else {
         // transposed intermediates [r][kx][Ny/2], partials [kx][slots][Ny], counters
         const size_t zb = (size_t)G.nz * op->ncol * (Ny / 2) * cs;
@@ -688,7 +728,7 @@ extern "C" gj_status gj_op_tune(gj_op *op, int P_row, int C_col, int L_grp, int 
     if (P_row > 0 && (P_row > 64 || row_smem(op->Nx, P_row, cs) > room)) {
         set_error("gj_op_tune: P_row too large for shared memory"); return GJ_ERR_ARG;
     }
-    if (C_col > 0 && (C_col > 64 || col_smem(op->Ny, C_col, 3, cs) > room)) {
+    if (C_col > 0 && (C_col > 64 || col_smem(op->Ny, C_col, C_col, cs) > room)) {
         set_error("gj_op_tune: C_col too large for shared memory"); return GJ_ERR_ARG;
     }
     if (L_grp > 0 && L_grp > op->nz) { set_error("gj_op_tune: L_grp above nz"); return GJ_ERR_ARG; }
@@ -696,9 +736,9 @@ extern "C" gj_status gj_op_tune(gj_op *op, int P_row, int C_col, int L_grp, int 
     if (radix_order >= 0 && (!plan_size(op->Nx, px, radix_order) || !plan_size(op->Ny, py, radix_order))) {
         set_error("gj_op_tune: radix_order must be 0, 1 or 2"); return GJ_ERR_ARG;
     }
-    if (P_row > 0) op->P_row = P_row;
-    if (C_col > 0) op->C_col = C_col;
-    if (L_grp > 0) op->L_grp = L_grp;
+    if (P_row > 0) { op->P_row = P_row; op->rows_tuned = true; }
+    if (C_col > 0) { op->C_col = C_col; op->cols_tuned = true; }
+    if (L_grp > 0) { op->L_grp = L_grp; op->layers_tuned = true; }
     if (radix_order >= 0) op->radix_order = radix_order;
     op->px = px;
     op->py = py;

@@ -18,14 +18,18 @@ inline OpView<R> view_of(const gj_op *op) {
     v.Y = static_cast<cpx<R> *>(op->Y);
     v.W = static_cast<cpx<R> *>(op->W);
     v.V = static_cast<cpx<R> *>(op->V);
+    v.cnt = op->cnt;
     v.real_spec = op->real_spec ? 1 : 0;
     v.rbase = 0;
     v.spec_r0 = 0;
     v.tcol = op->fast1024 ? op->Ny / 2 : 0;
+    v.split_half = op->fast || op->fast1024;  // the general kernels' spectra carry the factor
     return v;
 }
 
-inline size_t row_smem(int Nx, int P, size_t cs) { return (size_t)(2 * Nx * P + Nx) * cs; }
-inline size_t col_smem(int Ny, int C, int nbuf, size_t cs) { return (size_t)(nbuf * Ny * C + Ny) * cs; }
+// Shared memory of a row pass (two buffers of P lines and the twiddles) and of a column
+// pass (two buffers of B lines, `keep` more lines that stay, the twiddles).
+inline size_t row_smem(int Nx, int pitch, size_t cs) { return (size_t)(2 * Nx * pitch + Nx) * cs; }
+inline size_t col_smem(int Ny, int pitch, int keep, size_t cs) { return (size_t)(2 * Ny * pitch + Ny * keep + Ny) * cs; }
 
 }  // namespace gj
