@@ -19,7 +19,7 @@ ROOT = os.path.dirname(HERE)
 BUILD = os.path.join(ROOT, "_build", "gj")
 LIB = os.path.join(HERE, "libgj.so")
 SOURCES = ["general_solver_f32.cu", "general_solver_f64.cu", "general_cols_f32.cu", "general_cols_f64.cu",
-           "general_rows_f32.cu", "general_rows_f64.cu", "rrcg.cu", "matvec.cu", "setup.cu", "gramian.cu", "probe.cu",
+           "general_recompute_f32.cu", "general_recompute_f64.cu", "general_rows_f32.cu", "general_rows_f64.cu", "rrcg.cu", "matvec.cu", "setup.cu", "gramian.cu", "probe.cu",
            "api.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O3",

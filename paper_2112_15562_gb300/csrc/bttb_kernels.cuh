@@ -30,8 +30,6 @@ struct OpView {
     cpx<R> *V;           // fast path: residual-row spectra [ncol][256] (unused otherwise)
     int real_spec;       // fast path: spec holds the real, even spectrum of an even table for
                          // ky <= Ny/2 only, R[nz][ncol][even_spec_len(Ny)]
-    int rbase;           // first layer of a column launch (per-layer launches of the recompute mode)
-    int spec_r0;         // layer held at spec index 0 (0 when all layers are stored)
     int split_half;      // 1: the row passes halve the split spectra; 0: the factor is in `spec`
     int tcol;            // 0: Z, W, V row-major ([line][ncol]); > 0: transposed, line iy of layer r and
                          // bin k at ((r * ncol + k) * tcol + iy) (the N_y = 1024 column kernels' layout)
@@ -207,7 +205,6 @@ struct ColShape {
     int pitch1;      // of the C lines of the residual or summed spectrum
     unsigned mB, mC;
     int arrivals;    // layer groups of a column tile (1: the sum stays on chip)
-    int serial;      // 1: a launch per layer, which add to Y one after the other
 };
 
 template <typename C>
@@ -412,6 +409,78 @@ __global__ void __launch_bounds__(256) k_row_resid(OpView<R> op, PairMap pm, int
 // sum_r T^_r . FFT_y(Z_r); the last group of a tile to arrive takes the sum of all
 // groups (through Y) and writes W[jy] = IFFT_y(sum)[jy], jy < sy.  With one group the sum
 // never leaves the CTA.
+
+// Sources and sinks of the column passes.  Absent columns, layers and rows are clamped to
+// present ones and masked afterwards, so that a butterfly's loads are unconditional and go
+// out together: behind a branch each waited for the one before it (a layer of N = 256 took
+// 16 memory latencies; 128x128x32 FP32, both fields: 66 us for the forward columns).
+struct LineMap {  // line b of a group -> layer and column
+    unsigned mC;
+    int C, cols, rg, r1;
+    __device__ __forceinline__ void at(int b, int &r, int &c) const {
+        const int g = fast_div(b, mC);
+        c = b - g * C;
+        r = rg + g;
+    }
+    __device__ __forceinline__ bool clamp(int &r, int &c) const {
+        const bool ok = c < cols && r < r1;
+        c = min(c, cols - 1);
+        r = min(r, r1 - 1);
+        return ok;
+    }
+};
+template <typename R>
+struct FromZ {  // column elements of the row-pass output
+    const OpView<R> &op;
+    const cpx<R> *Z;  // column c0
+    LineMap lm;
+    __device__ __forceinline__ cpx<R> operator()(int j, int b) const {
+        int r, c;
+        lm.at(b, r, c);
+        const bool ok = lm.clamp(r, c) && j < op.ny;
+        const cpx<R> z = Z[((size_t)r * op.ny + min(j, op.ny - 1)) * op.ncol + c];
+        return ok ? z : czero<cpx<R>>();
+    }
+};
+template <typename R>
+struct IntoSum {  // times the layer's spectrum, added to this thread's own entry of acc
+    const OpView<R> &op;
+    const cpx<R> *T;  // column c0
+    LineMap lm;
+    cpx<R> *acc;
+    int pitch;
+    bool first;
+    __device__ __forceinline__ cpx<R> pre(int n, int b) const {
+        int r, c;
+        lm.at(b, r, c);
+        lm.clamp(r, c);
+        return __ldg(T + ((size_t)r * op.Ny + n) * op.ncol + c);
+    }
+    __device__ __forceinline__ void operator()(int n, int b, cpx<R> x, cpx<R> t) const {
+        int r, c;
+        lm.at(b, r, c);
+        cpx<R> y = cmul(x, t);
+        if (!lm.clamp(r, c)) y = czero<cpx<R>>();
+        cpx<R> *a = acc + n * pitch + b;
+        *a = first ? y : cadd(*a, y);
+    }
+};
+template <typename R>
+struct FromVhat {  // conj(spectrum) times the residual's column transform
+    const OpView<R> &op;
+    const cpx<R> *T;
+    LineMap lm;
+    const cpx<R> *vh;
+    int pitch1;
+    __device__ __forceinline__ cpx<R> operator()(int k, int b) const {
+        int r, c;
+        lm.at(b, r, c);
+        const cpx<R> v = vh[k * pitch1 + c];
+        lm.clamp(r, c);
+        return cmulc(v, __ldg(T + ((size_t)r * op.Ny + k) * op.ncol + c));
+    }
+};
+
 template <typename R>
 __global__ void __launch_bounds__(256) k_col_fwd(OpView<R> op0, OpView<R> op1, ColShape cs, const int *done) {
     using Cx = cpx<R>;
@@ -419,7 +488,7 @@ __global__ void __launch_bounds__(256) k_col_fwd(OpView<R> op0, OpView<R> op1, C
     const OpView<R> &op = blockIdx.z ? op1 : op0;
     const int C = cs.C, G = cs.G, pitch = cs.pitch;
     const int c0 = blockIdx.x * C;
-    const int r0 = op.rbase + blockIdx.y * cs.L;
+    const int r0 = blockIdx.y * cs.L;
     if (r0 >= op.nz || c0 >= op.ncol) return;
     const int r1 = min(r0 + cs.L, op.nz);
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -433,17 +502,9 @@ __global__ void __launch_bounds__(256) k_col_fwd(OpView<R> op0, OpView<R> op1, C
     load_twiddles(tw, op.twy, N);
     bool first = true;
     for (int rg = r0; rg < r1; rg += G) {
-        auto in = [&](int j, int b) {
-            const int g = fast_div(b, cs.mC), c = b - g * C, r = rg + g;
-            return (j < ny && c < cols && r < r1) ? op.Z[((size_t)r * ny + j) * ncol + c0 + c] : czero<Cx>();
-        };
-        auto out = [&](int n, int b, Cx x) {
-            const int g = fast_div(b, cs.mC), c = b - g * C, r = rg + g;
-            Cx y = czero<Cx>();
-            if (c < cols && r < r1) y = cmul(x, __ldg(op.spec + ((size_t)(r - op.spec_r0) * N + n) * ncol + c0 + c));
-            Cx *a = acc + n * pitch + b;  // this thread's own entry in every layer group
-            *a = first ? y : cadd(*a, y);
-        };
+        const LineMap lm{cs.mC, C, cols, rg, r1};
+        const FromZ<R> in{op, op.Z + c0, lm};
+        const IntoSum<R> out{op, op.spec + c0, lm, acc, pitch, first};
         fft_run<R, false, true, false>(op.py, C * G, cs.mB, pitch, bufA, bufB, tw, ny, N, in, out);
         first = false;
         if (!(op.py.nst & 1)) { Cx *t = bufA; bufA = bufB; bufB = t; }  // the last stage may still be reading bufA
@@ -454,23 +515,17 @@ __global__ void __launch_bounds__(256) k_col_fwd(OpView<R> op0, OpView<R> op1, C
         for (int g = 1; g < G; ++g) y = cadd(y, acc[k * pitch + g * C + c]);
         return y;
     };
-    // Groups meet in Y in the order of the layers, so that a product repeats bit for bit:
-    // the groups of one launch in a slot each, summed by the last to arrive; the launches of
-    // the recompute mode (one layer each) add to slot 0 one after the other.
+    // The groups of a tile meet in Y, a slot each, and the last to arrive adds them in the
+    // order of the layers, so that a product repeats bit for bit.
     const size_t plane = (size_t)N * ncol;
     Cx *Yt = op.Y + c0;
     const int slots = cs.arrivals;
-    const bool before = cs.serial && r0 > 0;
-    if (cs.serial ? r1 < op.nz : slots > 1) {
-        Cx *Ys = Yt + (cs.serial ? 0 : blockIdx.y * plane);
+    if (slots > 1) {
+        Cx *Ys = Yt + blockIdx.y * plane;
         for (int it = threadIdx.x; it < N * C; it += blockDim.x) {
             const int k = fast_div(it, cs.mC), c = it - k * C;
-            if (c < cols) {
-                const Cx t = tile_sum(k, c);
-                Ys[(size_t)k * ncol + c] = before ? cadd(Ys[(size_t)k * ncol + c], t) : t;
-            }
+            if (c < cols) Ys[(size_t)k * ncol + c] = tile_sum(k, c);
         }
-        if (cs.serial) return;
         __threadfence();
         __syncthreads();
         if (threadIdx.x == 0) last_in = atomicAdd(op.cnt + blockIdx.x, 1) == slots - 1;
@@ -480,10 +535,8 @@ __global__ void __launch_bounds__(256) k_col_fwd(OpView<R> op0, OpView<R> op1, C
         if (threadIdx.x == 0) op.cnt[blockIdx.x] = 0;
     }
     auto in = [&](int k, int c) {
-        if (c >= cols) return czero<Cx>();
-        const Cx *y = Yt + (size_t)k * ncol + c;
-        if (cs.serial) return before ? cadd(*y, tile_sum(k, c)) : tile_sum(k, c);
         if (slots == 1) return tile_sum(k, c);
+        const Cx *y = Yt + (size_t)k * ncol + min(c, cols - 1);  // (an absent column's result is dropped)
         Cx t = __ldcg(y);
         for (int s = 1; s < slots; ++s) t = cadd(t, __ldcg(y + s * plane));
         return t;
@@ -504,7 +557,7 @@ __global__ void __launch_bounds__(256) k_col_adj(OpView<R> op0, OpView<R> op1, C
     const OpView<R> &op = blockIdx.z ? op1 : op0;
     const int C = cs.C, G = cs.G, pitch1 = cs.pitch1;
     const int c0 = blockIdx.x * C;
-    const int r0 = op.rbase + blockIdx.y * cs.L;
+    const int r0 = blockIdx.y * cs.L;
     if (c0 >= op.ncol || r0 >= op.nz) return;
     const int r1 = min(r0 + cs.L, op.nz);
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -517,19 +570,15 @@ __global__ void __launch_bounds__(256) k_col_adj(OpView<R> op0, OpView<R> op1, C
     load_twiddles(tw, op.twy, N);
     {
         auto in = [&](int j, int c) {
-            return (j < op.sy && c < cols) ? op.W[(size_t)j * ncol + c0 + c] : czero<Cx>();
+            const Cx w = op.W[(size_t)min(j, op.sy - 1) * ncol + c0 + min(c, cols - 1)];
+            return (j < op.sy && c < cols) ? w : czero<Cx>();
         };
         auto out = [&](int n, int c, Cx x) { vh[n * pitch1 + c] = x; };
         fft_run<R, false, true, false>(op.py, C, cs.mC, pitch1, bufA, bufB, tw, op.sy, N, in, out);
     }
     __syncthreads();
     for (int rg = r0; rg < r1; rg += G) {
-        auto in = [&](int k, int b) {
-            const int g = fast_div(b, cs.mC), c = b - g * C, r = rg + g;
-            return (c < cols && r < r1)
-                       ? cmulc(vh[k * pitch1 + c], __ldg(op.spec + ((size_t)(r - op.spec_r0) * N + k) * ncol + c0 + c))
-                       : czero<Cx>();
-        };
+        const FromVhat<R> in{op, op.spec + c0, LineMap{cs.mC, C, cols, rg, r1}, vh, pitch1};
         auto out = [&](int n, int b, Cx x) {
             const int g = fast_div(b, cs.mC), c = b - g * C, r = rg + g;
             if (n < ny && c < cols && r < r1) op.Z[((size_t)r * ny + n) * ncol + c0 + c] = x;
@@ -537,6 +586,124 @@ __global__ void __launch_bounds__(256) k_col_adj(OpView<R> op0, OpView<R> op1, C
         fft_run<R, true, false, true>(op.py, C * G, cs.mB, cs.pitch, bufA, bufB, tw, N, ny, in, out);
         if (!(op.py.nst & 1)) { Cx *t = bufA; bufA = bufB; bufB = t; }  // the last stage may still be reading bufA
     }
+}
+
+// ---------------------------------------------------------------------------
+// Column passes of the recompute mode, one layer a launch: the FP64 column transform of
+// the layer's table rows (Zs) gives the layer's spectrum of a tile of C columns, which is
+// rounded to R, used at once and never leaves the CTA.  The FP64 part keeps the SM's two
+// FP64 lanes busy and the R part of other CTAs runs beside it.
+// even: the table is even in both offsets, so its row spectra are real and even in y: Zs
+// holds the rows 0 .. Ny/2, and two columns share one complex transform.
+
+struct RecShape {
+    int C, lines;  // columns per CTA; FP64 lines (C, or C / 2 when even)
+    unsigned mC, mlines;
+    int even;
+    int buf;  // bytes of a transform buffer: N lines FP64 or N C values of R
+};
+
+template <typename R>
+__device__ __forceinline__ void layer_spectrum(const OpView<R> &op, const RecShape &rs, int c0, int cols,
+                                               const double2 *Zs, double2 *bufA, double2 *bufB, const double2 *tw64,
+                                               cpx<R> *S) {
+    const int N = op.Ny, ncol = op.ncol, C = rs.C;
+    const double2 *Z = Zs + c0;
+    auto in = [&](int j, int l) {
+        if (rs.even) {
+            const double2 *row = Z + (size_t)(2 * j > N ? N - j : j) * ncol;
+            return make_double2(__ldg(&row[min(2 * l, cols - 1)].x), __ldg(&row[min(2 * l + 1, cols - 1)].x));
+        }
+        return __ldg(Z + (size_t)j * ncol + min(l, cols - 1));
+    };
+    auto out = [&](int k, int l, double2 x) {
+        if (rs.even) {
+            S[k * C + 2 * l] = mk<cpx<R>>((R)x.x, R(0));
+            S[k * C + 2 * l + 1] = mk<cpx<R>>((R)x.y, R(0));
+        } else {
+            S[k * C + l] = mk<cpx<R>>((R)x.x, (R)x.y);
+        }
+    };
+    fft_run<double, false, false, false>(op.py, rs.lines, rs.mlines, rs.lines, bufA, bufB, tw64, N, N, in, out);
+    __syncthreads();
+}
+
+// Y (+)= T^_r . FFT_y(Z_r); the first layer writes Y.
+template <typename R>
+struct IntoY {
+    cpx<R> *Y;  // column c0
+    const cpx<R> *S;
+    int ncol, C, cols, first;
+    __device__ __forceinline__ cpx<R> pre(int n, int c) const { return Y[(size_t)n * ncol + min(c, cols - 1)]; }
+    __device__ __forceinline__ void operator()(int n, int c, cpx<R> x, cpx<R> y) const {
+        const cpx<R> p = cmul(x, S[n * C + c]);
+        if (c < cols) Y[(size_t)n * ncol + c] = first ? p : cadd(y, p);
+    }
+};
+
+template <typename R>
+__global__ void __launch_bounds__(256) k_col_rec_fwd(OpView<R> op, RecShape rs, const double2 *Zs,
+                                                     const double2 *twy64, int r) {
+    using Cx = cpx<R>;
+    const int N = op.Ny, C = rs.C, c0 = blockIdx.x * C, cols = min(C, op.ncol - c0);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned char *bufA = smem_raw, *bufB = bufA + rs.buf;
+    double2 *tw64 = reinterpret_cast<double2 *>(bufB + rs.buf);
+    Cx *S = reinterpret_cast<Cx *>(tw64 + N), *tw = S + N * C;
+    load_twiddles(tw64, twy64, N);
+    load_twiddles(tw, op.twy, N);
+    layer_spectrum<R>(op, rs, c0, cols, Zs, reinterpret_cast<double2 *>(bufA), reinterpret_cast<double2 *>(bufB), tw64,
+                      S);
+    const FromZ<R> in{op, op.Z + c0, LineMap{rs.mC, C, cols, r, r + 1}};
+    const IntoY<R> out{op.Y + c0, S, op.ncol, C, cols, r == 0};
+    fft_run<R, false, true, false>(op.py, C, rs.mC, C, reinterpret_cast<Cx *>(bufA), reinterpret_cast<Cx *>(bufB), tw,
+                                   op.ny, N, in, out);
+}
+
+// Z_r = IFFT_y(conj(T^_r) . Y), rows iy < ny (Y = FFT_y of the residual rows).
+template <typename R>
+__global__ void __launch_bounds__(256) k_col_rec_adj(OpView<R> op, RecShape rs, const double2 *Zs,
+                                                     const double2 *twy64, int r) {
+    using Cx = cpx<R>;
+    const int N = op.Ny, C = rs.C, c0 = blockIdx.x * C, cols = min(C, op.ncol - c0), ncol = op.ncol, ny = op.ny;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned char *bufA = smem_raw, *bufB = bufA + rs.buf;
+    double2 *tw64 = reinterpret_cast<double2 *>(bufB + rs.buf);
+    Cx *S = reinterpret_cast<Cx *>(tw64 + N), *tw = S + N * C;
+    load_twiddles(tw64, twy64, N);
+    load_twiddles(tw, op.twy, N);
+    layer_spectrum<R>(op, rs, c0, cols, Zs, reinterpret_cast<double2 *>(bufA), reinterpret_cast<double2 *>(bufB), tw64,
+                      S);
+    const Cx *Y = op.Y + c0;
+    Cx *Z = op.Z + (size_t)r * ny * ncol + c0;
+    auto in = [&](int k, int c) { return cmulc(Y[(size_t)k * ncol + min(c, cols - 1)], S[k * C + c]); };
+    auto out = [&](int n, int c, Cx x) {
+        if (n < ny && c < cols) Z[(size_t)n * ncol + c] = x;
+    };
+    fft_run<R, true, false, true>(op.py, C, rs.mC, C, reinterpret_cast<Cx *>(bufA), reinterpret_cast<Cx *>(bufB), tw,
+                                  N, ny, in, out);
+}
+
+// One column transform of the whole plane: Y = FFT_y(W) (W has sy rows) or, INV,
+// W = IFFT_y(Y) cropped to sy rows.
+template <typename R, bool INV>
+__global__ void __launch_bounds__(256) k_col_plane(OpView<R> op, ColShape cs) {
+    using Cx = cpx<R>;
+    const int N = op.Ny, C = cs.C, c0 = blockIdx.x * C, cols = min(C, op.ncol - c0), ncol = op.ncol, sy = op.sy;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Cx *bufA = reinterpret_cast<Cx *>(smem_raw), *bufB = bufA + N * cs.pitch1, *tw = bufB + N * cs.pitch1;
+    load_twiddles(tw, op.twy, N);
+    const Cx *src = (INV ? op.Y : op.W) + c0;
+    Cx *dst = (INV ? op.W : op.Y) + c0;
+    const int rows_in = INV ? N : sy, rows_out = INV ? sy : N;
+    auto in = [&](int j, int c) {
+        const Cx w = src[(size_t)min(j, rows_in - 1) * ncol + min(c, cols - 1)];
+        return j < rows_in ? w : czero<Cx>();
+    };
+    auto out = [&](int n, int c, Cx x) {
+        if (n < rows_out && c < cols) dst[(size_t)n * ncol + c] = x;
+    };
+    fft_run<R, INV, !INV, INV>(op.py, C, cs.mC, cs.pitch1, bufA, bufB, tw, rows_in, rows_out, in, out);
 }
 
 }  // namespace gj

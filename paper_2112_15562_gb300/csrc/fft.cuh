@@ -16,6 +16,7 @@
 // Forward transforms use exp(-2 pi i jk/N); inverse ones are unnormalised.
 #pragma once
 #include <type_traits>
+#include <utility>
 
 #include "common.cuh"
 
@@ -46,6 +47,9 @@ __device__ __forceinline__ int fast_div(int n, unsigned m) { return m ? (int)__u
 // ---------------------------------------------------------------------------
 // Roots of unity as compile-time constants: sine and cosine of 2 pi K / N by their
 // Taylor series on the first octant (|x| <= pi/4: 13 terms leave less than 1e-26).
+
+// sqrt(2)/2
+template <typename R> __host__ __device__ constexpr R rsqrt2() { return R(0.70710678118654752440084436210485); }
 
 constexpr double root_sin_series(double x) {
     const double q = x * x;
@@ -93,7 +97,15 @@ __device__ __forceinline__ cpx<R> rot(cpx<R> a) {
     else if constexpr (2 * k == N) return mk<C>(-a.x, -a.y);
     else if constexpr (4 * k == N) return mul_mi<C, INV>(a);
     else if constexpr (4 * k == 3 * N) return mul_mi<C, !INV>(a);
-    else {
+    else if constexpr (8 * k % N == 0) {
+        // (+-1 -+ i) / sqrt 2: two additions, and the factor joins the additions that follow
+        constexpr R h = rsqrt2<R>();
+        constexpr int o = 8 * k / N;  // 1, 3, 5, 7
+        constexpr bool re = o == 1 || o == 7, im = (o == 1 || o == 3) == INV;  // signs of the root's parts
+        const R x = re == im ? a.x - a.y : a.x + a.y, y = re == im ? a.x + a.y : a.x - a.y;
+        // a (c + i d) with |c| = |d| = h: (c a.x - d a.y, d a.x + c a.y)
+        return mk<C>(re ? h * x : -h * x, im ? h * y : -h * y);
+    } else {
         constexpr R wr = (R)Root<k, N>::c, wi = (R)(INV ? Root<k, N>::s : -Root<k, N>::s);
         return mk<C>(a.x * wr - a.y * wi, a.x * wi + a.y * wr);
     }
@@ -238,6 +250,20 @@ __device__ __forceinline__ void dft(cpx<R> (&v)[RAD]) {
 // ones from r = (RAD + 1) / 2 on are absent when valid <= M (RAD + 1) / 2
 __device__ __forceinline__ bool half_enough(const FftStage &s, int valid) { return valid <= s.M * ((s.rad + 1) / 2); }
 
+// A sink with a member pre(n, b) has it called for every output before the inputs are
+// read: its loads are in flight during the butterfly.  The result is handed back to it.
+struct NoPre {};
+template <class Out, class = void> struct PreOf {
+    using T = NoPre;
+    static __device__ __forceinline__ T load(const Out &, int, int) { return T{}; }
+    template <class C> static __device__ __forceinline__ void store(const Out &out, int n, int b, C x, T) { out(n, b, x); }
+};
+template <class Out> struct PreOf<Out, decltype((void)&Out::pre)> {
+    using T = decltype(std::declval<const Out &>().pre(0, 0));
+    static __device__ __forceinline__ T load(const Out &out, int n, int b) { return out.pre(n, b); }
+    template <class C> static __device__ __forceinline__ void store(const Out &out, int n, int b, C x, T t) { out(n, b, x, t); }
+};
+
 template <typename R, int RAD, bool INV, bool TW, bool HIN, bool HOUT, class In, class Out>
 __device__ __forceinline__ void fft_stage(const FftStage &s, int B, unsigned mB, const cpx<R> *tw, const In &in,
                                           const Out &out) {
@@ -248,6 +274,10 @@ __device__ __forceinline__ void fft_stage(const FftStage &s, int B, unsigned mB,
     for (int it = threadIdx.x; it < total; it += blockDim.x) {
         const int j = fast_div(it, mB), b = it - j * B;
         const int k = TW ? j - fast_div(j, s.mNs) * s.Ns : 0;
+        const int d0 = (j - k) * RAD + k;
+        typename PreOf<Out>::T t[RAD];
+#pragma unroll
+        for (int r = 0; r < NO; ++r) t[r] = PreOf<Out>::load(out, d0 + r * s.Ns, b);
         C v[RAD];
 #pragma unroll
         for (int r = 0; r < RAD; ++r) v[r] = r < NZ ? in(j + r * s.M, b) : czero<C>();
@@ -257,9 +287,8 @@ __device__ __forceinline__ void fft_stage(const FftStage &s, int B, unsigned mB,
             for (int r = 1; r < RAD; ++r) v[r] = INV ? cmulc(v[r], tw[r * e]) : cmul(v[r], tw[r * e]);
         }
         dft<R, RAD, INV, NZ>(v);
-        const int d0 = (j - k) * RAD + k;
 #pragma unroll
-        for (int r = 0; r < NO; ++r) out(d0 + r * s.Ns, b, v[r]);
+        for (int r = 0; r < NO; ++r) PreOf<Out>::store(out, d0 + r * s.Ns, b, v[r], t[r]);
     }
 }
 

@@ -52,6 +52,31 @@ void gen_col_adj(const gj_op *o, const OpView<R> &v0, const OpView<R> &v1, int n
                    col_smem(o->Ny, s.pitch, s.pitch1, sizeof(cpx<R>)), st>>>(v0, v1, s, done);
 }
 
+template <typename R> void gen_rec_attr() {
+    allow_max_smem(k_col_rec_fwd<R>);
+    allow_max_smem(k_col_rec_adj<R>);
+    allow_max_smem(k_col_plane<R, false>);
+    allow_max_smem(k_col_plane<R, true>);
+}
+template <typename R> void gen_rec_fwd(const gj_op *o, const OpView<R> &v, int r, cudaStream_t st) {
+    const RecShape s = rec_shape(o->py, o->even_rows, sizeof(cpx<R>));
+    k_col_rec_fwd<R><<<(o->ncol + s.C - 1) / s.C, gen_threads(o->py.mmax, s.C), rec_smem(s, o->Ny, sizeof(cpx<R>)),
+                    st>>>(v, s, recompute_rows_out(o), recompute_twy64(o), r);
+}
+template <typename R> void gen_rec_adj(const gj_op *o, const OpView<R> &v, int r, cudaStream_t st) {
+    const RecShape s = rec_shape(o->py, o->even_rows, sizeof(cpx<R>));
+    k_col_rec_adj<R><<<(o->ncol + s.C - 1) / s.C, gen_threads(o->py.mmax, s.C), rec_smem(s, o->Ny, sizeof(cpx<R>)),
+                    st>>>(v, s, recompute_rows_out(o), recompute_twy64(o), r);
+}
+template <typename R> void gen_rec_plane(const gj_op *o, const OpView<R> &v, bool inverse, cudaStream_t st) {
+    const ColShape s = col_shape(o, 1, 1, sizeof(cpx<R>), true);
+    const dim3 g((o->ncol + s.C - 1) / s.C);
+    const int T = gen_threads(o->py.mmax, s.C);
+    const size_t sm = (size_t)(2 * s.pitch1 + 1) * o->Ny * sizeof(cpx<R>);
+    if (inverse) k_col_plane<R, true><<<g, T, sm, st>>>(v, s);
+    else k_col_plane<R, false><<<g, T, sm, st>>>(v, s);
+}
+
 }  // namespace gj
 
 // Explicit instantiations.
@@ -73,3 +98,8 @@ void gen_col_adj(const gj_op *o, const OpView<R> &v0, const OpView<R> &v1, int n
                                  cudaStream_t);                                                                  \
     template void gen_col_adj<R>(const gj_op *, const OpView<R> &, const OpView<R> &, int, int, const int *,     \
                                  cudaStream_t);
+#define GJ_RECOMPUTE(R)                                                                     \
+    template void gen_rec_attr<R>();                                                        \
+    template void gen_rec_fwd<R>(const gj_op *, const OpView<R> &, int, cudaStream_t);      \
+    template void gen_rec_adj<R>(const gj_op *, const OpView<R> &, int, cudaStream_t);      \
+    template void gen_rec_plane<R>(const gj_op *, const OpView<R> &, bool, cudaStream_t);

@@ -9,6 +9,7 @@ namespace gj {
 constexpr int kGenThreads = 256;             // most threads of a CTA
 constexpr size_t kGenSmem = 100 * 1024;      // shared memory up to which a shape may grow: two CTAs an SM
 constexpr int kGenCtas = 304;                // CTAs worth having in flight: two an SM
+constexpr int kGenGroups = 10;               // most layer groups of a column tile (partial sums to keep and to add)
 
 inline int gen_threads(int mmax, int lines) {
     const int t = (mmax * lines + 31) / 32 * 32;
@@ -51,38 +52,46 @@ inline int pick_layer_lines(const FftPlanDev &pl, int C, int L, size_t cs) {
     return G < 1 ? 1 : G;
 }
 
-// Layers per CTA: all of them when the column tiles alone fill the GPU (the layer sum
-// then never leaves the CTA), else so few that the CTAs do, but no fewer than a CTA takes
-// at a time.
-inline int pick_layers(const FftPlanDev &pl, int C, int tiles, int nz, size_t cs) {
-    const int G = pick_layer_lines(pl, C, nz, cs);
-    int groups = (kGenCtas + tiles - 1) / tiles;
-    if (groups > (nz + G - 1) / G) groups = (nz + G - 1) / G;
-    return (nz + groups - 1) / groups;
-}
-
-// Columns per CTA: a column tile's rows should fill 32-byte sectors (4 FP32 or 2 FP64
-// columns) when there are enough tiles and layers to fill the GPU, one column when not.
-inline int pick_col_tile(const FftPlanDev &pl, int ncol, int nz, int nf, size_t cs) {
-    int C = 8;
-    while (C > 1 && (C * pl.mmax > kGenThreads || col_smem(pl.N, odd_pitch(C), odd_pitch(C), cs) > kGenSmem)) C /= 2;
-    while (C > 1) {
-        const long long tiles = (long long)((ncol + C - 1) / C) * nf;
-        const int G = pick_layer_lines(pl, C, nz, cs);
-        if (tiles * ((nz + G - 1) / G) >= kGenCtas) break;
-        C /= 2;
+// Columns and layers per CTA of a column pass over nz layers of nf fields, by the time the
+// pass should take: every SM works off its CTAs, each ceil(L / G) group transforms and one
+// more (the residual's or the sum's), and a group transform takes its instructions' time
+// (FP64: the two lanes an SM has for it) or, when an SM has little to do, a chain of
+// latencies.  Fewer columns waste sectors of the layer spectra and intermediates (32 bytes
+// are four FP32 or two FP64 columns).  Fixed values (from gj_op_tune) are kept when positive.
+struct ColPick { int C, L; };
+inline ColPick pick_cols(const FftPlanDev &pl, int ncol, int nz, int nf, size_t cs, int fixC = 0, int fixL = 0) {
+    const bool wide = cs == 16;  // complex doubles
+    ColPick best{1, nz};
+    double least = 1e300;
+    for (int C = fixC > 0 ? fixC : 1; C <= (fixC > 0 ? fixC : 8); C *= 2) {
+        if (fixC <= 0 && C > 1 && (C * pl.mmax > kGenThreads || C >= 2 * ncol ||
+                                   col_smem(pl.N, odd_pitch(C), odd_pitch(C), cs) > kGenSmem))
+            break;
+        const double waste = wide ? (C == 1 ? 1.2 : 1.0) : (C == 1 ? 1.6 : C == 2 ? 1.25 : C == 4 ? 1.05 : 1.0);
+        const int tiles = (ncol + C - 1) / C * nf;
+        for (int groups = 1; groups <= nz && groups <= kGenGroups; ++groups) {
+            const int L = fixL > 0 ? (fixL < nz ? fixL : nz) : (nz + groups - 1) / groups;
+            const int G = pick_layer_lines(pl, C, L, cs);
+            const int ctas = tiles * ((nz + L - 1) / L);
+            const int per_sm = (ctas + 151) / 152;
+            const double work = (double)pl.N * C * G * (wide ? 15.0 : 0.5) / 1900.0, latency = 2.5;  // microseconds
+            const double t = ((L + G - 1) / G + 1) * std::max(per_sm * work * waste + 1.5 / per_sm, latency) +
+                             (ctas > tiles ? 1.0 + 0.2 * (ctas / tiles) : 0.0);
+            if (t < 0.98 * least) { least = t; best = ColPick{C, L}; }
+            if (fixL > 0) break;
+        }
     }
-    return C;
+    return best;
 }
 
-// layers: of the launch (1 in the recompute mode, whose launches share one sum)
 inline ColShape col_shape(const gj_op *o, int nf, int layers, size_t cs, bool adjoint) {
     ColShape s;
-    s.C = o->cols_tuned ? o->C_col : pick_col_tile(o->py, o->ncol, layers, nf, cs);
-    const int tiles = (o->ncol + s.C - 1) / s.C * nf;
-    s.L = o->layers_tuned ? std::min(o->L_grp, layers) : pick_layers(o->py, s.C, tiles, layers, cs);
+    const ColPick pick =
+        pick_cols(o->py, o->ncol, layers, nf, cs, o->cols_tuned ? o->C_col : 0, o->layers_tuned ? o->L_grp : 0);
+    s.C = pick.C;
+    s.L = pick.L;
     // the forward sums have room for gen_slots groups
-    if (!adjoint && !o->recompute) s.L = std::max(s.L, (layers + o->gen_slots - 1) / o->gen_slots);
+    if (!adjoint) s.L = std::max(s.L, (layers + o->gen_slots - 1) / o->gen_slots);
     s.G = pick_layer_lines(o->py, s.C, s.L, cs);
     const int B = s.C * s.G;
     const bool pad = col_smem(o->Ny, odd_pitch(B), adjoint ? odd_pitch(s.C) : odd_pitch(B), cs) <= kGenSmemMax;
@@ -91,7 +100,6 @@ inline ColShape col_shape(const gj_op *o, int nf, int layers, size_t cs, bool ad
     s.mB = div_magic(B);
     s.mC = div_magic(s.C);
     s.arrivals = (layers + s.L - 1) / s.L;
-    s.serial = o->recompute ? 1 : 0;
     return s;
 }
 
@@ -117,5 +125,30 @@ void gen_col_fwd(const gj_op *o, const OpView<R> &v0, const OpView<R> &v1, int n
 template <typename R>
 void gen_col_adj(const gj_op *o, const OpView<R> &v0, const OpView<R> &v1, int nf, int layers, const int *done,
                  cudaStream_t st);
+
+// Columns per CTA of the recompute mode's column passes (RecShape): two FP64 lines where
+// they fit two CTAs an SM.
+inline size_t rec_smem(const RecShape &s, int N, size_t cs) {
+    return 2 * (size_t)s.buf + (size_t)N * sizeof(double2) + (size_t)(s.C + 1) * N * cs;
+}
+inline RecShape rec_shape(const FftPlanDev &pl, bool even, size_t cs) {
+    RecShape s;
+    s.even = even ? 1 : 0;
+    for (s.lines = 2;; s.lines = 1) {
+        s.C = even ? 2 * s.lines : s.lines;
+        s.buf = pl.N * (int)std::max(s.lines * sizeof(double2), s.C * cs);
+        if (s.lines == 1 || (s.lines * pl.mmax <= kGenThreads && rec_smem(s, pl.N, cs) <= kGenSmem)) break;
+    }
+    s.mC = div_magic(s.C);
+    s.mlines = div_magic(s.lines);
+    return s;
+}
+
+// Recompute mode: layer r's launches after recompute_rows (FP64 rows of the layer's table in
+// Zs), and the one transform per product of the residual's or the summed spectrum's columns.
+template <typename R> void gen_rec_attr();
+template <typename R> void gen_rec_fwd(const gj_op *o, const OpView<R> &v, int r, cudaStream_t st);
+template <typename R> void gen_rec_adj(const gj_op *o, const OpView<R> &v, int r, cudaStream_t st);
+template <typename R> void gen_rec_plane(const gj_op *o, const OpView<R> &v, bool inverse, cudaStream_t st);
 
 }  // namespace gj

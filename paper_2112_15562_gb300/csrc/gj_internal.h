@@ -46,6 +46,8 @@ struct gj_op {
     // per-layer spectrum recomputation (GJ_SETUP_RECOMPUTE_SPECTRA): `spec` holds one
     // layer, rebuilt from the closed forms before each use
     bool recompute = false;
+    bool even_table = false;  // the table is even in both offsets: its spectrum is real and even
+    bool even_rows = false;   // recompute mode: an even table's transforms share rows and columns
     gj::gj_setup_scratch_impl *scratch = nullptr;
     int slots = 0;
     int col_grid = 0;      // CTAs of the persistent column kernels
@@ -70,8 +72,12 @@ int fast_col_items(int Ny, int nz);  // items per column of the fast column kern
 int fast_slots(int nfield, int ncol, int items_per_col, long long warps);
 bool fast1024_eligible(const gj_op *op);
 
-// rebuilds layer r's spectrum into spec (recompute mode; setup.cu)
-void recompute_layer(const gj_op *op, int r, cudaStream_t st);
+// recompute mode (setup.cu): the corner lattice of every depth plane, once per product;
+// then layer r's table and its FP64 row transforms, and where those are
+void recompute_begin(const gj_op *op, cudaStream_t st);
+void recompute_rows(const gj_op *op, int r, cudaStream_t st);
+const double2 *recompute_rows_out(const gj_op *op);
+const double2 *recompute_twy64(const gj_op *op);
 
 // enqueue products (matvec.cu)
 gj_status forward_enqueue(const gj_op *op, const void *m, void *d, cudaStream_t s);

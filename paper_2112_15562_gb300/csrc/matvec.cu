@@ -22,14 +22,14 @@ static void general_forward(const gj_op *a, const gj_op *b, const R *m0, const R
     gen_row_fwd<R>(a, v0, PairMap{a->nz * a->ny, 0, 0}, a->nx, v0.Z, v1.Z, LoadPlain2<R>{{m0, m1}, a->nx}, nullptr, st,
                    nf);
     if (a->recompute) {
-        // one layer at a time: rebuild its spectrum, then add its column products
+        // one layer at a time: rebuild its spectrum and add its column products
+        gen_rec_attr<R>();
+        recompute_begin(a, st);
         for (int r = 0; r < a->nz; ++r) {
-            recompute_layer(a, r, st);
-            OpView<R> vr = v0;
-            vr.rbase = r;
-            vr.spec_r0 = r;
-            gen_col_fwd<R>(a, vr, vr, 1, 1, nullptr, st);
+            recompute_rows(a, r, st);
+            gen_rec_fwd<R>(a, v0, r, st);
         }
+        gen_rec_plane<R>(a, v0, true, st);
     } else {
         gen_col_fwd<R>(a, v0, v1, nf, a->nz, nullptr, st);
     }
@@ -43,12 +43,12 @@ static void general_adjoint(const gj_op *a, const gj_op *b, const R *r0, const R
     const OpView<R> v0 = view_of<R>(a), v1 = view_of<R>(b ? b : a);
     gen_row_fwd<R>(a, v0, PairMap{a->sy, 0, 0}, a->sx, v0.W, v1.W, LoadPlain2<R>{{r0, r1}, a->sx}, nullptr, st, nf);
     if (a->recompute) {
+        gen_rec_attr<R>();
+        gen_rec_plane<R>(a, v0, false, st);
+        recompute_begin(a, st);
         for (int r = 0; r < a->nz; ++r) {
-            recompute_layer(a, r, st);
-            OpView<R> vr = v0;
-            vr.rbase = r;
-            vr.spec_r0 = r;
-            gen_col_adj<R>(a, vr, vr, 1, 1, nullptr, st);
+            recompute_rows(a, r, st);
+            gen_rec_adj<R>(a, v0, r, st);
         }
     } else {
         gen_col_adj<R>(a, v0, v1, nf, a->nz, nullptr, st);

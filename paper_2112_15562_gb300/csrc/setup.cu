@@ -90,109 +90,147 @@ __constant__ double kGL3w[3] = {0.55555555555555555556, 0.88888888888888888889, 
 // + 3 (c3 uv + c4 uw + c5 vw)) / R^5 (magnetic), by an n-point tensor rule in
 // precision F.  The integrand is smooth there and the sum has no cancellation to
 // speak of, so for an FP32 operator (whose spectra are rounded to FP32) the rule runs
-// in FP32, some 30 times the FP64 rate; FP64 operators keep FP64.
+// in FP32, some 60 times the FP64 rate; FP64 operators keep FP64.
+// The parts that keep their sign, or change it, when u or v does come out apart, so
+// that one evaluation serves the offsets (+-u, +-v): part[0] + su sv part[1] + su part[2]
+// + sv part[3] (gravity: part[0] alone).
 template <typename F> __device__ __forceinline__ F rsqrt_t(F x);
 template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return rsqrt(x); }
 template <> __device__ __forceinline__ float rsqrt_t<float>(float x) { return rsqrtf(x); }
 
 template <int NP, typename F>
-__device__ double far_cubature(double uc_, double hu_, double vc_, double hv_, double wc_, double hw_, int magnetic,
-                               const MagCoef &k) {
+__device__ __forceinline__ void far_cubature(F uc, F hu, F vc, F hv, F wc, F hw, int magnetic, const MagCoef &k,
+                                             F (&part)[4]) {
     const double *x = NP == 5 ? kGL5x : (NP == 4 ? kGL4x : kGL3x);
     const double *wt = NP == 5 ? kGL5w : (NP == 4 ? kGL4w : kGL3w);
-    const F uc = (F)uc_, hu = (F)hu_, vc = (F)vc_, hv = (F)hv_, wc = (F)wc_, hw = (F)hw_;
-    const F c0 = (F)k.c[0], c1 = (F)k.c[1], c2 = (F)k.c[2], c3 = (F)k.c[3], c4 = (F)k.c[4], c5 = (F)k.c[5];
-    F s = 0;
+    const F c0 = (F)k.c[0], c1 = (F)k.c[1], c2 = (F)k.c[2], tr = (F)(k.c[0] + k.c[1] + k.c[2]);
+    F s0 = 0, suv = 0, su = 0, sv = 0;
 #pragma unroll
     for (int a = 0; a < NP; ++a) {
         const F u = uc + hu * (F)x[a];
 #pragma unroll
         for (int b = 0; b < NP; ++b) {
             const F v = vc + hv * (F)x[b];
-            F sw = 0;
+            const F uv2 = u * u + v * v, wab = (F)(wt[a] * wt[b]);
+            F i3 = 0, i5 = 0, i5w = 0, i5ww = 0;  // sums over w of 1/R^3, 1/R^5, w/R^5, w^2/R^5 (gravity: w/R^3 in i3)
 #pragma unroll
             for (int c = 0; c < NP; ++c) {
                 const F w = wc + hw * (F)x[c];
-                const F r2 = u * u + v * v + w * w;
-                const F ir = rsqrt_t<F>(r2);
-                const F ir3 = ir * ir * ir;
-                F f;
+                const F ir = rsqrt_t<F>(uv2 + w * w);
+                const F ir2 = ir * ir, g3 = (F)wt[c] * ir * ir2;
                 if (magnetic) {
-                    const F q = c0 * (F(3) * u * u - r2) + c1 * (F(3) * v * v - r2) + c2 * (F(3) * w * w - r2) +
-                                F(3) * (c3 * u * v + c4 * u * w + c5 * v * w);
-                    f = q * ir3 * ir * ir;
+                    const F g5 = g3 * ir2, g5w = g5 * w;
+                    i3 += g3;
+                    i5 += g5;
+                    i5w += g5w;
+                    i5ww += g5w * w;
                 } else {
-                    f = w * ir3;
+                    i3 += g3 * w;
                 }
-                sw += (F)wt[c] * f;
             }
-            s += (F)(wt[a] * wt[b]) * sw;
+            if (magnetic) {
+                s0 += wab * (F(3) * ((c0 * u * u + c1 * v * v) * i5 + c2 * i5ww) - tr * i3);
+                suv += wab * (u * v) * i5;
+                su += wab * u * i5w;
+                sv += wab * v * i5w;
+            } else {
+                s0 += wab * i3;
+            }
         }
     }
-    return (double)s * hu_ * hv_ * hw_;
+    part[0] = s0;
+    part[1] = F(3) * (F)k.c[3] * suv;
+    part[2] = F(3) * (F)k.c[4] * su;
+    part[3] = F(3) * (F)k.c[5] * sv;
 }
 
-// Row-pass input of the setup: the circulant embedding of layer r's table,
-// T[c_y mod Ny][c_x mod Nx] = K(c_y + off_y, c_x + off_x) for c in
-// [-(n-1), s-1], zero elsewhere; K is the 8-corner sum of the lattice, or the
-// far-field cubature.
-struct LoadTable {
-    static constexpr int STAGE_U = 1;  // the fetch is the corner differences and the far-field cubature
+// Depth range of a layer (centre and half height below the stations), its squared
+// near-field radius, and the cubature's volume element times the scale of the spectra.
+struct LayerGeom { double wc, hw, near2, vol; };
+
+// The circulant tables of a build's layers, T[c_y mod Ny][c_x mod Nx] =
+// K(c_y + off_y, c_x + off_x) for c in [-(n-1), s-1] (the rest is not written: the row
+// pass takes it as zero).  K is the 8-corner sum of the lattice, or the far-field cubature.
+struct TableGeom {
     const double *lat;
-    int nbx1, nby1;
+    int nbx1, nby1, k0;  // lattice points, and the lattice plane of the build's first layer
     int Nx, Ny, sx, sy, nx, ny, off_x, off_y, a_max, b_max;
+    int a0, na, b0, nb;  // |c + off| runs over [a0, a0 + na) along y and [b0, b0 + nb) along x
     double scale;
-    double dx, dy;
-    const double *zw;  // depth planes of the build's layers (relative to the stations)
+    const double *axis;       // prism centres -|c + off| cell: [nb] along x, then [na] along y
+    const LayerGeom *layer;   // of the build's first layer
+    double hu, hv;            // half cells
     int magnetic;
-    int far32;  // far-field cubature in FP32 (FP32 operators)
     MagCoef mc;
-    template <typename F> __device__ double far(double uc, double vc, double wc, double hw, double dist,
-                                                double size) const {
-        return dist < 3.0 * kFar * size ? far_cubature<5, F>(uc, 0.5 * dx, vc, 0.5 * dy, wc, hw, magnetic, mc)
-             : dist < 8.0 * kFar * size ? far_cubature<4, F>(uc, 0.5 * dx, vc, 0.5 * dy, wc, hw, magnetic, mc)
-                                        : far_cubature<3, F>(uc, 0.5 * dx, vc, 0.5 * dy, wc, hw, magnetic, mc);
-    }
-    __device__ void init() {}
-    __device__ double value(int line, int j) const {
-        const int r = line / Ny, iy = line % Ny;
-        int cy, cx;
-        if (iy <= sy - 1) cy = iy; else if (iy >= Ny - (ny - 1)) cy = iy - Ny; else return 0.0;
-        if (j <= sx - 1) cx = j; else if (j >= Nx - (nx - 1)) cx = j - Nx; else return 0.0;
-        {
-            // the prism spans u in [-(cx + off_x) -+ 1/2] dx, v likewise, w in [zw[r], zw[r + 1]]
-            const double uc = -(double)(cx + off_x) * dx, vc = -(double)(cy + off_y) * dy;
-            const double w1 = zw[r], w2 = zw[r + 1];
-            const double wc = 0.5 * (w1 + w2), hw = 0.5 * (w2 - w1);
-            const double size = fmax(fmax(dx, dy), w2 - w1);
-            const double dist = sqrt(uc * uc + vc * vc + wc * wc);
-            if (dist >= kFar * size) {
-                const double v = far32 ? far<float>(uc, vc, wc, hw, dist, size) : far<double>(uc, vc, wc, hw, dist, size);
-                return v * scale;
+};
+
+// 8-corner sum at offsets (cy + off_y, cx + off_x) = (a, b), inside the lattice window
+__device__ __forceinline__ double corner_sum(const TableGeom &G, int r, int a, int b) {
+    const int e = G.b_max - b, f = G.a_max - a;
+    double s = 0.0;
+#pragma unroll
+    for (int dk = 0; dk < 2; ++dk)
+#pragma unroll
+        for (int df = 0; df < 2; ++df)
+#pragma unroll
+            for (int de = 0; de < 2; ++de) {
+                const double t = G.lat[((size_t)(G.k0 + r + dk) * G.nby1 + (f + df)) * G.nbx1 + (e + de)];
+                s += ((de + df + dk) & 1) ? t : -t;
             }
+    return s;
+}
+
+// One thread per (|a|, |b|) of a layer writes up to four entries.  The FP64 units of this
+// GPU do two operations a cycle and SM, so an entry's address, distance and rule must not
+// use them: evaluated entry by entry with FP64 distances inside the row transforms, a
+// 1023 x 1023 layer took 130 of the row pass's 190 us for an FP32 operator.
+template <typename F>
+__global__ void __launch_bounds__(128) k_table(TableGeom G, double *T) {
+    const int ib = blockIdx.x * blockDim.x + threadIdx.x;
+    const int ia = blockIdx.y, r = blockIdx.z;
+    if (ib >= G.nb) return;
+    const int a = G.a0 + ia, b = G.b0 + ib;
+    const LayerGeom lg = G.layer[r];
+    // offset (a, b) sees the prism centred at u = -b dx, v = -a dy
+    const F uc = (F)G.axis[ib], vc = (F)G.axis[G.nb + ia], wc = (F)lg.wc, hw = (F)lg.hw;
+    const F d2 = uc * uc + vc * vc + wc * wc, near2 = (F)lg.near2;
+    const bool far = d2 >= near2;
+    F part[4] = {0, 0, 0, 0};
+    if (far) {
+        const F hu = (F)G.hu, hv = (F)G.hv;
+        if (d2 < F(9) * near2) far_cubature<5, F>(uc, hu, vc, hv, wc, hw, G.magnetic, G.mc, part);
+        else if (d2 < F(64) * near2) far_cubature<4, F>(uc, hu, vc, hv, wc, hw, G.magnetic, G.mc, part);
+        else far_cubature<3, F>(uc, hu, vc, hv, wc, hw, G.magnetic, G.mc, part);
+    }
+    double *Tr = T + (size_t)r * G.Ny * G.Nx;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int sa = (q & 1) ? -1 : 1, sb = (q & 2) ? -1 : 1;
+        if ((sa < 0 && a == 0) || (sb < 0 && b == 0)) continue;
+        const int cy = sa * a - G.off_y, cx = sb * b - G.off_x;
+        if (cy < -(G.ny - 1) || cy > G.sy - 1 || cx < -(G.nx - 1) || cx > G.sx - 1) continue;
+        double v;
+        if (far) {
+            const F p = part[0] + (F)(sa * sb) * part[1] + (F)sb * part[2] + (F)sa * part[3];
+            v = (double)p * lg.vol;
+        } else {
+            v = corner_sum(G, r, sa * a, sb * b) * G.scale;
         }
-        const int e = b_max - (cx + off_x);
-        const int f = a_max - (cy + off_y);
-        if (e < 0 || e + 1 >= nbx1 || f < 0 || f + 1 >= nby1) {
-            // outside the lattice window (it covers every offset nearer than kFar prism
-            // sizes, so this is never taken): the cubature, in FP64
-            const double uc = -(double)(cx + off_x) * dx, vc = -(double)(cy + off_y) * dy;
-            const double w1 = zw[r], w2 = zw[r + 1];
-            const double size = fmax(fmax(dx, dy), w2 - w1);
-            const double dist = sqrt(uc * uc + vc * vc + 0.25 * (w1 + w2) * (w1 + w2));
-            return far<double>(uc, vc, 0.5 * (w1 + w2), 0.5 * (w2 - w1), dist, size) * scale;
-        }
-        double s = 0.0;
-#pragma unroll
-        for (int dk = 0; dk < 2; ++dk)
-#pragma unroll
-            for (int df = 0; df < 2; ++df)
-#pragma unroll
-                for (int de = 0; de < 2; ++de) {
-                    const double t = lat[((size_t)(r + dk) * nby1 + (f + df)) * nbx1 + (e + de)];
-                    s += ((de + df + dk) & 1) ? t : -t;
-                }
-        return s * scale;
+        Tr[(size_t)(cy < 0 ? cy + G.Ny : cy) * G.Nx + (cx < 0 ? cx + G.Nx : cx)] = v;
+    }
+}
+
+// Row-pass input of the setup: the tables, zero outside the offsets in use.
+struct LoadTable {
+    static constexpr int STAGE_U = 4;
+    const double *T;
+    int Nx, Ny, sx, sy, nx, ny;
+    unsigned mNy;
+    __device__ void init() {}
+    __device__ __forceinline__ double value(int line, int j) const {
+        const int iy = line - fast_div(line, mNy) * Ny;
+        const bool in = (iy <= sy - 1 || iy >= Ny - (ny - 1)) && (j <= sx - 1 || j >= Nx - (nx - 1));
+        return in ? T[(size_t)line * Nx + j] : 0.0;
     }
     __device__ __forceinline__ void fetch(int la, int lb, bool hb, int j, double &a, double &b) const {
         a = value(la, j);
@@ -389,11 +427,15 @@ static void free_op_memory(gj_op *op) {
     op->twx = op->twy = op->spec = op->Z = op->Y = op->W = op->V = op->twtab = nullptr;
 }
 
-// Work buffers of the spectrum build for `layers` consecutive layers: the FP64
-// corner lattice (layers + 1 depth planes), the FP64 row-pass output, the depths
-// and FP64 twiddles.  Kept by operators that rebuild their spectra per layer.
+// Work buffers of the spectrum build for `layers` consecutive layers at a time: the FP64
+// corner lattice (every depth plane: about 20 x 20 points each), the FP64 tables and
+// row-pass output, the depths and FP64 twiddles.  Kept by operators that rebuild their
+// spectra per layer.
 struct gj_setup_scratch_impl {
     double *lat = nullptr;
+    double *tab = nullptr;
+    double *axis = nullptr;
+    LayerGeom *layer = nullptr;
     double2 *Zs = nullptr;
     double *zw = nullptr;
     void *twx64 = nullptr, *twy64 = nullptr;
@@ -403,7 +445,7 @@ struct gj_setup_scratch_impl {
 
 static void scratch_free(gj_setup_scratch_impl *sc) {
     if (!sc) return;
-    cudaFree(sc->lat); cudaFree(sc->Zs); cudaFree(sc->zw);
+    cudaFree(sc->lat); cudaFree(sc->tab); cudaFree(sc->axis); cudaFree(sc->layer); cudaFree(sc->Zs); cudaFree(sc->zw);
     if (sc->own_tw) { cudaFree(sc->twx64); cudaFree(sc->twy64); }
     delete sc;
 }
@@ -429,6 +471,32 @@ static LatticeWindow lattice_window(const gj_op *op) {
     return w;
 }
 
+static MagCoef mag_coef(const gj_op *op) {
+    MagCoef mc{};
+    const double d2r = 3.14159265358979323846 / 180.0;
+    const double I = op->mag.incl_deg * d2r, D = op->mag.decl_deg * d2r;
+    const double t[3] = {std::cos(I) * std::sin(D), std::cos(I) * std::cos(D), std::sin(I)};
+    mc.c[0] = t[0] * t[0]; mc.c[1] = t[1] * t[1]; mc.c[2] = t[2] * t[2];
+    mc.c[3] = 2 * t[0] * t[1]; mc.c[4] = 2 * t[0] * t[2]; mc.c[5] = 2 * t[1] * t[2];
+    return mc;
+}
+
+static double table_scale(const gj_op *op) {
+    // the row passes of the build, and those of the general kernels, leave out the half of
+    // the real-line split: it is part of the spectra (a power of two: nothing rounds)
+    const double scale = (op->fast || op->fast1024 ? 0.5 : 0.25) / ((double)op->Nx * (double)op->Ny);
+    if (op->field == GJ_MAGNETIC) return scale * op->mag.F_nT / (4.0 * 3.14159265358979323846);
+    // G = 6.6743e-11 m^3 kg^-1 s^-2; g/cc -> kg/m^3 (1e3); m/s^2 -> mGal (1e5)
+    return scale * 6.6743e-11 * 1.0e3 * 1.0e5;
+}
+
+// range of |c + off| over c in [-(n-1), s-1]
+static void offset_span(int off, int s, int n, int &lo, int &count) {
+    const int first = off - (n - 1), last = off + s - 1;
+    lo = first > 0 ? first : (last < 0 ? -last : 0);
+    count = std::max(std::abs(first), std::abs(last)) - lo + 1;
+}
+
 static gj_status scratch_alloc(const gj_op *op, int layers, gj_setup_scratch_impl **out) {
     gj_setup_scratch_impl *sc = new (std::nothrow) gj_setup_scratch_impl();
     if (!sc) { set_error("setup scratch: host allocation failed"); return GJ_ERR_OOM; }
@@ -447,9 +515,26 @@ static gj_status scratch_alloc(const gj_op *op, int layers, gj_setup_scratch_imp
     const size_t plane = (size_t)lw.nbx1 * lw.nby1;
     std::vector<double> zw(op->nz + 1);
     for (int k = 0; k <= op->nz; ++k) zw[k] = op->z_edges[k] - op->station_z;
-    if ((e = cudaMalloc(&sc->lat, plane * (layers + 1) * sizeof(double))) != cudaSuccess ||
+    std::vector<LayerGeom> geom(op->nz);
+    for (int k = 0; k < op->nz; ++k) {
+        const double size = std::max(std::max(op->dx, op->dy), zw[k + 1] - zw[k]);
+        geom[k] = LayerGeom{0.5 * (zw[k] + zw[k + 1]), 0.5 * (zw[k + 1] - zw[k]), kFar * kFar * size * size,
+                            0.125 * op->dx * op->dy * (zw[k + 1] - zw[k]) * table_scale(op)};
+    }
+    int a0, na, b0, nb;
+    offset_span(op->off_y, op->sy, op->ny, a0, na);
+    offset_span(op->off_x, op->sx, op->nx, b0, nb);
+    std::vector<double> axis(nb + na);
+    for (int i = 0; i < nb; ++i) axis[i] = -(double)(b0 + i) * op->dx;
+    for (int i = 0; i < na; ++i) axis[nb + i] = -(double)(a0 + i) * op->dy;
+    if ((e = cudaMalloc(&sc->lat, plane * (op->nz + 1) * sizeof(double))) != cudaSuccess ||
+        (e = cudaMalloc(&sc->tab, (size_t)layers * op->Ny * op->Nx * sizeof(double))) != cudaSuccess ||
         (e = cudaMalloc(&sc->Zs, (size_t)layers * op->Ny * op->ncol * sizeof(double2))) != cudaSuccess ||
         (e = cudaMalloc(&sc->zw, zw.size() * sizeof(double))) != cudaSuccess ||
+        (e = cudaMalloc(&sc->axis, axis.size() * sizeof(double))) != cudaSuccess ||
+        (e = cudaMalloc(&sc->layer, geom.size() * sizeof(LayerGeom))) != cudaSuccess ||
+        (e = cudaMemcpy(sc->axis, axis.data(), axis.size() * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemcpy(sc->layer, geom.data(), geom.size() * sizeof(LayerGeom), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(sc->zw, zw.data(), zw.size() * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess) {
         scratch_free(sc);
         return cuda_fail(e, "setup scratch");
@@ -458,67 +543,71 @@ static gj_status scratch_alloc(const gj_op *op, int layers, gj_setup_scratch_imp
     return GJ_OK;
 }
 
-// Spectra of layers r0 .. r0 + count - 1 (count <= the scratch's layers) into
-// spec[0 .. count): corner lattice of the count + 1 depth planes, the circulant
-// embedding of each layer's table differenced from it while loading the FP64 row
-// transforms, FP64 column transforms, rounding to the operator's precision.
-// Enqueues only (no synchronisation).
-template <typename Rout>
-static void build_layers(const gj_op *op, const gj_setup_scratch_impl &sc, int r0, int count, cpx<Rout> *spec,
-                         cudaStream_t st) {
-    Lattice L;
+// The corner lattice of every depth plane (enqueues one launch).  A point is a chain of
+// FP64 logarithms and arctangents, so the points are spread one warp a block.
+static void build_lattice(const gj_op *op, const gj_setup_scratch_impl &sc, cudaStream_t st) {
     const LatticeWindow lw = lattice_window(op);
+    Lattice L;
     L.b_max = lw.b_max;
     L.a_max = lw.a_max;
     L.nbx1 = lw.nbx1;
     L.nby1 = lw.nby1;
-    L.nz1 = count + 1;
+    L.nz1 = op->nz + 1;
     L.dx = op->dx;
     L.dy = op->dy;
-    L.zw = sc.zw + r0;
-    MagCoef mc{};
-    // the row passes below, and those of the general kernels, leave out the half of the
-    // real-line split: it is part of the spectra (a power of two: nothing rounds)
-    double scale = (op->fast || op->fast1024 ? 0.5 : 0.25) / ((double)op->Nx * (double)op->Ny);
-    const int magnetic = op->field == GJ_MAGNETIC;
-    if (magnetic) {
-        const double d2r = 3.14159265358979323846 / 180.0;
-        const double I = op->mag.incl_deg * d2r, D = op->mag.decl_deg * d2r;
-        const double t[3] = {std::cos(I) * std::sin(D), std::cos(I) * std::cos(D), std::sin(I)};
-        mc.c[0] = t[0] * t[0]; mc.c[1] = t[1] * t[1]; mc.c[2] = t[2] * t[2];
-        mc.c[3] = 2 * t[0] * t[1]; mc.c[4] = 2 * t[0] * t[2]; mc.c[5] = 2 * t[1] * t[2];
-        scale *= op->mag.F_nT / (4.0 * 3.14159265358979323846);
-    } else {
-        // G = 6.6743e-11 m^3 kg^-1 s^-2; g/cc -> kg/m^3 (1e3); m/s^2 -> mGal (1e5)
-        scale *= 6.6743e-11 * 1.0e3 * 1.0e5;
-    }
-    const size_t lat_pts = (size_t)L.nbx1 * L.nby1 * L.nz1;
-    k_corner_lattice<<<(int)std::min<size_t>(1216, (lat_pts + 255) / 256), 256, 0, st>>>(L, magnetic, mc, sc.lat);
+    L.zw = sc.zw;
+    const size_t pts = (size_t)L.nbx1 * L.nby1 * L.nz1;
+    k_corner_lattice<<<(int)std::min<size_t>(4864, (pts + 31) / 32), 32, 0, st>>>(L, op->field == GJ_MAGNETIC,
+                                                                                 mag_coef(op), sc.lat);
+}
+
+// Tables of layers r0 .. r0 + count - 1 (count <= the scratch's layers), after
+// build_lattice, and their FP64 row transforms into the scratch's Zs.  half_rows: of an even
+// table, the rows 0 .. Ny/2 alone (one layer).  Enqueues only (no synchronisation).
+static OpView<double> build_rows(const gj_op *op, const gj_setup_scratch_impl &sc, int r0, int count, bool half_rows,
+                                 cudaStream_t st) {
+    const LatticeWindow lw = lattice_window(op);
+    TableGeom G;
+    G.lat = sc.lat; G.nbx1 = lw.nbx1; G.nby1 = lw.nby1; G.k0 = r0;
+    G.Nx = op->Nx; G.Ny = op->Ny; G.sx = op->sx; G.sy = op->sy; G.nx = op->nx; G.ny = op->ny;
+    G.off_x = op->off_x; G.off_y = op->off_y; G.a_max = lw.a_max; G.b_max = lw.b_max;
+    offset_span(op->off_y, op->sy, op->ny, G.a0, G.na);
+    offset_span(op->off_x, op->sx, op->nx, G.b0, G.nb);
+    G.scale = table_scale(op);
+    G.axis = sc.axis;
+    G.layer = sc.layer + r0;
+    G.hu = 0.5 * op->dx;
+    G.hv = 0.5 * op->dy;
+    G.magnetic = op->field == GJ_MAGNETIC;
+    G.mc = mag_coef(op);
+    const dim3 tg((G.nb + 127) / 128, G.na, count);
+    if (op->prec == GJ_FP32_MIXED) k_table<float><<<tg, 128, 0, st>>>(G, sc.tab);
+    else k_table<double><<<tg, 128, 0, st>>>(G, sc.tab);
 
     OpView<double> v{};
     v.sx = op->sx; v.sy = op->sy; v.nx = op->nx; v.ny = op->ny; v.nz = count;
     v.Nx = op->Nx; v.Ny = op->Ny; v.ncol = op->ncol; v.px = op->px; v.py = op->py;
     v.twx = static_cast<const double2 *>(sc.twx64);
     v.twy = static_cast<const double2 *>(sc.twy64);
-
-    LoadTable lt;
-    lt.lat = sc.lat; lt.nbx1 = L.nbx1; lt.nby1 = L.nby1;
-    lt.Nx = op->Nx; lt.Ny = op->Ny; lt.sx = op->sx; lt.sy = op->sy; lt.nx = op->nx; lt.ny = op->ny;
-    lt.off_x = op->off_x; lt.off_y = op->off_y; lt.a_max = L.a_max; lt.b_max = L.b_max;
-    lt.scale = scale;
-    lt.dx = op->dx; lt.dy = op->dy;
-    lt.zw = sc.zw + r0;
-    lt.magnetic = magnetic;
-    lt.far32 = op->prec == GJ_FP32_MIXED ? 1 : 0;
-    lt.mc = mc;
-    PairMap pm{count * op->Ny, 0, 0};
+    const LoadTable lt{sc.tab, op->Nx, op->Ny, op->sx, op->sy, op->nx, op->ny, div_magic(op->Ny)};
+    PairMap pm{half_rows ? op->Ny / 2 + 1 : count * op->Ny, 0, 0};
     const int npairs = (pm.nlines + 1) / 2;
     const RowShape rs = row_shape_of(op->px, pick_row_pairs(op->px, npairs, sizeof(double2)), sizeof(double2));
     k_row_fwd<double, LoadTable><<<(npairs + rs.P - 1) / rs.P, gen_threads(op->px.mmax, rs.P),
                                    row_smem(op->Nx, rs.pitch, sizeof(double2)), st>>>(v, pm, op->Nx, rs, sc.Zs, sc.Zs,
                                                                                      lt, nullptr);
+    return v;
+}
+
+// Spectra of layers r0 .. r0 + count - 1 into spec[0 .. count): the row transforms above,
+// column transforms, rounding to the operator's precision.
+template <typename Rout>
+static void build_layers(const gj_op *op, const gj_setup_scratch_impl &sc, int r0, int count, cpx<Rout> *spec,
+                         cudaStream_t st) {
+    const OpView<double> v = build_rows(op, sc, r0, count, false, st);
     ColShape cs{};
-    cs.C = pick_col_tile(op->py, op->ncol, count, 1, sizeof(double2));
+    cs.C = 2;
+    while (cs.C > 1 && (cs.C * op->py.mmax > kGenThreads || col_smem(op->Ny, cs.C, 0, sizeof(double2)) > kGenSmem)) cs.C /= 2;
     cs.G = 1;
     cs.pitch = cs.C;
     cs.mB = cs.mC = div_magic(cs.C);
@@ -533,13 +622,24 @@ static void set_build_attributes() {
     allow_max_smem(k_col_spec<double>);
 }
 
+// where layer r's spectrum starts, in complex values (the even real spectra: two values each)
+static size_t spec_offset(const gj_op *op, int r) {
+    return op->real_spec ? (size_t)r * op->ncol * even_spec_len(op->Ny) / 2 : (size_t)r * op->Ny * op->ncol;
+}
+
 template <typename Rout>
 static gj_status build_spectra(gj_op *op, cudaStream_t st) {
     gj_setup_scratch_impl *sc = nullptr;
-    gj_status rc = scratch_alloc(op, op->nz, &sc);
+    // as many layers at a time as fit a quarter of a gigabyte of tables and row transforms
+    const size_t per = (size_t)op->Ny * op->Nx * sizeof(double) + (size_t)op->Ny * op->ncol * sizeof(double2);
+    const int most = (int)std::max<size_t>(1, std::min<size_t>(op->nz, ((size_t)256 << 20) / per));
+    gj_status rc = scratch_alloc(op, most, &sc);
     if (rc != GJ_OK) return rc;
     set_build_attributes();
-    build_layers<Rout>(op, *sc, 0, op->nz, static_cast<cpx<Rout> *>(op->spec), st);
+    build_lattice(op, *sc, st);
+    for (int r = 0; r < op->nz; r += most)
+        build_layers<Rout>(op, *sc, r, std::min(most, op->nz - r),
+                           static_cast<cpx<Rout> *>(op->spec) + spec_offset(op, r), st);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     scratch_free(sc);
@@ -547,12 +647,13 @@ static gj_status build_spectra(gj_op *op, cudaStream_t st) {
     return GJ_OK;
 }
 
-void recompute_layer(const gj_op *op, int r, cudaStream_t st) {
-    if (op->prec == GJ_FP64)
-        build_layers<double>(op, *op->scratch, r, 1, static_cast<cpx<double> *>(op->spec), st);
-    else
-        build_layers<float>(op, *op->scratch, r, 1, static_cast<cpx<float> *>(op->spec), st);
+void recompute_begin(const gj_op *op, cudaStream_t st) { build_lattice(op, *op->scratch, st); }
+
+void recompute_rows(const gj_op *op, int r, cudaStream_t st) {
+    build_rows(op, *op->scratch, r, 1, op->even_rows, st);
 }
+const double2 *recompute_rows_out(const gj_op *op) { return op->scratch->Zs; }
+const double2 *recompute_twy64(const gj_op *op) { return static_cast<const double2 *>(op->scratch->twy64); }
 
 }  // namespace gj
 
@@ -602,6 +703,10 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
     op->Nx = Nx; op->Ny = Ny; op->ncol = Nx / 2 + 1;
     const size_t cs = 2 * elem_bytes(prec);
     op->recompute = (flags & GJ_SETUP_RECOMPUTE_SPECTRA) != 0;
+    // gravity over a station grid that covers the prisms with no offset: the table is even
+    // in both offsets, so its spectrum is real
+    op->even_table = field == GJ_GRAVITY && G.sx == G.nx && G.sy == G.ny && G.off_x == 0 && G.off_y == 0;
+    op->even_rows = op->recompute && op->even_table && rec_smem(rec_shape(op->py, true, cs), Ny, cs) <= kGenSmemMax;
     op->fast = !op->recompute && fast_eligible(op);
     if (op->fast) {
         int dev = 0, sms = 0;
@@ -611,9 +716,7 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
         const int ci = fast_col_items(Ny, G.nz);
         const long long warps = (long long)op->col_grid * f512::CWARPS;
         op->slots = std::max(fast_slots(1, 257, ci, warps), fast_slots(2, 257, ci, warps));
-        // gravity over a station grid that covers the prisms with no offset: the table
-        // is even in both offsets, so its spectrum is real
-        op->real_spec = field == GJ_GRAVITY && G.sx == G.nx && G.sy == G.ny && G.off_x == 0 && G.off_y == 0;
+        op->real_spec = op->even_table;
     }
     op->fast1024 = !op->recompute && fast1024_eligible(op);
     if (op->fast1024) {
@@ -623,7 +726,7 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
         op->col_grid = std::max(1, sms);
         const long long warps = (long long)op->col_grid * f1024::CWF;
         op->slots = std::max(fast_slots(1, op->ncol, G.nz, warps), fast_slots(2, op->ncol, G.nz, warps));
-        op->real_spec = field == GJ_GRAVITY && G.sx == G.nx && G.sy == G.ny && G.off_x == 0 && G.off_y == 0;
+        op->real_spec = op->even_table;
     }
     // the shapes of both fields' launches (single-field ones pick their own until tuned)
     const int layers = op->recompute ? 1 : G.nz;
@@ -632,8 +735,9 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
         op->P_row = 16;
         while (op->P_row > 1 && row_smem(Nx, odd_pitch(op->P_row), cs) > kGenSmem) op->P_row >>= 1;
     }
-    op->C_col = pick_col_tile(op->py, op->ncol, layers, 2, cs);
-    op->L_grp = pick_layers(op->py, op->C_col, (op->ncol + op->C_col - 1) / op->C_col * 2, layers, cs);
+    const ColPick both = pick_cols(op->py, op->ncol, layers, 2, cs);
+    op->C_col = both.C;
+    op->L_grp = both.L;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     gj_status rc;
     cudaError_t e;
@@ -660,11 +764,11 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
         // partial layer sums (as many groups as a launch of one field or of both makes; a
         // tuned L_grp makes no more) and arrival counters, which are zero between launches
         for (int nf = 1; nf <= 2 && !op->recompute; ++nf) {
-            const int C = pick_col_tile(op->py, op->ncol, layers, nf, cs);
-            const int L = pick_layers(op->py, C, (op->ncol + C - 1) / C * nf, layers, cs);
+            const int L = pick_cols(op->py, op->ncol, layers, nf, cs).L;
             op->gen_slots = std::max(op->gen_slots, (layers + L - 1) / L);
         }
-        const size_t sb = (size_t)op->gen_slots * Ny * op->ncol * cs, yb = sb + op->ncol * sizeof(int);
+        // (the recompute mode sums in the plane of `spec`)
+        const size_t sb = op->recompute ? 0 : (size_t)op->gen_slots * Ny * op->ncol * cs, yb = sb + op->ncol * sizeof(int);
         const size_t wb = (size_t)std::max(G.sy, 1) * op->ncol * cs;
         op->ws_bytes = zb + yb + wb;
         if ((e = cudaMalloc(&op->Z, zb)) != cudaSuccess) { rc = cuda_fail(e, "workspace"); goto fail; }

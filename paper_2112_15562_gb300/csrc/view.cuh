@@ -15,13 +15,12 @@ inline OpView<R> view_of(const gj_op *op) {
     v.twy = static_cast<const cpx<R> *>(op->twy);
     v.spec = static_cast<const cpx<R> *>(op->spec);
     v.Z = static_cast<cpx<R> *>(op->Z);
-    v.Y = static_cast<cpx<R> *>(op->Y);
+    // the recompute mode keeps no spectra: the plane they would take holds the layer sum
+    v.Y = static_cast<cpx<R> *>(op->recompute ? op->spec : op->Y);
     v.W = static_cast<cpx<R> *>(op->W);
     v.V = static_cast<cpx<R> *>(op->V);
     v.cnt = op->cnt;
     v.real_spec = op->real_spec ? 1 : 0;
-    v.rbase = 0;
-    v.spec_r0 = 0;
     v.tcol = op->fast1024 ? op->Ny / 2 : 0;
     v.split_half = op->fast || op->fast1024;  // the general kernels' spectra carry the factor
     return v;
