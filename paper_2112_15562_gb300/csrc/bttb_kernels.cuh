@@ -604,10 +604,10 @@ struct RecShape {
 };
 
 template <typename R>
-__device__ __forceinline__ void layer_spectrum(const OpView<R> &op, const RecShape &rs, int c0, int cols,
+__device__ __forceinline__ void layer_spectrum(int N, int ncol, const RecShape &rs, const FftPlanDev &py, int c0, int cols,
                                                const double2 *Zs, double2 *bufA, double2 *bufB, const double2 *tw64,
                                                cpx<R> *S) {
-    const int N = op.Ny, ncol = op.ncol, C = rs.C;
+    const int C = rs.C;
     const double2 *Z = Zs + c0;
     auto in = [&](int j, int l) {
         if (rs.even) {
@@ -624,7 +624,7 @@ __device__ __forceinline__ void layer_spectrum(const OpView<R> &op, const RecSha
             S[k * C + l] = mk<cpx<R>>((R)x.x, (R)x.y);
         }
     };
-    fft_run<double, false, false, false>(op.py, rs.lines, rs.mlines, rs.lines, bufA, bufB, tw64, N, N, in, out);
+    fft_run<double, false, false, false>(py, rs.lines, rs.mlines, rs.lines, bufA, bufB, tw64, N, N, in, out);
     __syncthreads();
 }
 
@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(256) k_col_rec_fwd(OpView<R> op, RecShape rs, 
     Cx *S = reinterpret_cast<Cx *>(tw64 + N), *tw = S + N * C;
     load_twiddles(tw64, twy64, N);
     load_twiddles(tw, op.twy, N);
-    layer_spectrum<R>(op, rs, c0, cols, Zs, reinterpret_cast<double2 *>(bufA), reinterpret_cast<double2 *>(bufB), tw64,
+    layer_spectrum<R>(N, op.ncol, rs, op.py, c0, cols, Zs, reinterpret_cast<double2 *>(bufA), reinterpret_cast<double2 *>(bufB), tw64,
                       S);
     const FromZ<R> in{op, op.Z + c0, LineMap{rs.mC, C, cols, r, r + 1}};
     const IntoY<R> out{op.Y + c0, S, op.ncol, C, cols, r == 0};
@@ -672,7 +672,7 @@ __global__ void __launch_bounds__(256) k_col_rec_adj(OpView<R> op, RecShape rs, 
     Cx *S = reinterpret_cast<Cx *>(tw64 + N), *tw = S + N * C;
     load_twiddles(tw64, twy64, N);
     load_twiddles(tw, op.twy, N);
-    layer_spectrum<R>(op, rs, c0, cols, Zs, reinterpret_cast<double2 *>(bufA), reinterpret_cast<double2 *>(bufB), tw64,
+    layer_spectrum<R>(N, op.ncol, rs, op.py, c0, cols, Zs, reinterpret_cast<double2 *>(bufA), reinterpret_cast<double2 *>(bufB), tw64,
                       S);
     const Cx *Y = op.Y + c0;
     Cx *Z = op.Z + (size_t)r * ny * ncol + c0;

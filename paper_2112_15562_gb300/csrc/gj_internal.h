@@ -47,7 +47,7 @@ struct gj_op {
     // layer, rebuilt from the closed forms before each use
     bool recompute = false;
     bool even_table = false;  // the table is even in both offsets: its spectrum is real and even
-    bool even_rows = false;   // recompute mode: an even table's transforms share rows and columns
+    bool even_rows = false;   // the build of an even table transforms half the rows, and columns in pairs
     gj::gj_setup_scratch_impl *scratch = nullptr;
     int slots = 0;
     int col_grid = 0;      // CTAs of the persistent column kernels

@@ -73,17 +73,19 @@ __global__ void k_corner_lattice(Lattice L, int magnetic, MagCoef mc, double *ou
 // beyond (relative error at most about 5e-13 there, against 1e-7 for the corner
 // sums at 100 sides).
 constexpr double kFar = 8.0;
-// Gauss-Legendre nodes and weights on [-1, 1]
-__constant__ double kGL5x[5] = {-0.90617984593866399280, -0.53846931010568309104, 0.0, 0.53846931010568309104,
-                                0.90617984593866399280};
-__constant__ double kGL5w[5] = {0.23692688505618908751, 0.47862867049936646804, 0.56888888888888888889,
-                                0.47862867049936646804, 0.23692688505618908751};
-__constant__ double kGL4x[4] = {-0.86113631159405257522, -0.33998104358485626480, 0.33998104358485626480,
-                                0.86113631159405257522};
-__constant__ double kGL4w[4] = {0.34785484513745385737, 0.65214515486254614263, 0.65214515486254614263,
-                                0.34785484513745385737};
-__constant__ double kGL3x[3] = {-0.77459666924148337704, 0.0, 0.77459666924148337704};
-__constant__ double kGL3w[3] = {0.55555555555555555556, 0.88888888888888888889, 0.55555555555555555556};
+// Gauss-Legendre nodes and weights on [-1, 1], as constants of the unrolled rules
+__host__ __device__ constexpr double gl_node(int np, int i) {
+    return np == 5 ? (i == 0 ? -0.90617984593866399280 : i == 1 ? -0.53846931010568309104 : i == 2 ? 0.0
+                      : i == 3 ? 0.53846931010568309104 : 0.90617984593866399280)
+         : np == 4 ? (i == 0 ? -0.86113631159405257522 : i == 1 ? -0.33998104358485626480
+                      : i == 2 ? 0.33998104358485626480 : 0.86113631159405257522)
+                   : (i == 0 ? -0.77459666924148337704 : i == 1 ? 0.0 : 0.77459666924148337704);
+}
+__host__ __device__ constexpr double gl_weight(int np, int i) {
+    return np == 5 ? (i == 0 || i == 4 ? 0.23692688505618908751 : i == 2 ? 0.56888888888888888889 : 0.47862867049936646804)
+         : np == 4 ? (i == 0 || i == 3 ? 0.34785484513745385737 : 0.65214515486254614263)
+                   : (i == 1 ? 0.88888888888888888889 : 0.55555555555555555556);
+}
 
 // The integral over [u1, u2] x [v1, v2] x [w1, w2] of w / R^3 (gravity) or of
 // t^T (d2(1/R)/dr dr) t = (c0 (3u^2 - R^2) + c1 (3v^2 - R^2) + c2 (3w^2 - R^2)
@@ -98,74 +100,75 @@ template <typename F> __device__ __forceinline__ F rsqrt_t(F x);
 template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return rsqrt(x); }
 template <> __device__ __forceinline__ float rsqrt_t<float>(float x) { return rsqrtf(x); }
 
-template <int NP, typename F>
-__device__ __forceinline__ void far_cubature(F uc, F hu, F vc, F hv, F wc, F hw, int magnetic, const MagCoef &k,
-                                             F (&part)[4]) {
-    const double *x = NP == 5 ? kGL5x : (NP == 4 ? kGL4x : kGL3x);
-    const double *wt = NP == 5 ? kGL5w : (NP == 4 ? kGL4w : kGL3w);
-    const F c0 = (F)k.c[0], c1 = (F)k.c[1], c2 = (F)k.c[2], tr = (F)(k.c[0] + k.c[1] + k.c[2]);
+// magnetic coefficients of the cubature, t = (c0, c1, c2) on the diagonal, c3 c4 c5 off it:
+// 3 (t . r)^2 - R^2 = au u^2 + av v^2 + aw w^2 + 3 c3 uv + 3 c4 uw + 3 c5 vw
+template <typename F> struct FarCoef { F au, av, aw, uv, uw, vw; };
+
+template <int NP, typename F, bool MAG>
+__device__ __forceinline__ void far_cubature(F uc, F hu, F vc, F hv, F wc, F hw, const FarCoef<F> &k, F (&part)[4]) {
     F s0 = 0, suv = 0, su = 0, sv = 0;
 #pragma unroll
     for (int a = 0; a < NP; ++a) {
-        const F u = uc + hu * (F)x[a];
+        const F u = uc + hu * (F)gl_node(NP, a), u2 = u * u;
 #pragma unroll
         for (int b = 0; b < NP; ++b) {
-            const F v = vc + hv * (F)x[b];
-            const F uv2 = u * u + v * v, wab = (F)(wt[a] * wt[b]);
-            F i3 = 0, i5 = 0, i5w = 0, i5ww = 0;  // sums over w of 1/R^3, 1/R^5, w/R^5, w^2/R^5 (gravity: w/R^3 in i3)
+            const F v = vc + hv * (F)gl_node(NP, b);
+            const F uv2 = u2 + v * v, e = MAG ? k.au * u2 + k.av * (v * v) : F(0);
+            const F wab = (F)(gl_weight(NP, a) * gl_weight(NP, b));
+            F i0 = 0, i5 = 0, i5w = 0;  // sums over w: the even part, 1/R^5, w/R^5 (gravity: w/R^3)
 #pragma unroll
             for (int c = 0; c < NP; ++c) {
-                const F w = wc + hw * (F)x[c];
-                const F ir = rsqrt_t<F>(uv2 + w * w);
-                const F ir2 = ir * ir, g3 = (F)wt[c] * ir * ir2;
-                if (magnetic) {
-                    const F g5 = g3 * ir2, g5w = g5 * w;
-                    i3 += g3;
+                const F w = wc + hw * (F)gl_node(NP, c), w2 = w * w;
+                const F ir = rsqrt_t<F>(uv2 + w2);
+                const F ir2 = ir * ir, g3 = (F)gl_weight(NP, c) * ir * ir2;
+                if (MAG) {
+                    const F g5 = g3 * ir2;
+                    i0 += g5 * (e + k.aw * w2);
                     i5 += g5;
-                    i5w += g5w;
-                    i5ww += g5w * w;
+                    i5w += g5 * w;
                 } else {
-                    i3 += g3 * w;
+                    i0 += g3 * w;
                 }
             }
-            if (magnetic) {
-                s0 += wab * (F(3) * ((c0 * u * u + c1 * v * v) * i5 + c2 * i5ww) - tr * i3);
+            s0 += wab * i0;
+            if (MAG) {
                 suv += wab * (u * v) * i5;
                 su += wab * u * i5w;
                 sv += wab * v * i5w;
-            } else {
-                s0 += wab * i3;
             }
         }
     }
     part[0] = s0;
-    part[1] = F(3) * (F)k.c[3] * suv;
-    part[2] = F(3) * (F)k.c[4] * su;
-    part[3] = F(3) * (F)k.c[5] * sv;
+    part[1] = MAG ? k.uv * suv : F(0);
+    part[2] = MAG ? k.uw * su : F(0);
+    part[3] = MAG ? k.vw * sv : F(0);
 }
 
 // Depth range of a layer (centre and half height below the stations), its squared
 // near-field radius, and the cubature's volume element times the scale of the spectra.
-struct LayerGeom { double wc, hw, near2, vol; };
+template <typename F> struct LayerGeom {
+    F wc, hw, near2;
+    double vol;
+};
 
 // The circulant tables of a build's layers, T[c_y mod Ny][c_x mod Nx] =
-// K(c_y + off_y, c_x + off_x) for c in [-(n-1), s-1] (the rest is not written: the row
-// pass takes it as zero).  K is the 8-corner sum of the lattice, or the far-field cubature.
-struct TableGeom {
+// K(c_y + off_y, c_x + off_x) for c in [-(n-1), s-1], zero elsewhere.  K is the 8-corner
+// sum of the lattice, or the far-field cubature.
+template <typename F> struct TableGeom {
     const double *lat;
     int nbx1, nby1, k0;  // lattice points, and the lattice plane of the build's first layer
     int Nx, Ny, sx, sy, nx, ny, off_x, off_y, a_max, b_max;
     int a0, na, b0, nb;  // |c + off| runs over [a0, a0 + na) along y and [b0, b0 + nb) along x
     double scale;
-    const double *axis;       // prism centres -|c + off| cell: [nb] along x, then [na] along y
-    const LayerGeom *layer;   // of the build's first layer
-    double hu, hv;            // half cells
-    int magnetic;
-    MagCoef mc;
+    const F *axis;              // prism centres -|c + off| cell: [nb] along x, then [na] along y
+    const LayerGeom<F> *layer;  // of the build's first layer
+    F hu, hv;                   // half cells
+    FarCoef<F> k;
 };
 
 // 8-corner sum at offsets (cy + off_y, cx + off_x) = (a, b), inside the lattice window
-__device__ __forceinline__ double corner_sum(const TableGeom &G, int r, int a, int b) {
+template <typename F>
+__device__ __forceinline__ double corner_sum(const TableGeom<F> &G, int r, int a, int b) {
     const int e = G.b_max - b, f = G.a_max - a;
     double s = 0.0;
 #pragma unroll
@@ -180,96 +183,103 @@ __device__ __forceinline__ double corner_sum(const TableGeom &G, int r, int a, i
     return s;
 }
 
-// One thread per (|a|, |b|) of a layer writes up to four entries.  The FP64 units of this
-// GPU do two operations a cycle and SM, so an entry's address, distance and rule must not
-// use them: evaluated entry by entry with FP64 distances inside the row transforms, a
-// 1023 x 1023 layer took 130 of the row pass's 190 us for an FP32 operator.
-template <typename F>
-__global__ void __launch_bounds__(128) k_table(TableGeom G, double *T) {
-    const int ib = blockIdx.x * blockDim.x + threadIdx.x;
-    const int ia = blockIdx.y, r = blockIdx.z;
-    if (ib >= G.nb) return;
-    const int a = G.a0 + ia, b = G.b0 + ib;
-    const LayerGeom lg = G.layer[r];
-    // offset (a, b) sees the prism centred at u = -b dx, v = -a dy
-    const F uc = (F)G.axis[ib], vc = (F)G.axis[G.nb + ia], wc = (F)lg.wc, hw = (F)lg.hw;
-    const F d2 = uc * uc + vc * vc + wc * wc, near2 = (F)lg.near2;
-    const bool far = d2 >= near2;
-    F part[4] = {0, 0, 0, 0};
-    if (far) {
-        const F hu = (F)G.hu, hv = (F)G.hv;
-        if (d2 < F(9) * near2) far_cubature<5, F>(uc, hu, vc, hv, wc, hw, G.magnetic, G.mc, part);
-        else if (d2 < F(64) * near2) far_cubature<4, F>(uc, hu, vc, hv, wc, hw, G.magnetic, G.mc, part);
-        else far_cubature<3, F>(uc, hu, vc, hv, wc, hw, G.magnetic, G.mc, part);
-    }
-    double *Tr = T + (size_t)r * G.Ny * G.Nx;
+// Two table rows and their FP64 row transform: a CTA takes the rows of offsets a and -a
+// (even: those of |a| = 2q and 2q + 1, all an even table needs), one thread per |b|
+// evaluates the prism once for every row and sign it serves.  The FP64 units of this GPU
+// do two operations a cycle and SM, so what decides an entry's address, distance and rule
+// must not use them (done entry by entry in FP64 inside the transform, a 1023 x 1023 layer
+// of an FP32 operator took 205 us; a table kernel of its own and the transform 75 us),
+// and evaluation in FP32 runs beside the FP64 butterflies of other CTAs.
+template <typename F, bool MAG>
+__global__ void __launch_bounds__(256) k_table_rows(TableGeom<F> G, OpView<double> op, RowShape rs, int even,
+                                                    double2 *Zs) {
+    using C = double2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = op.Nx, ncol = op.ncol, q = blockIdx.x, r = blockIdx.y;
+    int ia[2], iy[2];
+    bool ok[2];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int sa = (q & 1) ? -1 : 1, sb = (q & 2) ? -1 : 1;
-        if ((sa < 0 && a == 0) || (sb < 0 && b == 0)) continue;
-        const int cy = sa * a - G.off_y, cx = sb * b - G.off_x;
-        if (cy < -(G.ny - 1) || cy > G.sy - 1 || cx < -(G.nx - 1) || cx > G.sx - 1) continue;
-        double v;
-        if (far) {
-            const F p = part[0] + (F)(sa * sb) * part[1] + (F)sb * part[2] + (F)sa * part[3];
-            v = (double)p * lg.vol;
-        } else {
-            v = corner_sum(G, r, sa * a, sb * b) * G.scale;
+    for (int l = 0; l < 2; ++l) {
+        ia[l] = even ? 2 * q + l : q;
+        const int a = G.a0 + ia[l], cy = (even || l == 0 ? a : -a) - G.off_y;
+        ok[l] = ia[l] < G.na && cy >= -(G.ny - 1) && cy <= G.sy - 1 && !(!even && l == 1 && a == 0);
+        iy[l] = cy < 0 ? cy + G.Ny : cy;
+    }
+    if (!ok[0] && !ok[1]) return;
+    C *buf0 = reinterpret_cast<C *>(smem_raw), *buf1 = buf0 + N, *tw = buf1 + N;
+    load_twiddles(tw, op.twx, N);
+    for (int i = threadIdx.x; i < N; i += blockDim.x) buf0[i] = czero<C>();
+    __syncthreads();
+    const LayerGeom<F> lg = G.layer[r];
+    for (int ib = threadIdx.x; ib < G.nb; ib += blockDim.x) {
+        const F uc = G.axis[ib];  // offset (a, b) sees the prism centred at u = -b dx, v = -a dy
+        const int b = G.b0 + ib;
+        for (int l = 0; l < (even ? 2 : 1); ++l) {
+            const int il = l == 0 ? ia[0] : ia[1];
+            if (il >= G.na) break;
+            const F vc = G.axis[G.nb + il];
+            const F d2 = uc * uc + vc * vc + lg.wc * lg.wc;
+            const bool far = d2 >= lg.near2;
+            F part[4] = {0, 0, 0, 0};
+            if (far) {
+                if (d2 < F(9) * lg.near2) far_cubature<5, F, MAG>(uc, G.hu, vc, G.hv, lg.wc, lg.hw, G.k, part);
+                else if (d2 < F(64) * lg.near2) far_cubature<4, F, MAG>(uc, G.hu, vc, G.hv, lg.wc, lg.hw, G.k, part);
+                else far_cubature<3, F, MAG>(uc, G.hu, vc, G.hv, lg.wc, lg.hw, G.k, part);
+            }
+#pragma unroll
+            for (int sg = 0; sg < 4; ++sg) {  // signs of a and b
+                const int sa = (sg & 1) ? -1 : 1, sb = (sg & 2) ? -1 : 1;
+                if ((even && sa < 0) || (sb < 0 && b == 0)) continue;
+                const int comp = even ? l : (sg & 1), cx = sb * b - G.off_x;
+                if (!(comp ? ok[1] : ok[0]) || cx < -(G.nx - 1) || cx > G.sx - 1) continue;
+                double v;
+                if (far) v = (double)(part[0] + (F)(sa * sb) * part[1] + (F)sb * part[2] + (F)sa * part[3]) * lg.vol;
+                else v = corner_sum(G, r, sa * (G.a0 + il), sb * b) * G.scale;
+                reinterpret_cast<double *>(buf0 + (cx < 0 ? cx + N : cx))[comp] = v;
+            }
         }
-        Tr[(size_t)(cy < 0 ? cy + G.Ny : cy) * G.Nx + (cx < 0 ? cx + G.Nx : cx)] = v;
+    }
+    __syncthreads();
+    const C *X = fft_staged<double, false>(op.px, rs, buf0, buf1, tw, N, N);
+    C *out0 = Zs + ((size_t)r * G.Ny + iy[0]) * ncol, *out1 = Zs + ((size_t)r * G.Ny + iy[1]) * ncol;
+    for (int k = threadIdx.x; k < ncol; k += blockDim.x) {
+        const C zk = X[k], zm = X[k ? N - k : 0];
+        if (ok[0]) out0[k] = mk<C>(zk.x + zm.x, zk.y - zm.y);
+        if (ok[1]) out1[k] = mk<C>(zk.y + zm.y, zm.x - zk.x);
     }
 }
 
-// Row-pass input of the setup: the tables, zero outside the offsets in use.
-struct LoadTable {
-    static constexpr int STAGE_U = 4;
-    const double *T;
-    int Nx, Ny, sx, sy, nx, ny;
-    unsigned mNy;
-    __device__ void init() {}
-    __device__ __forceinline__ double value(int line, int j) const {
-        const int iy = line - fast_div(line, mNy) * Ny;
-        const bool in = (iy <= sy - 1 || iy >= Ny - (ny - 1)) && (j <= sx - 1 || j >= Nx - (nx - 1));
-        return in ? T[(size_t)line * Nx + j] : 0.0;
-    }
-    __device__ __forceinline__ void fetch(int la, int lb, bool hb, int j, double &a, double &b) const {
-        a = value(la, j);
-        b = hb ? value(lb, j) : 0.0;
-    }
-    __device__ __forceinline__ void flush(double *) const {}
-};
-
-// Column pass of the setup: spec[r] = FFT_y of the row-pass output of layer r.
+// Column pass of the setup: spec[r] = FFT_y of layer r's row transforms, rounded, in the
+// layout of the operator's kernels.
 template <typename Rout>
-__global__ void __launch_bounds__(256) k_col_spec(OpView<double> op, const double2 *Zs, cpx<Rout> *spec, ColShape cs,
+__global__ void __launch_bounds__(256) k_col_spec(OpView<double> op, RecShape rs, const double2 *Zs, cpx<Rout> *spec,
                                                   int transposed, int real_only) {
-    using Cx = double2;
-    const int c0 = blockIdx.x * cs.C;
-    const int r = blockIdx.y;
+    using Cx = cpx<Rout>;
+    const int N = op.Ny, ncol = op.ncol, C = rs.C, c0 = blockIdx.x * C, cols = min(C, ncol - c0), r = blockIdx.y;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int Ny = op.Ny, ncol = op.ncol;
-    const int cols = min(cs.C, ncol - c0);
-    Cx *bufA = reinterpret_cast<Cx *>(smem_raw);
-    Cx *bufB = bufA + Ny * cs.pitch;
-    Cx *tw = bufB + Ny * cs.pitch;
-    load_twiddles(tw, op.twy, Ny);
-    const Cx *Zr = Zs + (size_t)r * Ny * ncol;
-    cpx<Rout> *Sr = spec + (size_t)r * Ny * ncol;
-    const int ke = even_spec_len(Ny);
-    auto in = [&](int j, int c) { return c < cols ? Zr[(size_t)j * ncol + c0 + c] : czero<Cx>(); };
-    auto out = [&](int ky, int c, Cx x) {
-        if (c >= cols) return;
-        if (real_only) {
-            // the table is even in both offsets: the spectrum is real (its imaginary part
-            // is zero in exact arithmetic) and even in ky, so only ky <= Ny/2 is kept,
-            // as R[r][kx][ke] (fast path)
-            if (ky <= Ny / 2) reinterpret_cast<Rout *>(spec)[((size_t)r * ncol + c0 + c) * ke + ky] = (Rout)x.x;
-        } else {
-            const size_t at = transposed ? (size_t)(c0 + c) * Ny + ky : (size_t)ky * ncol + c0 + c;
-            Sr[at] = mk<cpx<Rout>>((Rout)x.x, (Rout)x.y);
+    unsigned char *bufA = smem_raw, *bufB = bufA + rs.buf;
+    double2 *tw64 = reinterpret_cast<double2 *>(bufB + rs.buf);
+    Cx *S = reinterpret_cast<Cx *>(tw64 + N);
+    load_twiddles(tw64, op.twy, N);
+    layer_spectrum<Rout>(N, ncol, rs, op.py, c0, cols, Zs + (size_t)r * N * ncol, reinterpret_cast<double2 *>(bufA),
+                         reinterpret_cast<double2 *>(bufB), tw64, S);
+    Cx *Sr = spec + (size_t)r * N * ncol;
+    if (real_only) {
+        // the table is even in both offsets: the spectrum is real and even in ky, so only
+        // ky <= Ny/2 is kept, as R[r][kx][ke] (fast paths)
+        const int ke = even_spec_len(N), h = N / 2 + 1;
+        Rout *out = reinterpret_cast<Rout *>(spec) + ((size_t)r * ncol + c0) * ke;
+        for (int c = 0; c < cols; ++c)
+            for (int k = threadIdx.x; k < h; k += blockDim.x) out[(size_t)c * ke + k] = S[k * C + c].x;
+    } else if (transposed) {
+        for (int c = 0; c < cols; ++c)
+            for (int k = threadIdx.x; k < N; k += blockDim.x) Sr[(size_t)(c0 + c) * N + k] = S[k * C + c];
+    } else {
+        for (int it = threadIdx.x; it < N * C; it += blockDim.x) {
+            const int k = fast_div(it, rs.mC), c = it - k * C;
+            if (c < cols) Sr[(size_t)k * ncol + c0 + c] = S[it];
         }
-    };
-    fft_run<double, false, false, false>(op.py, cs.C, cs.mB, cs.pitch, bufA, bufB, tw, Ny, Ny, in, out);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -428,14 +438,13 @@ static void free_op_memory(gj_op *op) {
 }
 
 // Work buffers of the spectrum build for `layers` consecutive layers at a time: the FP64
-// corner lattice (every depth plane: about 20 x 20 points each), the FP64 tables and
-// row-pass output, the depths and FP64 twiddles.  Kept by operators that rebuild their
+// corner lattice (every depth plane: about 20 x 20 points each), the FP64 row
+// transforms of the tables (rows outside the offsets in use stay zero), the geometry and
+// FP64 twiddles.  Kept by operators that rebuild their
 // spectra per layer.
 struct gj_setup_scratch_impl {
     double *lat = nullptr;
-    double *tab = nullptr;
-    double *axis = nullptr;
-    LayerGeom *layer = nullptr;
+    void *axis = nullptr, *layer = nullptr;  // TableGeom's, in the far field's precision
     double2 *Zs = nullptr;
     double *zw = nullptr;
     void *twx64 = nullptr, *twy64 = nullptr;
@@ -445,7 +454,7 @@ struct gj_setup_scratch_impl {
 
 static void scratch_free(gj_setup_scratch_impl *sc) {
     if (!sc) return;
-    cudaFree(sc->lat); cudaFree(sc->tab); cudaFree(sc->axis); cudaFree(sc->layer); cudaFree(sc->Zs); cudaFree(sc->zw);
+    cudaFree(sc->lat); cudaFree(sc->axis); cudaFree(sc->layer); cudaFree(sc->Zs); cudaFree(sc->zw);
     if (sc->own_tw) { cudaFree(sc->twx64); cudaFree(sc->twy64); }
     delete sc;
 }
@@ -497,6 +506,28 @@ static void offset_span(int off, int s, int n, int &lo, int &count) {
     count = std::max(std::abs(first), std::abs(last)) - lo + 1;
 }
 
+// TableGeom's axis and layer arrays in precision F (as bytes)
+template <typename F>
+static void table_geometry(const gj_op *op, const std::vector<double> &zw, std::vector<char> &axis,
+                           std::vector<char> &geom) {
+    int a0, na, b0, nb;
+    offset_span(op->off_y, op->sy, op->ny, a0, na);
+    offset_span(op->off_x, op->sx, op->nx, b0, nb);
+    axis.resize((nb + na) * sizeof(F));
+    geom.resize(op->nz * sizeof(LayerGeom<F>));
+    F *ax = reinterpret_cast<F *>(axis.data());
+    for (int i = 0; i < nb; ++i) ax[i] = (F)(-(double)(b0 + i) * op->dx);
+    for (int i = 0; i < na; ++i) ax[nb + i] = (F)(-(double)(a0 + i) * op->dy);
+    LayerGeom<F> *lg = reinterpret_cast<LayerGeom<F> *>(geom.data());
+    for (int k = 0; k < op->nz; ++k) {
+        const double size = std::max(std::max(op->dx, op->dy), zw[k + 1] - zw[k]);
+        lg[k].wc = (F)(0.5 * (zw[k] + zw[k + 1]));
+        lg[k].hw = (F)(0.5 * (zw[k + 1] - zw[k]));
+        lg[k].near2 = (F)(kFar * kFar * size * size);
+        lg[k].vol = 0.125 * op->dx * op->dy * (zw[k + 1] - zw[k]) * table_scale(op);
+    }
+}
+
 static gj_status scratch_alloc(const gj_op *op, int layers, gj_setup_scratch_impl **out) {
     gj_setup_scratch_impl *sc = new (std::nothrow) gj_setup_scratch_impl();
     if (!sc) { set_error("setup scratch: host allocation failed"); return GJ_ERR_OOM; }
@@ -515,26 +546,17 @@ static gj_status scratch_alloc(const gj_op *op, int layers, gj_setup_scratch_imp
     const size_t plane = (size_t)lw.nbx1 * lw.nby1;
     std::vector<double> zw(op->nz + 1);
     for (int k = 0; k <= op->nz; ++k) zw[k] = op->z_edges[k] - op->station_z;
-    std::vector<LayerGeom> geom(op->nz);
-    for (int k = 0; k < op->nz; ++k) {
-        const double size = std::max(std::max(op->dx, op->dy), zw[k + 1] - zw[k]);
-        geom[k] = LayerGeom{0.5 * (zw[k] + zw[k + 1]), 0.5 * (zw[k + 1] - zw[k]), kFar * kFar * size * size,
-                            0.125 * op->dx * op->dy * (zw[k + 1] - zw[k]) * table_scale(op)};
-    }
-    int a0, na, b0, nb;
-    offset_span(op->off_y, op->sy, op->ny, a0, na);
-    offset_span(op->off_x, op->sx, op->nx, b0, nb);
-    std::vector<double> axis(nb + na);
-    for (int i = 0; i < nb; ++i) axis[i] = -(double)(b0 + i) * op->dx;
-    for (int i = 0; i < na; ++i) axis[nb + i] = -(double)(a0 + i) * op->dy;
+    std::vector<char> axis, geom;
+    if (op->prec == GJ_FP32_MIXED) table_geometry<float>(op, zw, axis, geom);
+    else table_geometry<double>(op, zw, axis, geom);
+    const size_t zsb = (size_t)layers * op->Ny * op->ncol * sizeof(double2);
     if ((e = cudaMalloc(&sc->lat, plane * (op->nz + 1) * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&sc->tab, (size_t)layers * op->Ny * op->Nx * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&sc->Zs, (size_t)layers * op->Ny * op->ncol * sizeof(double2))) != cudaSuccess ||
+        (e = cudaMalloc(&sc->Zs, zsb)) != cudaSuccess || (e = cudaMemset(sc->Zs, 0, zsb)) != cudaSuccess ||
         (e = cudaMalloc(&sc->zw, zw.size() * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&sc->axis, axis.size() * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&sc->layer, geom.size() * sizeof(LayerGeom))) != cudaSuccess ||
-        (e = cudaMemcpy(sc->axis, axis.data(), axis.size() * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = cudaMemcpy(sc->layer, geom.data(), geom.size() * sizeof(LayerGeom), cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMalloc(&sc->axis, axis.size())) != cudaSuccess ||
+        (e = cudaMalloc(&sc->layer, geom.size())) != cudaSuccess ||
+        (e = cudaMemcpy(sc->axis, axis.data(), axis.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemcpy(sc->layer, geom.data(), geom.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(sc->zw, zw.data(), zw.size() * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess) {
         scratch_free(sc);
         return cuda_fail(e, "setup scratch");
@@ -562,40 +584,43 @@ static void build_lattice(const gj_op *op, const gj_setup_scratch_impl &sc, cuda
 }
 
 // Tables of layers r0 .. r0 + count - 1 (count <= the scratch's layers), after
-// build_lattice, and their FP64 row transforms into the scratch's Zs.  half_rows: of an even
-// table, the rows 0 .. Ny/2 alone (one layer).  Enqueues only (no synchronisation).
-static OpView<double> build_rows(const gj_op *op, const gj_setup_scratch_impl &sc, int r0, int count, bool half_rows,
-                                 cudaStream_t st) {
+// build_lattice, and their FP64 row transforms into the scratch's Zs (even_rows: the rows
+// 0 .. Ny/2 alone).  Enqueues only (no synchronisation).
+template <typename F>
+static void launch_table_rows(const gj_op *op, const gj_setup_scratch_impl &sc, int r0, int count,
+                              const OpView<double> &v, cudaStream_t st) {
     const LatticeWindow lw = lattice_window(op);
-    TableGeom G;
+    TableGeom<F> G;
     G.lat = sc.lat; G.nbx1 = lw.nbx1; G.nby1 = lw.nby1; G.k0 = r0;
     G.Nx = op->Nx; G.Ny = op->Ny; G.sx = op->sx; G.sy = op->sy; G.nx = op->nx; G.ny = op->ny;
     G.off_x = op->off_x; G.off_y = op->off_y; G.a_max = lw.a_max; G.b_max = lw.b_max;
     offset_span(op->off_y, op->sy, op->ny, G.a0, G.na);
     offset_span(op->off_x, op->sx, op->nx, G.b0, G.nb);
     G.scale = table_scale(op);
-    G.axis = sc.axis;
-    G.layer = sc.layer + r0;
-    G.hu = 0.5 * op->dx;
-    G.hv = 0.5 * op->dy;
-    G.magnetic = op->field == GJ_MAGNETIC;
-    G.mc = mag_coef(op);
-    const dim3 tg((G.nb + 127) / 128, G.na, count);
-    if (op->prec == GJ_FP32_MIXED) k_table<float><<<tg, 128, 0, st>>>(G, sc.tab);
-    else k_table<double><<<tg, 128, 0, st>>>(G, sc.tab);
+    G.axis = static_cast<const F *>(sc.axis);
+    G.layer = static_cast<const LayerGeom<F> *>(sc.layer) + r0;
+    G.hu = (F)(0.5 * op->dx);
+    G.hv = (F)(0.5 * op->dy);
+    const MagCoef mc = mag_coef(op);
+    const double tr = mc.c[0] + mc.c[1] + mc.c[2];
+    G.k = FarCoef<F>{(F)(3 * mc.c[0] - tr), (F)(3 * mc.c[1] - tr), (F)(3 * mc.c[2] - tr),
+                     (F)(3 * mc.c[3]),      (F)(3 * mc.c[4]),      (F)(3 * mc.c[5])};
+    const RowShape rs = row_shape_of(op->px, 1, sizeof(double2));
+    const dim3 grid(op->even_rows ? (G.na + 1) / 2 : G.na, count);
+    const int T = gen_threads(op->px.mmax, 1), even = op->even_rows ? 1 : 0;
+    const size_t sm = row_smem(op->Nx, rs.pitch, sizeof(double2));
+    if (op->field == GJ_MAGNETIC) k_table_rows<F, true><<<grid, T, sm, st>>>(G, v, rs, even, sc.Zs);
+    else k_table_rows<F, false><<<grid, T, sm, st>>>(G, v, rs, even, sc.Zs);
+}
 
+static OpView<double> build_rows(const gj_op *op, const gj_setup_scratch_impl &sc, int r0, int count, cudaStream_t st) {
     OpView<double> v{};
     v.sx = op->sx; v.sy = op->sy; v.nx = op->nx; v.ny = op->ny; v.nz = count;
     v.Nx = op->Nx; v.Ny = op->Ny; v.ncol = op->ncol; v.px = op->px; v.py = op->py;
     v.twx = static_cast<const double2 *>(sc.twx64);
     v.twy = static_cast<const double2 *>(sc.twy64);
-    const LoadTable lt{sc.tab, op->Nx, op->Ny, op->sx, op->sy, op->nx, op->ny, div_magic(op->Ny)};
-    PairMap pm{half_rows ? op->Ny / 2 + 1 : count * op->Ny, 0, 0};
-    const int npairs = (pm.nlines + 1) / 2;
-    const RowShape rs = row_shape_of(op->px, pick_row_pairs(op->px, npairs, sizeof(double2)), sizeof(double2));
-    k_row_fwd<double, LoadTable><<<(npairs + rs.P - 1) / rs.P, gen_threads(op->px.mmax, rs.P),
-                                   row_smem(op->Nx, rs.pitch, sizeof(double2)), st>>>(v, pm, op->Nx, rs, sc.Zs, sc.Zs,
-                                                                                     lt, nullptr);
+    if (op->prec == GJ_FP32_MIXED) launch_table_rows<float>(op, sc, r0, count, v, st);
+    else launch_table_rows<double>(op, sc, r0, count, v, st);
     return v;
 }
 
@@ -604,20 +629,19 @@ static OpView<double> build_rows(const gj_op *op, const gj_setup_scratch_impl &s
 template <typename Rout>
 static void build_layers(const gj_op *op, const gj_setup_scratch_impl &sc, int r0, int count, cpx<Rout> *spec,
                          cudaStream_t st) {
-    const OpView<double> v = build_rows(op, sc, r0, count, false, st);
-    ColShape cs{};
-    cs.C = 2;
-    while (cs.C > 1 && (cs.C * op->py.mmax > kGenThreads || col_smem(op->Ny, cs.C, 0, sizeof(double2)) > kGenSmem)) cs.C /= 2;
-    cs.G = 1;
-    cs.pitch = cs.C;
-    cs.mB = cs.mC = div_magic(cs.C);
-    k_col_spec<Rout><<<dim3((op->ncol + cs.C - 1) / cs.C, count), gen_threads(op->py.mmax, cs.C),
-                       col_smem(op->Ny, cs.pitch, 0, sizeof(double2)), st>>>(
-        v, sc.Zs, spec, cs, (op->fast || op->fast1024) ? 1 : 0, op->real_spec ? 1 : 0);
+    const OpView<double> v = build_rows(op, sc, r0, count, st);
+    const RecShape cs = rec_shape(op->py, op->even_rows, sizeof(cpx<Rout>));
+    k_col_spec<Rout><<<dim3((op->ncol + cs.C - 1) / cs.C, count), gen_threads(op->py.mmax, cs.lines),
+                       rec_smem(cs, op->Ny, sizeof(cpx<Rout>)), st>>>(v, cs, sc.Zs, spec,
+                                                                     (op->fast || op->fast1024) ? 1 : 0,
+                                                                     op->real_spec ? 1 : 0);
 }
 
 static void set_build_attributes() {
-    allow_max_smem(k_row_fwd<double, LoadTable>);
+    allow_max_smem(k_table_rows<float, false>);
+    allow_max_smem(k_table_rows<float, true>);
+    allow_max_smem(k_table_rows<double, false>);
+    allow_max_smem(k_table_rows<double, true>);
     allow_max_smem(k_col_spec<float>);
     allow_max_smem(k_col_spec<double>);
 }
@@ -630,8 +654,8 @@ static size_t spec_offset(const gj_op *op, int r) {
 template <typename Rout>
 static gj_status build_spectra(gj_op *op, cudaStream_t st) {
     gj_setup_scratch_impl *sc = nullptr;
-    // as many layers at a time as fit a quarter of a gigabyte of tables and row transforms
-    const size_t per = (size_t)op->Ny * op->Nx * sizeof(double) + (size_t)op->Ny * op->ncol * sizeof(double2);
+    // as many layers at a time as fit a quarter of a gigabyte of row transforms
+    const size_t per = (size_t)op->Ny * op->ncol * sizeof(double2);
     const int most = (int)std::max<size_t>(1, std::min<size_t>(op->nz, ((size_t)256 << 20) / per));
     gj_status rc = scratch_alloc(op, most, &sc);
     if (rc != GJ_OK) return rc;
@@ -650,7 +674,7 @@ static gj_status build_spectra(gj_op *op, cudaStream_t st) {
 void recompute_begin(const gj_op *op, cudaStream_t st) { build_lattice(op, *op->scratch, st); }
 
 void recompute_rows(const gj_op *op, int r, cudaStream_t st) {
-    build_rows(op, *op->scratch, r, 1, op->even_rows, st);
+    build_rows(op, *op->scratch, r, 1, st);
 }
 const double2 *recompute_rows_out(const gj_op *op) { return op->scratch->Zs; }
 const double2 *recompute_twy64(const gj_op *op) { return static_cast<const double2 *>(op->scratch->twy64); }
@@ -706,7 +730,7 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
     // gravity over a station grid that covers the prisms with no offset: the table is even
     // in both offsets, so its spectrum is real
     op->even_table = field == GJ_GRAVITY && G.sx == G.nx && G.sy == G.ny && G.off_x == 0 && G.off_y == 0;
-    op->even_rows = op->recompute && op->even_table && rec_smem(rec_shape(op->py, true, cs), Ny, cs) <= kGenSmemMax;
+    op->even_rows = op->even_table && rec_smem(rec_shape(op->py, true, cs), Ny, cs) <= kGenSmemMax;
     op->fast = !op->recompute && fast_eligible(op);
     if (op->fast) {
         int dev = 0, sms = 0;
