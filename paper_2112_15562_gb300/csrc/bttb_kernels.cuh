@@ -81,11 +81,8 @@ __device__ __forceinline__ void staged_loop(int total, Load load, Store store) {
         }
     }
 }
-// Batch of a row functor's staging loop: Pro::STAGE_U where the functor states it
-// (a functor whose fetch is long arithmetic keeps 1, so that its code is not
-// replicated), else 4.
-template <class F, class = void> struct StageU { static constexpr int value = 4; };
-template <class F> struct StageU<F, decltype((void)F::STAGE_U)> { static constexpr int value = F::STAGE_U; };
+// Elements of a row functor's loops in flight per thread.
+template <typename R> constexpr int kRowU = sizeof(R) == 8 ? 2 : 4;
 
 // ---------------------------------------------------------------------------
 // Plain functors.
@@ -99,12 +96,18 @@ struct LoadPlain {  // a = x0[la*pitch + j], b = x1[lb*pitch + j]
     const R *x1;
     int pitch;
     static constexpr int NPRE = 1;  // rows la of x0 and lb of x1, staged by the 512 team passes
-    static constexpr int STAGE_U = 8;
     __device__ const R *pre_src(int, int i) const { return i == 0 ? x0 : x1; }
     __device__ void init() {}
+    struct Raw { R a, b; };
+    __device__ __forceinline__ Raw load(int la, int lb, bool hb, int j) const {
+        return Raw{x0[(size_t)la * pitch + j], hb ? x1[(size_t)lb * pitch + j] : R(0)};
+    }
+    __device__ __forceinline__ void apply(const Raw &q, int, int, bool, int, R &a, R &b) const {
+        a = q.a;
+        b = q.b;
+    }
     __device__ __forceinline__ void fetch(int la, int lb, bool hb, int j, R &a, R &b) const {
-        a = x0[(size_t)la * pitch + j];
-        b = hb ? x1[(size_t)lb * pitch + j] : R(0);
+        apply(load(la, lb, hb, j), la, lb, hb, j, a, b);
     }
     // elements j0 + k * stride (k < K) below n; zero beyond
     template <int K, bool PRE = false>
@@ -131,9 +134,14 @@ struct StorePlain {
     __device__ const R *pre_src(int, int) const { return nullptr; }
     __device__ __forceinline__ void prefetch(int, int, bool, int, int) const {}
     __device__ void init() {}
-    __device__ __forceinline__ void store(int la, int lb, bool hb, int j, R a, R b) const {
+    struct Raw {};
+    __device__ __forceinline__ Raw load(int, int, bool, int) const { return Raw{}; }
+    __device__ __forceinline__ void apply(const Raw &, int la, int lb, bool hb, int j, R a, R b) const {
         y0[(size_t)la * pitch + j] = a;
         if (hb) y1[(size_t)lb * pitch + j] = b;
+    }
+    __device__ __forceinline__ void store(int la, int lb, bool hb, int j, R a, R b) const {
+        apply(Raw{}, la, lb, hb, j, a, b);
     }
     template <int K, bool PRE = false>
     __device__ __forceinline__ void store_batch(int la, int lb, bool hb, int j0, int stride, int n, const R (&a)[K],
@@ -312,21 +320,25 @@ __global__ void __launch_bounds__(256) k_row_fwd(OpView<R> op, PairMap pm, int n
     const int q0 = blockIdx.x * P;
     const int np = pm.npairs();
     const unsigned mn = div_magic(n_in);
-    staged_loop<StageU<Pro>::value>(
+    auto &&fn = field_functor(pro, field);
+    using Raw = decltype(fn.load(0, 0, false, 0));
+    staged_loop<kRowU<R>>(
         n_in * P,
         [&](int it) {
+            const int p = fast_div(it, mn), j = it - p * n_in, q = q0 + p;
+            int la, lb; bool hb;
+            pm.lines(min(q, np - 1), la, lb, hb);
+            return fn.load(la, lb, hb, j);
+        },
+        [&](int it, const Raw &raw) {
             const int p = fast_div(it, mn), j = it - p * n_in, q = q0 + p;
             R a = 0, b = 0;
             if (q < np) {
                 int la, lb; bool hb;
                 pm.lines(q, la, lb, hb);
-                field_functor(pro, field).fetch(la, lb, hb, j, a, b);
+                fn.apply(raw, la, lb, hb, j, a, b);
             }
-            return mk<C>(a, b);
-        },
-        [&](int it, C z) {
-            const int p = fast_div(it, mn), j = it - p * n_in;
-            buf0[j * rs.pitch + p] = z;
+            buf0[j * rs.pitch + p] = mk<C>(a, b);
         });
     __syncthreads();
     const C *X = fft_staged<R, false>(op.px, rs, buf0, buf1, tw, n_in, N);
@@ -357,14 +369,24 @@ __global__ void __launch_bounds__(256) k_row_inv(OpView<R> op, PairMap pm, int n
     __syncthreads();
     const C *X = fft_staged<R, true>(op.px, rs, buf0, buf1, tw, N, n_out);
     const unsigned mn = div_magic(n_out);
-    for (int it = threadIdx.x; it < n_out * P; it += blockDim.x) {
-        const int p = fast_div(it, mn), j = it - p * n_out, q = q0 + p;
-        if (q >= np) continue;
-        int la, lb; bool hb;
-        pm.lines(q, la, lb, hb);
-        const C z = X[j * rs.pitch + p];
-        field_functor(epi, field).store(la, lb, hb, j, z.x, z.y);
-    }
+    auto &&fn = field_functor(epi, field);
+    using Raw = decltype(fn.load(0, 0, false, 0));
+    staged_loop<kRowU<R>>(
+        n_out * P,
+        [&](int it) {
+            const int p = fast_div(it, mn), j = it - p * n_out;
+            int la, lb; bool hb;
+            pm.lines(min(q0 + p, np - 1), la, lb, hb);
+            return fn.load(la, lb, hb, j);
+        },
+        [&](int it, const Raw &raw) {
+            const int p = fast_div(it, mn), j = it - p * n_out, q = q0 + p;
+            if (q >= np) return;
+            int la, lb; bool hb;
+            pm.lines(q, la, lb, hb);
+            const C z = X[j * rs.pitch + p];
+            fn.apply(raw, la, lb, hb, j, z.x, z.y);
+        });
     epi.flush(red);
 }
 
@@ -392,12 +414,18 @@ __global__ void __launch_bounds__(256) k_row_resid(OpView<R> op, PairMap pm, int
     __syncthreads();
     C *X = fft_staged<R, true>(op.px, rs, buf0, buf1, tw, N, n_out);
     const unsigned mn = div_magic(n_out);
-    for (int it = threadIdx.x; it < n_out * P; it += blockDim.x) {
-        const int p = fast_div(it, mn), j = it - p * n_out;
-        C z = X[j * rs.pitch + p];
-        if (q0 + p < np) epi.residual(q0 + p, j, z.x, z.y);
-        X[j * rs.pitch + p] = z;
-    }
+    staged_loop<kRowU<R>>(
+        n_out * P,
+        [&](int it) {
+            const int p = fast_div(it, mn), j = it - p * n_out;
+            return epi.load(min(q0 + p, np - 1), 0, true, j);
+        },
+        [&](int it, const typename Epi::Raw &raw) {
+            const int p = fast_div(it, mn), j = it - p * n_out;
+            C z = X[j * rs.pitch + p];
+            if (q0 + p < np) epi.residual(raw, z.x, z.y);
+            X[j * rs.pitch + p] = z;
+        });
     __syncthreads();
     const C *Y = fft_staged<R, false>(op.px, rs, X, X == buf0 ? buf1 : buf0, tw, n_out, N);
     split_lines<R>(op, pm, rs, q0, Y, out0, out1);
@@ -533,13 +561,35 @@ __global__ void __launch_bounds__(256) k_col_fwd(OpView<R> op0, OpView<R> op1, C
         if (!last_in) return;
         __threadfence();
         if (threadIdx.x == 0) op.cnt[blockIdx.x] = 0;
+        // Two elements and four slots of loads in flight a thread.  (Summed inside the inverse
+        // transform's first stage, every input waited for its slots one by one: the sums of
+        // eight groups cost 16 us of a 128x128x32 product's 45 us column pass.)
+        staged_loop<2>(
+            N * C,
+            [&](int it) {
+                const int k = fast_div(it, cs.mC), c = it - k * C;
+                const Cx *y = Yt + (size_t)k * ncol + min(c, cols - 1);  // (an absent column's result is dropped)
+                Cx t = __ldcg(y);
+                for (int s = 1; s < slots; s += 4) {
+                    Cx v[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) v[u] = s + u < slots ? __ldcg(y + (s + u) * plane) : czero<Cx>();
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) t = cadd(t, v[u]);
+                }
+                return t;
+            },
+            [&](int it, Cx t) {
+                const int k = fast_div(it, cs.mC), c = it - k * C;
+                acc[k * pitch + c] = t;
+            });
+        __syncthreads();
     }
+    const int Gs = slots > 1 ? 1 : G;  // the sum of all groups sits in the lines of the first layer
     auto in = [&](int k, int c) {
-        if (slots == 1) return tile_sum(k, c);
-        const Cx *y = Yt + (size_t)k * ncol + min(c, cols - 1);  // (an absent column's result is dropped)
-        Cx t = __ldcg(y);
-        for (int s = 1; s < slots; ++s) t = cadd(t, __ldcg(y + s * plane));
-        return t;
+        Cx y = acc[k * pitch + c];
+        for (int g = 1; g < Gs; ++g) y = cadd(y, acc[k * pitch + g * C + c]);
+        return y;
     };
     auto out = [&](int n, int c, Cx x) {
         if (n < op.sy && c < cols) op.W[(size_t)n * ncol + c0 + c] = x;

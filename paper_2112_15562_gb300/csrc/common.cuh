@@ -60,34 +60,79 @@ __device__ __forceinline__ double block_sum(double v, double *scratch) {
     return r;
 }
 
+// Sums K values over the 32 lanes of a warp together: at the first steps half of the lanes
+// hand over half of the values, so that four sums take six FP64 additions a lane and not
+// twenty (the FP64 units do two a cycle and SM: the solver's row passes spent up to 40 % of
+// their time there).  On return lane l holds the sum of value (l >> 4) of two, or of
+// 2 (l >> 4) + ((l >> 3) & 1) of four.
+__device__ __forceinline__ double warp_sums2(double v0, double v1) {
+    const bool up = threadIdx.x & 16;
+    double t = (up ? v1 : v0) + __shfl_xor_sync(0xffffffffu, up ? v0 : v1, 16);
+    for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+__device__ __forceinline__ double warp_sums4(double v0, double v1, double v2, double v3) {
+    const bool up = threadIdx.x & 16, up8 = threadIdx.x & 8;
+    const double a = (up ? v2 : v0) + __shfl_xor_sync(0xffffffffu, up ? v0 : v2, 16);
+    const double b = (up ? v3 : v1) + __shfl_xor_sync(0xffffffffu, up ? v1 : v3, 16);
+    double t = (up8 ? b : a) + __shfl_xor_sync(0xffffffffu, up8 ? a : b, 8);
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+
 // Adds per-thread partials acc[0..K) into out[0..K) (one double atomic per
-// block per entry).  All K sums share one pass: warp shuffles, one barrier, and
-// the first warp finishes.  `scratch` holds at least K * warps doubles (the fast
-// kernels reserve 128: K <= 4 with up to 32 warps).
+// block per entry).  All K sums share one pass: warp sums, one barrier, and
+// the first warp finishes.  `scratch` holds at least 4 * warps doubles (the kernels
+// reserve 128: up to 32 warps).
 // All threads must call it.
 template <int K, typename A>
 __device__ __forceinline__ void block_accumulate(const A *acc, double *out, double *scratch) {
+    static_assert(K >= 2 && K <= 4, "two to four sums");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nw = (blockDim.x + 31) >> 5;
-    double v[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        v[k] = (double)acc[k];
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-    }
+    double t;
+    if constexpr (K == 2) t = warp_sums2((double)acc[0], (double)acc[1]);
+    else t = warp_sums4((double)acc[0], (double)acc[1], (double)acc[2], K > 3 ? (double)acc[K - 1] : 0.0);
     __syncthreads();  // scratch may still be in use by an earlier call
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < K; ++k) scratch[k * nw + warp] = v[k];
+    if constexpr (K == 2) {
+        if ((lane & 15) == 0) scratch[(lane >> 4) * nw + warp] = t;
+    } else {
+        if ((lane & 7) == 0) scratch[(lane >> 3) * nw + warp] = t;
+    }
     __syncthreads();
     if (warp == 0) {
+        // sixteen lanes per value
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            double t = lane < nw ? scratch[k * nw + lane] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0 && out) atomicAdd(out + k, t);
+        for (int k = 0; k < K; k += 2) {
+            const int mine = k + (lane >> 4);
+            double s = 0.0;
+            if (mine < K)
+                for (int w = lane & 15; w < nw; w += 16) s += scratch[mine * nw + w];
+            for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if ((lane & 15) == 0 && mine < K && out) atomicAdd(out + mine, s);
         }
     }
+}
+
+// ---------------------------------------------------------------------------
+// asynchronous global -> shared copies (cp.async), completed per thread by groups
+
+__device__ __forceinline__ uint32_t s_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async(float2 *dst, const float2 *src) { cp_async8(dst, src); }
+__device__ __forceinline__ void cp_async(double2 *dst, const double2 *src) { cp_async16(dst, src); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int NPEND>
+__device__ __forceinline__ void cp_async_wait() {  // at most NPEND of the newest groups still in flight
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(NPEND) : "memory");
 }
 
 // Allows launches of `f` with any dynamic shared memory up to the device's opt-in

@@ -249,23 +249,12 @@ __device__ __forceinline__ void inv512(cpx<R> (&v)[16], cpx<R> *buf, const TW &t
 // ---------------------------------------------------------------------------
 // TMA bulk copies and mbarriers
 
-__device__ __forceinline__ uint32_t s_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// asynchronous global -> shared copies (cp.async), completed per thread by groups
-__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s_addr(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async8(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s_addr(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s_addr(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int NPEND>
-__device__ __forceinline__ void cp_async_wait() {  // at most NPEND of the newest groups still in flight
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(NPEND) : "memory");
-}
+using gj::cp_async16;
+using gj::cp_async4;
+using gj::cp_async8;
+using gj::cp_async_commit;
+using gj::cp_async_wait;
+using gj::s_addr;
 
 __device__ __forceinline__ void mbar_init(uint64_t *bar) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_addr(bar)) : "memory");

@@ -17,7 +17,7 @@ void gen_row_fwd(const gj_op *o, const OpView<R> &v, const PairMap &pm, int n_in
                         const Pro &pro, const int *done, cudaStream_t st, int nf) {
     const int np = pm.joint ? pm.nlines : (pm.nlines + 1) / 2;
     const RowShape rs = row_shape(o, np * nf, sizeof(cpx<R>));
-    k_row_fwd<R, Pro><<<dim3((np + rs.P - 1) / rs.P, nf), gen_threads(o->px.mmax, rs.P),
+    k_row_fwd<R, Pro><<<dim3((np + rs.P - 1) / rs.P, nf), row_threads(o->px, rs.P, (long long)np * nf),
                         row_smem(o->Nx, rs.pitch, sizeof(cpx<R>)), st>>>(v, pm, n_in, rs, out0, out1, pro, done);
 }
 template <typename R, class Epi>
@@ -25,7 +25,7 @@ void gen_row_inv(const gj_op *o, const OpView<R> &v, const PairMap &pm, int n_ou
                         const cpx<R> *in1, const Epi &epi, const int *done, cudaStream_t st, int nf) {
     const int np = pm.joint ? pm.nlines : (pm.nlines + 1) / 2;
     const RowShape rs = row_shape(o, np * nf, sizeof(cpx<R>));
-    k_row_inv<R, Epi><<<dim3((np + rs.P - 1) / rs.P, nf), gen_threads(o->px.mmax, rs.P),
+    k_row_inv<R, Epi><<<dim3((np + rs.P - 1) / rs.P, nf), row_threads(o->px, rs.P, (long long)np * nf),
                         row_smem(o->Nx, rs.pitch, sizeof(cpx<R>)), st>>>(v, pm, n_out, rs, in0, in1, epi, done);
 }
 template <typename R, class Epi>
@@ -33,7 +33,7 @@ void gen_row_resid(const gj_op *o, const OpView<R> &v, const PairMap &pm, int n_
                           const cpx<R> *in1, cpx<R> *out0, cpx<R> *out1, const Epi &epi, const int *done,
                           cudaStream_t st) {
     const RowShape rs = row_shape(o, pm.nlines, sizeof(cpx<R>));
-    k_row_resid<R, Epi><<<(pm.nlines + rs.P - 1) / rs.P, gen_threads(o->px.mmax, rs.P),
+    k_row_resid<R, Epi><<<(pm.nlines + rs.P - 1) / rs.P, row_threads(o->px, rs.P, pm.nlines),
                           row_smem(o->Nx, rs.pitch, sizeof(cpx<R>)), st>>>(v, pm, n_out, rs, in0, in1, out0, out1, epi,
                                                                           done);
 }

@@ -7,7 +7,7 @@
 namespace gj {
 
 constexpr int kGenThreads = 256;             // most threads of a CTA
-constexpr size_t kGenSmem = 100 * 1024;      // shared memory up to which a shape may grow: two CTAs an SM
+constexpr size_t kGenSmem = 110 * 1024;      // shared memory up to which a shape may grow: two CTAs an SM
 constexpr int kGenCtas = 304;                // CTAs worth having in flight: two an SM
 constexpr int kGenGroups = 10;               // most layer groups of a column tile (partial sums to keep and to add)
 
@@ -28,6 +28,13 @@ inline int pick_row_pairs(const FftPlanDev &pl, long long npairs, size_t cs) {
            row_smem(pl.N, odd_pitch(2 * P), cs) <= kGenSmem)
         P *= 2;
     return P;
+}
+
+// Threads of a row pass: the widest stage's butterflies; when there are few CTAs, enough that
+// the staging and epilogue loops are one or two elements long (each is a memory latency).
+inline int row_threads(const FftPlanDev &pl, int P, long long npairs) {
+    const int t = gen_threads(pl.mmax, P);
+    return (npairs + P - 1) / P > kGenCtas ? t : std::max(t, gen_threads((pl.N + 1) / 2, P));
 }
 
 inline RowShape row_shape_of(const FftPlanDev &pl, int P, size_t cs) {
@@ -52,31 +59,48 @@ inline int pick_layer_lines(const FftPlanDev &pl, int C, int L, size_t cs) {
     return G < 1 ? 1 : G;
 }
 
-// Columns and layers per CTA of a column pass over nz layers of nf fields, by the time the
-// pass should take: every SM works off its CTAs, each ceil(L / G) group transforms and one
-// more (the residual's or the sum's), and a group transform takes its instructions' time
-// (FP64: the two lanes an SM has for it) or, when an SM has little to do, a chain of
-// latencies.  Fewer columns waste sectors of the layer spectra and intermediates (32 bytes
-// are four FP32 or two FP64 columns).  Fixed values (from gj_op_tune) are kept when positive.
+// Columns and layers per CTA of a column pass over nz layers of nf fields.  Fixed values
+// (from gj_op_tune) are kept when positive.
+//
+// FP32 passes wait for latencies: four columns fill a 32-byte sector of the spectra and
+// intermediates, and two CTAs an SM keep enough in flight; more layer groups only add partial
+// sums.  Problems too small for that take one column a CTA.  (Forward / adjoint of both
+// fields, us: 148x146x20 at 300x294 48 / 43 so, 53 / 40 with eight columns, 58 / 49 with one;
+// 300x200x30 at 400x600 118 / 94, 121 / 103 and 168 / 126 (two).)
+//
+// FP64 passes are bound by the two FP64 lanes of an SM: the shape with the least work on the
+// fullest SM, where a CTA costs its group transforms, one more for the residual (adjoint) or
+// a share of the sums (forward), and on average one CTA of imbalance.
 struct ColPick { int C, L; };
-inline ColPick pick_cols(const FftPlanDev &pl, int ncol, int nz, int nf, size_t cs, int fixC = 0, int fixL = 0) {
+inline ColPick pick_cols(const FftPlanDev &pl, int ncol, int nz, int nf, size_t cs, bool adjoint, int fixC = 0,
+                         int fixL = 0) {
     const bool wide = cs == 16;  // complex doubles
-    ColPick best{1, nz};
+    auto fits = [&](int C) { return col_smem(pl.N, odd_pitch(C), odd_pitch(C), cs) <= kGenSmem; };
+    auto tiles_of = [&](int C) { return (ncol + C - 1) / C * nf; };
+    ColPick best{fixC > 0 ? fixC : 1, nz};
+    if (!wide) {
+        if (fixC <= 0) {
+            best.C = 4;
+            while (best.C > 1 && !fits(best.C)) best.C /= 2;
+            const int G = pick_layer_lines(pl, best.C, nz, cs);
+            if (tiles_of(best.C) * ((nz + G - 1) / G) < kGenCtas / 2) best.C = 1;
+        }
+        const int tiles = tiles_of(best.C), G = pick_layer_lines(pl, best.C, nz, cs);
+        int groups = std::max(1, (kGenCtas + tiles / 2) / tiles);
+        groups = std::min(std::min(groups, kGenGroups), (nz + G - 1) / G);
+        best.L = fixL > 0 ? std::min(fixL, nz) : (nz + groups - 1) / groups;
+        return best;
+    }
     double least = 1e300;
-    for (int C = fixC > 0 ? fixC : 1; C <= (fixC > 0 ? fixC : 8); C *= 2) {
-        if (fixC <= 0 && C > 1 && (C * pl.mmax > kGenThreads || C >= 2 * ncol ||
-                                   col_smem(pl.N, odd_pitch(C), odd_pitch(C), cs) > kGenSmem))
-            break;
-        const double waste = wide ? (C == 1 ? 1.2 : 1.0) : (C == 1 ? 1.6 : C == 2 ? 1.25 : C == 4 ? 1.05 : 1.0);
-        const int tiles = (ncol + C - 1) / C * nf;
+    for (int C = fixC > 0 ? fixC : 1; C <= (fixC > 0 ? fixC : 4); C *= 2) {
+        if (fixC <= 0 && C > 1 && (C * pl.mmax > kGenThreads || C >= 2 * ncol || !fits(C))) break;
         for (int groups = 1; groups <= nz && groups <= kGenGroups; ++groups) {
-            const int L = fixL > 0 ? (fixL < nz ? fixL : nz) : (nz + groups - 1) / groups;
-            const int G = pick_layer_lines(pl, C, L, cs);
-            const int ctas = tiles * ((nz + L - 1) / L);
-            const int per_sm = (ctas + 151) / 152;
-            const double work = (double)pl.N * C * G * (wide ? 15.0 : 0.5) / 1900.0, latency = 2.5;  // microseconds
-            const double t = ((L + G - 1) / G + 1) * std::max(per_sm * work * waste + 1.5 / per_sm, latency) +
-                             (ctas > tiles ? 1.0 + 0.2 * (ctas / tiles) : 0.0);
+            const int L = fixL > 0 ? std::min(fixL, nz) : (nz + groups - 1) / groups;
+            const int G = pick_layer_lines(pl, C, L, cs), n = (nz + L - 1) / L;
+            const double work = (double)pl.N * C * G * 15.0 / 1900.0, latency = 2.5;  // microseconds
+            const double t = ((L + G - 1) / G + (adjoint ? 1.0 : 0.3)) *
+                                 std::max((tiles_of(C) * n / 152.0 + 1.0) * work, latency) +
+                             (n > 1 && !adjoint ? 1.5 + 0.2 * n : 0.0);
             if (t < 0.98 * least) { least = t; best = ColPick{C, L}; }
             if (fixL > 0) break;
         }
@@ -87,7 +111,7 @@ inline ColPick pick_cols(const FftPlanDev &pl, int ncol, int nz, int nf, size_t 
 inline ColShape col_shape(const gj_op *o, int nf, int layers, size_t cs, bool adjoint) {
     ColShape s;
     const ColPick pick =
-        pick_cols(o->py, o->ncol, layers, nf, cs, o->cols_tuned ? o->C_col : 0, o->layers_tuned ? o->L_grp : 0);
+        pick_cols(o->py, o->ncol, layers, nf, cs, adjoint, o->cols_tuned ? o->C_col : 0, o->layers_tuned ? o->L_grp : 0);
     s.C = pick.C;
     s.L = pick.L;
     // the forward sums have room for gen_slots groups

@@ -45,33 +45,20 @@ struct FieldVecs {
     R *mtp[2];             // W_{k-1} m_{k-1} (previous-model anchor only), else null
 };
 
-template <typename R> __device__ __forceinline__ R rsqrt_t(R x);
-template <> __device__ __forceinline__ float rsqrt_t<float>(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return rsqrt(x); }
-
-// Diagonal of W = W_depth W_hard W_L at cell c of layer r (Eq. W, Eq. WL).
-template <typename R>
-__device__ __forceinline__ R weight(const FieldVecs<R> &F, int i, int p, R eps2, int r, size_t c, R m) {
-    R w = F.wdep[i][r];
-    if (F.whard[i]) w *= F.whard[i][c];
-    if (p == 1) {
-        const R d = m - (F.mapr[i] ? F.mapr[i][c] : R(0));
-        w *= rsqrt_t<R>(sqrt(d * d + eps2));
-    }
-    return w;
-}
-
 // The L1 reweighting factor of Eq. WL and its reciprocal for p = 1 (1 for p = 2):
 // ((m - m_apr)^2 + eps^2)^(-1/4) and ((m - m_apr)^2 + eps^2)^(1/4).
-template <typename R>
-__device__ __forceinline__ void lp_factors(int p, R d, R eps2, R &wl, R &inv_wl) {
+template <typename R> __device__ __forceinline__ void lp_factors(int p, R d, R eps2, R &wl, R &inv_wl);
+// FP64: two reciprocal square roots, u = q^-2, q = (d^2 + eps^2) u, q^-1/2 (a square root, a
+// reciprocal one and a division by the weight took twice the FP64 instructions)
+template <>
+__device__ __forceinline__ void lp_factors<double>(int p, double d, double eps2, double &wl, double &inv_wl) {
     if (p == 1) {
-        const R q = sqrt(d * d + eps2);
-        wl = rsqrt_t<R>(q);
-        inv_wl = sqrt(q);
+        const double x = d * d + eps2, q = x * rsqrt(x);
+        wl = rsqrt(q);
+        inv_wl = q * wl;
     } else {
-        wl = R(1);
-        inv_wl = R(1);
+        wl = 1.0;
+        inv_wl = 1.0;
     }
 }
 // One hardware reciprocal square root (relative error about 1e-7; arguments below
@@ -94,6 +81,34 @@ __device__ __forceinline__ void lp_factors<float>(int p, float d, float eps2, fl
     }
 }
 
+// The general kernels' form: FP32 keeps the full range of eps^2 (no flush of small arguments).
+template <typename R>
+__device__ __forceinline__ void lp_factors_full(int p, R d, R eps2, R &wl, R &inv_wl) { lp_factors<R>(p, d, eps2, wl, inv_wl); }
+template <>
+__device__ __forceinline__ void lp_factors_full<float>(int p, float d, float eps2, float &wl, float &inv_wl) {
+    if (p == 1) {
+        const float q = sqrtf(d * d + eps2);
+        wl = rsqrtf(q);
+        inv_wl = sqrtf(q);
+    } else {
+        wl = 1.0f;
+        inv_wl = 1.0f;
+    }
+}
+
+// The solver scalars that a pass uses, in precision R, for every thread: one warp reads and
+// converts them (a conversion is FP64 work) and the block shares them.  All threads call;
+// ends with a barrier.
+template <typename R, int N, class Get>
+__device__ __forceinline__ void share_scalars(R (&v)[N], const Get &get) {
+    static_assert(N <= 32, "one warp");
+    __shared__ R sh[N];
+    if (threadIdx.x < N) sh[threadIdx.x] = (R)get((int)threadIdx.x);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = sh[i];
+}
+
 // Forward of m with the pending model update (RRCG:7-8 and the bounds) and the
 // Gramian sums of the updated models.
 template <typename R, bool OPT = true>
@@ -108,33 +123,61 @@ struct ProModel {
     __device__ void init() {
         upd = S->pending_update;
         gsp = S->gspace;
-        eps2 = (R)S->eps2;
+        R v[7];
+        share_scalars<R>(v, [&](int i) {
+            return *(i < 2 ? S->s + i : i < 4 ? S->lo + (i - 2) : i < 6 ? S->hi + (i - 4) : &S->eps2);
+        });
+        eps2 = v[6];
         for (int i = 0; i < 2; ++i) {
-            s[i] = (R)S->s[i]; lo[i] = (R)S->lo[i]; hi[i] = (R)S->hi[i]; pw[i] = S->p[i];
+            s[i] = v[i]; lo[i] = v[2 + i]; hi[i] = v[4 + i]; pw[i] = S->p[i];
         }
         acc[0] = acc[1] = acc[2] = 0;
     }
-    __device__ __forceinline__ void fetch(int la, int lb, bool, int j, R &a, R &b) {
+    // the general kernels' per-element form in two steps, so that the loads of several elements
+    // are in flight before the first store
+    struct Raw { R m[2], p[2], wh[2], ma[2]; };
+    __device__ __forceinline__ Raw load(int la, int, bool, int j) const {
+        const size_t c = (size_t)la * nx + j;
+        Raw q;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            q.m[i] = F.m[i][c];
+            q.p[i] = upd ? F.p[i][c] : R(0);
+            q.wh[i] = (OPT && F.whard[i]) ? F.whard[i][c] : R(1);
+            q.ma[i] = (OPT && F.mapr[i]) ? F.mapr[i][c] : R(0);
+        }
+        return q;
+    }
+    __device__ __forceinline__ void apply(const Raw &q, int la, int, bool, int j, R &a, R &b) {
         const size_t c = (size_t)la * nx + j;
         const int r = la / ny;
         R mv[2], gv[2];
+#pragma unroll
         for (int i = 0; i < 2; ++i) {
-            R mi = F.m[i][c];
+            R mi = q.m[i], wl, iwl;
             if (upd) {
-                const R w = weight(F, i, pw[i], eps2, r, c, mi);
-                if (OPT && F.mtp[i]) F.mtp[i][c] = w * mi;  // W_k m_k, the next anchor
-                mi = mi - s[i] * F.p[i][c] / w;
+                lp_factors_full<R>(pw[i], mi - q.ma[i], eps2, wl, iwl);
+                R inv_w = iwl * F.iwdep[i][r];
+                if (OPT && F.whard[i]) inv_w /= q.wh[i];
+                if (OPT && F.mtp[i]) F.mtp[i][c] = F.wdep[i][r] * q.wh[i] * wl * mi;  // W_k m_k, the next anchor
+                mi = mi - s[i] * q.p[i] * inv_w;
                 mi = fmin(fmax(mi, lo[i]), hi[i]);
                 F.m[i][c] = mi;
             }
-            mv[i] = mi;
-            gv[i] = gsp ? weight(F, i, pw[i], eps2, r, c, mi) * mi : mi;  // Gramian space
+            mv[i] = gv[i] = mi;
+            if (gsp) {  // the Gramian of the weighted models
+                lp_factors_full<R>(pw[i], mi - q.ma[i], eps2, wl, iwl);
+                gv[i] = F.wdep[i][r] * q.wh[i] * wl * mi;
+            }
         }
         acc[0] += gv[0] * gv[0];
         acc[1] += gv[1] * gv[1];
         acc[2] += gv[0] * gv[1];
         a = mv[0];
         b = mv[1];
+    }
+    __device__ __forceinline__ void fetch(int la, int lb, bool hb, int j, R &a, R &b) {
+        apply(load(la, lb, hb, j), la, lb, hb, j, a, b);
     }
     // rows a line needs in every launch (m, p), staged ahead by the persistent row
     // pass as pre[a][field][j]; the optional rows are read in place
@@ -213,26 +256,24 @@ struct EpiResidual {
     int sx;
     R acc[2];
     __device__ void init() { acc[0] = acc[1] = 0; }
-    __device__ __forceinline__ void store(int la, int, bool, int j, R a, R b) {
+    // y of both fields in a, b becomes W_d r~ (two steps, as in ProModel)
+    struct Raw { R w[2], d[2]; };
+    __device__ __forceinline__ Raw load(int la, int, bool, int j) const {
         const size_t t = (size_t)la * sx + j;
-        const R y[2] = {a, b};
-        for (int i = 0; i < 2; ++i) {
-            const R w = F.wd[i][t];
-            const R rt = w * (y[i] - F.dobs[i][t]);
-            acc[i] += rt * rt;
-            F.v[i][t] = w * rt;
-        }
+        return Raw{{F.wd[0][t], F.wd[1][t]}, {F.dobs[0][t], F.dobs[1][t]}};
     }
-    // fused form of the general kernels: y of both fields in a, b becomes W_d r~
-    __device__ __forceinline__ void residual(int la, int j, R &a, R &b) {
+    __device__ __forceinline__ void residual(const Raw &q, R &a, R &b) {
+        const R r0 = q.w[0] * (a - q.d[0]), r1 = q.w[1] * (b - q.d[1]);
+        acc[0] += r0 * r0;
+        acc[1] += r1 * r1;
+        a = q.w[0] * r0;
+        b = q.w[1] * r1;
+    }
+    __device__ __forceinline__ void store(int la, int lb, bool hb, int j, R a, R b) {
+        residual(load(la, lb, hb, j), a, b);
         const size_t t = (size_t)la * sx + j;
-        R *y[2] = {&a, &b};
-        for (int i = 0; i < 2; ++i) {
-            const R w = F.wd[i][t];
-            const R rt = w * (*y[i] - F.dobs[i][t]);
-            acc[i] += rt * rt;
-            *y[i] = w * rt;
-        }
+        F.v[0][t] = a;
+        F.v[1][t] = b;
     }
     // fused form, in two steps so that the loads can be issued before the transform:
     // resid_load fetches W_d and d; resid_apply takes y in a, b and returns v = W_d r~
@@ -331,29 +372,56 @@ struct EpiGradient {
     int pw[2], gsp, prev;
     R acc[2];
     __device__ void init() {
-        for (int i = 0; i < 2; ++i) { alpha[i] = (R)S->alpha[i]; lam[i] = (R)S->lam[i]; pw[i] = S->p[i]; }
-        eps2 = (R)S->eps2;
-        g11 = (R)S->G[0]; g22 = (R)S->G[1]; g12 = (R)S->G[2];
+        R v[8];
+        share_scalars<R>(v, [&](int i) {
+            return *(i < 2 ? S->alpha + i : i < 4 ? S->lam + (i - 2) : i < 7 ? S->G + (i - 4) : &S->eps2);
+        });
+        for (int i = 0; i < 2; ++i) { alpha[i] = v[i]; lam[i] = v[2 + i]; pw[i] = S->p[i]; }
+        eps2 = v[7];
+        g11 = v[4]; g22 = v[5]; g12 = v[6];
         gsp = S->gspace;
         prev = S->anchor == GJ_ANCHOR_PREVIOUS && S->k > 0;  // W_{k-1} m_{k-1} exists from k = 1
         acc[0] = acc[1] = 0;
     }
-    __device__ __forceinline__ void store(int la, int, bool, int j, R a, R b) {
+    struct Raw { R m[2], wh[2], ma[2], an[2]; };
+    __device__ __forceinline__ Raw load(int la, int, bool, int j) const {
+        const size_t c = (size_t)la * nx + j;
+        Raw q;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            q.m[i] = F.m[i][c];
+            q.wh[i] = (OPT && F.whard[i]) ? F.whard[i][c] : R(1);
+            q.ma[i] = (OPT && F.mapr[i]) ? F.mapr[i][c] : R(0);
+            q.an[i] = (OPT && prev) ? F.mtp[i][c] : R(0);
+        }
+        return q;
+    }
+    __device__ __forceinline__ void apply(const Raw &q, int la, int, bool, int j, R a, R b) {
         const size_t c = (size_t)la * nx + j;
         const int r = la / ny;
-        const R mm[2] = {F.m[0][c], F.m[1][c]};
-        const R w[2] = {weight(F, 0, pw[0], eps2, r, c, mm[0]), weight(F, 1, pw[1], eps2, r, c, mm[1])};
+        R w[2], inv_w[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            R wl, iwl;
+            lp_factors_full<R>(pw[i], q.m[i] - q.ma[i], eps2, wl, iwl);
+            w[i] = F.wdep[i][r] * wl;
+            inv_w[i] = iwl * F.iwdep[i][r];
+            if (OPT && F.whard[i]) { w[i] *= q.wh[i]; inv_w[i] /= q.wh[i]; }
+        }
         // ascent directions in the chosen space (RRCG:2-3 or Eq. steepestascenta/b)
-        const R u0 = gsp ? w[0] * mm[0] : mm[0], u1 = gsp ? w[1] * mm[1] : mm[1];
+        const R u0 = gsp ? w[0] * q.m[0] : q.m[0], u1 = gsp ? w[1] * q.m[1] : q.m[1];
         const R lG[2] = {g22 * u0 - g12 * u1, g11 * u1 - g12 * u0};
         const R g[2] = {a, b};
+#pragma unroll
         for (int i = 0; i < 2; ++i) {
-            const R ma = (OPT && F.mapr[i]) ? F.mapr[i][c] : R(0);
-            const R anchor = (OPT && prev) ? F.mtp[i][c] : w[i] * ma;
-            const R li = g[i] / w[i] + alpha[i] * (w[i] * mm[i] - anchor) + lam[i] * lG[i];
+            const R anchor = (OPT && prev) ? q.an[i] : w[i] * q.ma[i];
+            const R li = g[i] * inv_w[i] + alpha[i] * (w[i] * q.m[i] - anchor) + lam[i] * lG[i];
             F.l[i][c] = li;
             acc[i] += li * li;
         }
+    }
+    __device__ __forceinline__ void store(int la, int lb, bool hb, int j, R a, R b) {
+        apply(load(la, lb, hb, j), la, lb, hb, j, a, b);
     }
     static constexpr int NPRE = 1;  // m, staged ahead by the persistent row pass
     __device__ const R *pre_src(int, int i) const { return F.m[i]; }
@@ -417,31 +485,54 @@ struct ProDirection {
     R acc[4];  // (p,l)_0, (p,l)_1, ||p||^2_0, ||p||^2_1
     __device__ void init() {
         first = S->k == 0;
-        eps2 = (R)S->eps2;
         for (int i = 0; i < 2; ++i) pw[i] = S->p[i];
-        if (S->per_field) {
-            for (int i = 0; i < 2; ++i) beta[i] = S->ll_prev[i] > 0 ? (R)(S->ll[i] / S->ll_prev[i]) : R(0);
-        } else {
-            const double den = S->ll_prev[0] + S->ll_prev[1];
-            const R b = den > 0 ? (R)((S->ll[0] + S->ll[1]) / den) : R(0);
-            beta[0] = beta[1] = b;
-        }
+        R v[3];
+        share_scalars<R>(v, [&](int i) {
+            if (i == 2) return S->eps2;
+            const double num = S->per_field ? S->ll[i] : S->ll[0] + S->ll[1];
+            const double den = S->per_field ? S->ll_prev[i] : S->ll_prev[0] + S->ll_prev[1];
+            return den > 0 ? num / den : 0.0;
+        });
+        beta[0] = v[0];
+        beta[1] = v[1];
+        eps2 = v[2];
         acc[0] = acc[1] = acc[2] = acc[3] = 0;
     }
-    __device__ __forceinline__ void fetch(int la, int, bool, int j, R &a, R &b) {
+    struct Raw { R l[2], p[2], m[2], wh[2], ma[2]; };
+    __device__ __forceinline__ Raw load(int la, int, bool, int j) const {
+        const size_t c = (size_t)la * nx + j;
+        Raw q;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            q.l[i] = F.l[i][c];
+            q.p[i] = first ? R(0) : F.p[i][c];
+            q.m[i] = F.m[i][c];
+            q.wh[i] = (OPT && F.whard[i]) ? F.whard[i][c] : R(1);
+            q.ma[i] = (OPT && F.mapr[i]) ? F.mapr[i][c] : R(0);
+        }
+        return q;
+    }
+    __device__ __forceinline__ void apply(const Raw &q, int la, int, bool, int j, R &a, R &b) {
         const size_t c = (size_t)la * nx + j;
         const int r = la / ny;
         R x[2];
+#pragma unroll
         for (int i = 0; i < 2; ++i) {
-            const R li = F.l[i][c];
-            const R pi = first ? li : li + beta[i] * F.p[i][c];
+            const R pi = first ? q.l[i] : q.l[i] + beta[i] * q.p[i];
+            R wl, iwl;
+            lp_factors_full<R>(pw[i], q.m[i] - q.ma[i], eps2, wl, iwl);
+            R inv_w = iwl * F.iwdep[i][r];
+            if (OPT && F.whard[i]) inv_w /= q.wh[i];
             F.p[i][c] = pi;
-            acc[i] += pi * li;
+            acc[i] += pi * q.l[i];
             acc[2 + i] += pi * pi;
-            x[i] = pi / weight(F, i, pw[i], eps2, r, c, F.m[i][c]);
+            x[i] = pi * inv_w;
         }
         a = x[0];
         b = x[1];
+    }
+    __device__ __forceinline__ void fetch(int la, int lb, bool hb, int j, R &a, R &b) {
+        apply(load(la, lb, hb, j), la, lb, hb, j, a, b);
     }
     static constexpr int NPRE = 3;  // l, p, m, staged ahead by the persistent row pass
     __device__ const R *pre_src(int a, int i) const {
@@ -507,11 +598,18 @@ struct EpiQNorm {
     int sx;
     R acc[2];
     __device__ void init() { acc[0] = acc[1] = 0; }
-    __device__ __forceinline__ void store(int la, int, bool, int j, R a, R b) {
+    struct Raw { R w[2]; };
+    __device__ __forceinline__ Raw load(int la, int, bool, int j) const {
         const size_t t = (size_t)la * sx + j;
-        const R q0 = F.wd[0][t] * a, q1 = F.wd[1][t] * b;
+        return Raw{{F.wd[0][t], F.wd[1][t]}};
+    }
+    __device__ __forceinline__ void apply(const Raw &q, int, int, bool, int, R a, R b) {
+        const R q0 = q.w[0] * a, q1 = q.w[1] * b;
         acc[0] += q0 * q0;
         acc[1] += q1 * q1;
+    }
+    __device__ __forceinline__ void store(int la, int lb, bool hb, int j, R a, R b) {
+        apply(load(la, lb, hb, j), la, lb, hb, j, a, b);
     }
     // batched form (the 512 kernels): prefetch loads W_d of line la, elements
     // lane + 32 k, before the transform; store_batch(j0 = lane or lane + 128) uses them

@@ -759,7 +759,7 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
         op->P_row = 16;
         while (op->P_row > 1 && row_smem(Nx, odd_pitch(op->P_row), cs) > kGenSmem) op->P_row >>= 1;
     }
-    const ColPick both = pick_cols(op->py, op->ncol, layers, 2, cs);
+    const ColPick both = pick_cols(op->py, op->ncol, layers, 2, cs, false);
     op->C_col = both.C;
     op->L_grp = both.L;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
@@ -788,7 +788,7 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
         // partial layer sums (as many groups as a launch of one field or of both makes; a
         // tuned L_grp makes no more) and arrival counters, which are zero between launches
         for (int nf = 1; nf <= 2 && !op->recompute; ++nf) {
-            const int L = pick_cols(op->py, op->ncol, layers, nf, cs).L;
+            const int L = pick_cols(op->py, op->ncol, layers, nf, cs, false).L;
             op->gen_slots = std::max(op->gen_slots, (layers + L - 1) / L);
         }
         // (the recompute mode sums in the plane of `spec`)
