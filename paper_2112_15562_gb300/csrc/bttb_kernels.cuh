@@ -307,14 +307,16 @@ template <typename R, class Pro>
 __global__ void __launch_bounds__(256) k_row_fwd(OpView<R> op, PairMap pm, int n_in, RowShape rs,
                                                  cpx<R> *out0, cpx<R> *out1, Pro pro, const int *done) {
     using C = cpx<R>;
-    if (stopped(done)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int N = op.Nx, P = rs.P;
     C *buf0 = reinterpret_cast<C *>(smem_raw);
     C *buf1 = buf0 + N * rs.pitch;
     C *tw = buf1 + N * rs.pitch;
     __shared__ double red[128];
+    pdl_go();
     load_twiddles(tw, op.twx, N);
+    pdl_wait();
+    if (stopped(done)) return;
     pro.init();
     const int field = blockIdx.y;
     const int q0 = blockIdx.x * P;
@@ -353,14 +355,16 @@ __global__ void __launch_bounds__(256) k_row_inv(OpView<R> op, PairMap pm, int n
                                                  const cpx<R> *in0, const cpx<R> *in1, Epi epi,
                                                  const int *done) {
     using C = cpx<R>;
-    if (stopped(done)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int N = op.Nx, P = rs.P;
     C *buf0 = reinterpret_cast<C *>(smem_raw);
     C *buf1 = buf0 + N * rs.pitch;
     C *tw = buf1 + N * rs.pitch;
     __shared__ double red[128];
+    pdl_go();
     load_twiddles(tw, op.twx, N);
+    pdl_wait();
+    if (stopped(done)) return;
     epi.init();
     const int field = blockIdx.y;
     const int q0 = blockIdx.x * P;
@@ -399,14 +403,16 @@ __global__ void __launch_bounds__(256) k_row_resid(OpView<R> op, PairMap pm, int
                                                    const cpx<R> *in0, const cpx<R> *in1, cpx<R> *out0, cpx<R> *out1,
                                                    Epi epi, const int *done) {
     using C = cpx<R>;
-    if (stopped(done)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int N = op.Nx, P = rs.P;
     C *buf0 = reinterpret_cast<C *>(smem_raw);
     C *buf1 = buf0 + N * rs.pitch;
     C *tw = buf1 + N * rs.pitch;
     __shared__ double red[128];
+    pdl_go();
     load_twiddles(tw, op.twx, N);
+    pdl_wait();
+    if (stopped(done)) return;
     epi.init();
     const int q0 = blockIdx.x * P;
     const int np = pm.npairs();
@@ -512,7 +518,7 @@ struct FromVhat {  // conj(spectrum) times the residual's column transform
 template <typename R>
 __global__ void __launch_bounds__(256) k_col_fwd(OpView<R> op0, OpView<R> op1, ColShape cs, const int *done) {
     using Cx = cpx<R>;
-    if (stopped(done)) return;
+    pdl_go();
     const OpView<R> &op = blockIdx.z ? op1 : op0;
     const int C = cs.C, G = cs.G, pitch = cs.pitch;
     const int c0 = blockIdx.x * C;
@@ -528,6 +534,8 @@ __global__ void __launch_bounds__(256) k_col_fwd(OpView<R> op0, OpView<R> op1, C
     Cx *acc = bufB + N * pitch;
     Cx *tw = acc + N * pitch;
     load_twiddles(tw, op.twy, N);
+    pdl_wait();
+    if (stopped(done)) return;
     bool first = true;
     for (int rg = r0; rg < r1; rg += G) {
         const LineMap lm{cs.mC, C, cols, rg, r1};
@@ -603,7 +611,7 @@ __global__ void __launch_bounds__(256) k_col_fwd(OpView<R> op0, OpView<R> op1, C
 template <typename R>
 __global__ void __launch_bounds__(256) k_col_adj(OpView<R> op0, OpView<R> op1, ColShape cs, const int *done) {
     using Cx = cpx<R>;
-    if (stopped(done)) return;
+    pdl_go();
     const OpView<R> &op = blockIdx.z ? op1 : op0;
     const int C = cs.C, G = cs.G, pitch1 = cs.pitch1;
     const int c0 = blockIdx.x * C;
@@ -618,6 +626,8 @@ __global__ void __launch_bounds__(256) k_col_adj(OpView<R> op0, OpView<R> op1, C
     Cx *vh = bufB + N * cs.pitch;
     Cx *tw = vh + N * pitch1;
     load_twiddles(tw, op.twy, N);
+    pdl_wait();
+    if (stopped(done)) return;
     {
         auto in = [&](int j, int c) {
             const Cx w = op.W[(size_t)min(j, op.sy - 1) * ncol + c0 + min(c, cols - 1)];
@@ -702,6 +712,8 @@ __global__ void __launch_bounds__(256) k_col_rec_fwd(OpView<R> op, RecShape rs, 
     Cx *S = reinterpret_cast<Cx *>(tw64 + N), *tw = S + N * C;
     load_twiddles(tw64, twy64, N);
     load_twiddles(tw, op.twy, N);
+    pdl_wait();
+    pdl_go();  // only now: the next layer's table rows may rely on everything before this kernel
     layer_spectrum<R>(N, op.ncol, rs, op.py, c0, cols, Zs, reinterpret_cast<double2 *>(bufA), reinterpret_cast<double2 *>(bufB), tw64,
                       S);
     const FromZ<R> in{op, op.Z + c0, LineMap{rs.mC, C, cols, r, r + 1}};
@@ -722,6 +734,8 @@ __global__ void __launch_bounds__(256) k_col_rec_adj(OpView<R> op, RecShape rs, 
     Cx *S = reinterpret_cast<Cx *>(tw64 + N), *tw = S + N * C;
     load_twiddles(tw64, twy64, N);
     load_twiddles(tw, op.twy, N);
+    pdl_wait();
+    pdl_go();  // only now: the next layer's table rows may rely on everything before this kernel
     layer_spectrum<R>(N, op.ncol, rs, op.py, c0, cols, Zs, reinterpret_cast<double2 *>(bufA), reinterpret_cast<double2 *>(bufB), tw64,
                       S);
     const Cx *Y = op.Y + c0;
@@ -743,6 +757,7 @@ __global__ void __launch_bounds__(256) k_col_plane(OpView<R> op, ColShape cs) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Cx *bufA = reinterpret_cast<Cx *>(smem_raw), *bufB = bufA + N * cs.pitch1, *tw = bufB + N * cs.pitch1;
     load_twiddles(tw, op.twy, N);
+    pdl_wait();
     const Cx *src = (INV ? op.Y : op.W) + c0;
     Cx *dst = (INV ? op.W : op.Y) + c0;
     const int rows_in = INV ? N : sy, rows_out = INV ? sy : N;

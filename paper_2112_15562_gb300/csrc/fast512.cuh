@@ -404,7 +404,6 @@ struct ColItem {
 template <typename R>
 __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_fwd512(View2<R> V, const int *done) {
     using C = cpx<R>;
-    if (stopped(done) || op_failed(V.err)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int ZB = H * sizeof(C), TB = N * sizeof(C);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
@@ -420,6 +419,9 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_fwd512(View2<R> V, const
     if (threadIdx.x == 0) mbar_init(&tabbar);
     mbar_fence_init();
     __syncthreads();
+    pdl_go();
+    pdl_wait();
+    if (stopped(done) || op_failed(V.err)) return;
     TabTw<R> tw;
     tw.bind(tab);
     const int nz = V.op[0].nz, sy = V.op[0].sy;
@@ -549,7 +551,6 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_fwd512(View2<R> V, const
 template <typename R>
 __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_adj512(View2<R> V, const int *done) {
     using C = cpx<R>;
-    if (stopped(done) || op_failed(V.err)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int TB = N * sizeof(C);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
@@ -564,6 +565,9 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_adj512(View2<R> V, const
     if (threadIdx.x == 0) mbar_init(&tabbar);
     mbar_fence_init();
     __syncthreads();
+    pdl_go();
+    pdl_wait();
+    if (stopped(done) || op_failed(V.err)) return;
     TabTw<R> tw;
     tw.bind(tab);
     const int nz = V.op[0].nz, ny = V.op[0].ny;
@@ -701,7 +705,6 @@ __device__ __forceinline__ void inv256h(cpx<R> (&v)[16], cpx<R> *buf, const TW &
 template <typename R>
 __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_fwd256(View2<R> V, const int *done) {
     using C = cpx<R>;
-    if (stopped(done) || op_failed(V.err)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int ZB = H2 * sizeof(C), TB = N2 * sizeof(C);  // one layer's column of Zt / St
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
@@ -717,6 +720,9 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_fwd256(View2<R> V, const
     if (threadIdx.x == 0) mbar_init(&tabbar);
     mbar_fence_init();
     __syncthreads();
+    pdl_go();
+    pdl_wait();
+    if (stopped(done) || op_failed(V.err)) return;
     TabTw<R> tw;
     tw.bind(tab);
     const int nz = V.op[0].nz, sy = V.op[0].sy, nzp = (nz + 1) >> 1;
@@ -852,7 +858,6 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_fwd256(View2<R> V, const
 template <typename R>
 __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_adj256(View2<R> V, const int *done) {
     using C = cpx<R>;
-    if (stopped(done) || op_failed(V.err)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int TB = N2 * sizeof(C);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
@@ -867,6 +872,9 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_adj256(View2<R> V, const
     if (threadIdx.x == 0) mbar_init(&tabbar);
     mbar_fence_init();
     __syncthreads();
+    pdl_go();
+    pdl_wait();
+    if (stopped(done) || op_failed(V.err)) return;
     TabTw<R> tw;
     tw.bind(tab);
     const int nz = V.op[0].nz, ny = V.op[0].ny, nzp = (nz + 1) >> 1;

@@ -69,6 +69,8 @@ __global__ void __launch_bounds__(NW * 32, 2) k_row_fwd512(View2<R> V, int joint
                                                            int out_sel, Pro pro, const int *done) {
     using C = cpx<R>;
     constexpr int FFTS = NW * FPW;
+    pdl_go();
+    pdl_wait();
     if (stopped(done)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *tile = reinterpret_cast<C *>(smem_raw);  // [FFTS][N + 1]
@@ -179,6 +181,8 @@ __global__ void __launch_bounds__(NW * 32, 2) k_row_inv512(View2<R> V, int joint
                                                            int in_sel, Epi epi, const int *done) {
     using C = cpx<R>;
     constexpr int FFTS = NW * FPW;
+    pdl_go();
+    pdl_wait();
     if (stopped(done)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *tile = reinterpret_cast<C *>(smem_raw);  // [NC][2 FFTS + 1]
@@ -407,6 +411,8 @@ __global__ void __launch_bounds__(NW * 32, 1) k_row_fwd512t(View2<R> V, int nz, 
     using C = cpx<R>;
     static_assert(NW % TEAM == 0, "whole teams");
     constexpr int NT = NW / TEAM, LPG = TeamMode<PAIR>::LPG;
+    pdl_go();
+    pdl_wait();
     if (stopped(done)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -567,6 +573,8 @@ __global__ void __launch_bounds__(NW * 32, 2) k_row_resid512(View2<R> V, int nli
                                                              const int *done) {
     using C = cpx<R>;
     constexpr int FFTS = NW;  // one joint transform per warp
+    pdl_go();
+    pdl_wait();
     if (stopped(done)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *tile = reinterpret_cast<C *>(smem_raw);  // [NC][2 NW + 1], later [NW][N + 1]

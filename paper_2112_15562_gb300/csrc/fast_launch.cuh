@@ -64,22 +64,22 @@ template <typename R, int NW, int FPW, class Pro>
 inline void row_fwd(const View2<R> &V, int joint, int nlines, int lpl, int n_in, int out_sel, const Pro &pro,
                     const int *done, cudaStream_t st, int nfield = 1) {
     const int per = (joint ? 1 : 2) * NW * FPW;
-    k_row_fwd512<R, Pro, NW, FPW><<<dim3((nlines + per - 1) / per, nfield), NW * 32, smem_row_fwd<R, NW, FPW>(), st>>>(
-        V, joint, nlines, lpl, n_in, out_sel, pro, done);
+    launch_after(k_row_fwd512<R, Pro, NW, FPW>, dim3((nlines + per - 1) / per, nfield), dim3(NW * 32),
+                 smem_row_fwd<R, NW, FPW>(), st, V, joint, nlines, lpl, n_in, out_sel, pro, done);
 }
 
 template <typename R, int NW, int FPW, class Epi>
 inline void row_inv(const View2<R> &V, int joint, int nlines, int lpl, int n_out, int in_sel, const Epi &epi,
                     const int *done, cudaStream_t st, int nfield = 1) {
     const int per = (joint ? 1 : 2) * NW * FPW;
-    k_row_inv512<R, Epi, NW, FPW><<<dim3((nlines + per - 1) / per, nfield), NW * 32, smem_row_inv<R, NW, FPW>(), st>>>(
-        V, joint, nlines, lpl, n_out, in_sel, epi, done);
+    launch_after(k_row_inv512<R, Epi, NW, FPW>, dim3((nlines + per - 1) / per, nfield), dim3(NW * 32),
+                 smem_row_inv<R, NW, FPW>(), st, V, joint, nlines, lpl, n_out, in_sel, epi, done);
 }
 
 template <typename R, int NW, class Epi>
 inline void row_resid(const View2<R> &V, int nlines, int n_out, const Epi &epi, const int *done, cudaStream_t st) {
-    k_row_resid512<R, Epi, NW><<<(nlines + NW - 1) / NW, NW * 32, smem_row_resid<R, NW>(), st>>>(V, nlines, n_out, epi,
-                                                                                                 done);
+    launch_after(k_row_resid512<R, Epi, NW>, dim3((nlines + NW - 1) / NW), dim3(NW * 32), smem_row_resid<R, NW>(), st, V,
+                 nlines, n_out, epi, done);
 }
 
 // persistent team row passes over nz layers of lpl lines (grid: one CTA per SM);
@@ -87,8 +87,8 @@ inline void row_resid(const View2<R> &V, int nlines, int n_out, const Epi &epi, 
 template <typename R, bool PAIR = false, class Pro>
 inline void row_fwd_t(const View2<R> &V, int grid, int nz, int lpl, int n_in, int out_sel, const Pro &pro,
                       const int *done, cudaStream_t st) {
-    k_row_fwd512t<R, Pro, kRowNW, PAIR><<<grid, kRowNW * 32, smem_row_t<R, kRowNW, Pro::NPRE>(), st>>>(
-        V, nz, lpl, n_in, out_sel, pro, done);
+    launch_after(k_row_fwd512t<R, Pro, kRowNW, PAIR>, dim3(grid), dim3(kRowNW * 32), smem_row_t<R, kRowNW, Pro::NPRE>(),
+                 st, V, nz, lpl, n_in, out_sel, pro, done);
 }
 template <typename R, bool PAIR = false, class Epi>
 inline void row_inv_t(const View2<R> &V, int grid, int nz, int lpl, int n_out, int in_sel, const Epi &epi,
@@ -101,17 +101,17 @@ inline void row_inv_t(const View2<R> &V, int grid, int nz, int lpl, int n_out, i
 template <typename R>
 inline void col_fwd(const View2<R> &V, int grid, const int *done, cudaStream_t st) {
     if (V.op[0].Ny == N2)
-        k_col_fwd256<R><<<grid, CWARPS * 32, smem_col_fwd256<R>(), st>>>(V, done);
+        launch_after(k_col_fwd256<R>, dim3(grid), dim3(CWARPS * 32), smem_col_fwd256<R>(), st, V, done);
     else
-        k_col_fwd512<R><<<grid, CWARPS * 32, smem_col_fwd<R>(), st>>>(V, done);
+        launch_after(k_col_fwd512<R>, dim3(grid), dim3(CWARPS * 32), smem_col_fwd<R>(), st, V, done);
 }
 
 template <typename R>
 inline void col_adj(const View2<R> &V, int grid, const int *done, cudaStream_t st) {
     if (V.op[0].Ny == N2)
-        k_col_adj256<R><<<grid, CWARPS * 32, smem_col_adj256<R>(), st>>>(V, done);
+        launch_after(k_col_adj256<R>, dim3(grid), dim3(CWARPS * 32), smem_col_adj256<R>(), st, V, done);
     else
-        k_col_adj512<R><<<grid, CWARPS * 32, smem_col_adj<R>(), st>>>(V, done);
+        launch_after(k_col_adj512<R>, dim3(grid), dim3(CWARPS * 32), smem_col_adj<R>(), st, V, done);
 }
 
 }  // namespace f512

@@ -117,8 +117,16 @@ __device__ void scalars_after_direction(SolverDev *S) {
 }
 
 // one warp each (launched as <<<1, 32>>>)
-__global__ void k_scalars_after_residual(SolverDev *S) { scalar_step_on_copy<scalars_after_residual>(S); }
-__global__ void k_scalars_after_direction(SolverDev *S) { scalar_step_on_copy<scalars_after_direction>(S); }
+__global__ void k_scalars_after_residual(SolverDev *S) {
+    pdl_go();
+    pdl_wait();
+    scalar_step_on_copy<scalars_after_residual>(S);
+}
+__global__ void k_scalars_after_direction(SolverDev *S) {
+    pdl_go();
+    pdl_wait();
+    scalar_step_on_copy<scalars_after_direction>(S);
+}
 
 // The report of the solver state into device memory (one thread): the same fields
 // as gj_rrcg_report_get, without a host round trip.
@@ -357,7 +365,7 @@ struct SolverLaunch {
             // residual, Phi and the residual rows' spectra for the adjoint, in one pass
             EpiResidual<R> er{F, sv->S, o->sx};
             row_resid<R, kDataNW>(V2, o->sy, o->sx, er, done, st);
-            k_scalars_after_residual<<<1, 32, 0, st>>>(sv->S);
+            launch_after(k_scalars_after_residual, dim3(1), dim3(32), 0, st, sv->S);
             return;
         }
         PairMap pc{o->nz * o->ny, 1, o->ny};
@@ -371,7 +379,7 @@ struct SolverLaunch {
             if (rows1024) f1024::row_inv<R>(v0, ps, o->sx, v0.W, v1.W, o->twtab, er, done, st);
         if (!rows1024)
             gen_row_resid<R>(o, v0, ps, o->sx, v0.W, v1.W, fast1024 ? v0.V : v0.W, fast1024 ? v1.V : v1.W, er, done, st);
-        k_scalars_after_residual<<<1, 32, 0, st>>>(sv->S);
+        launch_after(k_scalars_after_residual, dim3(1), dim3(32), 0, st, sv->S);
     }
 
     void body(cudaStream_t st) {
@@ -394,7 +402,7 @@ struct SolverLaunch {
             forward_columns(st);
             EpiQNorm<R> eq{F, sv->S, o->sx};
             row_inv<R, kDataNW, kDataFPW>(V2, 1, o->sy, o->sy, o->sx, 1, eq, done, st);
-            k_scalars_after_direction<<<1, 32, 0, st>>>(sv->S);
+            launch_after(k_scalars_after_direction, dim3(1), dim3(32), 0, st, sv->S);
             head(st);
             return;
         }
@@ -415,7 +423,7 @@ struct SolverLaunch {
         forward_columns(st);
         EpiQNorm<R> eq{F, sv->S, o->sx};
         rows_inv(ps, o->sx, v0.W, v1.W, eq, done, st);
-        k_scalars_after_direction<<<1, 32, 0, st>>>(sv->S);
+        launch_after(k_scalars_after_direction, dim3(1), dim3(32), 0, st, sv->S);
         // model update, its forward product and the chi^2 scalars
         head(st);
     }

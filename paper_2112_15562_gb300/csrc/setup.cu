@@ -54,6 +54,7 @@ struct Lattice {
 };
 
 __global__ void k_corner_lattice(Lattice L, int magnetic, MagCoef mc, double *out) {
+    pdl_wait();  // (the launch before may still read the lattice)
     const size_t total = (size_t)L.nbx1 * L.nby1 * L.nz1;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const int e = (int)(i % L.nbx1);
@@ -192,7 +193,7 @@ __device__ __forceinline__ double corner_sum(const TableGeom<F> &G, int r, int a
 // and evaluation in FP32 runs beside the FP64 butterflies of other CTAs.
 template <typename F, bool MAG>
 __global__ void __launch_bounds__(256) k_table_rows(TableGeom<F> G, OpView<double> op, RowShape rs, int even,
-                                                    double2 *Zs) {
+                                                    int after_lattice, double2 *Zs) {
     using C = double2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int N = op.Nx, ncol = op.ncol, q = blockIdx.x, r = blockIdx.y;
@@ -206,6 +207,9 @@ __global__ void __launch_bounds__(256) k_table_rows(TableGeom<F> G, OpView<doubl
         iy[l] = cy < 0 ? cy + G.Ny : cy;
     }
     if (!ok[0] && !ok[1]) return;
+    // Launches after the first of a build follow a column launch that started its own work
+    // when everything before it was complete: the lattice is there, and only Zs is waited for.
+    if (after_lattice) pdl_wait();
     C *buf0 = reinterpret_cast<C *>(smem_raw), *buf1 = buf0 + N, *tw = buf1 + N;
     load_twiddles(tw, op.twx, N);
     for (int i = threadIdx.x; i < N; i += blockDim.x) buf0[i] = czero<C>();
@@ -241,6 +245,8 @@ __global__ void __launch_bounds__(256) k_table_rows(TableGeom<F> G, OpView<doubl
     }
     __syncthreads();
     const C *X = fft_staged<double, false>(op.px, rs, buf0, buf1, tw, N, N);
+    if (!after_lattice) pdl_wait();  // the column launch before this one may still read Zs
+    pdl_go();
     C *out0 = Zs + ((size_t)r * G.Ny + iy[0]) * ncol, *out1 = Zs + ((size_t)r * G.Ny + iy[1]) * ncol;
     for (int k = threadIdx.x; k < ncol; k += blockDim.x) {
         const C zk = X[k], zm = X[k ? N - k : 0];
@@ -261,6 +267,8 @@ __global__ void __launch_bounds__(256) k_col_spec(OpView<double> op, RecShape rs
     double2 *tw64 = reinterpret_cast<double2 *>(bufB + rs.buf);
     Cx *S = reinterpret_cast<Cx *>(tw64 + N);
     load_twiddles(tw64, op.twy, N);
+    pdl_wait();
+    pdl_go();
     layer_spectrum<Rout>(N, ncol, rs, op.py, c0, cols, Zs + (size_t)r * N * ncol, reinterpret_cast<double2 *>(bufA),
                          reinterpret_cast<double2 *>(bufB), tw64, S);
     Cx *Sr = spec + (size_t)r * N * ncol;
@@ -579,8 +587,8 @@ static void build_lattice(const gj_op *op, const gj_setup_scratch_impl &sc, cuda
     L.dy = op->dy;
     L.zw = sc.zw;
     const size_t pts = (size_t)L.nbx1 * L.nby1 * L.nz1;
-    k_corner_lattice<<<(int)std::min<size_t>(4864, (pts + 31) / 32), 32, 0, st>>>(L, op->field == GJ_MAGNETIC,
-                                                                                 mag_coef(op), sc.lat);
+    launch_after(k_corner_lattice, dim3((unsigned)std::min<size_t>(4864, (pts + 31) / 32)), dim3(32), 0, st, L,
+                 op->field == GJ_MAGNETIC, mag_coef(op), sc.lat);
 }
 
 // Tables of layers r0 .. r0 + count - 1 (count <= the scratch's layers), after
@@ -589,6 +597,7 @@ static void build_lattice(const gj_op *op, const gj_setup_scratch_impl &sc, cuda
 template <typename F>
 static void launch_table_rows(const gj_op *op, const gj_setup_scratch_impl &sc, int r0, int count,
                               const OpView<double> &v, cudaStream_t st) {
+    const bool after_lattice = r0 == 0;  // the builds go through the layers in order
     const LatticeWindow lw = lattice_window(op);
     TableGeom<F> G;
     G.lat = sc.lat; G.nbx1 = lw.nbx1; G.nby1 = lw.nby1; G.k0 = r0;
@@ -609,8 +618,8 @@ static void launch_table_rows(const gj_op *op, const gj_setup_scratch_impl &sc, 
     const dim3 grid(op->even_rows ? (G.na + 1) / 2 : G.na, count);
     const int T = gen_threads(op->px.mmax, 1), even = op->even_rows ? 1 : 0;
     const size_t sm = row_smem(op->Nx, rs.pitch, sizeof(double2));
-    if (op->field == GJ_MAGNETIC) k_table_rows<F, true><<<grid, T, sm, st>>>(G, v, rs, even, sc.Zs);
-    else k_table_rows<F, false><<<grid, T, sm, st>>>(G, v, rs, even, sc.Zs);
+    launch_after(op->field == GJ_MAGNETIC ? k_table_rows<F, true> : k_table_rows<F, false>, grid, dim3(T), sm, st, G, v,
+                 rs, even, after_lattice ? 1 : 0, sc.Zs);
 }
 
 static OpView<double> build_rows(const gj_op *op, const gj_setup_scratch_impl &sc, int r0, int count, cudaStream_t st) {
@@ -631,10 +640,9 @@ static void build_layers(const gj_op *op, const gj_setup_scratch_impl &sc, int r
                          cudaStream_t st) {
     const OpView<double> v = build_rows(op, sc, r0, count, st);
     const RecShape cs = rec_shape(op->py, op->even_rows, sizeof(cpx<Rout>));
-    k_col_spec<Rout><<<dim3((op->ncol + cs.C - 1) / cs.C, count), gen_threads(op->py.mmax, cs.lines),
-                       rec_smem(cs, op->Ny, sizeof(cpx<Rout>)), st>>>(v, cs, sc.Zs, spec,
-                                                                     (op->fast || op->fast1024) ? 1 : 0,
-                                                                     op->real_spec ? 1 : 0);
+    launch_after(k_col_spec<Rout>, dim3((op->ncol + cs.C - 1) / cs.C, count), dim3(gen_threads(op->py.mmax, cs.lines)),
+                 rec_smem(cs, op->Ny, sizeof(cpx<Rout>)), st, v, cs, sc.Zs, spec, (op->fast || op->fast1024) ? 1 : 0,
+                 op->real_spec ? 1 : 0);
 }
 
 static void set_build_attributes() {
