@@ -254,7 +254,7 @@ gj_status gj_gramian_value_grad(int64_t n, gj_precision precision,
  * is an interface for such callers.)
  *
  * The call allocates nothing: no cudaMalloc, cudaMallocAsync or cudaFree.  Its
- * reduction scratch is a fixed 131,096-byte device array inside the library,
+ * reduction scratch is a fixed 9,736-byte device array inside the library,
  * which every GPU that loads the library holds until the process exits.  The
  * first call on each device looks up that array's device address
  * (cudaGetSymbolAddress, with the device current); make that first call before

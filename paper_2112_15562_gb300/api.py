@@ -15,13 +15,12 @@ _FIELD = {"gravity": L.GJ_GRAVITY, "magnetic": L.GJ_MAGNETIC, L.GJ_GRAVITY: L.GJ
           L.GJ_MAGNETIC: L.GJ_MAGNETIC}
 
 
-def _stream(stream=None) -> ct.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ct.c_void_p(s.cuda_stream)
+def _stream(stream=None) -> int:
+    return (torch.cuda.current_stream() if stream is None else stream).cuda_stream
 
 
-def _ptr(t: Optional[torch.Tensor]) -> Optional[ct.c_void_p]:
-    return None if t is None else ct.c_void_p(t.data_ptr())
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
+    return None if t is None else t.data_ptr()
 
 
 def _vec(t: torch.Tensor, dtype, n: int, name: str) -> torch.Tensor:

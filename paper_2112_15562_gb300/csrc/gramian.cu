@@ -1,4 +1,6 @@
 // The Gramian coupling term (Eq. Gramian) and its ascent directions (RRCG:2-3).
+#include <algorithm>
+#include <map>
 #include <mutex>
 #include <string>
 
@@ -6,78 +8,240 @@
 
 namespace gj {
 
-// Pass 1: per-block partial sums of (m1,m1), (m2,m2), (m1,m2).  Products and the
-// per-thread sums use the vector precision; block and grid sums use FP64.
-template <typename R>
-__global__ void __launch_bounds__(256) k_gram_dots(int64_t n, const R *m1, const R *m2, double *part) {
+// Both passes stream the vectors: 2 n R in, then 2 n R in (from L2 where they fit) and 2 n R
+// out.  A thread keeps eight 16-byte loads in flight, the products of sixteen elements at most
+// go into an FP32 partial sum before FP64 takes it, and the sums over blocks happen inside
+// the two launches (every block of the second sums the first's partials, the last block to
+// finish sums the second's), where two one-block launches of 4 to 6 us each stood before.
+// 2.6 M values FP32, us: partial sums 13.7 + 6.4 and directions 16.4 + 4.5 before.
+constexpr int kGramBlocks = 304;    // two blocks an SM
+constexpr int kGramThreads = 256;
+constexpr int kGramChunk = 16;      // elements of a thread between FP64 additions
+// scratch: 3 partial sums a block, 1 residual sum a block, the ticket
+constexpr int kGramDoubles = 4 * kGramBlocks + 1;
+
+template <typename R> struct Vec16;
+template <> struct Vec16<float> { using T = float4; static constexpr int N = 4; };
+template <> struct Vec16<double> { using T = double2; static constexpr int N = 2; };
+
+// Calls f(k, x, y) for the elements of this thread's chunks, k < kGramChunk a compile-time
+// position in the chunk, and chunk_done() after each chunk.  VEC: 16-byte loads (aligned
+// vectors), else one element a load.  get(i, x, y) when they are one element, else in vectors.
+template <typename R, bool VEC, class Each, class Done>
+__device__ __forceinline__ void gram_chunks(int64_t n, const R *__restrict__ m1, const R *__restrict__ m2, Each each,
+                                            Done done) {
+    const int64_t thread = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, threads = (int64_t)gridDim.x * blockDim.x;
+    if constexpr (VEC) {
+        using V = typename Vec16<R>::T;
+        constexpr int N = Vec16<R>::N, U = 4;  // vectors of each input in flight (N U <= kGramChunk elements)
+        const int64_t nv = n / N;
+        const V *a = reinterpret_cast<const V *>(m1), *b = reinterpret_cast<const V *>(m2);
+        for (int64_t v0 = thread; v0 < nv; v0 += U * threads) {
+            V x[U], y[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t v = v0 + u * threads;
+                if (v < nv) { x[u] = a[v]; y[u] = b[v]; }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t v = v0 + u * threads;
+                if (v < nv) each(v * N, reinterpret_cast<const R(&)[N]>(x[u]), reinterpret_cast<const R(&)[N]>(y[u]));
+            }
+            done();
+        }
+        for (int64_t i = nv * N + thread; i < n; i += threads) {  // the last n % N elements
+            const R x[1] = {m1[i]}, y[1] = {m2[i]};
+            each(i, x, y);
+            done();
+        }
+    } else {
+        for (int64_t i0 = thread; i0 < n; i0 += kGramChunk * threads) {
+            R x[kGramChunk], y[kGramChunk];
+#pragma unroll
+            for (int u = 0; u < kGramChunk; ++u) {
+                const int64_t i = i0 + u * threads;
+                if (i < n) { x[u] = m1[i]; y[u] = m2[i]; }
+            }
+#pragma unroll
+            for (int u = 0; u < kGramChunk; ++u) {
+                const int64_t i = i0 + u * threads;
+                const R xu[1] = {x[u]}, yu[1] = {y[u]};
+                if (i < n) each(i, xu, yu);
+            }
+            done();
+        }
+    }
+}
+
+// (m1,m1), (m2,m2), (m1,m2): part[c nb + block].  Also zeroes the second pass's ticket.
+template <typename R, bool VEC>
+__global__ void __launch_bounds__(kGramThreads) k_gram_dots(int64_t n, const R *m1, const R *m2, double *part,
+                                                            unsigned *ticket) {
     __shared__ double red[32];
+    pdl_go();
+    pdl_wait();
+    double s11 = 0, s22 = 0, s12 = 0;
     R a11 = 0, a22 = 0, a12 = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const R x = m1[i], y = m2[i];
-        a11 += x * x; a22 += y * y; a12 += x * y;
-    }
-    const double s11 = block_sum((double)a11, red);
-    const double s22 = block_sum((double)a22, red);
-    const double s12 = block_sum((double)a12, red);
+    gram_chunks<R, VEC>(
+        n, m1, m2,
+        [&](int64_t, const auto &x, const auto &y) {
+            constexpr int N = (int)(sizeof(x) / sizeof(R));
+#pragma unroll
+            for (int k = 0; k < N; ++k) { a11 += x[k] * x[k]; a22 += y[k] * y[k]; a12 += x[k] * y[k]; }
+        },
+        [&]() {
+            s11 += (double)a11; s22 += (double)a22; s12 += (double)a12;
+            a11 = a22 = a12 = 0;
+        });
+    s11 = block_sum(s11, red);
+    s22 = block_sum(s22, red);
+    s12 = block_sum(s12, red);
     if (threadIdx.x == 0) {
-        part[3 * blockIdx.x + 0] = s11;
-        part[3 * blockIdx.x + 1] = s22;
-        part[3 * blockIdx.x + 2] = s12;
+        const int nb = gridDim.x;
+        part[blockIdx.x] = s11;
+        part[nb + blockIdx.x] = s22;
+        part[2 * nb + blockIdx.x] = s12;
+        if (blockIdx.x == 0) *ticket = 0;
     }
 }
 
-// Pass 2 (one block): fixed-order sum of the partials into sums[0..3).
-__global__ void k_gram_finish(int nb, const double *part, double *sums) {
-    __shared__ double red[32];
-    for (int c = 0; c < 3; ++c) {
-        double t = 0.0;
-        for (int b = threadIdx.x; b < nb; b += blockDim.x) t += part[3 * b + c];
-        t = block_sum(t, red);
-        if (threadIdx.x == 0) sums[c] = t;
-    }
-}
-
-// Pass 3: ascent directions and ||m2 - (a12/a11) m1||^2 partials, which give
+// Ascent directions, and ||m2 - (a12/a11) m1||^2, which gives
 // S = a11 ||m2 - (a12/a11) m1||^2 without the cancellation of a11 a22 - a12^2.
-template <typename R>
-__global__ void __launch_bounds__(256) k_gram_dirs(int64_t n, const R *m1, const R *m2, const double *sums,
-                                                   R *l1, R *l2, double *part) {
-    __shared__ double red[32];
-    const double a11 = sums[0], a22 = sums[1], a12 = sums[2];
-    const R c11 = (R)a11, c22 = (R)a22, c12 = (R)a12;
-    const R ratio = a11 > 0 ? (R)(a12 / a11) : R(0);
-    R res = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const R x = m1[i], y = m2[i];
-        if (l1) l1[i] = c22 * x - c12 * y;
-        if (l2) l2[i] = c11 * y - c12 * x;
-        const R d = y - ratio * x;
-        res += d * d;
+template <typename R, bool VEC>
+__global__ void __launch_bounds__(kGramThreads) k_gram_dirs(int64_t n, const R *m1, const R *m2, const double *part,
+                                                            R *l1, R *l2, double *part2, unsigned *ticket, double *S) {
+    __shared__ double red[32], sums[3];
+    __shared__ R coef[4];
+    __shared__ bool last;
+    const int nb = gridDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pdl_wait();
+    if (warp < 3) {  // one warp a sum, in a fixed order
+        double t = 0.0;
+        for (int b = lane; b < nb; b += 32) t += part[warp * nb + b];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) sums[warp] = t;
     }
-    const double s = block_sum((double)res, red);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
-__global__ void k_gram_value(int nb, const double *part, const double *sums, double *S) {
-    __shared__ double red[32];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        coef[0] = (R)sums[0];
+        coef[1] = (R)sums[1];
+        coef[2] = (R)sums[2];
+        coef[3] = sums[0] > 0 ? (R)(sums[2] / sums[0]) : R(0);
+    }
+    __syncthreads();
+    const R c11 = coef[0], c22 = coef[1], c12 = coef[2], ratio = coef[3];
+    double s = 0;
+    R res = 0;
+    gram_chunks<R, VEC>(
+        n, m1, m2,
+        [&](int64_t i, const auto &x, const auto &y) {
+            constexpr int N = (int)(sizeof(x) / sizeof(R));
+            R u[N], v[N];
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                u[k] = c22 * x[k] - c12 * y[k];
+                v[k] = c11 * y[k] - c12 * x[k];
+                const R d = y[k] - ratio * x[k];
+                res += d * d;
+            }
+            if constexpr (N > 1) {
+                using V = typename Vec16<R>::T;
+                if (l1) *reinterpret_cast<V *>(l1 + i) = reinterpret_cast<const V &>(u);
+                if (l2) *reinterpret_cast<V *>(l2 + i) = reinterpret_cast<const V &>(v);
+            } else {
+                if (l1) l1[i] = u[0];
+                if (l2) l2[i] = v[0];
+            }
+        },
+        [&]() {
+            s += (double)res;
+            res = 0;
+        });
+    s = block_sum(s, red);
+    if (threadIdx.x == 0) {
+        part2[blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == (unsigned)nb - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
     double t = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) t += part[b];
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) t += __ldcg(part2 + b);
     t = block_sum(t, red);
     if (threadIdx.x == 0) *S = sums[0] > 0 ? sums[0] * t : 0.0;
+}
+
+// The two launches on a scratch of kGramDoubles doubles.
+template <typename R, bool VEC>
+static cudaError_t gramian_kernels(int64_t n, const R *m1, const R *m2, double *S, R *l1, R *l2, double *scratch,
+                                   cudaStream_t st) {
+    const int64_t per = (int64_t)kGramThreads * kGramChunk;
+    const int nb = (int)std::min<int64_t>(kGramBlocks, (n + per - 1) / per);
+    double *part = scratch, *part2 = scratch + 3 * kGramBlocks;
+    unsigned *ticket = reinterpret_cast<unsigned *>(scratch + 4 * kGramBlocks);
+    launch_after(k_gram_dots<R, VEC>, dim3(nb), dim3(kGramThreads), 0, st, n, m1, m2, part, ticket);
+    launch_after(k_gram_dirs<R, VEC>, dim3(nb), dim3(kGramThreads), 0, st, n, m1, m2, part, l1, l2, part2, ticket, S);
+    return cudaGetLastError();
+}
+template <typename R>
+static cudaError_t gramian_on(int64_t n, const void *m1, const void *m2, double *S, void *l1, void *l2,
+                              double *scratch, cudaStream_t st) {
+    // 16-byte loads and stores where every vector starts on 16 bytes
+    const uintptr_t at = (uintptr_t)m1 | (uintptr_t)m2 | (uintptr_t)l1 | (uintptr_t)l2;
+    return (at & 15) == 0 ? gramian_kernels<R, true>(n, (const R *)m1, (const R *)m2, S, (R *)l1, (R *)l2, scratch, st)
+                          : gramian_kernels<R, false>(n, (const R *)m1, (const R *)m2, S, (R *)l1, (R *)l2, scratch, st);
+}
+
+// Scratch comes from a memory pool of the library's own, one per device, which keeps up to
+// kPoolKeep bytes between calls (the default pool gives its memory back at every
+// synchronisation: the next allocation then cost some 200 us on the host).  Blocks are
+// stream-ordered, so calls on any streams and threads have scratch of their own.  Under stream
+// capture, or if the pool cannot be made, the default pool serves.
+constexpr uint64_t kPoolKeep = 32 << 20;  // (a pool reserves memory in large pieces)
+static cudaMemPool_t scratch_pool(int dev) {
+    static std::mutex mu;
+    static std::map<int, cudaMemPool_t> pools;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = pools.find(dev);
+    if (it != pools.end()) return it->second;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = kPoolKeep;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+        cudaGetLastError();
+        pool = nullptr;
+    } else if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        cudaMemPoolDestroy(pool);
+        pool = nullptr;
+    }
+    pools[dev] = pool;
+    return pool;
+}
+static cudaError_t scratch_take(double **p, size_t doubles, cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e != cudaSuccess) return e;
+    int dev = 0;
+    if (cap == cudaStreamCaptureStatusNone) {
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+        if (cudaMemPool_t pool = scratch_pool(dev))
+            return cudaMallocFromPoolAsync(reinterpret_cast<void **>(p), doubles * sizeof(double), pool, st);
+    }
+    return cudaMallocAsync(reinterpret_cast<void **>(p), doubles * sizeof(double), st);
 }
 
 template <typename R>
 static gj_status gramian_launch(int64_t n, const void *m1, const void *m2, double *S, void *l1, void *l2,
                                 cudaStream_t st) {
-    const int nb = (int)std::min<int64_t>(4 * 152, std::max<int64_t>(1, (n + 255) / 256));
     double *scratch = nullptr;
-    GJ_CUDA(cudaMallocAsync(&scratch, (3 * nb + 3) * sizeof(double), st));
-    double *part = scratch, *sums = scratch + 3 * nb;
-    k_gram_dots<R><<<nb, 256, 0, st>>>(n, (const R *)m1, (const R *)m2, part);
-    k_gram_finish<<<1, 256, 0, st>>>(nb, part, sums);
-    k_gram_dirs<R><<<nb, 256, 0, st>>>(n, (const R *)m1, (const R *)m2, sums, (R *)l1, (R *)l2, part);
-    k_gram_value<<<1, 256, 0, st>>>(nb, part, sums, S);
-    cudaError_t e = cudaGetLastError();
+    GJ_CUDA(scratch_take(&scratch, kGramDoubles, st));
+    cudaError_t e = gramian_on<R>(n, m1, m2, S, l1, l2, scratch, st);
     cudaFreeAsync(scratch, st);
     if (e != cudaSuccess) return cuda_fail(e, "gramian launch");
     return GJ_OK;
@@ -132,7 +296,7 @@ template <typename R>
 static gj_status pearson_launch(int64_t n, const void *a, const void *b, double *r, cudaStream_t st) {
     const int nb = (int)std::min<int64_t>(2 * 152, std::max<int64_t>(1, (n + 255) / 256));
     double *scratch = nullptr;
-    GJ_CUDA(cudaMallocAsync(&scratch, 5 * (size_t)nb * sizeof(double), st));
+    GJ_CUDA(scratch_take(&scratch, 5 * (size_t)nb, st));
     k_sums2<R><<<nb, 256, 0, st>>>(n, (const R *)a, (const R *)b, scratch);
     k_centred3<R><<<nb, 256, 0, st>>>(n, (const R *)a, (const R *)b, scratch, nb, scratch + 2 * nb);
     k_pearson_finish<<<1, 1, 0, st>>>(nb, scratch + 2 * nb, r);
@@ -169,13 +333,11 @@ extern "C" gj_status gj_gramian_value_grad(int64_t n, gj_precision prec, const v
 namespace gj {
 namespace {
 
-constexpr int kNoAllocMaxBlocks = 4096;             // partial sums per call
-constexpr int64_t kNoAllocChunk = 4096;             // elements per block
-constexpr int64_t kNoAllocMaxN = (int64_t)kNoAllocMaxBlocks * kNoAllocChunk;  // 16,777,216
-constexpr int kNoAllocDoubles = 3 * kNoAllocMaxBlocks + 3 + kNoAllocMaxBlocks;  // 131,096 bytes
+constexpr int64_t kNoAllocMaxN = 16777216;
+
 constexpr int kMaxDevices = 64;
 
-static __device__ __align__(256) double g_noalloc_scratch[kNoAllocDoubles];
+static __device__ __align__(256) double g_noalloc_scratch[kGramDoubles];
 
 std::mutex g_noalloc_mu;
 double *g_noalloc_addr[kMaxDevices] = {};
@@ -205,16 +367,8 @@ gj_status gramian_launch_noalloc(int64_t n, const void *m1, const void *m2, doub
     double *scratch = nullptr;
     gj_status rc = noalloc_scratch(&scratch);
     if (rc != GJ_OK) return rc;
-    const int nb = (int)((n + kNoAllocChunk - 1) / kNoAllocChunk);
-    double *part = scratch;                                  // 3 per block
-    double *sums = scratch + 3 * kNoAllocMaxBlocks;          // 3
-    double *part2 = sums + 3;                                // 1 per block
     // every slot that is read is written earlier in the same call: nothing needs clearing
-    k_gram_dots<R><<<nb, 256, 0, st>>>(n, (const R *)m1, (const R *)m2, part);
-    k_gram_finish<<<1, 256, 0, st>>>(nb, part, sums);
-    k_gram_dirs<R><<<nb, 256, 0, st>>>(n, (const R *)m1, (const R *)m2, sums, (R *)l1, (R *)l2, part2);
-    k_gram_value<<<1, 256, 0, st>>>(nb, part2, sums, S);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = gramian_on<R>(n, m1, m2, S, l1, l2, scratch, st);
     return e == cudaSuccess ? GJ_OK : cuda_fail(e, "gramian (no allocation) launch");
 }
 
