@@ -12,6 +12,8 @@
 // columns (W -> Y = V^) -> per layer conj(T^_r) V^ and inverse columns (Y -> Z)
 // -> inverse rows cropped to the prisms (Z -> g).
 #pragma once
+#include <utility>
+
 #include "fft.cuh"
 
 namespace gj {
@@ -81,6 +83,36 @@ __device__ __forceinline__ void staged_loop(int total, Load load, Store store) {
         }
     }
 }
+// The same with the first batch taken apart: loads(...) issues it, stores(...) hands it over and
+// runs the rest of the loop, so that other loads and waits can stand between the two.
+template <int U, class Load>
+struct FirstBatch {
+    decltype(std::declval<Load>()(0)) v[U];
+    __device__ __forceinline__ void loads(int total, const Load &load) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int it = threadIdx.x + u * (int)blockDim.x;
+            if (it < total) v[u] = load(it);
+        }
+    }
+    template <class Store>
+    __device__ __forceinline__ void stores(int total, const Load &load, const Store &store) {
+        for (int it0 = threadIdx.x; it0 < total;) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int it = it0 + u * (int)blockDim.x;
+                if (it < total) store(it, v[u]);
+            }
+            it0 += U * blockDim.x;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int it = it0 + u * (int)blockDim.x;
+                if (it < total) v[u] = load(it);
+            }
+        }
+    }
+};
+
 // Elements of a row functor's loops in flight per thread.
 template <typename R> constexpr int kRowU = sizeof(R) == 8 ? 2 : 4;
 
@@ -97,10 +129,17 @@ struct LoadPlain {  // a = x0[la*pitch + j], b = x1[lb*pitch + j]
     int pitch;
     static constexpr int NPRE = 1;  // rows la of x0 and lb of x1, staged by the 512 team passes
     __device__ const R *pre_src(int, int i) const { return i == 0 ? x0 : x1; }
+    using Real = R;
+    static constexpr int NS = 0;
+    __device__ __forceinline__ R scalar(int) const { return R(0); }
+    __device__ __forceinline__ void begin() {}
+    __device__ __forceinline__ void set(const R *) {}
     __device__ void init() {}
     struct Raw { R a, b; };
     __device__ __forceinline__ Raw load(int la, int lb, bool hb, int j) const {
-        return Raw{x0[(size_t)la * pitch + j], hb ? x1[(size_t)lb * pitch + j] : R(0)};
+        const R a = x0[(size_t)la * pitch + j];
+        const R b = *(hb ? x1 + (size_t)lb * pitch + j : x0 + (size_t)la * pitch + j);  // (no branch between loads)
+        return Raw{a, hb ? b : R(0)};
     }
     __device__ __forceinline__ void apply(const Raw &q, int, int, bool, int, R &a, R &b) const {
         a = q.a;
@@ -133,6 +172,11 @@ struct StorePlain {
     static constexpr int NPRE = 0;  // reads nothing
     __device__ const R *pre_src(int, int) const { return nullptr; }
     __device__ __forceinline__ void prefetch(int, int, bool, int, int) const {}
+    using Real = R;
+    static constexpr int NS = 0;
+    __device__ __forceinline__ R scalar(int) const { return R(0); }
+    __device__ __forceinline__ void begin() {}
+    __device__ __forceinline__ void set(const R *) {}
     __device__ void init() {}
     struct Raw {};
     __device__ __forceinline__ Raw load(int, int, bool, int) const { return Raw{}; }
@@ -167,6 +211,11 @@ struct LoadPlain2 {  // field f: lines la and lb of x[f]
     const R *x[2];
     int pitch;
     static constexpr int NPRE = LoadPlain<R>::NPRE;
+    using Real = R;
+    static constexpr int NS = 0;
+    __device__ __forceinline__ R scalar(int) const { return R(0); }
+    __device__ __forceinline__ void begin() {}
+    __device__ __forceinline__ void set(const R *) {}
     __device__ void init() {}
     __device__ void flush(double *) const {}
     __device__ LoadPlain<R> of(int f) const {  // a select, not an indexed load
@@ -179,6 +228,11 @@ struct StorePlain2 {  // field f: lines la and lb of y[f]
     R *y[2];
     int pitch;
     static constexpr int NPRE = StorePlain<R>::NPRE;
+    using Real = R;
+    static constexpr int NS = 0;
+    __device__ __forceinline__ R scalar(int) const { return R(0); }
+    __device__ __forceinline__ void begin() {}
+    __device__ __forceinline__ void set(const R *) {}
     __device__ void init() {}
     __device__ void flush(double *) const {}
     __device__ StorePlain<R> of(int f) const {  // a select, not an indexed load
@@ -219,6 +273,15 @@ template <typename C>
 __device__ __forceinline__ void load_twiddles(C *tw, const C *src, int N) {
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = src[i];
 }
+// the same as asynchronous copies: the caller waits (cp_async_wait) before a barrier that
+// precedes the first use
+template <typename C>
+__device__ __forceinline__ void copy_twiddles(C *tw, const C *src, int N) {
+    for (int i = threadIdx.x; i < N; i += blockDim.x) cp_async(tw + i, src + i);
+    cp_async_commit();
+}
+// The stop flag of a solve, read but not yet waited for (see stopped).
+__device__ __forceinline__ int stop_flag(const int *done) { return done ? __ldcg(done) : 0; }
 
 // In-place forward transform of P lines staged in buf0 (elements < valid): returns the
 // buffer that holds the result (buf0 or buf1).  Ends with a barrier.
@@ -263,41 +326,41 @@ __device__ __forceinline__ void split_lines(const OpView<R> &op, const PairMap &
     }
 }
 
-// The Hermitian-extended A + i B of P pairs of half spectra into buf (each read once).
+// The Hermitian-extended A + i B of P pairs of half spectra into a buffer (each read once).
 template <typename R>
-__device__ __forceinline__ void stage_spectra(const OpView<R> &op, const PairMap &pm, const RowShape &rs, int q0,
-                                              const cpx<R> *in0, const cpx<R> *in1, cpx<R> *buf) {
+struct SpectraStage {
     using C = cpx<R>;
     struct Two { C a, b; };
-    const int N = op.Nx, ncol = op.ncol, np = pm.npairs();
-    const unsigned mcol = div_magic(ncol);
-    auto at = [&](int it, int &p, int &k) {
+    const OpView<R> &op;
+    PairMap pm;
+    RowShape rs;
+    int q0;
+    const C *in0, *in1;
+    unsigned mcol;
+    __device__ __forceinline__ void at(int it, int &p, int &k) const {
         if (op.tcol) { k = fast_div(it, rs.mP); p = it - k * rs.P; }
-        else { p = fast_div(it, mcol); k = it - p * ncol; }
-    };
-    staged_loop<4>(
-        ncol * rs.P,
-        [&](int it) {
-            int p, k;
-            at(it, p, k);
-            Two t{czero<C>(), czero<C>()};
-            if (q0 + p < np) {
-                int la, lb; bool hb;
-                pm.lines(q0 + p, la, lb, hb);
-                t.a = in0[pm.at(la, k, ncol, op.tcol)];
-                if (hb) t.b = in1[pm.at(lb, k, ncol, op.tcol)];
-            }
-            return t;
-        },
-        [&](int it, Two t) {
-            int p, k;
-            at(it, p, k);
-            const bool self = k == 0 || 2 * k == N;
-            if (self) { t.a.y = 0; t.b.y = 0; }
-            buf[k * rs.pitch + p] = mk<C>(t.a.x - t.b.y, t.a.y + t.b.x);
-            if (!self) buf[(N - k) * rs.pitch + p] = mk<C>(t.a.x + t.b.y, t.b.x - t.a.y);
-        });
-}
+        else { p = fast_div(it, mcol); k = it - p * op.ncol; }
+    }
+    __device__ __forceinline__ Two operator()(int it) const {
+        int p, k;
+        at(it, p, k);
+        const int np = pm.npairs();
+        int la, lb; bool hb;
+        pm.lines(min(q0 + p, np - 1), la, lb, hb);
+        Two t{in0[pm.at(la, k, op.ncol, op.tcol)], czero<C>()};
+        if (hb) t.b = in1[pm.at(lb, k, op.ncol, op.tcol)];
+        return t;
+    }
+    __device__ __forceinline__ void put(C *buf, int it, Two t) const {
+        int p, k;
+        at(it, p, k);
+        const int N = op.Nx;
+        const bool self = k == 0 || 2 * k == N;
+        if (self) { t.a.y = 0; t.b.y = 0; }
+        buf[k * rs.pitch + p] = mk<C>(t.a.x - t.b.y, t.a.y + t.b.x);
+        if (!self) buf[(N - k) * rs.pitch + p] = mk<C>(t.a.x + t.b.y, t.b.x - t.a.y);
+    }
+};
 
 // ---------------------------------------------------------------------------
 // Row pass, real -> half spectrum.  Pro::fetch(la, lb, hasb, j, a, b) supplies the
@@ -308,40 +371,53 @@ __global__ void __launch_bounds__(256) k_row_fwd(OpView<R> op, PairMap pm, int n
                                                  cpx<R> *out0, cpx<R> *out1, Pro pro, const int *done) {
     using C = cpx<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = op.Nx, P = rs.P;
+    const int N = op.Nx, P = rs.P, ncol = op.ncol;
     C *buf0 = reinterpret_cast<C *>(smem_raw);
     C *buf1 = buf0 + N * rs.pitch;
     C *tw = buf1 + N * rs.pitch;
     __shared__ double red[128];
+    __shared__ R sc[8];
     pdl_go();
-    load_twiddles(tw, op.twx, N);
+    copy_twiddles(tw, op.twx, N);
     pdl_wait();
-    if (stopped(done)) return;
-    pro.init();
+    // the stop flag, the functor's scalars and the first elements: one memory latency for all
+    const int stop = stop_flag(done);
+    pro.begin();
+    static_assert(Pro::NS <= 8, "scalars");
+    R mine = R(0);
+    if (threadIdx.x < Pro::NS) mine = pro.scalar((int)threadIdx.x);
     const int field = blockIdx.y;
     const int q0 = blockIdx.x * P;
     const int np = pm.npairs();
     const unsigned mn = div_magic(n_in);
-    auto &&fn = field_functor(pro, field);
-    using Raw = decltype(fn.load(0, 0, false, 0));
-    staged_loop<kRowU<R>>(
-        n_in * P,
-        [&](int it) {
-            const int p = fast_div(it, mn), j = it - p * n_in, q = q0 + p;
+    auto load = [&](int it) {
+        const int p = fast_div(it, mn), j = it - p * n_in, q = q0 + p;
+        int la, lb; bool hb;
+        pm.lines(min(q, np - 1), la, lb, hb);
+        return field_functor(pro, field).load(la, lb, hb, j);
+    };
+    FirstBatch<kRowU<R>, decltype(load)> first;
+    first.loads(n_in * P, load);
+    if (stop) {
+        cp_async_wait<0>();
+        return;
+    }
+    if constexpr (Pro::NS > 0) {
+        if (threadIdx.x < Pro::NS) sc[threadIdx.x] = mine;
+        __syncthreads();
+    }
+    pro.set(sc);
+    first.stores(n_in * P, load, [&](int it, const auto &raw) {
+        const int p = fast_div(it, mn), j = it - p * n_in, q = q0 + p;
+        R a = 0, b = 0;
+        if (q < np) {
             int la, lb; bool hb;
-            pm.lines(min(q, np - 1), la, lb, hb);
-            return fn.load(la, lb, hb, j);
-        },
-        [&](int it, const Raw &raw) {
-            const int p = fast_div(it, mn), j = it - p * n_in, q = q0 + p;
-            R a = 0, b = 0;
-            if (q < np) {
-                int la, lb; bool hb;
-                pm.lines(q, la, lb, hb);
-                fn.apply(raw, la, lb, hb, j, a, b);
-            }
-            buf0[j * rs.pitch + p] = mk<C>(a, b);
-        });
+            pm.lines(q, la, lb, hb);
+            field_functor(pro, field).apply(raw, la, lb, hb, j, a, b);
+        }
+        buf0[j * rs.pitch + p] = mk<C>(a, b);
+    });
+    cp_async_wait<0>();
     __syncthreads();
     const C *X = fft_staged<R, false>(op.px, rs, buf0, buf1, tw, n_in, N);
     split_lines<R>(op, pm, rs, q0, X, field ? out1 : out0, pm.joint ? out1 : (field ? out1 : out0));
@@ -356,21 +432,35 @@ __global__ void __launch_bounds__(256) k_row_inv(OpView<R> op, PairMap pm, int n
                                                  const int *done) {
     using C = cpx<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = op.Nx, P = rs.P;
+    const int N = op.Nx, P = rs.P, ncol = op.ncol;
     C *buf0 = reinterpret_cast<C *>(smem_raw);
     C *buf1 = buf0 + N * rs.pitch;
     C *tw = buf1 + N * rs.pitch;
     __shared__ double red[128];
+    __shared__ R sc[8];
     pdl_go();
-    load_twiddles(tw, op.twx, N);
+    copy_twiddles(tw, op.twx, N);
     pdl_wait();
-    if (stopped(done)) return;
-    epi.init();
+    const int stop = stop_flag(done);
+    epi.begin();
+    static_assert(Epi::NS <= 8, "scalars");
+    R mine = R(0);
+    if (threadIdx.x < Epi::NS) mine = epi.scalar((int)threadIdx.x);
     const int field = blockIdx.y;
     const int q0 = blockIdx.x * P;
     const int np = pm.npairs();
-    stage_spectra<R>(op, pm, rs, q0, field ? in1 : in0, pm.joint ? in1 : (field ? in1 : in0), buf0);
+    const SpectraStage<R> ss{op, pm, rs, q0, field ? in1 : in0, pm.joint ? in1 : (field ? in1 : in0), div_magic(ncol)};
+    FirstBatch<4, SpectraStage<R>> first;
+    first.loads(ncol * P, ss);
+    if (stop) {
+        cp_async_wait<0>();
+        return;
+    }
+    if (threadIdx.x < Epi::NS) sc[threadIdx.x] = mine;
+    first.stores(ncol * P, ss, [&](int it, const auto &t) { ss.put(buf0, it, t); });
+    cp_async_wait<0>();
     __syncthreads();
+    epi.set(sc);
     const C *X = fft_staged<R, true>(op.px, rs, buf0, buf1, tw, N, n_out);
     const unsigned mn = div_magic(n_out);
     auto &&fn = field_functor(epi, field);
@@ -404,19 +494,27 @@ __global__ void __launch_bounds__(256) k_row_resid(OpView<R> op, PairMap pm, int
                                                    Epi epi, const int *done) {
     using C = cpx<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = op.Nx, P = rs.P;
+    const int N = op.Nx, P = rs.P, ncol = op.ncol;
     C *buf0 = reinterpret_cast<C *>(smem_raw);
     C *buf1 = buf0 + N * rs.pitch;
     C *tw = buf1 + N * rs.pitch;
     __shared__ double red[128];
     pdl_go();
-    load_twiddles(tw, op.twx, N);
+    copy_twiddles(tw, op.twx, N);
     pdl_wait();
-    if (stopped(done)) return;
-    epi.init();
+    const int stop = stop_flag(done);
     const int q0 = blockIdx.x * P;
     const int np = pm.npairs();
-    stage_spectra<R>(op, pm, rs, q0, in0, in1, buf0);
+    const SpectraStage<R> ss{op, pm, rs, q0, in0, in1, div_magic(ncol)};
+    FirstBatch<4, SpectraStage<R>> first;
+    first.loads(ncol * P, ss);
+    if (stop) {
+        cp_async_wait<0>();
+        return;
+    }
+    epi.set(nullptr);
+    first.stores(ncol * P, ss, [&](int it, const auto &t) { ss.put(buf0, it, t); });
+    cp_async_wait<0>();
     __syncthreads();
     C *X = fft_staged<R, true>(op.px, rs, buf0, buf1, tw, N, n_out);
     const unsigned mn = div_magic(n_out);
@@ -593,12 +691,15 @@ __global__ void __launch_bounds__(256) k_col_fwd(OpView<R> op0, OpView<R> op1, C
             });
         __syncthreads();
     }
-    const int Gs = slots > 1 ? 1 : G;  // the sum of all groups sits in the lines of the first layer
-    auto in = [&](int k, int c) {
-        Cx y = acc[k * pitch + c];
-        for (int g = 1; g < Gs; ++g) y = cadd(y, acc[k * pitch + g * C + c]);
-        return y;
-    };
+    if (slots == 1 && G > 1) {
+        // (inside the inverse's first stage a thread added the layers of every input in turn)
+        for (int it = threadIdx.x; it < N * C; it += blockDim.x) {
+            const int k = fast_div(it, cs.mC), c = it - k * C;
+            acc[k * pitch + c] = tile_sum(k, c);
+        }
+        __syncthreads();
+    }
+    auto in = [&](int k, int c) { return acc[k * pitch + c]; };  // the sum of all layers
     auto out = [&](int n, int c, Cx x) {
         if (n < op.sy && c < cols) op.W[(size_t)n * ncol + c0 + c] = x;
     };

@@ -101,6 +101,14 @@ __device__ __forceinline__ void block_accumulate(const A *acc, double *out, doub
     }
     __syncthreads();
     if (warp == 0) {
+        if (nw <= 8) {  // few warps: one lane a value (an FP64 addition holds its scheduler for 64 cycles)
+            if (lane < K) {
+                double s = scratch[lane * nw];
+                for (int w = 1; w < nw; ++w) s += scratch[lane * nw + w];
+                if (out) atomicAdd(out + lane, s);
+            }
+            return;
+        }
         // sixteen lanes per value
 #pragma unroll
         for (int k = 0; k < K; k += 2) {

@@ -96,17 +96,19 @@ __device__ __forceinline__ void lp_factors_full<float>(int p, float d, float eps
     }
 }
 
-// The solver scalars that a pass uses, in precision R, for every thread: one warp reads and
-// converts them (a conversion is FP64 work) and the block shares them.  All threads call;
-// ends with a barrier.
-template <typename R, int N, class Get>
-__device__ __forceinline__ void share_scalars(R (&v)[N], const Get &get) {
-    static_assert(N <= 32, "one warp");
-    __shared__ R sh[N];
-    if (threadIdx.x < N) sh[threadIdx.x] = (R)get((int)threadIdx.x);
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < N; ++i) v[i] = sh[i];
+// The solver scalars that a pass uses, in precision R, for every thread: lane i of one warp
+// reads and converts scalar(i) (a conversion is FP64 work), the block shares them, and
+// set() takes them.  Functors with NS scalars inherit init() from here (all threads call it);
+// the general kernels take the steps apart, so that these loads overlap with the data's.
+template <class Fn>
+__device__ __forceinline__ void init_scalars(Fn &fn) {
+    using R = typename Fn::Real;
+    __shared__ R sh[Fn::NS > 0 ? Fn::NS : 1];
+    if constexpr (Fn::NS > 0) {
+        if (threadIdx.x < Fn::NS) sh[threadIdx.x] = fn.scalar((int)threadIdx.x);
+        __syncthreads();
+    }
+    fn.set(sh);
 }
 
 // Forward of m with the pending model update (RRCG:7-8 and the bounds) and the
@@ -120,18 +122,24 @@ struct ProModel {
     int upd, pw[2], gsp;
     R s[2], lo[2], hi[2], eps2;
     R acc[3];
-    __device__ void init() {
+    using Real = R;
+    static constexpr int NS = 7;
+    __device__ __forceinline__ R scalar(int i) const {
+        return (R)*(i < 2 ? S->s + i : i < 4 ? S->lo + (i - 2) : i < 6 ? S->hi + (i - 4) : &S->eps2);
+    }
+    __device__ __forceinline__ void begin() {  // what load() needs, and the other integers
         upd = S->pending_update;
         gsp = S->gspace;
-        R v[7];
-        share_scalars<R>(v, [&](int i) {
-            return *(i < 2 ? S->s + i : i < 4 ? S->lo + (i - 2) : i < 6 ? S->hi + (i - 4) : &S->eps2);
-        });
+        for (int i = 0; i < 2; ++i) pw[i] = S->p[i];
+    }
+    __device__ __forceinline__ void set(const R *v) {
         eps2 = v[6];
-        for (int i = 0; i < 2; ++i) {
-            s[i] = v[i]; lo[i] = v[2 + i]; hi[i] = v[4 + i]; pw[i] = S->p[i];
-        }
+        for (int i = 0; i < 2; ++i) { s[i] = v[i]; lo[i] = v[2 + i]; hi[i] = v[4 + i]; }
         acc[0] = acc[1] = acc[2] = 0;
+    }
+    __device__ void init() {
+        begin();
+        init_scalars(*this);
     }
     // the general kernels' per-element form in two steps, so that the loads of several elements
     // are in flight before the first store
@@ -142,7 +150,7 @@ struct ProModel {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             q.m[i] = F.m[i][c];
-            q.p[i] = upd ? F.p[i][c] : R(0);
+            q.p[i] = F.p[i][c];  // (zero before the first direction; unconditional, so that no load waits for upd)
             q.wh[i] = (OPT && F.whard[i]) ? F.whard[i][c] : R(1);
             q.ma[i] = (OPT && F.mapr[i]) ? F.mapr[i][c] : R(0);
         }
@@ -255,7 +263,12 @@ struct EpiResidual {
     SolverDev *S;
     int sx;
     R acc[2];
-    __device__ void init() { acc[0] = acc[1] = 0; }
+    using Real = R;
+    static constexpr int NS = 0;
+    __device__ __forceinline__ R scalar(int) const { return R(0); }
+    __device__ __forceinline__ void begin() {}
+    __device__ __forceinline__ void set(const R *) { acc[0] = acc[1] = 0; }
+    __device__ void init() { set(nullptr); }
     // y of both fields in a, b becomes W_d r~ (two steps, as in ProModel)
     struct Raw { R w[2], d[2]; };
     __device__ __forceinline__ Raw load(int la, int, bool, int j) const {
@@ -371,17 +384,25 @@ struct EpiGradient {
     R alpha[2], lam[2], eps2, g11, g22, g12;
     int pw[2], gsp, prev;
     R acc[2];
-    __device__ void init() {
-        R v[8];
-        share_scalars<R>(v, [&](int i) {
-            return *(i < 2 ? S->alpha + i : i < 4 ? S->lam + (i - 2) : i < 7 ? S->G + (i - 4) : &S->eps2);
-        });
-        for (int i = 0; i < 2; ++i) { alpha[i] = v[i]; lam[i] = v[2 + i]; pw[i] = S->p[i]; }
-        eps2 = v[7];
-        g11 = v[4]; g22 = v[5]; g12 = v[6];
+    using Real = R;
+    static constexpr int NS = 8;
+    __device__ __forceinline__ R scalar(int i) const {
+        return (R)*(i < 2 ? S->alpha + i : i < 4 ? S->lam + (i - 2) : i < 7 ? S->G + (i - 4) : &S->eps2);
+    }
+    __device__ __forceinline__ void begin() {
         gsp = S->gspace;
         prev = S->anchor == GJ_ANCHOR_PREVIOUS && S->k > 0;  // W_{k-1} m_{k-1} exists from k = 1
+        for (int i = 0; i < 2; ++i) pw[i] = S->p[i];
+    }
+    __device__ __forceinline__ void set(const R *v) {
+        for (int i = 0; i < 2; ++i) { alpha[i] = v[i]; lam[i] = v[2 + i]; }
+        eps2 = v[7];
+        g11 = v[4]; g22 = v[5]; g12 = v[6];
         acc[0] = acc[1] = 0;
+    }
+    __device__ void init() {
+        begin();
+        init_scalars(*this);
     }
     struct Raw { R m[2], wh[2], ma[2], an[2]; };
     __device__ __forceinline__ Raw load(int la, int, bool, int j) const {
@@ -483,20 +504,27 @@ struct ProDirection {
     R beta[2], eps2;
     int first, pw[2];
     R acc[4];  // (p,l)_0, (p,l)_1, ||p||^2_0, ||p||^2_1
-    __device__ void init() {
+    using Real = R;
+    static constexpr int NS = 3;
+    __device__ __forceinline__ R scalar(int i) const {
+        if (i == 2) return (R)S->eps2;
+        const double num = S->per_field ? S->ll[i] : S->ll[0] + S->ll[1];
+        const double den = S->per_field ? S->ll_prev[i] : S->ll_prev[0] + S->ll_prev[1];
+        return den > 0 ? (R)(num / den) : R(0);
+    }
+    __device__ __forceinline__ void begin() {
         first = S->k == 0;
         for (int i = 0; i < 2; ++i) pw[i] = S->p[i];
-        R v[3];
-        share_scalars<R>(v, [&](int i) {
-            if (i == 2) return S->eps2;
-            const double num = S->per_field ? S->ll[i] : S->ll[0] + S->ll[1];
-            const double den = S->per_field ? S->ll_prev[i] : S->ll_prev[0] + S->ll_prev[1];
-            return den > 0 ? num / den : 0.0;
-        });
+    }
+    __device__ __forceinline__ void set(const R *v) {
         beta[0] = v[0];
         beta[1] = v[1];
         eps2 = v[2];
         acc[0] = acc[1] = acc[2] = acc[3] = 0;
+    }
+    __device__ void init() {
+        begin();
+        init_scalars(*this);
     }
     struct Raw { R l[2], p[2], m[2], wh[2], ma[2]; };
     __device__ __forceinline__ Raw load(int la, int, bool, int j) const {
@@ -505,7 +533,7 @@ struct ProDirection {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             q.l[i] = F.l[i][c];
-            q.p[i] = first ? R(0) : F.p[i][c];
+            q.p[i] = F.p[i][c];
             q.m[i] = F.m[i][c];
             q.wh[i] = (OPT && F.whard[i]) ? F.whard[i][c] : R(1);
             q.ma[i] = (OPT && F.mapr[i]) ? F.mapr[i][c] : R(0);
@@ -597,7 +625,12 @@ struct EpiQNorm {
     SolverDev *S;
     int sx;
     R acc[2];
-    __device__ void init() { acc[0] = acc[1] = 0; }
+    using Real = R;
+    static constexpr int NS = 0;
+    __device__ __forceinline__ R scalar(int) const { return R(0); }
+    __device__ __forceinline__ void begin() {}
+    __device__ __forceinline__ void set(const R *) { acc[0] = acc[1] = 0; }
+    __device__ void init() { set(nullptr); }
     struct Raw { R w[2]; };
     __device__ __forceinline__ Raw load(int la, int, bool, int j) const {
         const size_t t = (size_t)la * sx + j;
