@@ -70,8 +70,21 @@ inline int pick_layer_lines(const FftPlanDev &pl, int C, int L, size_t cs) {
 //
 // FP64 passes are bound by the two FP64 lanes of an SM: the shape with the least work on the
 // fullest SM, where a CTA costs its group transforms, one more for the residual (adjoint) or
-// a share of the sums (forward), and on average one CTA of imbalance.
+// a share of the sums (forward), some 2 us of its own, and one or two CTAs of imbalance;
+// single columns waste half of each sector.  (Forward of both fields, us: 200x180x20 at
+// 360x400 463 with four columns and two layers, 591 with one and ten; 256x256x40 at 512x512
+// 1007 with two and five, 1064 with one and twenty.)
 struct ColPick { int C, L; };
+// FP64 work of B lines relative to full warps on the four schedulers of an SM (half of what a
+// CTA leaves idle is taken by the others).
+inline double fp64_fill(const FftPlanDev &pl, int B) {
+    double f = 0.0;
+    for (int s = 0; s < pl.nst; ++s) {
+        const int items = pl.st[s].M * B, warps = (items + 31) / 32;
+        f += (warps + 3) / 4 * 128.0 / items / pl.nst;
+    }
+    return 0.5 + 0.5 * f;
+}
 inline ColPick pick_cols(const FftPlanDev &pl, int ncol, int nz, int nf, size_t cs, bool adjoint, int fixC = 0,
                          int fixL = 0) {
     const bool wide = cs == 16;  // complex doubles
@@ -93,14 +106,16 @@ inline ColPick pick_cols(const FftPlanDev &pl, int ncol, int nz, int nf, size_t 
     }
     double least = 1e300;
     for (int C = fixC > 0 ? fixC : 1; C <= (fixC > 0 ? fixC : 4); C *= 2) {
-        if (fixC <= 0 && C > 1 && (C * pl.mmax > kGenThreads || C >= 2 * ncol || !fits(C))) break;
+        if (fixC <= 0 && C > 1 && (C * pl.mmax > 2 * kGenThreads || C >= 2 * ncol || !fits(C))) break;
+        const double waste = C == 1 ? 1.2 : 1.0;
         for (int groups = 1; groups <= nz && groups <= kGenGroups; ++groups) {
             const int L = fixL > 0 ? std::min(fixL, nz) : (nz + groups - 1) / groups;
             const int G = pick_layer_lines(pl, C, L, cs), n = (nz + L - 1) / L;
-            const double work = (double)pl.N * C * G * 15.0 / 1900.0, latency = 2.5;  // microseconds
+            const double work = (double)pl.N * C * G * 15.0 / 1900.0 * waste * fp64_fill(pl, C * G);  // microseconds
+            const double ctas = tiles_of(C) * n / 152.0;
             const double t = ((L + G - 1) / G + (adjoint ? 1.0 : 0.3)) *
-                                 std::max((tiles_of(C) * n / 152.0 + 1.0) * work, latency) +
-                             (n > 1 && !adjoint ? 1.5 + 0.2 * n : 0.0);
+                                 std::max((ctas + (adjoint ? 1.0 : 2.0)) * work, 2.5) +
+                             2.0 * ctas + (n > 1 && !adjoint ? 1.5 + 0.2 * n : 0.0);
             if (t < 0.98 * least) { least = t; best = ColPick{C, L}; }
             if (fixL > 0) break;
         }
@@ -118,7 +133,9 @@ inline ColShape col_shape(const gj_op *o, int nf, int layers, size_t cs, bool ad
     if (!adjoint) s.L = std::max(s.L, (layers + o->gen_slots - 1) / o->gen_slots);
     s.G = pick_layer_lines(o->py, s.C, s.L, cs);
     const int B = s.C * s.G;
-    const bool pad = col_smem(o->Ny, odd_pitch(B), adjoint ? odd_pitch(s.C) : odd_pitch(B), cs) <= kGenSmemMax;
+    // an odd pitch where it fits; an FP64 adjoint pass takes the space for another CTA instead
+    // (256x256x40 at 512x512, both fields: 991 -> 952 us; the forward pass lost, 1007 -> 1045)
+    const bool pad = !(adjoint && cs == 16) && col_smem(o->Ny, odd_pitch(B), adjoint ? odd_pitch(s.C) : odd_pitch(B), cs) <= kGenSmemMax;
     s.pitch = pad ? odd_pitch(B) : B;
     s.pitch1 = pad ? odd_pitch(s.C) : s.C;
     s.mB = div_magic(B);
