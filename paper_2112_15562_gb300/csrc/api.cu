@@ -1,6 +1,8 @@
 // Error reporting and library metadata.
 #include <stdio.h>
 
+#include <map>
+#include <mutex>
 #include <string>
 
 #include "gj_internal.h"
@@ -15,6 +17,38 @@ gj_status cuda_fail(cudaError_t e, const char *what) {
     std::string m = std::string(what) + ": " + cudaGetErrorName(e) + " (" + cudaGetErrorString(e) + ")";
     set_error(m);
     return e == cudaErrorMemoryAllocation ? GJ_ERR_OOM : GJ_ERR_CUDA;
+}
+
+constexpr uint64_t kPoolKeep = 128 << 20;  // (a pool reserves memory in pieces of 32 MB)
+static cudaMemPool_t own_pool(int dev) {
+    static std::mutex mu;
+    static std::map<int, cudaMemPool_t> pools;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = pools.find(dev);
+    if (it != pools.end()) return it->second;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = kPoolKeep;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+        cudaGetLastError();
+        pool = nullptr;
+    } else if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        cudaMemPoolDestroy(pool);
+        pool = nullptr;
+    }
+    pools[dev] = pool;
+    return pool;
+}
+cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t st) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (cudaMemPool_t pool = own_pool(dev)) return cudaMallocFromPoolAsync(p, bytes, pool, st);
+    return cudaMallocAsync(p, bytes, st);
 }
 
 }  // namespace gj

@@ -62,6 +62,12 @@ int  autotune_size(int minN);               // smallest 7-smooth N >= minN
 size_t elem_bytes(gj_precision p);           // bytes of one real value
 void make_twiddles(int N, std::vector<double> &re, std::vector<double> &im);
 
+// Stream-ordered device memory from a pool of the library's own, one per device, which keeps
+// up to 128 MB between uses and gives the rest back at the next synchronisation (the default
+// pool gives everything back, and an allocation then costs some 100 us; so does cudaMalloc).
+// Any stream or thread may call; free with cudaFreeAsync in the stream, or with cudaFree.
+cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t st);
+
 template <typename R> struct OpView;
 template <typename R> OpView<R> view_of(const gj_op *op);
 

@@ -1,6 +1,5 @@
 // The Gramian coupling term (Eq. Gramian) and its ascent directions (RRCG:2-3).
 #include <algorithm>
-#include <map>
 #include <mutex>
 #include <string>
 
@@ -194,45 +193,12 @@ static cudaError_t gramian_on(int64_t n, const void *m1, const void *m2, double 
                           : gramian_kernels<R, false>(n, (const R *)m1, (const R *)m2, S, (R *)l1, (R *)l2, scratch, st);
 }
 
-// Scratch comes from a memory pool of the library's own, one per device, which keeps up to
-// kPoolKeep bytes between calls (the default pool gives its memory back at every
-// synchronisation: the next allocation then cost some 200 us on the host).  Blocks are
-// stream-ordered, so calls on any streams and threads have scratch of their own.  Under stream
-// capture, or if the pool cannot be made, the default pool serves.
-constexpr uint64_t kPoolKeep = 32 << 20;  // (a pool reserves memory in large pieces)
-static cudaMemPool_t scratch_pool(int dev) {
-    static std::mutex mu;
-    static std::map<int, cudaMemPool_t> pools;
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = pools.find(dev);
-    if (it != pools.end()) return it->second;
-    cudaMemPoolProps props{};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = dev;
-    cudaMemPool_t pool = nullptr;
-    uint64_t keep = kPoolKeep;
-    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
-        cudaGetLastError();
-        pool = nullptr;
-    } else if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-        cudaGetLastError();
-        cudaMemPoolDestroy(pool);
-        pool = nullptr;
-    }
-    pools[dev] = pool;
-    return pool;
-}
+// Under stream capture the default pool serves: the block becomes a node of the graph.
 static cudaError_t scratch_take(double **p, size_t doubles, cudaStream_t st) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(st, &cap);
     if (e != cudaSuccess) return e;
-    int dev = 0;
-    if (cap == cudaStreamCaptureStatusNone) {
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if (cudaMemPool_t pool = scratch_pool(dev))
-            return cudaMallocFromPoolAsync(reinterpret_cast<void **>(p), doubles * sizeof(double), pool, st);
-    }
+    if (cap == cudaStreamCaptureStatusNone) return pool_alloc(reinterpret_cast<void **>(p), doubles * sizeof(double), st);
     return cudaMallocAsync(reinterpret_cast<void **>(p), doubles * sizeof(double), st);
 }
 

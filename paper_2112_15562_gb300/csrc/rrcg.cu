@@ -144,9 +144,32 @@ __global__ void k_report(const SolverDev *S, const int *err, gj_rrcg_report *rep
     rep->S_G = S->SG_last;
 }
 
+// W_d = 1 / sigma (s values, field blockIdx.y) and 1 / W_depth (nz values) of both fields.
 template <typename R>
-__global__ void k_reciprocal(int n, const R *sigma, R *wd) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) wd[i] = R(1) / sigma[i];
+struct Reciprocals {
+    const R *sigma[2], *wdep[2];
+    R *wd[2], *iwdep[2];
+    int s, nz;
+};
+template <typename R>
+__global__ void k_reciprocals(Reciprocals<R> q) {
+    const int f = blockIdx.y, i0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    for (int i = i0; i < q.s; i += step) q.wd[f][i] = R(1) / q.sigma[f][i];
+    for (int i = i0; i < q.nz; i += step) q.iwdep[f][i] = R(1) / q.wdep[f][i];
+}
+template <typename R>
+static void launch_reciprocals(R *buf, size_t n, size_t s, int nz, const void *const sigma[2],
+                               const void *const w_depth[2], cudaStream_t st) {
+    Reciprocals<R> q;
+    for (int i = 0; i < 2; ++i) {
+        q.sigma[i] = static_cast<const R *>(sigma[i]);
+        q.wdep[i] = static_cast<const R *>(w_depth[i]);
+        q.wd[i] = buf + 4 * n + (2 + i) * s;
+        q.iwdep[i] = buf + 4 * n + 4 * s + (size_t)i * nz;
+    }
+    q.s = (int)s;
+    q.nz = nz;
+    k_reciprocals<R><<<dim3(64, 2), 256, 0, st>>>(q);
 }
 
 }  // namespace gj
@@ -463,11 +486,16 @@ static gj_status check_ops(const gj_op *const ops[2]) {
 
 }  // namespace gj
 
-extern "C" gj_status gj_rrcg_create(const gj_op *const ops[2], const gj_rrcg_params *P,
-                                    const void *const dobs[2], const void *const sigma[2],
-                                    const void *const m_apr[2], const void *const w_depth[2],
-                                    const void *const w_hard[2], void *const m[2], gj_rrcg_hist *hist,
-                                    gj_stream_t stream, gj_rrcg **out) {
+// Creation was host time: two cudaMalloc, four small launches, and two cudaFree at the end (each a
+// device-wide synchronisation).  One stream-ordered block of the library's pool and one launch
+// for the reciprocals take their place: create and destroy of a 256 x 256 x 40 solver went from
+// 258 + 110 to 157 + 28 us, six uneven ones from 1540 + 350 to 900 + 25 us.  wait: the solver is
+// ready for any stream on return.  The one-shot solve stays in its stream and does not wait, so
+// that its graph is captured while the first residual runs (70 us).
+static gj_status rrcg_create(const gj_op *const ops[2], const gj_rrcg_params *P, const void *const dobs[2],
+                             const void *const sigma[2], const void *const m_apr[2], const void *const w_depth[2],
+                             const void *const w_hard[2], void *const m[2], gj_rrcg_hist *hist, gj_stream_t stream,
+                             bool wait, gj_rrcg **out) {
     if (!out) { set_error("gj_rrcg_create: out is NULL"); return GJ_ERR_ARG; }
     *out = nullptr;
     gj_status rc = check_ops(ops);
@@ -490,6 +518,13 @@ extern "C" gj_status gj_rrcg_create(const gj_op *const ops[2], const gj_rrcg_par
     if (P->gramian_space != GJ_GRAMIAN_ORIGINAL && P->gramian_space != GJ_GRAMIAN_WEIGHTED) {
         set_error("gj_rrcg_create: bad gramian_space"); return GJ_ERR_ARG;
     }
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    GJ_CUDA(cudaStreamIsCapturing(st, &cap));
+    if (cap != cudaStreamCaptureStatusNone) {
+        set_error("gj_rrcg_create: the stream is being captured");
+        return GJ_ERR_CUDA;
+    }
     gj_rrcg *sv = new (std::nothrow) gj_rrcg();
     if (!sv) { set_error("gj_rrcg_create: host allocation failed"); return GJ_ERR_OOM; }
     const gj_op *o = ops[0];
@@ -504,15 +539,19 @@ extern "C" gj_status gj_rrcg_create(const gj_op *const ops[2], const gj_rrcg_par
     }
     sv->hist = hist;
     sv->prev_anchor = P->anchor == GJ_ANCHOR_PREVIOUS;
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const size_t es = elem_bytes(o->prec);
     const size_t n = (size_t)o->nx * o->ny * o->nz, s = (size_t)o->sx * o->sy;
     cudaError_t e;
-    if ((e = cudaMalloc(&sv->S, sizeof(SolverDev))) != cudaSuccess) { delete sv; return cuda_fail(e, "solver state"); }
+    // one block: the state, then the vectors
     const size_t nbuf = 4 * n + 4 * s + 2 * (size_t)o->nz + (sv->prev_anchor ? 2 * n : 0);
-    if ((e = cudaMalloc(&sv->buf, nbuf * es)) != cudaSuccess) {
-        cudaFree(sv->S); delete sv; return cuda_fail(e, "solver vectors");
+    constexpr size_t kStateBytes = (sizeof(SolverDev) + 255) / 256 * 256;
+    void *blk = nullptr;
+    if ((e = pool_alloc(&blk, kStateBytes + nbuf * es, st)) != cudaSuccess) {
+        delete sv;
+        return cuda_fail(e, "solver state and vectors");
     }
+    sv->S = static_cast<SolverDev *>(blk);
+    sv->buf = static_cast<char *>(blk) + kStateBytes;
     SolverDev h{};
     h.kmax = P->kmax;
     h.stop_on_chi2 = P->stop_on_chi2;
@@ -530,31 +569,27 @@ extern "C" gj_status gj_rrcg_create(const gj_op *const ops[2], const gj_rrcg_par
     h.hist = hist;
     cudaMemcpyAsync(sv->S, &h, sizeof(h), cudaMemcpyHostToDevice, st);
     cudaMemsetAsync(sv->buf, 0, 4 * n * es, st);
-    // W_d = 1 / sigma
-    for (int i = 0; i < 2; ++i) {
-        void *wd = static_cast<char *>(sv->buf) + (4 * n + (2 + i) * s) * es;
-        if (o->prec == GJ_FP64)
-            k_reciprocal<double><<<64, 256, 0, st>>>((int)s, (const double *)sigma[i], (double *)wd);
-        else
-            k_reciprocal<float><<<64, 256, 0, st>>>((int)s, (const float *)sigma[i], (float *)wd);
-    }
-    // 1 / W_depth
-    for (int i = 0; i < 2; ++i) {
-        void *iw = static_cast<char *>(sv->buf) + (4 * n + 4 * s + (size_t)i * o->nz) * es;
-        if (o->prec == GJ_FP64)
-            k_reciprocal<double><<<1, 256, 0, st>>>(o->nz, (const double *)w_depth[i], (double *)iw);
-        else
-            k_reciprocal<float><<<1, 256, 0, st>>>(o->nz, (const float *)w_depth[i], (float *)iw);
-    }
+    if (o->prec == GJ_FP64) launch_reciprocals(static_cast<double *>(sv->buf), n, s, o->nz, sigma, w_depth, st);
+    else launch_reciprocals(static_cast<float *>(sv->buf), n, s, o->nz, sigma, w_depth, st);
     if (o->prec == GJ_FP64) run_head<double>(sv, st); else run_head<float>(sv, st);
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess && wait) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
-        cudaFree(sv->S); cudaFree(sv->buf); delete sv;
+        cudaStreamSynchronize(st);  // (freeing pool memory does not wait for its kernels)
+        cudaFree(sv->S);
+        delete sv;
         return cuda_fail(e, "gj_rrcg_create");
     }
     *out = sv;
     return GJ_OK;
+}
+
+extern "C" gj_status gj_rrcg_create(const gj_op *const ops[2], const gj_rrcg_params *P,
+                                    const void *const dobs[2], const void *const sigma[2],
+                                    const void *const m_apr[2], const void *const w_depth[2],
+                                    const void *const w_hard[2], void *const m[2], gj_rrcg_hist *hist,
+                                    gj_stream_t stream, gj_rrcg **out) {
+    return rrcg_create(ops, P, dobs, sigma, m_apr, w_depth, w_hard, m, hist, stream, true, out);
 }
 
 extern "C" gj_status gj_rrcg_iterate(gj_rrcg *sv, int iters, int use_graph, gj_stream_t stream) {
@@ -708,8 +743,7 @@ extern "C" void gj_rrcg_destroy(gj_rrcg *sv) {
     for (auto g : sv->seg_graph) cudaGraphDestroy(g);
     for (auto *v : {&sv->eager_pairs, &sv->graph_pairs, &sv->free_pairs})
         for (auto &p : *v) { cudaEventDestroy(p.a); cudaEventDestroy(p.b); }
-    cudaFree(sv->S);
-    cudaFree(sv->buf);
+    cudaFree(sv->S);  // (the vectors are in the same block)
     delete sv;
 }
 
@@ -736,7 +770,7 @@ extern "C" gj_status gj_rrcg_joint_solve(const gj_op *const ops[2], const gj_rrc
                                          gj_rrcg_report *rep, gj_stream_t stream) {
     if (!rep) { set_error("gj_rrcg_joint_solve: rep is NULL"); return GJ_ERR_ARG; }
     gj_rrcg *sv = nullptr;
-    gj_status rc = gj_rrcg_create(ops, P, dobs, sigma, m_apr, w_depth, w_hard, m, hist, stream, &sv);
+    gj_status rc = rrcg_create(ops, P, dobs, sigma, m_apr, w_depth, w_hard, m, hist, stream, false, &sv);
     if (rc != GJ_OK) return rc;
     // Iterations go in chunks of eight graph replays.  The stop flag of chunk c - 1 is
     // copied into page-locked memory behind it and read while chunk c runs, so the
@@ -922,9 +956,9 @@ extern "C" gj_status gj_rrcg_joint_solve_host(const gj_op *const ops[2], const g
     if (m_apr && (m_apr[0] || m_apr[1])) per += n;
     if (w_hard && (w_hard[0] || w_hard[1])) per += n;
     char *blk = nullptr;
-    cudaError_t e = cudaMalloc(&blk, 2 * per * es);
-    if (e != cudaSuccess) return cuda_fail(e, "gj_rrcg_joint_solve_host: device buffers");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    cudaError_t e = pool_alloc(reinterpret_cast<void **>(&blk), 2 * per * es, st);
+    if (e != cudaSuccess) return cuda_fail(e, "gj_rrcg_joint_solve_host: device buffers");
     const void *d_dobs[2], *d_sig[2], *d_wdep[2], *d_mapr[2] = {nullptr, nullptr}, *d_wh[2] = {nullptr, nullptr};
     void *d_m[2];
     char *at = blk;
@@ -949,6 +983,7 @@ extern "C" gj_status gj_rrcg_joint_solve_host(const gj_op *const ops[2], const g
         }
     }
     if (e != cudaSuccess) {
+        cudaStreamSynchronize(st);  // (freeing pool memory does not wait for the copies)
         cudaFree(blk);
         return cuda_fail(e, "gj_rrcg_joint_solve_host: copies in");
     }
@@ -957,7 +992,10 @@ extern "C" gj_status gj_rrcg_joint_solve_host(const gj_op *const ops[2], const g
         for (int i = 0; i < 2 && e == cudaSuccess; ++i)
             e = cudaMemcpyAsync(m[i], d_m[i], n * es, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) rc = cuda_fail(e, "gj_rrcg_joint_solve_host: copies out");
+        if (e != cudaSuccess) {
+            cudaStreamSynchronize(st);
+            rc = cuda_fail(e, "gj_rrcg_joint_solve_host: copies out");
+        }
     }
     cudaFree(blk);
     return rc;
