@@ -369,7 +369,7 @@ def run_ours(args, rank, world, local_rank):
     # roofline of the dominant kernel: the spectrum multiply-and-sum column pass
     o = ops[0].info
     kname = ("k_col_fwd512 (persistent layer-summed spectrum multiply + inverse column FFT, both fields)"
-             if o.fast_path else "k_col_fwd_mac (layer-summed spectrum multiply, both fields)")
+             if o.fast_path else "k_col_fwd (layer-summed spectrum multiply + inverse column FFT, both fields)")
     traffic, traffic_note = profiled_traffic(o.fast_path)
     S_mag = o.nz * o.Ny * o.ncol * 8
     S_grav_min = even_spectrum_bytes(o, 4)
@@ -393,7 +393,7 @@ def run_ours(args, rank, world, local_rank):
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f32 (f64 scalars)", "data": "synthetic", "config": dict(CONFIG),
-            "roofline": roof, "clocks": ck, "gpu_launches": (10 if o.fast_path else 14) * args.steps,
+            "roofline": roof, "clocks": ck, "gpu_launches": 10 * args.steps,
             "iteration": {"algorithmic_bytes": iter_alg,
                           "algorithmic_GBs": iter_alg / (ms_per_step * 1e-3) / 1e9,
                           "frac_of_hbm": iter_alg / (ms_per_step * 1e-3) / 1e9 / hbm,

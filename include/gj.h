@@ -127,13 +127,15 @@ gj_status gj_bttb_setup(const gj_grid *grid, gj_field field, const gj_mag *mag,
 /* Setup flags for gj_bttb_setup_ex. */
 enum {
     /* Keep one layer's spectrum instead of all n_z: every product rebuilds each
-     * layer's spectrum from the closed-form prism fields (FP64 corner lattice of
-     * the layer's two depth planes, FP64 2-D FFT of its circulant table, rounded to
-     * the operator's precision) just before using it (Sec. 2.7.1 applied per
-     * layer).  The spectra are bit-identical to the stored ones; the cost is the
-     * setup work of one layer per layer per product.  Served by the general
-     * kernels (never the warp-FFT fast path); products only: the joint solver
-     * rejects such operators with GJ_ERR_UNSUPPORTED. */
+     * layer's spectrum from the closed-form prism fields (the FP64 corner lattice of
+     * every depth plane's near-field window once per product; per layer the FP64 2-D
+     * FFT of its circulant table, rounded to the operator's precision on chip, column
+     * by column) as the column pass uses it (Sec. 2.7.1 applied per layer).  The
+     * spectra are those of a stored operator up to the rounding of the FP64 build; the
+     * cost is the setup work of every layer per product.  The one spectrum plane that
+     * is kept holds the layer sum.  Served by the general kernels (never the warp-FFT
+     * fast path); products only: the joint solver rejects such operators with
+     * GJ_ERR_UNSUPPORTED. */
     GJ_SETUP_RECOMPUTE_SPECTRA = 1
 };
 
@@ -154,8 +156,9 @@ gj_status gj_op_info(const gj_op *op, gj_op_info_t *info);
  * of the autotuner (the paper has no counterpart).  P_row: line pairs per CTA of
  * the row passes; C_col: columns per CTA of the column passes; L_grp: layers per
  * CTA of the layer-summed spectrum multiply; radix_order: the radix plan of the
- * transforms (0: radix 8 first, then the odd primes ascending; 1: the same stages
- * reversed; 2: radix 4 for the power-of-two part).  A value <= 0 (or < 0 for
+ * transforms (0: the cheapest stages of radix 2 to 17; 1: the same stages reversed;
+ * 2: radix 4 for the power-of-two part, then the odd primes).  L_grp is raised where the
+ * layer groups would outnumber the operator's partial-sum slots.  A value <= 0 (or < 0 for
  * radix_order) keeps the current choice.  Any choice gives the same products up
  * to rounding.  Synchronous, host-side only; GJ_ERR_ARG if a tile does not fit
  * in shared memory.  Not for operators in use on another stream.
@@ -222,10 +225,10 @@ gj_status gj_g_adjoint(const gj_op *op, const void *r, void *g, gj_stream_t stre
 /*
  * gj_g_forward_pair / gj_g_adjoint_pair - the products of two operators in one
  * call: d[i] = A_i m[i] (or g[i] = A_i^T r[i]) for i = 0, 1, with the vectors as in
- * gj_g_forward / gj_g_adjoint.  When both operators are on the warp-FFT fast path
- * with the same grid and padded size (the gravity and magnetic operators of one joint problem), the
- * persistent column passes take both fields' columns in one launch, which fills the
- * GPU better than two single-field calls; the row passes stay per field, so that
+ * gj_g_forward / gj_g_adjoint.  When both operators are served by the same kernels
+ * with the same grid, padded size and launch shapes (the gravity and magnetic operators
+ * of one joint problem), each pass is one launch over both fields, which fills the GPU
+ * better than two single-field calls; a transform never mixes the fields, so that
  * the results round as the single-field products do.  Otherwise the call runs the
  * two products one after the other.  The two operators must differ
  * (each owns its workspace); failures as for the single products.

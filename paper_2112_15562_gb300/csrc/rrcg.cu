@@ -486,6 +486,15 @@ static gj_status check_ops(const gj_op *const ops[2]) {
 
 }  // namespace gj
 
+// A solver is not made under stream capture: its memory would be a node of the graph.
+static gj_status not_capturing(cudaStream_t st, const char *what) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    GJ_CUDA(cudaStreamIsCapturing(st, &cap));
+    if (cap == cudaStreamCaptureStatusNone) return GJ_OK;
+    set_error(std::string(what) + ": the stream is being captured");
+    return GJ_ERR_CUDA;
+}
+
 // Creation was host time: two cudaMalloc, four small launches, and two cudaFree at the end (each a
 // device-wide synchronisation).  One stream-ordered block of the library's pool and one launch
 // for the reciprocals take their place: create and destroy of a 256 x 256 x 40 solver went from
@@ -519,12 +528,7 @@ static gj_status rrcg_create(const gj_op *const ops[2], const gj_rrcg_params *P,
         set_error("gj_rrcg_create: bad gramian_space"); return GJ_ERR_ARG;
     }
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    GJ_CUDA(cudaStreamIsCapturing(st, &cap));
-    if (cap != cudaStreamCaptureStatusNone) {
-        set_error("gj_rrcg_create: the stream is being captured");
-        return GJ_ERR_CUDA;
-    }
+    if ((rc = not_capturing(st, "gj_rrcg_create")) != GJ_OK) return rc;
     gj_rrcg *sv = new (std::nothrow) gj_rrcg();
     if (!sv) { set_error("gj_rrcg_create: host allocation failed"); return GJ_ERR_OOM; }
     const gj_op *o = ops[0];
@@ -957,6 +961,7 @@ extern "C" gj_status gj_rrcg_joint_solve_host(const gj_op *const ops[2], const g
     if (w_hard && (w_hard[0] || w_hard[1])) per += n;
     char *blk = nullptr;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    if ((rc = not_capturing(st, "gj_rrcg_joint_solve_host")) != GJ_OK) return rc;
     cudaError_t e = pool_alloc(reinterpret_cast<void **>(&blk), 2 * per * es, st);
     if (e != cudaSuccess) return cuda_fail(e, "gj_rrcg_joint_solve_host: device buffers");
     const void *d_dobs[2], *d_sig[2], *d_wdep[2], *d_mapr[2] = {nullptr, nullptr}, *d_wh[2] = {nullptr, nullptr};
@@ -996,6 +1001,8 @@ extern "C" gj_status gj_rrcg_joint_solve_host(const gj_op *const ops[2], const g
             cudaStreamSynchronize(st);
             rc = cuda_fail(e, "gj_rrcg_joint_solve_host: copies out");
         }
+    } else {
+        cudaStreamSynchronize(st);  // a refused solve leaves the copies in behind
     }
     cudaFree(blk);
     return rc;

@@ -127,3 +127,26 @@ def test_solver_creation_refuses_a_capturing_stream():
     sv.close()
     for op in ops:
         op.close()
+
+
+def test_refused_host_solve_leaves_nothing_behind():
+    """A parameter refused after the inputs were copied in; the next solve is that of a fresh start."""
+    gj = lib()
+    g = synth.uniform_grid(8, 8, 8, 8, 3, 40.0)
+    ops = [gj.bttb_setup(g, "gravity", precision="fp64"), gj.bttb_setup(g, "magnetic", MAG, precision="fp64")]
+    rng = np.random.default_rng(11)
+    data = [rng.standard_normal(g.s) for _ in range(2)]
+    ones = lambda n: [np.ones(n) for _ in range(2)]
+    models = []
+    for refuse in (False, True):
+        if refuse:
+            with pytest.raises(gj.GJError):
+                gj.rrcg_joint_solve_host(ops, gj.solver_params(kmax=3, lo=(2.0, 0.0), hi=(1.0, 0.1)), data, ones(g.s),
+                                         ones(g.nz), [np.zeros(g.n) for _ in range(2)])
+        m = [np.zeros(g.n) for _ in range(2)]
+        gj.rrcg_joint_solve_host(ops, gj.solver_params(kmax=3), data, ones(g.s), ones(g.nz), m)
+        models.append(m)
+    for i in range(2):
+        assert np.array_equal(models[0][i], models[1][i])
+    for op in ops:
+        op.close()
