@@ -2,17 +2,14 @@
 // 256 stations per direction (the zero-padded half of every transform is never
 // read or computed).
 //
-// Warp FFT.  512 = 16 x 32, one warp: lane l holds x[l + 32 j] (j < 8; the upper half of the
-// inputs is zero), takes a pruned 16-point DFT over j, multiplies by W512^(l a), transposes
-// through a swizzled shared-memory tile and takes the 32-point DFT over l in two halves:
-// lane (h, a) = a + 16 h reads all 32 values of a, folds y_l +- y_(l + 16), multiplies by
-// W32^(h l) and takes a 16-point DFT for the outputs of parity h.  Lane k then holds
-// X[k + 32 k1] in register k1.  The inverse runs the same steps backwards and forms the
-// outputs n < 256 only, y[lane + 32 j].  Lines and spectra are in the layout that the row and
-// column passes load and store, lane by lane, so nothing is redistributed around a transform.
-// (The split by output parity first, a 256-point transform per half-warp, read every input
-// twice, joined the halves of the inverse with 32 shuffles and as many selects, and passed
-// each line through shared memory once more.)
+// Warp FFT.  A pruned 512-point transform of 256 inputs x[n] splits into its even
+// and odd outputs, X[2k + h] = FFT256(x[n] W512^(h n))[k]; half-warp h computes one
+// of them.  Each 256-point transform is 16 x 16: lane l holds x[l + 16 j]
+// (j < 16), takes a 16-point DFT over j, multiplies by W256^(l k2), transposes
+// through a swizzled shared-memory tile and takes a second 16-point DFT over l.
+// Lane (h, k2) then holds X[2(k2 + 16 k1) + h] = X[lambda + 32 k1] in register k1,
+// lambda = 2 k2 + h.  The inverse runs the same steps backwards and returns
+// y[n], n < 256, with the even/odd halves combined across the two half-warps.
 //
 // Layouts (per field): row-pass output Zt[r][kx][iy] (kx < 257, iy < 256),
 // spectra St[r][kx][ky] (ky < 512), inverse-column output Wt[kx][jy].  Every
@@ -71,10 +68,12 @@ __device__ __forceinline__ void tw_col(cpx<R> (&y)[16]) {
     y[N2 + 12] = w16<R, INV, N2 * 3>(y[N2 + 12]);
 }
 
-// The 16-point DFT after its first four 4-point ones.
+// 16-point DFT in place, natural order in and out.
 template <typename R, bool INV>
-__device__ __forceinline__ void dft16_tail(cpx<R> (&x)[16]) {
+__device__ __forceinline__ void dft16(cpx<R> (&x)[16]) {
     using C = cpx<R>;
+#pragma unroll
+    for (int n2 = 0; n2 < 4; ++n2) dft4<R, INV>(x[n2], x[n2 + 4], x[n2 + 8], x[n2 + 12]);
     tw_col<R, INV, 1>(x);
     tw_col<R, INV, 2>(x);
     tw_col<R, INV, 3>(x);
@@ -88,14 +87,6 @@ __device__ __forceinline__ void dft16_tail(cpx<R> (&x)[16]) {
     }
 #pragma unroll
     for (int i = 0; i < 16; ++i) x[i] = o[i];
-}
-
-// 16-point DFT in place, natural order in and out.
-template <typename R, bool INV>
-__device__ __forceinline__ void dft16(cpx<R> (&x)[16]) {
-#pragma unroll
-    for (int n2 = 0; n2 < 4; ++n2) dft4<R, INV>(x[n2], x[n2 + 4], x[n2 + 8], x[n2 + 12]);
-    dft16_tail<R, INV>(x);
 }
 
 // cos(pi j / 16) for j = 0..8 (W32^j = cos(pi j/16) - i sin(pi j/16))
@@ -118,129 +109,141 @@ __device__ __forceinline__ cpx<R> w32c(int j) {  // W32^j for 0 <= j < 16 (j kno
     return mk<cpx<R>>((R)c, (R)(-sn));
 }
 
-// First stage of the 16-point DFT of x[0..7] (x[8..15] zero), then as dft16.
-template <typename R, bool INV>
-__device__ __forceinline__ void dft16_lo8(cpx<R> (&x)[16]) {
-    using C = cpx<R>;
-#pragma unroll
-    for (int n2 = 0; n2 < 4; ++n2) {  // dft4(a, b, 0, 0)
-        const C a = x[n2], b = x[n2 + 4], m = mul_mi<C, INV>(b);
-        x[n2] = cadd(a, b);
-        x[n2 + 4] = cadd(a, m);
-        x[n2 + 8] = csub(a, b);
-        x[n2 + 12] = csub(a, m);
-    }
-    dft16_tail<R, INV>(x);
-}
-
-// a + s b, s = +-1 (one paired instruction in FP32)
-template <typename R>
-__device__ __forceinline__ cpx<R> cadds(cpx<R> a, R s, cpx<R> b) {
-    if constexpr (sizeof(R) == 4) return __ffma2_rn(b, make_float2(s, s), a);
-    else return mk<cpx<R>>(fma(s, b.x, a.x), fma(s, b.y, a.y));
-}
-
-// Per-lane twiddles of the 512-point transform, W512^(lane k) for k < 16, as
-// lo[k & 3] * hi[k >> 2] (lo[0] = hi[0] = 1): twelve registers.
+// Per-lane twiddles, l = lane & 15.  Inverse form (load_inv): W256^(l k) =
+// lo[k & 3] * hi[k >> 2] and pre = W512^l.  Forward form (load_fwd): the odd
+// half-warp's factor W512^l is folded into hi, so that
+// lo[k & 3] * hi[k >> 2] = W512^(h l) W256^(l k) and the odd half only needs the
+// constant factors W32^j before its first DFT (W512^(l + 16 j) = W512^l W32^j).
 template <typename R>
 struct LaneTw {
-    cpx<R> lo[4], hi[4];
-    __device__ void load(const cpx<R> *__restrict__ tw512) {  // tw512[k] = W512^k (global, read-only)
-        const int lane = threadIdx.x & 31;
+    cpx<R> lo[4], hi[4], pre;
+    __device__ void load_inv(const cpx<R> *__restrict__ tw512) {  // tw512[k] = W512^k (global, read-only)
+        const int l = threadIdx.x & 15;
 #pragma unroll
-        for (int k = 1; k < 4; ++k) {
-            lo[k] = __ldg(tw512 + lane * k);
-            hi[k] = __ldg(tw512 + 4 * lane * k);
+        for (int k = 0; k < 4; ++k) {
+            lo[k] = __ldg(tw512 + ((2 * l * k) & 511));
+            hi[k] = __ldg(tw512 + ((8 * l * k) & 511));
+        }
+        pre = __ldg(tw512 + l);
+    }
+    __device__ void load_fwd(const cpx<R> *__restrict__ tw512) {
+        load_inv(tw512);
+        if (threadIdx.x & 16) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) hi[k] = cmul(hi[k], pre);
         }
     }
-    __device__ __forceinline__ cpx<R> at(int k) const {  // 0 < k < 16, known at compile time
-        return (k >> 2) == 0 ? lo[k & 3] : ((k & 3) == 0 ? hi[k >> 2] : cmul(lo[k & 3], hi[k >> 2]));
+    // twiddle of output k of the first DFT: W256^(l k) (times W512^(h l) in the forward form)
+    template <bool INV> __device__ __forceinline__ cpx<R> mul256(cpx<R> a, int k) const {
+        const cpx<R> w = (k >> 2) == 0 ? lo[k & 3] : ((k & 3) == 0 ? hi[k >> 2] : cmul(lo[k & 3], hi[k >> 2]));
+        return INV ? cmulc(a, w) : cmul(a, w);
     }
+    __device__ __forceinline__ cpx<R> fwd_tw(cpx<R> a, int k) const {  // forward form, includes k = 0
+        const cpx<R> w = (k & 3) == 0 ? hi[k >> 2] : cmul(lo[k & 3], hi[k >> 2]);
+        return cmul(a, w);
+    }
+    // combine twiddle of the inverse, W512^(l + 16 j) (j known at compile time)
+    __device__ __forceinline__ cpx<R> cmb(int j) const { return cmul(pre, w32c<R>(j)); }
 };
 
 // The same twiddles read from a per-CTA shared-memory table (no per-lane products,
-// no twiddle registers), rows of 32 lanes, l = lane & 15:
-//   [k < 16]  W512^(lane k)                    (at)
-//   [16 + k]  W256^(l k), the 256 transforms'  (mul256)
+// no twiddle registers), rows of 32 lanes (h, l):
+//   [k < 16]       forward W512^(h l + 2 l k)  (fwd_tw)
+//   [16 + k]       inverse W256^(l k) = W512^(2 l k)  (mul256)
+//   [32 + jj < 40] combine W512^(l + 16 (8 h + jj))  (cmb)
 // The entries are the operator's W512 table itself, so they carry no product rounding.
 template <typename R>
 struct TabTw {
-    static constexpr int WORDS = 32 * 32;
+    static constexpr int WORDS = 40 * 32;
     const cpx<R> *t;  // shared
     int lane;
     // every thread of the CTA, followed by a barrier before first use
     __device__ static void build(cpx<R> *t, const cpx<R> *__restrict__ tw512) {
         for (int i = threadIdx.x; i < WORDS; i += blockDim.x) {
-            const int row = i >> 5, ln = i & 31;
-            t[i] = __ldg(tw512 + (row < 16 ? ln * row : 2 * (ln & 15) * (row - 16)));
+            const int row = i >> 5, ln = i & 31, h = ln >> 4, l = ln & 15;
+            const int e = row < 16 ? h * l + 2 * l * row : (row < 32 ? 2 * l * (row - 16) : l + 16 * (8 * h + row - 32));
+            t[i] = __ldg(tw512 + (e & 511));
         }
     }
     __device__ void bind(const cpx<R> *tab) { t = tab; lane = threadIdx.x & 31; }
-    __device__ __forceinline__ cpx<R> at(int k) const { return t[k * 32 + lane]; }
     template <bool INV> __device__ __forceinline__ cpx<R> mul256(cpx<R> a, int k) const {
         const cpx<R> w = t[(16 + k) * 32 + lane];
         return INV ? cmulc(a, w) : cmul(a, w);
     }
+    __device__ __forceinline__ cpx<R> fwd_tw(cpx<R> a, int k) const { return cmul(a, t[k * 32 + lane]); }
+    __device__ __forceinline__ cpx<R> cmb(int j) const { return t[(32 + (j & 7)) * 32 + lane]; }
 };
+
+// Parity-split position of spectrum index k (0 <= k < 512) in a staging row, so
+// that the lanes of a half-warp (one parity, consecutive k/2) hit consecutive words.
+__device__ __forceinline__ int ppos(int k) { return ((k & 1) << 8) | (k >> 1); }
+// and of column kx (0 <= kx <= 256) in the inverse passes' staging tile
+__device__ __forceinline__ int kpos(int kx) { return (kx & 1) ? 129 + (kx >> 1) : (kx >> 1); }
 
 // Real, even spectra (the gravity table over stations that cover the prisms) keep
 // ky <= N/2 only: KE values per column (a multiple of four, so that columns start on
-// 16 bytes).  Spectrum index ky = lane + 32 k1 of the 512 transform's lane layout
+// 16 bytes).  Spectrum index ky = lambda + 32 k1 of the 512 transform's lane layout
 // reads entry min(ky, 512 - ky), which k1 (a compile-time index) decides.
 constexpr int KE = even_spec_len(N), KEB = KE * (int)sizeof(float);  // FP32, the fast path's precision
-__device__ __forceinline__ int even_pos512(int lane, int k1) { return k1 < 8 ? lane + 32 * k1 : N - 32 * k1 - lane; }
+__device__ __forceinline__ int even_pos512(int lam, int k1) { return k1 < 8 ? lam + 32 * k1 : N - 32 * k1 - lam; }
 
-// swizzled tile of 16 columns: entry (row, col) at row * 16 + (col ^ (row mod 16))
-__device__ __forceinline__ int swz(int row, int col) { return row * 16 + (col ^ (row & 15)); }
+// swizzled 16 x 16 tile of one half-warp: entry (row, col) at row*16 + (col ^ row)
+__device__ __forceinline__ int swz(int row, int col) { return row * 16 + (col ^ row); }
 
-// Forward pruned 512-point transform.  In: v[j] = x[lane + 32 j], j < 8 (the upper
-// registers are not read).  Out: v[k1] = X[lane + 32 k1].  buf: this warp's 512-entry tile.
-// tw: LaneTw or TabTw.
+// Forward pruned 512-point transform.  In: v[j] = x[l + 16 j] (both halves).
+// Out: lane (h, k2) v[k1] = X[lambda + 32 k1].  buf: this warp's 512-entry tile.
+// tw: LaneTw in the forward form (load_fwd), or TabTw.
 template <typename R, class TW>
 __device__ __forceinline__ void fwd512(cpx<R> (&v)[16], cpx<R> *buf, const TW &tw) {
-    const int lane = threadIdx.x & 31, h = lane >> 4, a = lane & 15;
-    dft16_lo8<R, false>(v);  // over j -> index a
-#pragma unroll
-    for (int k = 1; k < 16; ++k) v[k] = cmul(v[k], tw.at(k));
-    __syncwarp();
-#pragma unroll
-    for (int k = 0; k < 16; ++k) buf[swz(lane, k)] = v[k];
-    __syncwarp();
-    // outputs b = 2 k1 + h of the 32-point DFT over l: y_l + (-1)^h y_(l + 16), times W32^(h l)
-    const R s = h ? R(-1) : R(1);
-#pragma unroll
-    for (int r = 0; r < 16; ++r) v[r] = cadds<R>(buf[swz(r, a)], s, buf[swz(r + 16, a)]);
+    const int lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
+    cpx<R> *t = buf + h * 256;
     if (h) {
 #pragma unroll
-        for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], w32c<R>(r));
+        for (int j = 1; j < 16; ++j) v[j] = cmul(v[j], w32c<R>(j));
     }
+    dft16<R, false>(v);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = tw.fwd_tw(v[k], k);
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 16; ++k) t[swz(l, k)] = v[k];
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = t[swz(r, l)];
     dft16<R, false>(v);
 }
 
-// Inverse (unnormalised).  In: v[k1] = Y[lane + 32 k1].  Out: out[j] = y[lane + 32 j], j < 8.
+// Inverse (tw in the inverse form, load_inv): in lane (h, k2) v[k1] = Y[lambda + 32 k1].  Out (unnormalised): every
+// lane of both halves holds y[n] for n = l + 16 j with j in [8h, 8h + 8):
+// out[jj] = y[l + 16 (8h + jj)], jj < 8.
 template <typename R, class TW>
 __device__ __forceinline__ void inv512(cpx<R> (&v)[16], cpx<R> *buf, const TW &tw, cpx<R> (&out)[8]) {
-    const int lane = threadIdx.x & 31, h = lane >> 4, a = lane & 15;
-    dft16<R, true>(v);  // over k1 -> index l < 16
-    if (h) {
-#pragma unroll
-        for (int l = 1; l < 16; ++l) v[l] = cmulc(v[l], w32c<R>(l));
-    }
-    __syncwarp();
+    const int lane = threadIdx.x & 31, h = lane >> 4, k2 = lane & 15;
     cpx<R> *t = buf + h * 256;
+    dft16<R, true>(v);  // over k1 -> index l
 #pragma unroll
-    for (int l = 0; l < 16; ++l) t[swz(a, l)] = v[l];
+    for (int l = 1; l < 16; ++l) v[l] = tw.template mul256<true>(v[l], l);
     __syncwarp();
-    // this lane as l: the sums over the output parities h, + for l < 16 and - beyond
-    const R s = h ? R(-1) : R(1);
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        v[k] = cadds<R>(buf[swz(k, a)], s, buf[256 + swz(k, a)]);
-        if (k > 0) v[k] = cmulc(v[k], tw.at(k));
+    for (int l = 0; l < 16; ++l) t[swz(k2, l)] = v[l];
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = t[swz(r, k2)];
+    dft16<R, true>(v);  // over k2 -> j ; now v[j] = z_h[k2 + 16 j] (this lane's l = k2)
+    // y[n] = z_0[n] + W512^-n z_1[n]
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        cpx<R> o;
+        o.x = __shfl_xor_sync(0xffffffffu, v[j].x, 16);
+        o.y = __shfl_xor_sync(0xffffffffu, v[j].y, 16);
+        const bool mine = (j >> 3) == h;
+        if (mine) {
+            const cpx<R> z0 = h ? o : v[j];
+            const cpx<R> z1 = h ? v[j] : o;
+            const cpx<R> w = tw.cmb(j);  // W512^(l + 16 j)
+            out[j & 7] = cadd(z0, cmulc(z1, w));
+        }
     }
-    dft16<R, true>(v);  // over a -> index j, of which j < 8 are kept
-#pragma unroll
-    for (int j = 0; j < 8; ++j) out[j] = v[j];
 }
 
 // ---------------------------------------------------------------------------
@@ -403,7 +406,7 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_fwd512(View2<R> V, const
     using C = cpx<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int ZB = H * sizeof(C), TB = N * sizeof(C);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
     unsigned char *wbase = smem_raw + (size_t)warp * (CSTAGES * (ZB + TB) + N * sizeof(C));
     C *zs = reinterpret_cast<C *>(wbase);                          // CSTAGES x 256
     C *ts = reinterpret_cast<C *>(wbase + CSTAGES * ZB);            // CSTAGES x 512
@@ -431,6 +434,7 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_fwd512(View2<R> V, const
     if ((long long)blockIdx.x * CWARPS < Wt) load_twtab<R>(tab, V.twtab, &tabbar);
     if (w >= Wt) return;
     const int t0 = (int)seg_begin(w, T, Wt), t1 = (int)seg_begin(w + 1, T, Wt);
+    const int lam = 2 * l + h;
     ColItem cu, ci;  // the item being consumed; (lane 0) the next one to issue
     cu.set(t0, nz, V.nfield);
     ci = cu;
@@ -468,20 +472,20 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_fwd512(View2<R> V, const
         C v[16];
         const bool real_t = V.op[cu.fld].real_spec;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = zs[s * H + lane + 32 * j];
+        for (int j = 0; j < 16; ++j) v[j] = zs[s * H + l + 16 * j];
         fwd512<R>(v, xbuf, tw);
         // multiply by the layer's spectrum straight from the stage, then release it
         if (real_t) {
             const R *tr = reinterpret_cast<const R *>(ts + s * N);
 #pragma unroll
             for (int k1 = 0; k1 < 16; ++k1) {
-                const R tt = tr[even_pos512(lane, k1)];
+                const R tt = tr[even_pos512(lam, k1)];
                 acc[k1] = mk<C>(acc[k1].x + v[k1].x * tt, acc[k1].y + v[k1].y * tt);
             }
         } else {
 #pragma unroll
             for (int k1 = 0; k1 < 16; ++k1) {  // acc += v * t, four fused multiply-adds
-                const C t = ts[s * N + lane + 32 * k1];
+                const C t = ts[s * N + lam + 32 * k1];
                 acc[k1].x = fma(v[k1].x, t.x, acc[k1].x);
                 acc[k1].x = fma(-v[k1].y, t.y, acc[k1].x);
                 acc[k1].y = fma(v[k1].x, t.y, acc[k1].y);
@@ -502,7 +506,7 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_fwd512(View2<R> V, const
                 const int slot = (int)(w - wf), nslots = (int)(wl - wf + 1);
                 C *Pc = V.P[fld] + (size_t)kx * V.slots * N;
 #pragma unroll
-                for (int k1 = 0; k1 < 16; ++k1) Pc[(size_t)slot * N + lane + 32 * k1] = acc[k1];
+                for (int k1 = 0; k1 < 16; ++k1) Pc[(size_t)slot * N + lam + 32 * k1] = acc[k1];
                 __threadfence();
                 __syncwarp();
                 int old = 0;
@@ -515,7 +519,7 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_fwd512(View2<R> V, const
                     for (int sl = 0; sl < nslots; ++sl) {
 #pragma unroll
                         for (int k1 = 0; k1 < 16; ++k1)
-                            acc[k1] = cadd(acc[k1], __ldcg(Pc + (size_t)sl * N + lane + 32 * k1));
+                            acc[k1] = cadd(acc[k1], __ldcg(Pc + (size_t)sl * N + lam + 32 * k1));
                     }
                     if (lane == 0) V.cnt[fld][kx] = 0;
                 } else {
@@ -530,7 +534,7 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_fwd512(View2<R> V, const
             C *Wc = op.W + (size_t)kx * H;
 #pragma unroll
             for (int jj = 0; jj < 8; ++jj) {
-                const int n = lane + 32 * jj;
+                const int n = l + 16 * (8 * h + jj);
                 if (n < sy) Wc[n] = out[jj];
             }
 #pragma unroll
@@ -549,7 +553,7 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_adj512(View2<R> V, const
     using C = cpx<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int TB = N * sizeof(C);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
     unsigned char *wbase = smem_raw + (size_t)warp * (CSTAGES * TB + N * sizeof(C));
     C *ts = reinterpret_cast<C *>(wbase);
     C *xbuf = reinterpret_cast<C *>(wbase + CSTAGES * TB);
@@ -576,6 +580,7 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_adj512(View2<R> V, const
     if ((long long)blockIdx.x * CWARPS < Wt) load_twtab<R>(tab, V.twtab, &tabbar);
     if (w >= Wt) return;
     const int t0 = (int)seg_begin(w, T, Wt), t1 = (int)seg_begin(w + 1, T, Wt);
+    const int lam = 2 * l + h;
     ColItem cu, ci;  // the item being consumed; (lane 0) the next one to issue
     cu.set(t0, nz, V.nfield);
     ci = cu;
@@ -607,7 +612,7 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_adj512(View2<R> V, const
             // V^ = FFT512 of the residual column (rows >= sy are zero)
             const C *Wc = op.V + (size_t)kx * H;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) vh[j] = Wc[lane + 32 * j];
+            for (int j = 0; j < 16; ++j) vh[j] = Wc[l + 16 * j];
             fwd512<R>(vh, xbuf, tw);
         }
         const int s = (t - t0) % CSTAGES;
@@ -619,12 +624,12 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_adj512(View2<R> V, const
             const R *tr = reinterpret_cast<const R *>(ts + s * N);
 #pragma unroll
             for (int k1 = 0; k1 < 16; ++k1) {
-                const R tt = tr[even_pos512(lane, k1)];
+                const R tt = tr[even_pos512(lam, k1)];
                 v[k1] = mk<C>(vh[k1].x * tt, vh[k1].y * tt);
             }
         } else {
 #pragma unroll
-            for (int k1 = 0; k1 < 16; ++k1) v[k1] = cmulc(vh[k1], ts[s * N + lane + 32 * k1]);
+            for (int k1 = 0; k1 < 16; ++k1) v[k1] = cmulc(vh[k1], ts[s * N + lam + 32 * k1]);
         }
         __syncwarp();
         if (lane == 0 && ti < t1) issue();
@@ -633,7 +638,7 @@ __global__ void __launch_bounds__(CWARPS * 32, 1) k_col_adj512(View2<R> V, const
         C *Zc = op.Z + ((size_t)r * NC + kx) * H;
 #pragma unroll
         for (int jj = 0; jj < 8; ++jj) {
-            const int n = lane + 32 * jj;
+            const int n = l + 16 * (8 * h + jj);
             if (n < ny) Zc[n] = out[jj];
         }
     }
@@ -662,7 +667,9 @@ template <typename R, class TW>
 __device__ __forceinline__ void fwd256h(cpx<R> (&v)[16], cpx<R> *buf, const TW &tw) {
     const int lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
     cpx<R> *t = buf + h * 256;
-    dft16_lo8<R, false>(v);  // over j -> index a
+#pragma unroll
+    for (int j = 8; j < 16; ++j) v[j] = czero<cpx<R>>();
+    dft16<R, false>(v);  // over j -> index a; the zero half folds away
 #pragma unroll
     for (int k = 1; k < 16; ++k) v[k] = tw.template mul256<false>(v[k], k);  // W256^(l a)
     __syncwarp();

@@ -41,20 +41,26 @@ __device__ __forceinline__ void write_half_spectra(const cpx<R> *tile, const Vie
     const C *row = tile + f * (N + 1);
     const int kstep = blockDim.x / FFTS;
     for (int kx = threadIdx.x / FFTS; kx < NC; kx += kstep) {
-        const C zk = row[kx];
-        const C zm = row[(N - kx) & (N - 1)];
+        const C zk = row[ppos(kx)];
+        const C zm = row[ppos((N - kx) & (N - 1))];
         if (ha) oa[kx * hy] = mk<C>(R(0.5) * (zk.x + zm.x), R(0.5) * (zk.y - zm.y));
         if (hb) ob[kx * hy] = mk<C>(R(0.5) * (zk.y + zm.y), R(-0.5) * (zk.x - zm.x));
     }
 }
 
-// Real input a + i b held as a[i], b[i] for elements lane + 32 i: the transform's own
-// layout.  Result in v (lane layout).
+// Real input a + i b held as a[i], b[i] for elements lane + 32 i: redistribute
+// through the warp tile and run the forward transform.  Result in v (lane layout).
 template <typename R, class TW>
 __device__ __forceinline__ void fwd512_from_lines(const R (&a)[8], const R (&b)[8], cpx<R> *buf, const TW &tw,
                                                   cpx<R> (&v)[16]) {
+    using C = cpx<R>;
+    const int lane = threadIdx.x & 31, l = lane & 15;
+    __syncwarp();
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = mk<cpx<R>>(a[i], b[i]);
+    for (int i = 0; i < 8; ++i) buf[lane + 32 * i] = mk<C>(a[i], b[i]);
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = buf[l + 16 * j];
     fwd512<R>(v, buf, tw);
 }
 
@@ -74,8 +80,8 @@ __global__ void __launch_bounds__(NW * 32, 2) k_row_fwd512(View2<R> V, int joint
     pro.init();
     __syncthreads();
     LaneTw<R> tw;
-    tw.load(V.op[0].twx);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    tw.load_fwd(V.op[0].twx);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
     const int base = blockIdx.x * (joint ? FFTS : 2 * FFTS);
     const int field = blockIdx.y;  // single mode: the field of this CTA's lines (grid y = fields)
     C *buf = xb + warp * N;
@@ -98,8 +104,9 @@ __global__ void __launch_bounds__(NW * 32, 2) k_row_fwd512(View2<R> V, int joint
         }
         C v[16];
         fwd512_from_lines<R>(a, b, buf, tw, v);
+        const int lam = 2 * l + h;
 #pragma unroll
-        for (int k1 = 0; k1 < 16; ++k1) tile[f * (N + 1) + lane + 32 * k1] = v[k1];
+        for (int k1 = 0; k1 < 16; ++k1) tile[f * (N + 1) + ppos(lam + 32 * k1)] = v[k1];
     }
     __syncthreads();
     write_half_spectra<R, FFTS>(tile, V, joint, base, nlines, lpl, out_sel, field);
@@ -126,7 +133,7 @@ __device__ __forceinline__ void stage_half_spectra(cpx<R> *tile, const View2<R> 
     // every copy in flight at once; sources past the last line read as zero (their
     // lane may pair with a valid line in the same complex transform)
     for (int kx = kx0; kx < NC; kx += kstep) {
-        C *dst = tile + kx * P + s;
+        C *dst = tile + kpos(kx) * P + s;
         if (ok) cp_async8(dst, in + (size_t)kx * hy);
         else *dst = czero<C>();
     }
@@ -141,19 +148,30 @@ __device__ __forceinline__ void inv512_to_lines(const cpx<R> *tile, int sa, int 
                                                 R (&a)[8], R (&b)[8]) {
     using C = cpx<R>;
     constexpr int P = 2 * FFTS + 1;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
+    const int lam = 2 * l + h;
     C v[16];
 #pragma unroll
     for (int k1 = 0; k1 < 16; ++k1) {
-        const int kk = k1 < 8 ? lane + 32 * k1 : N - 32 * k1 - lane;
-        C A = tile[kk * P + sa], B = tile[kk * P + sb];
-        if ((k1 == 0 || k1 == 8) && lane == 0) { A.y = 0; B.y = 0; }  // kk = 0, 256
-        v[k1] = k1 < 8 ? mk<C>(A.x - B.y, A.y + B.x) : mk<C>(A.x + B.y, B.x - A.y);
+        const int k = lam + 32 * k1;
+        const bool lo = k <= H;
+        const int kk = lo ? k : N - k;
+        C A = tile[kpos(kk) * P + sa], B = tile[kpos(kk) * P + sb];
+        if (kk == 0 || kk == H) { A.y = 0; B.y = 0; }
+        v[k1] = lo ? mk<C>(A.x - B.y, A.y + B.x) : mk<C>(A.x + B.y, B.x - A.y);
     }
     C out[8];
     inv512<R>(v, buf, tw, out);
+    __syncwarp();
 #pragma unroll
-    for (int i = 0; i < 8; ++i) { a[i] = out[i].x; b[i] = out[i].y; }
+    for (int jj = 0; jj < 8; ++jj) buf[l + 16 * (8 * h + jj)] = out[jj];
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const C y = buf[lane + 32 * i];
+        a[i] = y.x;
+        b[i] = y.y;
+    }
 }
 
 // Inverse row pass: half spectra in[r][kx][iy] -> real lines, cropped to n_out,
@@ -177,7 +195,7 @@ __global__ void __launch_bounds__(NW * 32, 2) k_row_inv512(View2<R> V, int joint
     stage_half_spectra<R, FFTS>(tile, V, joint, base, nlines, lpl, in_sel, field);
     __syncthreads();
     LaneTw<R> tw;
-    tw.load(V.op[0].twx);
+    tw.load_inv(V.op[0].twx);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     C *buf = xb + warp * N;
     for (int s2 = 0; s2 < FPW; ++s2) {
@@ -206,22 +224,22 @@ __global__ void __launch_bounds__(NW * 32, 2) k_row_inv512(View2<R> V, int joint
 // range of the aligned groups of the layers (a layer's last group may hold fewer
 // lines), so that no launch ends in a partial wave.  Two modes:
 //   joint: both fields of a line in one complex transform; a group is four lines,
-//          warp k takes line k; the tile is stage[field][slot < 4][kx] with slot
-//          stride 260 (4 mod 16);
+//          warp k takes line k; the tile is stage[field][slot < 4][kq(kx)] with slot
+//          stride 274 (2 mod 16);
 //   pair:  one field, two lines per transform (warp k: lines 2k and 2k + 1); a group
-//          is eight lines; the tile is stage[slot < 8][kx] with slot stride 258
-//          (2 mod 16).
+//          is eight lines; the tile is stage[slot < 8][kq(kx)] with slot stride 273
+//          (1 mod 16).
 // The half spectra of a group sit in a double-buffered team tile and move to or from
-// the transposed layout out[r][kx][iy] as whole 32-byte sectors.  With these strides a
-// half-warp's 16 consecutive columns of one slot, and its (column, slot) pairs of a
-// group store or load (4 x 4 or 2 x 8), each fall in 16 distinct bank pairs.  One named
-// barrier per group and team.
+// the transposed layout out[r][kx][iy] as whole 32-byte sectors.  kq puts even
+// columns first and odd ones from 136 on; with these strides a half-warp's 16
+// consecutive columns of one slot, and its (column, slot) pairs of a group store or
+// load, each fall in 16 distinct bank pairs.  One named barrier per group and team.
 // The functor rows read in every launch are staged one transform ahead with
 // asynchronous copies.
 
 constexpr int TEAM = 4;                  // warps per team
-constexpr int LS = 260, FS = TEAM * LS;  // joint tile: slot and field strides (complex words)
-constexpr int LSP = 258;                 // pair tile: slot stride (8 slots fit in 2 FS)
+constexpr int LS = 274, FS = TEAM * LS;  // joint tile: slot and field strides (complex words)
+constexpr int LSP = 273;                 // pair tile: slot stride (8 slots fit in 2 FS)
 template <bool PAIR> struct TeamMode {
     static constexpr int LPG = PAIR ? 2 * TEAM : TEAM;  // lines per group
     static constexpr int GPT = PAIR ? 8 : 4;            // slots one thread row of a store covers
@@ -231,14 +249,18 @@ __device__ __forceinline__ void team_barrier(int team) {  // barrier 0 stays wit
     asm volatile("bar.sync %0, %1;\n" ::"r"(1 + team), "r"(TEAM * 32) : "memory");
 }
 
-// Z = FFT(a + i b) in the lane layout (v[k1] = Z[lane + 32 k1]) -> the half
+__device__ __forceinline__ int kq(int kx) { return (kx & 1) ? 136 + (kx >> 1) : (kx >> 1); }
+
+// Z = FFT(a + i b) in the lane layout (v[k1] = Z[lambda + 32 k1]) -> the half
 // spectra A = (Z[kx] + conj Z[N - kx]) / 2 and B = (Z[kx] - conj Z[N - kx]) / 2i,
-// kx = 0..256, at sa[kx] and sb[kx].  For lane != 0, Z[N - kx] sits in lane 32 - lane
-// at k1' = 15 - k1; lane 0 holds it at 16 - k1.
+// kx = 0..256, at sa[kq(kx)] and sb[kq(kx)].  For lambda != 0, Z[N - kx] sits in
+// lane (h, 16 - l - h) at k1' = 15 - k1; lane 0 (lambda = 0) holds it at 16 - k1.
 template <typename R>
 __device__ __forceinline__ void split_to_stage(const cpx<R> (&v)[16], cpx<R> *sa, cpx<R> *sb) {
     using C = cpx<R>;
-    const int lane = threadIdx.x & 31, partner = (32 - lane) & 31;
+    const int lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
+    const int partner = h ? 31 - l : ((16 - l) & 15);
+    const int q0 = h * 136 + l;  // kq(lambda + 32 k1) = q0 + 16 k1
 #pragma unroll
     for (int k1 = 0; k1 < 8; ++k1) {
         C zm;
@@ -246,27 +268,28 @@ __device__ __forceinline__ void split_to_stage(const cpx<R> (&v)[16], cpx<R> *sa
         zm.y = __shfl_sync(0xffffffffu, v[15 - k1].y, partner);
         if (lane == 0) zm = v[(16 - k1) & 15];
         const C zk = v[k1];
-        sa[lane + 32 * k1] = mk<C>(R(0.5) * (zk.x + zm.x), R(0.5) * (zk.y - zm.y));
-        sb[lane + 32 * k1] = mk<C>(R(0.5) * (zk.y + zm.y), R(-0.5) * (zk.x - zm.x));
+        sa[q0 + 16 * k1] = mk<C>(R(0.5) * (zk.x + zm.x), R(0.5) * (zk.y - zm.y));
+        sb[q0 + 16 * k1] = mk<C>(R(0.5) * (zk.y + zm.y), R(-0.5) * (zk.x - zm.x));
     }
     if (lane == 0) {  // kx = 256 is its own partner
-        sa[H] = mk<C>(v[8].x, R(0));
-        sb[H] = mk<C>(v[8].y, R(0));
+        sa[kq(H)] = mk<C>(v[8].x, R(0));
+        sb[kq(H)] = mk<C>(v[8].y, R(0));
     }
 }
 
 // Slots g < ng of a team tile -> out[kx * hy + g] (joint: field 0 to oa, field 1 to
 // ob; pair: eight slots to oa; hy = the column stride).  The team's 128 threads take (g, kx) =
-// (tid % GPT, tid / GPT + (128 / GPT) i).
+// (tid % GPT, tid / GPT + (128 / GPT) i): kx advances by 32 or 16, keeping its parity,
+// so kq(kx) advances by half of that.
 template <typename R, bool PAIR>
 __device__ __forceinline__ void team_store(const cpx<R> *stage, cpx<R> *oa, cpx<R> *ob, int ng, int tid, int hy) {
     constexpr int GPT = TeamMode<PAIR>::GPT, KS = 128 / GPT;
     const int g = tid % GPT;
     if (g >= ng) return;
     int kx = tid / GPT;
-    const cpx<R> *sa = stage + g * (PAIR ? LSP : LS) + kx;
+    const cpx<R> *sa = stage + g * (PAIR ? LSP : LS) + kq(kx);
     size_t o = (size_t)kx * hy + g;
-    for (; kx < NC; kx += KS, sa += KS, o += (size_t)KS * hy) {
+    for (; kx < NC; kx += KS, sa += KS / 2, o += (size_t)KS * hy) {
         oa[o] = sa[0];
         if (!PAIR) ob[o] = sa[FS];
     }
@@ -281,9 +304,9 @@ __device__ __forceinline__ void team_load(cpx<R> *stage, const cpx<R> *ia, const
     const int g = tid % GPT;
     if (g >= ng) return;
     int kx = tid / GPT;
-    cpx<R> *sa = stage + g * (PAIR ? LSP : LS) + kx;
+    cpx<R> *sa = stage + g * (PAIR ? LSP : LS) + kq(kx);
     size_t o = (size_t)kx * hy + g;
-    for (; kx < NC; kx += KS, sa += KS, o += (size_t)KS * hy) {
+    for (; kx < NC; kx += KS, sa += KS / 2, o += (size_t)KS * hy) {
         cp_async8(sa, ia + o);
         if (!PAIR) cp_async8(sa + FS, ib + o);
     }
@@ -295,19 +318,30 @@ template <typename R, class TW>
 __device__ __forceinline__ void stage_to_lines(const cpx<R> *sa, const cpx<R> *sb, bool has_b, cpx<R> *buf,
                                                const TW &tw, R (&a)[8], R (&b)[8]) {
     using C = cpx<R>;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
+    const int lam = 2 * l + h;
     C v[16];
 #pragma unroll
     for (int k1 = 0; k1 < 16; ++k1) {
-        const int kk = k1 < 8 ? lane + 32 * k1 : N - 32 * k1 - lane;
-        C A = sa[kk], B = has_b ? sb[kk] : czero<C>();
-        if ((k1 == 0 || k1 == 8) && lane == 0) { A.y = 0; B.y = 0; }  // kk = 0, 256
-        v[k1] = k1 < 8 ? mk<C>(A.x - B.y, A.y + B.x) : mk<C>(A.x + B.y, B.x - A.y);
+        const int k = lam + 32 * k1;
+        const bool lo = k <= H;
+        const int kk = lo ? k : N - k;
+        C A = sa[kq(kk)], B = has_b ? sb[kq(kk)] : czero<C>();
+        if (kk == 0 || kk == H) { A.y = 0; B.y = 0; }
+        v[k1] = lo ? mk<C>(A.x - B.y, A.y + B.x) : mk<C>(A.x + B.y, B.x - A.y);
     }
     C out[8];
     inv512<R>(v, buf, tw, out);
+    __syncwarp();
 #pragma unroll
-    for (int i = 0; i < 8; ++i) { a[i] = out[i].x; b[i] = out[i].y; }
+    for (int jj = 0; jj < 8; ++jj) buf[l + 16 * (8 * h + jj)] = out[jj];
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const C y = buf[lane + 32 * i];
+        a[i] = y.x;
+        b[i] = y.y;
+    }
 }
 
 // Stages the functor's rows into pre[a][i][H] (n elements each): source i = 0 from
@@ -389,7 +423,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_row_fwd512t(View2<R> V, int nz, 
     __shared__ double red[128];
     pro.init();
     LaneTw<R> tw;
-    tw.load(V.op[0].twx);
+    tw.load_fwd(V.op[0].twx);
     const int gpl = (lpl + LPG - 1) / LPG;
     // pair mode with both fields in V: the groups of field 0, then those of field 1
     const long long NG1 = (long long)nz * gpl;
@@ -466,7 +500,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_row_inv512t(View2<R> V, int nz, 
     __shared__ double red[128];
     epi.init();
     LaneTw<R> tw;
-    tw.load(V.op[0].twx);
+    tw.load_inv(V.op[0].twx);
     const int gpl = (lpl + LPG - 1) / LPG;
     // pair mode with both fields in V: the groups of field 0, then those of field 1
     const long long NG1 = (long long)nz * gpl;
@@ -552,8 +586,8 @@ __global__ void __launch_bounds__(NW * 32, 2) k_row_resid512(View2<R> V, int nli
     stage_half_spectra<R, FFTS>(tile, V, 1, base, nlines, nlines, 1);
     __syncthreads();
     LaneTw<R> tw;
-    tw.load(V.op[0].twx);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    tw.load_inv(V.op[0].twx);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
     C *buf = xb + warp * N;
     const int f = warp;
     const int line = base + f;
@@ -562,6 +596,7 @@ __global__ void __launch_bounds__(NW * 32, 2) k_row_resid512(View2<R> V, int nli
     if (ok) epi.template resid_load<8>(line, lane, 32, n_out, wv, dv);
     R a[8], b[8];
     inv512_to_lines<R, FFTS>(tile, f, FFTS + f, buf, tw, a, b);
+    tw.load_fwd(V.op[0].twx);
     if (ok) {
         epi.template resid_apply<8>(lane, 32, n_out, wv, dv, a, b);  // a, b <- v of both fields
     } else {
@@ -571,8 +606,9 @@ __global__ void __launch_bounds__(NW * 32, 2) k_row_resid512(View2<R> V, int nli
     C v[16];
     fwd512_from_lines<R>(a, b, buf, tw, v);
     __syncthreads();  // every warp is done reading the staged input
+    const int lam = 2 * l + h;
 #pragma unroll
-    for (int k1 = 0; k1 < 16; ++k1) tile[f * (N + 1) + lane + 32 * k1] = v[k1];
+    for (int k1 = 0; k1 < 16; ++k1) tile[f * (N + 1) + ppos(lam + 32 * k1)] = v[k1];
     __syncthreads();
     write_half_spectra<R, FFTS>(tile, V, 1, base, nlines, nlines, 2);
     epi.flush(red);
