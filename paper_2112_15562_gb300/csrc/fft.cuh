@@ -153,17 +153,33 @@ __device__ __forceinline__ void dft_prime(cpx<R> (&v)[P]) {
         else { a[j] = cadd(v[j], v[P - j]); b[j] = csub(v[j], v[P - j]); }
     });
     const C x0 = v[0];
-    C sum = x0;
-    static_for<1, Hh + 1>([&](auto J) { sum = cadd(sum, a[J]); });
-    v[0] = sum;
+    C mid = x0, dif = x0;  // radix 5
+    if constexpr (P == 5) {
+        // (c1 + c2) / 2 = -1/4, (c1 - c2) / 2 = sqrt(5) / 4: equal inputs cancel exactly, where
+        // rounded c1 and c2 leave 1e-8 of them in every output
+        const C t = cadd(a[1], a[2]);
+        v[0] = cadd(x0, t);
+        mid = mk<C>(x0.x - R(0.25) * t.x, x0.y - R(0.25) * t.y);
+        dif = csub(a[1], a[2]);
+    } else {
+        C sum = x0;
+        static_for<1, Hh + 1>([&](auto J) { sum = cadd(sum, a[J]); });
+        v[0] = sum;
+    }
     static_for<1, Hh + 1>([&](auto Q) {
         constexpr int q = Q;
         C A = x0, Bs = czero<C>();
+        if constexpr (P == 5) {
+            constexpr R k = (R)(q == 1 ? 0.55901699437494742410 : -0.55901699437494742410);
+            A = mk<C>(mid.x + k * dif.x, mid.y + k * dif.y);
+        }
         static_for<1, Hh + 1>([&](auto J) {
             constexpr int j = J;
             constexpr R c = (R)Root<(j * q) % P, P>::c, s = (R)Root<(j * q) % P, P>::s;
-            A.x += c * a[j].x;
-            A.y += c * a[j].y;
+            if constexpr (P != 5) {
+                A.x += c * a[j].x;
+                A.y += c * a[j].y;
+            }
             if constexpr (j == 1) { Bs.x = s * b[j].x; Bs.y = s * b[j].y; }
             else { Bs.x += s * b[j].x; Bs.y += s * b[j].y; }
         });
