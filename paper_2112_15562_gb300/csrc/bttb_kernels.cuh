@@ -204,8 +204,8 @@ struct StorePlain {
 
 // ---------------------------------------------------------------------------
 // Two fields' single-field products in one launch (the pair calls): a functor per
-// field, the one of field f taken with field_functor(pro, f).  Every other functor
-// serves its launch's lines as it is.
+// field, the one of field f taken with field_functor(pro, f).  The solver's data-line
+// epilogues take the field there too; every other functor serves its launch's lines as it is.
 template <typename R>
 struct LoadPlain2 {  // field f: lines la and lb of x[f]
     const R *x[2];
@@ -481,13 +481,17 @@ __global__ void __launch_bounds__(256) k_row_inv(OpView<R> op, PairMap pm, int n
             const C z = X[j * rs.pitch + p];
             fn.apply(raw, la, lb, hb, j, z.x, z.y);
         });
-    epi.flush(red);
+    fn.flush(red);
 }
 
-// Data-line pass of the solver (joint lines): inverse rows of the cropped forward
-// product, the residual epilogue (epi.residual turns the two fields' data into W_d r~),
-// and the forward rows of the result for the adjoint's column pass.  out may be in: a
-// CTA reads its lines before it writes them.
+// Data-line pass of the solver: inverse rows of the cropped forward product, the residual
+// epilogue (residual turns the predicted data into W_d r~), and the forward rows of the
+// result for the adjoint's column pass.  out may be in: a CTA reads its lines before it
+// writes them.  Two lines of one field share a transform (grid y = field): magnetic data are
+// some 200 times the gravity data and W_d r~ the other way round, and a transform that carried
+// a line of each rounded each field by the larger one (50x30x10 FP32, 20 iterations, the worst
+// of ten surveys: Phi and the models off by up to 7.7e-6, by 1.7e-7 and 2.5e-7 since, in the same
+// time).
 template <typename R, class Epi>
 __global__ void __launch_bounds__(256) k_row_resid(OpView<R> op, PairMap pm, int n_out, RowShape rs,
                                                    const cpx<R> *in0, const cpx<R> *in1, cpx<R> *out0, cpx<R> *out1,
@@ -503,9 +507,12 @@ __global__ void __launch_bounds__(256) k_row_resid(OpView<R> op, PairMap pm, int
     copy_twiddles(tw, op.twx, N);
     pdl_wait();
     const int stop = stop_flag(done);
+    const int field = blockIdx.y;
     const int q0 = blockIdx.x * P;
     const int np = pm.npairs();
-    const SpectraStage<R> ss{op, pm, rs, q0, in0, in1, div_magic(ncol)};
+    const C *in = field ? in1 : in0;
+    C *out = field ? out1 : out0;
+    const SpectraStage<R> ss{op, pm, rs, q0, in, in, div_magic(ncol)};
     FirstBatch<4, SpectraStage<R>> first;
     first.loads(ncol * P, ss);
     if (stop) {
@@ -518,22 +525,29 @@ __global__ void __launch_bounds__(256) k_row_resid(OpView<R> op, PairMap pm, int
     __syncthreads();
     C *X = fft_staged<R, true>(op.px, rs, buf0, buf1, tw, N, n_out);
     const unsigned mn = div_magic(n_out);
+    auto &&fn = field_functor(epi, field);
     staged_loop<kRowU<R>>(
         n_out * P,
         [&](int it) {
             const int p = fast_div(it, mn), j = it - p * n_out;
-            return epi.load(min(q0 + p, np - 1), 0, true, j);
+            int la, lb; bool hb;
+            pm.lines(min(q0 + p, np - 1), la, lb, hb);
+            return fn.load(la, lb, hb, j);
         },
         [&](int it, const typename Epi::Raw &raw) {
             const int p = fast_div(it, mn), j = it - p * n_out;
             C z = X[j * rs.pitch + p];
-            if (q0 + p < np) epi.residual(raw, z.x, z.y);
+            if (q0 + p < np) {
+                int la, lb; bool hb;
+                pm.lines(q0 + p, la, lb, hb);
+                fn.residual(raw, hb, z.x, z.y);
+            }
             X[j * rs.pitch + p] = z;
         });
     __syncthreads();
     const C *Y = fft_staged<R, false>(op.px, rs, X, X == buf0 ? buf1 : buf0, tw, n_out, N);
-    split_lines<R>(op, pm, rs, q0, Y, out0, out1);
-    epi.flush(red);
+    split_lines<R>(op, pm, rs, q0, Y, out, out);
+    fn.flush(red);
 }
 
 // ---------------------------------------------------------------------------

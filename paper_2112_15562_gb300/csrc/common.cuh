@@ -82,15 +82,28 @@ __device__ __forceinline__ double warp_sums4(double v0, double v1, double v2, do
 
 // Adds per-thread partials acc[0..K) into out[0..K) (one double atomic per
 // block per entry).  All K sums share one pass: warp sums, one barrier, and
-// the first warp finishes.  `scratch` holds at least 4 * warps doubles (the kernels
+// the first warp finishes (whose `out` counts).  `scratch` holds at least 4 * warps doubles (the kernels
 // reserve 128: up to 32 warps).
 // All threads must call it.
 template <int K, typename A>
 __device__ __forceinline__ void block_accumulate(const A *acc, double *out, double *scratch) {
-    static_assert(K >= 2 && K <= 4, "two to four sums");
+    static_assert(K >= 1 && K <= 4, "one to four sums");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nw = (blockDim.x + 31) >> 5;
     double t;
+    if constexpr (K == 1) {
+        t = (double)acc[0];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        __syncthreads();  // scratch may still be in use by an earlier call
+        if (lane == 0) scratch[warp] = t;
+        __syncthreads();
+        if (warp == 0) {
+            t = lane < nw ? scratch[lane] : 0.0;
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0 && out) atomicAdd(out, t);
+        }
+        return;
+    }
     if constexpr (K == 2) t = warp_sums2((double)acc[0], (double)acc[1]);
     else t = warp_sums4((double)acc[0], (double)acc[1], (double)acc[2], K > 3 ? (double)acc[K - 1] : 0.0);
     __syncthreads();  // scratch may still be in use by an earlier call

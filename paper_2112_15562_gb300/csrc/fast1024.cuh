@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(RW * 32, RCTA) k_row_inv1024(OpView<R> op, Pai
             if (n < n_out) field_functor(epi, blockIdx.y).store(la, lb, hb, n, out[jj].x, out[jj].y);
         }
     }
-    epi.flush(red);
+    field_functor(epi, blockIdx.y).flush(red);
 }
 
 template <typename R> inline size_t smem_row() {

@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(NW * 32, 2) k_row_inv512(View2<R> V, int joint
             field_functor(epi, field).template store_batch<4>(la, lb, hb, lane + 128, 32, n_out, a1, b1);
         }
     }
-    epi.flush(red);
+    field_functor(epi, field).flush(red);
 }
 
 // ---------------------------------------------------------------------------
@@ -564,15 +564,16 @@ __global__ void __launch_bounds__(NW * 32, 1) k_row_inv512t(View2<R> V, int nz, 
     epi.flush(red);
 }
 
-// Fused data-line pass of the solver: for station row jy of both fields, inverse
+// Fused data-line pass of the solver: for two station rows of one field (grid y), inverse
 // row transform of W (the cropped forward product), the residual epilogue
 // (r~ = W_d (A m - d), v = W_d r~, Phi partials), then the forward row transform
-// of v written to V[kx][jy] for the adjoint's column pass.
+// of v written to V[kx][jy] for the adjoint's column pass.  The fields share no transform:
+// their data differ by two orders of magnitude, and so would each other's rounding.
 template <typename R, class Epi, int NW>
 __global__ void __launch_bounds__(NW * 32, 2) k_row_resid512(View2<R> V, int nlines, int n_out, Epi epi,
                                                              const int *done) {
     using C = cpx<R>;
-    constexpr int FFTS = NW;  // one joint transform per warp
+    constexpr int FFTS = NW;  // one transform per warp
     pdl_go();
     pdl_wait();
     if (stopped(done)) return;
@@ -582,23 +583,25 @@ __global__ void __launch_bounds__(NW * 32, 2) k_row_resid512(View2<R> V, int nli
     C *tws = xb + NW * N;
     __shared__ double red[128];
     epi.init();
-    const int base = blockIdx.x * FFTS;
-    stage_half_spectra<R, FFTS>(tile, V, 1, base, nlines, nlines, 1);
+    const int base = blockIdx.x * 2 * FFTS, field = blockIdx.y;
+    stage_half_spectra<R, FFTS>(tile, V, 0, base, nlines, nlines, 1, field);
     __syncthreads();
     LaneTw<R> tw;
     tw.load_inv(V.op[0].twx);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = lane >> 4, l = lane & 15;
     C *buf = xb + warp * N;
     const int f = warp;
-    const int line = base + f;
-    const bool ok = line < nlines;
-    R wv[2][8], dv[2][8];  // W_d and d of the line, loaded during the transform
-    if (ok) epi.template resid_load<8>(line, lane, 32, n_out, wv, dv);
+    int la, lb;
+    bool ha, hb;
+    pair_lines(0, base, f, nlines, la, lb, ha, hb);
+    auto &&fn = field_functor(epi, field);
+    R wv[2][8], dv[2][8];  // W_d and d of the lines, loaded during the transform
+    if (ha) fn.template resid_load<8>(la, lb, hb, lane, 32, n_out, wv, dv);
     R a[8], b[8];
-    inv512_to_lines<R, FFTS>(tile, f, FFTS + f, buf, tw, a, b);
+    inv512_to_lines<R, FFTS>(tile, 2 * f, 2 * f + 1, buf, tw, a, b);
     tw.load_fwd(V.op[0].twx);
-    if (ok) {
-        epi.template resid_apply<8>(lane, 32, n_out, wv, dv, a, b);  // a, b <- v of both fields
+    if (ha) {
+        fn.template resid_apply<8>(lane, 32, n_out, hb, wv, dv, a, b);  // a, b <- v of both lines
     } else {
 #pragma unroll
         for (int i = 0; i < 8; ++i) a[i] = b[i] = R(0);
@@ -610,8 +613,8 @@ __global__ void __launch_bounds__(NW * 32, 2) k_row_resid512(View2<R> V, int nli
 #pragma unroll
     for (int k1 = 0; k1 < 16; ++k1) tile[f * (N + 1) + ppos(lam + 32 * k1)] = v[k1];
     __syncthreads();
-    write_half_spectra<R, FFTS>(tile, V, 1, base, nlines, nlines, 2);
-    epi.flush(red);
+    write_half_spectra<R, FFTS>(tile, V, 0, base, nlines, nlines, 2, field);
+    fn.flush(red);
 }
 
 // shared-memory bytes of each row kernel

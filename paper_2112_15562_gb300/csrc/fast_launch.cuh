@@ -58,7 +58,7 @@ inline void set_col_attr() {
 }
 
 // out_sel / in_sel: 0 = Z, 1 = W, 2 = V
-// nfield = 2 (single mode, with LoadPlain2 / StorePlain2): the lines of both fields,
+// nfield = 2 (single mode, functors that take the field): the lines of both fields,
 // grid y = field
 template <typename R, int NW, int FPW, class Pro>
 inline void row_fwd(const View2<R> &V, int joint, int nlines, int lpl, int n_in, int out_sel, const Pro &pro,
@@ -78,8 +78,8 @@ inline void row_inv(const View2<R> &V, int joint, int nlines, int lpl, int n_out
 
 template <typename R, int NW, class Epi>
 inline void row_resid(const View2<R> &V, int nlines, int n_out, const Epi &epi, const int *done, cudaStream_t st) {
-    launch_after(k_row_resid512<R, Epi, NW>, dim3((nlines + NW - 1) / NW), dim3(NW * 32), smem_row_resid<R, NW>(), st, V,
-                 nlines, n_out, epi, done);
+    launch_after(k_row_resid512<R, Epi, NW>, dim3((nlines + 2 * NW - 1) / (2 * NW), 2), dim3(NW * 32),
+                 smem_row_resid<R, NW>(), st, V, nlines, n_out, epi, done);
 }
 
 // persistent team row passes over nz layers of lpl lines (grid: one CTA per SM);
@@ -143,7 +143,7 @@ inline int row_grid(const PairMap &pm) {
     const int np = pm.joint ? pm.nlines : (pm.nlines + 1) / 2;
     return (np + RW - 1) / RW;
 }
-// nfield = 2 (pairs of one field's lines, LoadPlain2 / StorePlain2): both fields in one
+// nfield = 2 (pairs of one field's lines, functors that take the field): both fields in one
 // launch, grid y = field, field 1's buffers in o1 / i1
 template <typename R, class Pro>
 inline void row_fwd(const OpView<R> &v, const PairMap &pm, int n_in, cpx<R> *o0, cpx<R> *o1, const void *tab,

@@ -31,10 +31,12 @@ void gen_row_inv(const gj_op *o, const OpView<R> &v, const PairMap &pm, int n_ou
 }
 template <typename R, class Epi>
 void gen_row_resid(const gj_op *o, const OpView<R> &v, const PairMap &pm, int n_out, const cpx<R> *in0,
-                   const cpx<R> *in1, cpx<R> *out0, cpx<R> *out1, const Epi &epi, const int *done, cudaStream_t st) {
-    const RowShape rs = row_shape(o, pm.nlines, sizeof(cpx<R>));
-    launch_after(k_row_resid<R, Epi>, dim3((pm.nlines + rs.P - 1) / rs.P), dim3(row_threads(o->px, rs.P, pm.nlines)),
-                 row_smem(o->Nx, rs.pitch, sizeof(cpx<R>)), st, v, pm, n_out, rs, in0, in1, out0, out1, epi, done);
+                   const cpx<R> *in1, cpx<R> *out0, cpx<R> *out1, const Epi &epi, const int *done, cudaStream_t st,
+                   int nf) {
+    const int np = (pm.nlines + 1) / 2;
+    const RowShape rs = row_shape(o, (long long)np * nf, sizeof(cpx<R>));
+    launch_after(k_row_resid<R, Epi>, dim3((np + rs.P - 1) / rs.P, nf),
+                 dim3(row_threads(o->px, rs.P, (long long)np * nf)), row_smem(o->Nx, rs.pitch, sizeof(cpx<R>)), st, v, pm, n_out, rs, in0, in1, out0, out1, epi, done);
 }
 template <typename R>
 void gen_col_fwd(const gj_op *o, const OpView<R> &v0, const OpView<R> &v1, int nf, int layers, const int *done,
@@ -88,7 +90,8 @@ template <typename R> void gen_rec_plane(const gj_op *o, const OpView<R> &v, boo
 #define GJ_ROW_RESID(R, EPI)                                                                                    \
     template void gen_row_resid_attr<R, EPI>();                                                                 \
     template void gen_row_resid<R, EPI>(const gj_op *, const OpView<R> &, const PairMap &, int, const cpx<R> *, \
-                                        const cpx<R> *, cpx<R> *, cpx<R> *, const EPI &, const int *, cudaStream_t);
+                                        const cpx<R> *, cpx<R> *, cpx<R> *, const EPI &, const int *, cudaStream_t, \
+                                        int);
 #define GJ_COLS(R)                                                                                               \
     template void gen_col_attr<R>();                                                                             \
     template void gen_col_fwd<R>(const gj_op *, const OpView<R> &, const OpView<R> &, int, int, const int *,     \

@@ -146,7 +146,8 @@ inline ColShape col_shape(const gj_op *o, int nf, int layers, size_t cs, bool ad
 
 // Launches (general_impl.cuh; instantiated by general_*.cu, one translation unit per
 // precision and pass, because a kernel holds every codelet).  The attribute calls are
-// made once before a capture.  grid y of the rows: fields (LoadPlain2 / StorePlain2).
+// made once before a capture.  grid y of the rows: fields (LoadPlain2 / StorePlain2, the
+// solver's data-line epilogues).
 template <typename R, class Pro> void gen_row_fwd_attr();
 template <typename R, class Pro>
 void gen_row_fwd(const gj_op *o, const OpView<R> &v, const PairMap &pm, int n_in, cpx<R> *out0, cpx<R> *out1,
@@ -158,7 +159,8 @@ void gen_row_inv(const gj_op *o, const OpView<R> &v, const PairMap &pm, int n_ou
 template <typename R, class Epi> void gen_row_resid_attr();
 template <typename R, class Epi>
 void gen_row_resid(const gj_op *o, const OpView<R> &v, const PairMap &pm, int n_out, const cpx<R> *in0,
-                   const cpx<R> *in1, cpx<R> *out0, cpx<R> *out1, const Epi &epi, const int *done, cudaStream_t st);
+                   const cpx<R> *in1, cpx<R> *out0, cpx<R> *out1, const Epi &epi, const int *done, cudaStream_t st,
+                   int nf);
 template <typename R> void gen_col_attr();
 template <typename R>
 void gen_col_fwd(const gj_op *o, const OpView<R> &v0, const OpView<R> &v1, int nf, int layers, const int *done,

@@ -292,7 +292,7 @@ struct SolverLaunch {
             f1024::set_col_attr<R>();
             f1024::set_row_fwd_attr<R, ProModel<R>>();
             f1024::set_row_fwd_attr<R, ProDirection<R>>();
-            f1024::set_row_fwd_attr<R, LoadPair<R>>();
+            f1024::set_row_fwd_attr<R, LoadPlain2<R>>();
             f1024::set_row_inv_attr<R, EpiResidual<R>>();
             f1024::set_row_inv_attr<R, EpiGradient<R>>();
             f1024::set_row_inv_attr<R, EpiQNorm<R>>();
@@ -306,8 +306,9 @@ struct SolverLaunch {
         gen_col_attr<R>();
     }
 
-    // Row passes of the general path over both fields (joint pair maps): the block FFT
-    // kernels, or at N_x = 1024 with the N_y = 1024 columns the warp-FFT row kernels.
+    // Row passes of the general path over both fields (cell lines: a line of each field a
+    // transform; data lines: nf = 2 and two lines of one field): the block FFT kernels, or at
+    // N_x = 1024 with the N_y = 1024 columns the warp-FFT row kernels.
     template <class Pro>
     void rows_fwd(const PairMap &pm, int n_in, cpx<R> *o0, cpx<R> *o1, const Pro &pro, const int *done,
                   cudaStream_t st) {
@@ -319,12 +320,12 @@ struct SolverLaunch {
     }
     template <class Epi>
     void rows_inv(const PairMap &pm, int n_out, const cpx<R> *i0, const cpx<R> *i1, const Epi &epi, const int *done,
-                  cudaStream_t st) {
+                  cudaStream_t st, int nf = 1) {
         if constexpr (std::is_same_v<R, float>) if (rows1024) {
-            f1024::row_inv<R>(v0, pm, n_out, i0, i1, sv->op[0]->twtab, epi, done, st);
+            f1024::row_inv<R>(v0, pm, n_out, i0, i1, sv->op[0]->twtab, epi, done, st, nf);
             return;
         }
-        gen_row_inv<R>(sv->op[0], v0, pm, n_out, i0, i1, epi, done, st);
+        gen_row_inv<R>(sv->op[0], v0, pm, n_out, i0, i1, epi, done, st, nf);
     }
 
     // Forward columns (Y = sum_r T^_r FFT_y(Z_r)) and inverse columns, both fields.
@@ -395,13 +396,14 @@ struct SolverLaunch {
         ProModel<R> pm{F, sv->S, o->nx, o->ny};
         rows_fwd(pc, o->nx, v0.Z, v1.Z, pm, done, st);
         forward_columns(st);
-        PairMap ps{o->sy, 1, o->sy};
+        PairMap ps{o->sy, 0, o->sy};
         EpiResidual<R> er{F, sv->S, o->sx};
         // residual, Phi and the residual rows' spectra for the adjoint, in one pass
         if constexpr (std::is_same_v<R, float>)
-            if (rows1024) f1024::row_inv<R>(v0, ps, o->sx, v0.W, v1.W, o->twtab, er, done, st);
+            if (rows1024) f1024::row_inv<R>(v0, ps, o->sx, v0.W, v1.W, o->twtab, er, done, st, 2);
         if (!rows1024)
-            gen_row_resid<R>(o, v0, ps, o->sx, v0.W, v1.W, fast1024 ? v0.V : v0.W, fast1024 ? v1.V : v1.W, er, done, st);
+            gen_row_resid<R>(o, v0, ps, o->sx, v0.W, v1.W, fast1024 ? v0.V : v0.W, fast1024 ? v1.V : v1.W, er, done, st,
+                             2);
         launch_after(k_scalars_after_residual, dim3(1), dim3(32), 0, st, sv->S);
     }
 
@@ -424,17 +426,18 @@ struct SolverLaunch {
             }
             forward_columns(st);
             EpiQNorm<R> eq{F, sv->S, o->sx};
-            row_inv<R, kDataNW, kDataFPW>(V2, 1, o->sy, o->sy, o->sx, 1, eq, done, st);
+            row_inv<R, kDataNW, kDataFPW>(V2, 0, o->sy, o->sy, o->sx, 1, eq, done, st, 2);
             launch_after(k_scalars_after_direction, dim3(1), dim3(32), 0, st, sv->S);
             head(st);
             return;
         }
-        PairMap ps{o->sy, 1, o->sy};
+        PairMap ps{o->sy, 0, o->sy};
         PairMap pc{o->nz * o->ny, 1, o->ny};
         // adjoint: the residual rows' spectra (head) -> per-layer conj-spectrum columns -> Z
         if constexpr (std::is_same_v<R, float>) {
             if (rows1024)
-                f1024::row_fwd<R>(v0, ps, o->sx, v0.V, v1.V, o->twtab, LoadPair<R>{F.v[0], F.v[1], o->sx}, done, st);
+                f1024::row_fwd<R>(v0, ps, o->sx, v0.V, v1.V, o->twtab, LoadPlain2<R>{{F.v[0], F.v[1]}, o->sx}, done, st,
+                                  2);
             if (fast1024) f1024::col_adj<R>(V2, grid, done, st);
         }
         if (!fast1024) gen_col_adj<R>(o, v0, v1, 2, o->nz, done, st);
@@ -445,7 +448,7 @@ struct SolverLaunch {
         rows_fwd(pc, o->nx, v0.Z, v1.Z, pd, done, st);
         forward_columns(st);
         EpiQNorm<R> eq{F, sv->S, o->sx};
-        rows_inv(ps, o->sx, v0.W, v1.W, eq, done, st);
+        rows_inv(ps, o->sx, v0.W, v1.W, eq, done, st, 2);
         launch_after(k_scalars_after_direction, dim3(1), dim3(32), 0, st, sv->S);
         // model update, its forward product and the chi^2 scalars
         head(st);

@@ -256,56 +256,64 @@ struct ProModel {
     __device__ void flush(double *red) { block_accumulate<3>(acc, S->G, red); }
 };
 
+// The data-line epilogues: a launch serves both fields (grid y), a transform two lines la
+// and lb of one of them, which field_functor(epi, field) selects; hb: line lb exists.
+
 // Residual epilogue: r~ = W_d (A m - d), v = W_d r~, Phi partials (RRCG:1).
 template <typename R>
 struct EpiResidual {
     FieldVecs<R> F;
     SolverDev *S;
     int sx;
-    R acc[2];
+    int fld;
+    R acc;
     using Real = R;
     static constexpr int NS = 0;
     __device__ __forceinline__ R scalar(int) const { return R(0); }
     __device__ __forceinline__ void begin() {}
-    __device__ __forceinline__ void set(const R *) { acc[0] = acc[1] = 0; }
+    __device__ __forceinline__ void set(const R *) { acc = 0; }
     __device__ void init() { set(nullptr); }
-    // y of both fields in a, b becomes W_d r~ (two steps, as in ProModel)
+    __device__ __forceinline__ const R *wd() const { return fld ? F.wd[1] : F.wd[0]; }  // (selects, not indexed loads)
+    __device__ __forceinline__ const R *dobs() const { return fld ? F.dobs[1] : F.dobs[0]; }
+    // y of both lines in a, b becomes W_d r~ (two steps, as in ProModel)
     struct Raw { R w[2], d[2]; };
-    __device__ __forceinline__ Raw load(int la, int, bool, int j) const {
-        const size_t t = (size_t)la * sx + j;
-        return Raw{{F.wd[0][t], F.wd[1][t]}, {F.dobs[0][t], F.dobs[1][t]}};
+    __device__ __forceinline__ Raw load(int la, int lb, bool hb, int j) const {
+        const size_t t = (size_t)la * sx + j, u = (size_t)(hb ? lb : la) * sx + j;
+        return Raw{{wd()[t], wd()[u]}, {dobs()[t], dobs()[u]}};
     }
-    __device__ __forceinline__ void residual(const Raw &q, R &a, R &b) {
-        const R r0 = q.w[0] * (a - q.d[0]), r1 = q.w[1] * (b - q.d[1]);
-        acc[0] += r0 * r0;
-        acc[1] += r1 * r1;
+    __device__ __forceinline__ void residual(const Raw &q, bool hb, R &a, R &b) {
+        const R r0 = q.w[0] * (a - q.d[0]), r1 = hb ? q.w[1] * (b - q.d[1]) : R(0);
+        acc += r0 * r0;
+        acc += r1 * r1;
         a = q.w[0] * r0;
         b = q.w[1] * r1;
     }
     __device__ __forceinline__ void store(int la, int lb, bool hb, int j, R a, R b) {
-        residual(load(la, lb, hb, j), a, b);
-        const size_t t = (size_t)la * sx + j;
-        F.v[0][t] = a;
-        F.v[1][t] = b;
+        residual(load(la, lb, hb, j), hb, a, b);
+        R *v = fld ? F.v[1] : F.v[0];
+        v[(size_t)la * sx + j] = a;
+        if (hb) v[(size_t)lb * sx + j] = b;
     }
     // fused form, in two steps so that the loads can be issued before the transform:
-    // resid_load fetches W_d and d; resid_apply takes y in a, b and returns v = W_d r~
+    // resid_load fetches W_d and d (zero where there is no element); resid_apply takes y of
+    // both lines in a, b and returns v = W_d r~
     template <int K>
-    __device__ __forceinline__ void resid_load(int la, int j0, int stride, int n, R (&w)[2][K], R (&d)[2][K]) const {
-        const size_t t0 = (size_t)la * sx;
+    __device__ __forceinline__ void resid_load(int la, int lb, bool hb, int j0, int stride, int n, R (&w)[2][K],
+                                               R (&d)[2][K]) const {
+        const R *w0 = wd() + (size_t)la * sx, *w1 = wd() + (size_t)lb * sx;
+        const R *d0 = dobs() + (size_t)la * sx, *d1 = dobs() + (size_t)lb * sx;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int j = j0 + k * stride;
             const bool ok = j < n;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                w[i][k] = ok ? F.wd[i][t0 + j] : R(0);
-                d[i][k] = ok ? F.dobs[i][t0 + j] : R(0);
-            }
+            w[0][k] = ok ? w0[j] : R(0);
+            d[0][k] = ok ? d0[j] : R(0);
+            w[1][k] = ok && hb ? w1[j] : R(0);
+            d[1][k] = ok && hb ? d1[j] : R(0);
         }
     }
     template <int K>
-    __device__ __forceinline__ void resid_apply(int j0, int stride, int n, const R (&w)[2][K], const R (&d)[2][K],
+    __device__ __forceinline__ void resid_apply(int j0, int stride, int n, bool hb, const R (&w)[2][K], const R (&d)[2][K],
                                                 R (&a)[K], R (&b)[K]) {
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -313,67 +321,19 @@ struct EpiResidual {
             const bool ok = j < n;
             const R r0 = w[0][k] * (a[k] - d[0][k]);
             const R r1 = w[1][k] * (b[k] - d[1][k]);
-            if (ok) {
-                acc[0] += r0 * r0;
-                acc[1] += r1 * r1;
-            }
+            if (ok) acc += r0 * r0;
+            if (ok && hb) acc += r1 * r1;
             a[k] = ok ? w[0][k] * r0 : R(0);
-            b[k] = ok ? w[1][k] * r1 : R(0);
+            b[k] = ok && hb ? w[1][k] * r1 : R(0);
         }
     }
-    template <int K>
-    __device__ __forceinline__ void store_batch(int la, int, bool, int j0, int stride, int n, const R (&a)[K],
-                                                const R (&b)[K]) {
-        const size_t t0 = (size_t)la * sx;
-        R w[2][K], d[2][K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            const bool ok = j < n;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                w[i][k] = ok ? F.wd[i][t0 + j] : R(0);
-                d[i][k] = ok ? F.dobs[i][t0 + j] : R(0);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            if (j >= n) continue;
-            const R y[2] = {a[k], b[k]};
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const R rt = w[i][k] * (y[i] - d[i][k]);
-                acc[i] += rt * rt;
-                F.v[i][t0 + j] = w[i][k] * rt;
-            }
-        }
-    }
-    __device__ void flush(double *red) { block_accumulate<2>(acc, S->phi, red); }
+    __device__ void flush(double *red) { block_accumulate<1>(&acc, S->phi + fld, red); }
 };
-
 template <typename R>
-struct LoadPair {
-    const R *x0;
-    const R *x1;
-    int pitch;
-    __device__ void init() {}
-    __device__ __forceinline__ void fetch(int la, int lb, bool, int j, R &a, R &b) const {
-        a = x0[(size_t)la * pitch + j];
-        b = x1[(size_t)lb * pitch + j];
-    }
-    template <int K>
-    __device__ __forceinline__ void fetch_batch(int la, int lb, bool, int j0, int stride, int n, R (&a)[K],
-                                                R (&b)[K]) const {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int j = j0 + k * stride;
-            a[k] = j < n ? x0[(size_t)la * pitch + j] : R(0);
-            b[k] = j < n ? x1[(size_t)lb * pitch + j] : R(0);
-        }
-    }
-    __device__ void flush(double *) {}
-};
+__device__ __forceinline__ EpiResidual<R> &field_functor(EpiResidual<R> &p, int f) {
+    p.fld = f;
+    return p;
+}
 
 // Gradient epilogue (RRCG:2-4): l = W^-1 A^T v + alpha (W m - W m_apr) + lambda l_G.
 template <typename R, bool OPT = true>
@@ -624,52 +584,60 @@ struct EpiQNorm {
     FieldVecs<R> F;
     SolverDev *S;
     int sx;
-    R acc[2];
+    int fld;
+    R acc;
     using Real = R;
     static constexpr int NS = 0;
     __device__ __forceinline__ R scalar(int) const { return R(0); }
     __device__ __forceinline__ void begin() {}
-    __device__ __forceinline__ void set(const R *) { acc[0] = acc[1] = 0; }
+    __device__ __forceinline__ void set(const R *) { acc = 0; }
     __device__ void init() { set(nullptr); }
+    __device__ __forceinline__ const R *wd() const { return fld ? F.wd[1] : F.wd[0]; }
     struct Raw { R w[2]; };
-    __device__ __forceinline__ Raw load(int la, int, bool, int j) const {
-        const size_t t = (size_t)la * sx + j;
-        return Raw{{F.wd[0][t], F.wd[1][t]}};
+    __device__ __forceinline__ Raw load(int la, int lb, bool hb, int j) const {
+        return Raw{{wd()[(size_t)la * sx + j], wd()[(size_t)(hb ? lb : la) * sx + j]}};
     }
-    __device__ __forceinline__ void apply(const Raw &q, int, int, bool, int, R a, R b) {
-        const R q0 = q.w[0] * a, q1 = q.w[1] * b;
-        acc[0] += q0 * q0;
-        acc[1] += q1 * q1;
+    __device__ __forceinline__ void apply(const Raw &q, int, int, bool hb, int, R a, R b) {
+        const R q0 = q.w[0] * a, q1 = hb ? q.w[1] * b : R(0);
+        acc += q0 * q0;
+        acc += q1 * q1;
     }
     __device__ __forceinline__ void store(int la, int lb, bool hb, int j, R a, R b) {
         apply(load(la, lb, hb, j), la, lb, hb, j, a, b);
     }
-    // batched form (the 512 kernels): prefetch loads W_d of line la, elements
+    // batched form (the 512 kernels): prefetch loads W_d of lines la and lb, elements
     // lane + 32 k, before the transform; store_batch(j0 = lane or lane + 128) uses them
     R wq[2][8];
-    __device__ __forceinline__ void prefetch(int la, int, bool, int lane, int n) {
-        const size_t t0 = (size_t)la * sx;
+    __device__ __forceinline__ void prefetch(int la, int lb, bool hb, int lane, int n) {
+        const R *w0 = wd() + (size_t)la * sx, *w1 = wd() + (size_t)lb * sx;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int j = lane + 32 * k;
-            wq[0][k] = j < n ? F.wd[0][t0 + j] : R(0);
-            wq[1][k] = j < n ? F.wd[1][t0 + j] : R(0);
+            wq[0][k] = j < n ? w0[j] : R(0);
+            wq[1][k] = j < n && hb ? w1[j] : R(0);
         }
     }
     template <int K>
-    __device__ __forceinline__ void store_batch(int, int, bool, int j0, int stride, int n, const R (&a)[K],
+    __device__ __forceinline__ void store_batch(int, int, bool hb, int j0, int stride, int n, const R (&a)[K],
                                                 const R (&b)[K]) {
         const int o = (j0 - (int)(threadIdx.x & 31)) / 32;  // 0 or 4
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int j = j0 + k * stride;
             if (j >= n) continue;
-            const R q0 = wq[0][o + k] * a[k], q1 = wq[1][o + k] * b[k];
-            acc[0] += q0 * q0;
-            acc[1] += q1 * q1;
+            const R q0 = wq[0][o + k] * a[k];
+            acc += q0 * q0;
+            if (!hb) continue;
+            const R q1 = wq[1][o + k] * b[k];
+            acc += q1 * q1;
         }
     }
-    __device__ void flush(double *red) { block_accumulate<2>(acc, S->qq, red); }
+    __device__ void flush(double *red) { block_accumulate<1>(&acc, S->qq + fld, red); }
 };
+template <typename R>
+__device__ __forceinline__ EpiQNorm<R> &field_functor(EpiQNorm<R> &p, int f) {
+    p.fld = f;
+    return p;
+}
 
 }  // namespace gj
