@@ -388,9 +388,9 @@ __global__ void __launch_bounds__(CWA * 32, 1) k_col_adj1024(View2<R> V, const i
 }
 
 // ---------------------------------------------------------------------------
-// Row passes for N_x = 1024 (with the N_y = 1024 column kernels): real lines <->
-// half spectra in the transposed layout, through the general kernels' per-element
-// functors.  A CTA of RW warps runs one complex transform per warp: two lines of one
+// Row passes for N_x = 1024 and lines of at most 512 values (with the N_y = 1024 column
+// kernels): real lines <-> half spectra in the transposed layout, through the general
+// kernels' per-element functors.  A CTA of RW warps runs one complex transform per warp: two lines of one
 // field (pair map, joint = 0) or one line of each field (joint = 1).  The half
 // spectra of the CTA's lines meet in a shared tile [k < 513][slot], a transform's two
 // lines side by side (one 16-byte word), and move to or from the transposed layout with

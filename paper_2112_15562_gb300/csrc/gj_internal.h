@@ -43,6 +43,7 @@ struct gj_op {
     // kernels with the general row kernels writing and reading transposed Z, W, V;
     // spectra, partials, counters and the error word as on the fast path
     bool fast1024 = false;
+    bool rows1024 = false;  // with the warp-FFT row kernels: N_x = 1024 and at most 512 values a line
     // per-layer spectrum recomputation (GJ_SETUP_RECOMPUTE_SPECTRA): `spec` holds one
     // layer, rebuilt from the closed forms before each use
     bool recompute = false;

@@ -66,7 +66,7 @@ static void fast1024_forward(const gj_op *a, const gj_op *b, const float *m0, co
     gen_row_fwd_attr<R, LoadPlain2<R>>();
     gen_row_inv_attr<R, StorePlain2<R>>();
     f1024::set_col_attr<R>();
-    const bool rows1024 = a->Nx == 1024;  // warp-FFT rows as well
+    const bool rows1024 = a->rows1024;  // warp-FFT rows as well
     if (rows1024) {
         f1024::set_row_fwd_attr<R, LoadPlain<R>>();
         f1024::set_row_inv_attr<R, StorePlain<R>>();
@@ -116,7 +116,7 @@ static void fast1024_adjoint(const gj_op *a, const gj_op *b, const float *r0, co
     gen_row_fwd_attr<R, LoadPlain2<R>>();
     gen_row_inv_attr<R, StorePlain2<R>>();
     f1024::set_col_attr<R>();
-    const bool rows1024 = a->Nx == 1024;
+    const bool rows1024 = a->rows1024;
     if (rows1024) {
         f1024::set_row_fwd_attr<R, LoadPlain<R>>();
         f1024::set_row_inv_attr<R, StorePlain<R>>();

@@ -229,7 +229,7 @@ struct SolverLaunch {
     f512::View2<R> V2;
     bool fast = false;
     bool fast1024 = false;  // general row kernels (transposed intermediates) + N_y = 1024 column kernels
-    bool rows1024 = false;  // fast1024 with N_x = 1024: the warp-FFT row kernels of fast1024.cuh
+    bool rows1024 = false;  // with the warp-FFT row kernels of fast1024.cuh
     FieldVecs<R> F;
     int grid;  // CTAs of the persistent fast-path launches
 
@@ -241,7 +241,7 @@ struct SolverLaunch {
         if constexpr (std::is_same_v<R, float>) {
             fast = o->fast && sv->op[1]->fast;
             fast1024 = o->fast1024 && sv->op[1]->fast1024;
-            rows1024 = fast1024 && o->Nx == 1024;
+            rows1024 = fast1024 && o->rows1024;
             if (fast || fast1024) V2 = f512::make_view2<R>(sv->op[0], sv->op[1]);
         }
         const int n = o->nx * o->ny * o->nz, s = o->sx * o->sy;
@@ -307,8 +307,8 @@ struct SolverLaunch {
     }
 
     // Row passes of the general path over both fields (cell lines: a line of each field a
-    // transform; data lines: nf = 2 and two lines of one field): the block FFT kernels, or at
-    // N_x = 1024 with the N_y = 1024 columns the warp-FFT row kernels.
+    // transform; data lines: nf = 2 and two lines of one field): the block FFT kernels, or
+    // (rows1024) the warp-FFT row kernels that go with the N_y = 1024 columns.
     template <class Pro>
     void rows_fwd(const PairMap &pm, int n_in, cpx<R> *o0, cpx<R> *o1, const Pro &pro, const int *done,
                   cudaStream_t st) {

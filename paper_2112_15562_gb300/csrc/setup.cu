@@ -415,6 +415,8 @@ int fast_slots(int nfield, int ncol, int nz, long long warps) {
 bool fast1024_eligible(const gj_op *op) {
     return op->prec == GJ_FP32_MIXED && !op->fast && op->Ny == 1024 && op->ny <= 512 && op->sy <= 512;
 }
+// its row kernels hold 512 values of a line (16 a lane); longer lines take the general ones
+bool rows1024_eligible(const gj_op *op) { return op->fast1024 && op->Nx == 1024 && op->nx <= 512 && op->sx <= 512; }
 
 static gj_status upload_twiddles(int N, gj_precision prec, void **out) {
     std::vector<double> re, im;
@@ -751,6 +753,7 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
         op->real_spec = op->even_table;
     }
     op->fast1024 = !op->recompute && fast1024_eligible(op);
+    op->rows1024 = rows1024_eligible(op);
     if (op->fast1024) {
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
