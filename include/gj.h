@@ -366,7 +366,10 @@ gj_status gj_rrcg_joint_solve_host(const gj_op *const ops[2], const gj_rrcg_para
 
 /* Stepwise form of the same solve: a solver object holds the state (search
  * directions, scalars) and enqueues whole iterations without host round trips;
- * the stop test runs on the device and later iterations become no-ops. */
+ * the stop test runs on the device and later iterations become no-ops.  Everything
+ * that one iteration leaves for the next belongs to the solver, so that products of
+ * its operators, or iterations of another solver on them, may come in between when
+ * they are ordered (one stream, or explicit events). */
 typedef struct gj_rrcg gj_rrcg;
 
 gj_status gj_rrcg_create(const gj_op *const ops[2], const gj_rrcg_params *params,

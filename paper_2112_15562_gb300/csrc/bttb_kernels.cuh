@@ -29,7 +29,7 @@ struct OpView {
     cpx<R> *Y;           // [slots][Ny][ncol]  layer groups' partial sums
     int *cnt;            // [ncol]         arrivals of a column tile's layer groups, zero between launches
     cpx<R> *W;           // [max(sy, ...)][ncol]  inverse-column output / residual rows
-    cpx<R> *V;           // fast path: residual-row spectra [ncol][256] (unused otherwise)
+    cpx<R> *V;           // fast paths: data-row spectra [ncol][Ny/2] of the adjoint (unused otherwise)
     int real_spec;       // fast path: spec holds the real, even spectrum of an even table for
                          // ky <= Ny/2 only, R[nz][ncol][even_spec_len(Ny)]
     int split_half;      // 1: the row passes halve the split spectra; 0: the factor is in `spec`
@@ -486,8 +486,7 @@ __global__ void __launch_bounds__(256) k_row_inv(OpView<R> op, PairMap pm, int n
 
 // Data-line pass of the solver: inverse rows of the cropped forward product, the residual
 // epilogue (residual turns the predicted data into W_d r~), and the forward rows of the
-// result for the adjoint's column pass.  out may be in: a CTA reads its lines before it
-// writes them.  Two lines of one field share a transform (grid y = field): magnetic data are
+// result for the adjoint's column pass.  Two lines of one field share a transform (grid y = field): magnetic data are
 // some 200 times the gravity data and W_d r~ the other way round, and a transform that carried
 // a line of each rounded each field by the larger one (50x30x10 FP32, 20 iterations, the worst
 // of ten surveys: Phi and the models off by up to 7.7e-6, by 1.7e-7 and 2.5e-7 since, in the same

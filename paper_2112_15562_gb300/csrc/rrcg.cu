@@ -182,6 +182,7 @@ struct gj_rrcg {
     const gj_op *op[2];
     gj_precision prec;
     SolverDev *S = nullptr;   // device
+    void *vhat = nullptr;     // spectra of the residual's rows, both fields (vhat_values)
     void *buf = nullptr;      // p, l (2 fields each, n), v (2 x s), wd (2 x s)
     const void *dobs[2], *mapr[2], *wdep[2], *whard[2];
     bool prev_anchor = false;
@@ -222,10 +223,21 @@ static void cut_segment(gj_rrcg *sv, cudaStream_t st) {
     if (e != cudaSuccess && sv->cap_err == cudaSuccess) sv->cap_err = e;
 }
 
+// The residual's row spectra are written by the end of one iteration and read by the next, so
+// they are the solver's own: an operator's workspace serves any other call in between (its
+// products, another solver).  Complex values of one field, in the layout of the operator's
+// column passes (transposed: rows beyond the stations stay zero); none where the rows are
+// transformed from v at the start of an iteration.
+static size_t vhat_values(const gj_op *o) {
+    if (o->rows1024) return 0;
+    return (size_t)o->ncol * (o->fast || o->fast1024 ? o->Ny / 2 : o->sy);
+}
+
 template <typename R>
 struct SolverLaunch {
     gj_rrcg *sv;
     OpView<R> v0, v1;
+    cpx<R> *vhat[2];
     f512::View2<R> V2;
     bool fast = false;
     bool fast1024 = false;  // general row kernels (transposed intermediates) + N_y = 1024 column kernels
@@ -244,6 +256,10 @@ struct SolverLaunch {
             rows1024 = fast1024 && o->rows1024;
             if (fast || fast1024) V2 = f512::make_view2<R>(sv->op[0], sv->op[1]);
         }
+        vhat[0] = static_cast<cpx<R> *>(sv->vhat);
+        vhat[1] = vhat[0] + vhat_values(o);
+        if ((fast || fast1024) && !rows1024)
+            for (int i = 0; i < 2; ++i) V2.op[i].V = vhat[i];
         const int n = o->nx * o->ny * o->nz, s = o->sx * o->sy;
         R *b = static_cast<R *>(sv->buf);
         for (int i = 0; i < 2; ++i) {
@@ -402,8 +418,7 @@ struct SolverLaunch {
         if constexpr (std::is_same_v<R, float>)
             if (rows1024) f1024::row_inv<R>(v0, ps, o->sx, v0.W, v1.W, o->twtab, er, done, st, 2);
         if (!rows1024)
-            gen_row_resid<R>(o, v0, ps, o->sx, v0.W, v1.W, fast1024 ? v0.V : v0.W, fast1024 ? v1.V : v1.W, er, done, st,
-                             2);
+            gen_row_resid<R>(o, v0, ps, o->sx, v0.W, v1.W, vhat[0], vhat[1], er, done, st, 2);
         launch_after(k_scalars_after_residual, dim3(1), dim3(32), 0, st, sv->S);
     }
 
@@ -440,7 +455,12 @@ struct SolverLaunch {
                                   2);
             if (fast1024) f1024::col_adj<R>(V2, grid, done, st);
         }
-        if (!fast1024) gen_col_adj<R>(o, v0, v1, 2, o->nz, done, st);
+        if (!fast1024) {
+            OpView<R> a0 = v0, a1 = v1;
+            a0.W = vhat[0];
+            a1.W = vhat[1];
+            gen_col_adj<R>(o, a0, a1, 2, o->nz, done, st);
+        }
         EpiGradient<R> eg{F, sv->S, o->nx, o->ny};
         rows_inv(pc, o->nx, v0.Z, v1.Z, eg, done, st);
         // direction and its forward product
@@ -549,16 +569,18 @@ static gj_status rrcg_create(const gj_op *const ops[2], const gj_rrcg_params *P,
     const size_t es = elem_bytes(o->prec);
     const size_t n = (size_t)o->nx * o->ny * o->nz, s = (size_t)o->sx * o->sy;
     cudaError_t e;
-    // one block: the state, then the vectors
+    // one block: the state, the residual's row spectra, then the vectors
+    const size_t vhat_bytes = (2 * vhat_values(o) * 2 * es + 255) / 256 * 256;
     const size_t nbuf = 4 * n + 4 * s + 2 * (size_t)o->nz + (sv->prev_anchor ? 2 * n : 0);
     constexpr size_t kStateBytes = (sizeof(SolverDev) + 255) / 256 * 256;
     void *blk = nullptr;
-    if ((e = pool_alloc(&blk, kStateBytes + nbuf * es, st)) != cudaSuccess) {
+    if ((e = pool_alloc(&blk, kStateBytes + vhat_bytes + nbuf * es, st)) != cudaSuccess) {
         delete sv;
         return cuda_fail(e, "solver state and vectors");
     }
     sv->S = static_cast<SolverDev *>(blk);
-    sv->buf = static_cast<char *>(blk) + kStateBytes;
+    sv->vhat = static_cast<char *>(blk) + kStateBytes;
+    sv->buf = static_cast<char *>(sv->vhat) + vhat_bytes;
     SolverDev h{};
     h.kmax = P->kmax;
     h.stop_on_chi2 = P->stop_on_chi2;
@@ -575,7 +597,7 @@ static gj_status rrcg_create(const gj_op *const ops[2], const gj_rrcg_params *P,
     }
     h.hist = hist;
     cudaMemcpyAsync(sv->S, &h, sizeof(h), cudaMemcpyHostToDevice, st);
-    cudaMemsetAsync(sv->buf, 0, 4 * n * es, st);
+    cudaMemsetAsync(sv->vhat, 0, vhat_bytes + 4 * n * es, st);
     if (o->prec == GJ_FP64) launch_reciprocals(static_cast<double *>(sv->buf), n, s, o->nz, sigma, w_depth, st);
     else launch_reciprocals(static_cast<float *>(sv->buf), n, s, o->nz, sigma, w_depth, st);
     if (o->prec == GJ_FP64) run_head<double>(sv, st); else run_head<float>(sv, st);
