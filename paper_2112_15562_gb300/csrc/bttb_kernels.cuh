@@ -113,6 +113,13 @@ struct FirstBatch {
     }
 };
 
+// Static shared memory of the row passes: block_accumulate's scratch (four sums of the eight
+// warps) and the functors' scalars.  gj_op_tune accepts tiles up to what is left beside
+// kStaticSmem, so it must stay below that.
+constexpr int kRowSums = 4 * 8, kRowScalars = 8;
+constexpr size_t kStaticSmem = 1024;
+static_assert((kRowSums + kRowScalars) * sizeof(double) <= kStaticSmem, "a tile that gj_op_tune accepts must launch");
+
 // Elements of a row functor's loops in flight per thread.
 template <typename R> constexpr int kRowU = sizeof(R) == 8 ? 2 : 4;
 
@@ -375,15 +382,15 @@ __global__ void __launch_bounds__(256) k_row_fwd(OpView<R> op, PairMap pm, int n
     C *buf0 = reinterpret_cast<C *>(smem_raw);
     C *buf1 = buf0 + N * rs.pitch;
     C *tw = buf1 + N * rs.pitch;
-    __shared__ double red[128];
-    __shared__ R sc[8];
+    __shared__ double red[kRowSums];
+    __shared__ R sc[kRowScalars];
     pdl_go();
     copy_twiddles(tw, op.twx, N);
     pdl_wait();
     // the stop flag, the functor's scalars and the first elements: one memory latency for all
     const int stop = stop_flag(done);
     pro.begin();
-    static_assert(Pro::NS <= 8, "scalars");
+    static_assert(Pro::NS <= kRowScalars, "scalars");
     R mine = R(0);
     if (threadIdx.x < Pro::NS) mine = pro.scalar((int)threadIdx.x);
     const int field = blockIdx.y;
@@ -436,14 +443,14 @@ __global__ void __launch_bounds__(256) k_row_inv(OpView<R> op, PairMap pm, int n
     C *buf0 = reinterpret_cast<C *>(smem_raw);
     C *buf1 = buf0 + N * rs.pitch;
     C *tw = buf1 + N * rs.pitch;
-    __shared__ double red[128];
-    __shared__ R sc[8];
+    __shared__ double red[kRowSums];
+    __shared__ R sc[kRowScalars];
     pdl_go();
     copy_twiddles(tw, op.twx, N);
     pdl_wait();
     const int stop = stop_flag(done);
     epi.begin();
-    static_assert(Epi::NS <= 8, "scalars");
+    static_assert(Epi::NS <= kRowScalars, "scalars");
     R mine = R(0);
     if (threadIdx.x < Epi::NS) mine = epi.scalar((int)threadIdx.x);
     const int field = blockIdx.y;
@@ -501,7 +508,7 @@ __global__ void __launch_bounds__(256) k_row_resid(OpView<R> op, PairMap pm, int
     C *buf0 = reinterpret_cast<C *>(smem_raw);
     C *buf1 = buf0 + N * rs.pitch;
     C *tw = buf1 + N * rs.pitch;
-    __shared__ double red[128];
+    __shared__ double red[kRowSums];
     pdl_go();
     copy_twiddles(tw, op.twx, N);
     pdl_wait();

@@ -82,8 +82,7 @@ __device__ __forceinline__ double warp_sums4(double v0, double v1, double v2, do
 
 // Adds per-thread partials acc[0..K) into out[0..K) (one double atomic per
 // block per entry).  All K sums share one pass: warp sums, one barrier, and
-// the first warp finishes (whose `out` counts).  `scratch` holds at least 4 * warps doubles (the kernels
-// reserve 128: up to 32 warps).
+// the first warp finishes (whose `out` counts).  `scratch` holds at least 4 * warps doubles.
 // All threads must call it.
 template <int K, typename A>
 __device__ __forceinline__ void block_accumulate(const A *acc, double *out, double *scratch) {

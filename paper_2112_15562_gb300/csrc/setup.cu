@@ -863,7 +863,7 @@ extern "C" gj_status gj_op_tune(gj_op *op, int P_row, int C_col, int L_grp, int 
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     const size_t cs = 2 * elem_bytes(op->prec);
-    const size_t room = (size_t)optin - 1024;  // the kernels' static reduction scratch
+    const size_t room = (size_t)optin - kStaticSmem;
     if (P_row > 0 && (P_row > 64 || row_smem(op->Nx, P_row, cs) > room)) {
         set_error("gj_op_tune: P_row too large for shared memory"); return GJ_ERR_ARG;
     }
