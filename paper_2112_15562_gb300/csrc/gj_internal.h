@@ -66,8 +66,24 @@ void make_twiddles(int N, std::vector<double> &re, std::vector<double> &im);
 // Stream-ordered device memory from a pool of the library's own, one per device, which keeps
 // up to 128 MB between uses and gives the rest back at the next synchronisation (the default
 // pool gives everything back, and an allocation then costs some 100 us; so does cudaMalloc).
-// Any stream or thread may call; free with cudaFreeAsync in the stream, or with cudaFree.
+// Any stream or thread may call; free with cudaFreeAsync in the stream, or with cudaFree once
+// the kernels on it are done: unlike cudaMalloc's memory, it is given back without waiting.
 cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t st);
+
+// Makes `dev` the current device until the end of the scope.
+class DeviceScope {
+    int before = 0;
+    bool other = false;
+public:
+    explicit DeviceScope(int dev) {
+        other = cudaGetDevice(&before) == cudaSuccess && before != dev && cudaSetDevice(dev) == cudaSuccess;
+    }
+    ~DeviceScope() {
+        if (other) cudaSetDevice(before);
+    }
+    DeviceScope(const DeviceScope &) = delete;
+    DeviceScope &operator=(const DeviceScope &) = delete;
+};
 
 template <typename R> struct OpView;
 template <typename R> OpView<R> view_of(const gj_op *op);

@@ -181,6 +181,7 @@ struct ProfilePair { cudaEvent_t a, b; };
 struct gj_rrcg {
     const gj_op *op[2];
     gj_precision prec;
+    int dev = 0;              // the device that the solver was made on
     SolverDev *S = nullptr;   // device
     void *vhat = nullptr;     // spectra of the residual's rows, both fields (vhat_values)
     void *buf = nullptr;      // p, l (2 fields each, n), v (2 x s), wd (2 x s)
@@ -557,6 +558,11 @@ static gj_status rrcg_create(const gj_op *const ops[2], const gj_rrcg_params *P,
     const gj_op *o = ops[0];
     sv->op[0] = ops[0]; sv->op[1] = ops[1];
     sv->prec = o->prec;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&sv->dev)) != cudaSuccess) {
+        delete sv;
+        return cuda_fail(e, "gj_rrcg_create");
+    }
     for (int i = 0; i < 2; ++i) {
         sv->dobs[i] = dobs[i];
         sv->mapr[i] = m_apr ? m_apr[i] : nullptr;
@@ -568,7 +574,6 @@ static gj_status rrcg_create(const gj_op *const ops[2], const gj_rrcg_params *P,
     sv->prev_anchor = P->anchor == GJ_ANCHOR_PREVIOUS;
     const size_t es = elem_bytes(o->prec);
     const size_t n = (size_t)o->nx * o->ny * o->nz, s = (size_t)o->sx * o->sy;
-    cudaError_t e;
     // one block: the state, the residual's row spectra, then the vectors
     const size_t vhat_bytes = (2 * vhat_values(o) * 2 * es + 255) / 256 * 256;
     const size_t nbuf = 4 * n + 4 * s + 2 * (size_t)o->nz + (sv->prev_anchor ? 2 * n : 0);
@@ -765,6 +770,7 @@ extern "C" gj_status gj_rrcg_profile_read(gj_rrcg *sv, int *launches, double *to
 
 extern "C" void gj_rrcg_destroy(gj_rrcg *sv) {
     if (!sv) return;
+    DeviceScope scope(sv->dev);  // whatever device is current: its kernels are the ones to wait for
     cudaDeviceSynchronize();
     if (sv->exec) cudaGraphExecDestroy(sv->exec);
     if (sv->graph) cudaGraphDestroy(sv->graph);

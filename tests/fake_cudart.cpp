@@ -1,0 +1,115 @@
+// A stand-in for the CUDA runtime with two devices and no kernels, linked with the library's
+// objects so that their host code runs without a GPU.  Device memory is host memory.  It keeps
+// which device is current, which devices have kernels or copies that nothing has waited for, and
+// which device owns each block of pool memory, and counts blocks given back while their device
+// was still at work (freeing pool memory does not wait).
+#include <cuda_runtime_api.h>
+#include <stdlib.h>
+#include <string.h>
+
+#include <map>
+
+namespace {
+int current = 0, early_frees = 0, launches = 0;
+bool busy[2] = {false, false};
+std::map<void *, int> pool_blocks;
+cudaError_t give(void **p, size_t bytes) {
+    *p = calloc(1, bytes ? bytes : 1);
+    return *p ? cudaSuccess : cudaErrorMemoryAllocation;
+}
+cudaError_t handle(void *out) {
+    *static_cast<void **>(out) = malloc(1);
+    return cudaSuccess;
+}
+}  // namespace
+
+extern "C" {
+int fake_early_frees() { return early_frees; }
+int fake_launches() { return launches; }
+int fake_pool_blocks() { return (int)pool_blocks.size(); }
+
+cudaError_t cudaGetDevice(int *d) { *d = current; return cudaSuccess; }
+cudaError_t cudaSetDevice(int d) { current = d; return cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() { busy[current] = false; return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { busy[current] = false; return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr a, int) {
+    *v = a == cudaDevAttrMultiProcessorCount ? 4 : a == cudaDevAttrMaxSharedMemoryPerBlockOptin ? 227 * 1024 : 0;
+    return cudaSuccess;
+}
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+const char *cudaGetErrorName(cudaError_t) { return "fake"; }
+const char *cudaGetErrorString(cudaError_t) { return "fake"; }
+
+cudaError_t cudaMalloc(void **p, size_t n) { return give(p, n); }
+cudaError_t cudaMallocAsync(void **p, size_t n, cudaStream_t) { return give(p, n); }
+cudaError_t cudaMallocFromPoolAsync(void **p, size_t n, cudaMemPool_t, cudaStream_t) {
+    cudaError_t e = give(p, n);
+    if (e == cudaSuccess) pool_blocks[*p] = current;
+    return e;
+}
+cudaError_t cudaFree(void *p) {
+    auto it = pool_blocks.find(p);
+    if (it != pool_blocks.end()) {
+        early_frees += busy[it->second];
+        pool_blocks.erase(it);
+    }
+    free(p);
+    return cudaSuccess;
+}
+cudaError_t cudaFreeAsync(void *p, cudaStream_t) { pool_blocks.erase(p); free(p); return cudaSuccess; }
+cudaError_t cudaMemPoolCreate(cudaMemPool_t *p, const cudaMemPoolProps *) { return handle(p); }
+cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *) { return cudaSuccess; }
+cudaError_t cudaMemPoolDestroy(cudaMemPool_t) { return cudaSuccess; }
+cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { return give(p, n); }
+cudaError_t cudaGetSymbolAddress(void **, const void *) { return cudaErrorNotSupported; }
+cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { memcpy(d, s, n); return cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) {
+    busy[current] = true;
+    memcpy(d, s, n);
+    return cudaSuccess;
+}
+cudaError_t cudaMemset(void *d, int v, size_t n) { memset(d, v, n); return cudaSuccess; }
+cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t) {
+    busy[current] = true;
+    memset(d, v, n);
+    return cudaSuccess;
+}
+
+static cudaError_t launched() {
+    busy[current] = true;
+    ++launches;
+    return cudaSuccess;
+}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *, const void *, void **) { return launched(); }
+cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3, dim3, void **, size_t, cudaStream_t) { return launched(); }
+cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *) { *k = nullptr; return cudaSuccess; }
+unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, void *) { return 0; }
+cudaError_t __cudaPopCallConfiguration(dim3 *, dim3 *, size_t *, void *) { return cudaSuccess; }
+void **__cudaRegisterFatBinary(void *p) { return (void **)p; }
+void __cudaRegisterFatBinaryEnd(void **) {}
+void __cudaUnregisterFatBinary(void **) {}
+void __cudaRegisterFunction(void **, const char *, char *, const char *, int, uint3 *, uint3 *, dim3 *, dim3 *, int *) {}
+void __cudaRegisterVar(void **, char *, char *, const char *, int, size_t, int, int) {}
+cudaError_t cudaFuncGetAttributes(cudaFuncAttributes *a, const void *) { memset(a, 0, sizeof *a); return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void *, cudaFuncAttribute, int) { return cudaSuccess; }
+
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s) {
+    *s = cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return handle(s); }
+cudaError_t cudaStreamDestroy(cudaStream_t s) { free(s); return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *g) { return handle(g); }
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t *x, cudaGraph_t, unsigned long long) { return handle(x); }
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return launched(); }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t x) { free(x); return cudaSuccess; }
+cudaError_t cudaGraphDestroy(cudaGraph_t g) { free(g); return cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t *e) { return handle(e); }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return handle(e); }
+cudaError_t cudaEventDestroy(cudaEvent_t e) { free(e); return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { *ms = 0; return cudaSuccess; }
+}

@@ -1,0 +1,75 @@
+"""The library's host code against a stand-in for the CUDA runtime with two devices
+(fake_cudart.cpp): what it allocates, waits for and frees, and on which device.  No GPU."""
+import ctypes as ct
+import glob
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    from paper_2112_15562_gb300 import _lib, build
+
+    def objects():
+        return [os.path.join(build.BUILD, s.replace(".cu", ".o")) for s in build.SOURCES]
+
+    build.build(force=not all(os.path.exists(o) for o in objects()))
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build._nvcc()))))
+    include = [d for d in (os.path.join(cuda, "include"), *glob.glob(os.path.join(cuda, "targets", "*", "include")))
+               if os.path.exists(os.path.join(d, "cuda_runtime_api.h"))]
+    out = str(tmp_path_factory.mktemp("fake") / "libgj_fake.so")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", include[0],
+                    os.path.join(ROOT, "tests", "fake_cudart.cpp"), *objects(), "-o", out], check=True)
+    real, _lib._lib, path, _lib.LIB_PATH = _lib._lib, None, _lib.LIB_PATH, out
+    try:
+        yield _lib.load()
+    finally:
+        _lib._lib, _lib.LIB_PATH = real, path
+
+
+def solver(lib, kmax=5):
+    """A solver over 4 x 4 x 2 cells in FP64; returns (handle, operators, keep-alive)."""
+    from paper_2112_15562_gb300 import _lib as L
+    from paper_2112_15562_gb300.api import solver_params
+
+    z = (ct.c_double * 3)(0.0, 10.0, 20.0)
+    g = L.Grid(4, 4, 4, 4, 2, 10.0, 10.0, ct.cast(z, ct.POINTER(ct.c_double)), 0.0, 0, 0)
+    mag = L.Mag(50000.0, 60.0, 10.0)
+    ops = (ct.c_void_p * 2)()
+    for i in range(2):
+        h = ct.c_void_p()
+        assert lib.gj_bttb_setup(ct.byref(g), 1 + i, ct.byref(mag), 0, 0, 0, None, ct.byref(h)) == 0
+        ops[i] = h.value
+    keep = [(ct.c_double * n)(*([1.0] * n)) for n in (16, 16, 2, 32) for _ in range(2)]
+    pair = lambda k: (ct.c_void_p * 2)(*[ct.addressof(x) for x in keep[2 * k:2 * k + 2]])
+    P = solver_params(kmax=kmax)
+    h = ct.c_void_p()
+    assert lib.gj_rrcg_create(ops, ct.byref(P), pair(0), pair(1), None, pair(2), None, pair(3), None, None, ct.byref(h)) == 0
+    return h, ops, keep
+
+
+@pytest.mark.parametrize("current", [0, 1])
+def test_a_solver_is_freed_after_its_own_device_is_done(lib, current):
+    """Its block is pool memory, which is given back without waiting: destroying it while another
+    device is current has to wait for the device that it was made on, and leaves the caller's
+    device current."""
+    before, blocks = lib.fake_early_frees(), lib.fake_pool_blocks()
+    assert lib.cudaSetDevice(0) == 0
+    h, ops, keep = solver(lib)
+    n = lib.fake_launches()
+    assert lib.gj_rrcg_iterate(h, 2, 0, None) == 0 and lib.fake_launches() > n
+    assert lib.fake_pool_blocks() == blocks + 1
+    lib.cudaSetDevice(current)
+    lib.gj_rrcg_destroy(h)
+    dev = ct.c_int(-1)
+    lib.cudaGetDevice(ct.byref(dev))
+    assert dev.value == current
+    assert lib.fake_pool_blocks() == blocks
+    assert lib.fake_early_frees() == before
+    lib.cudaSetDevice(0)
+    for op in ops:
+        lib.gj_op_destroy(op)
