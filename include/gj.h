@@ -129,7 +129,8 @@ gj_status gj_bttb_setup(const gj_grid *grid, gj_field field, const gj_mag *mag,
 enum {
     /* Keep one layer's spectrum instead of all n_z: every product rebuilds each
      * layer's spectrum from the closed-form prism fields (the FP64 corner lattice of
-     * every depth plane's near-field window once per product; per layer the FP64 2-D
+     * every depth plane's near-field window once per product, or of each layer's two
+     * planes where all of them are large; per layer the FP64 2-D
      * FFT of its circulant table, rounded to the operator's precision on chip, column
      * by column) as the column pass uses it (Sec. 2.7.1 applied per layer).  The
      * spectra are those of a stored operator up to the rounding of the FP64 build; the

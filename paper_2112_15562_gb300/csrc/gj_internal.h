@@ -95,8 +95,9 @@ int fast_col_items(int Ny, int nz);  // items per column of the fast column kern
 int fast_slots(int nfield, int ncol, int items_per_col, long long warps);
 bool fast1024_eligible(const gj_op *op);
 
-// recompute mode (setup.cu): the corner lattice of every depth plane, once per product;
-// then layer r's table and its FP64 row transforms, and where those are
+// recompute mode (setup.cu): the corner lattice of every depth plane, once per product (or, where
+// that is large, each layer's two planes with the layer); then layer r's table and its FP64 row
+// transforms, and where those are
 void recompute_begin(const gj_op *op, cudaStream_t st);
 void recompute_rows(const gj_op *op, int r, cudaStream_t st);
 const double2 *recompute_rows_out(const gj_op *op);

@@ -157,12 +157,12 @@ template <typename F> struct LayerGeom {
 // sum of the lattice, or the far-field cubature.
 template <typename F> struct TableGeom {
     const double *lat;
-    int nbx1, nby1, k0;  // lattice points, and the lattice plane of the build's first layer
+    int nbx1, nby1, k0;  // lattice points, and the lattice plane of the launch's first layer
     int Nx, Ny, sx, sy, nx, ny, off_x, off_y, a_max, b_max;
     int a0, na, b0, nb;  // |c + off| runs over [a0, a0 + na) along y and [b0, b0 + nb) along x
     double scale;
     const F *axis;              // prism centres -|c + off| cell: [nb] along x, then [na] along y
-    const LayerGeom<F> *layer;  // of the build's first layer
+    const LayerGeom<F> *layer;  // of the launch's first layer
     F hu, hv;                   // half cells
     FarCoef<F> k;
 };
@@ -207,8 +207,9 @@ __global__ void __launch_bounds__(256) k_table_rows(TableGeom<F> G, OpView<doubl
         iy[l] = cy < 0 ? cy + G.Ny : cy;
     }
     if (!ok[0] && !ok[1]) return;
-    // Launches after the first of a build follow a column launch that started its own work
-    // when everything before it was complete: the lattice is there, and only Zs is waited for.
+    // Where one lattice serves the whole build, launches after the first follow a column launch
+    // that started its own work when everything before it was complete: the lattice is there,
+    // and only Zs is waited for.
     if (after_lattice) pdl_wait();
     C *buf0 = reinterpret_cast<C *>(smem_raw), *buf1 = buf0 + N, *tw = buf1 + N;
     load_twiddles(tw, op.twx, N);
@@ -448,10 +449,10 @@ static void free_op_memory(gj_op *op) {
 }
 
 // Work buffers of the spectrum build for `layers` consecutive layers at a time: the FP64
-// corner lattice (every depth plane: about 20 x 20 points each), the FP64 row
-// transforms of the tables (rows outside the offsets in use stay zero), the geometry and
-// FP64 twiddles.  Kept by operators that rebuild their
-// spectra per layer.
+// corner lattice (the depth planes of lat_layers consecutive layers: about 20 x 20 points each
+// for cubic cells), the FP64 row transforms of the tables (rows outside the offsets in use stay
+// zero), the geometry and FP64 twiddles.  Kept by operators that rebuild their spectra per
+// layer.
 struct gj_setup_scratch_impl {
     double *lat = nullptr;
     void *axis = nullptr, *layer = nullptr;  // TableGeom's, in the far field's precision
@@ -459,7 +460,7 @@ struct gj_setup_scratch_impl {
     double *zw = nullptr;
     void *twx64 = nullptr, *twy64 = nullptr;
     bool own_tw = false;
-    int layers = 0;
+    int layers = 0, lat_layers = 0;
 };
 
 static void scratch_free(gj_setup_scratch_impl *sc) {
@@ -538,10 +539,22 @@ static void table_geometry(const gj_op *op, const std::vector<double> &zw, std::
     }
 }
 
-static gj_status scratch_alloc(const gj_op *op, int layers, gj_setup_scratch_impl **out) {
+// Layers that the corner lattice of a rebuilding operator covers at a time: all (one launch a
+// product) while their planes take no more than one layer's row transforms, or a megabyte;
+// layers much thicker than the cells are wide spread the near field over the whole grid, where
+// all planes would outweigh the spectra that the operator does not keep: then one.
+constexpr size_t kLatticeKeep = 1 << 20;
+static int kept_lattice_layers(const gj_op *op) {
+    const LatticeWindow lw = lattice_window(op);
+    const size_t all = (size_t)lw.nbx1 * lw.nby1 * (op->nz + 1) * sizeof(double);
+    return all <= std::max(kLatticeKeep, (size_t)op->Ny * op->ncol * sizeof(double2)) ? op->nz : 1;
+}
+
+static gj_status scratch_alloc(const gj_op *op, int layers, int lat_layers, gj_setup_scratch_impl **out) {
     gj_setup_scratch_impl *sc = new (std::nothrow) gj_setup_scratch_impl();
     if (!sc) { set_error("setup scratch: host allocation failed"); return GJ_ERR_OOM; }
     sc->layers = layers;
+    sc->lat_layers = lat_layers;
     gj_status rc = GJ_OK;
     cudaError_t e;
     if (op->prec == GJ_FP64) {
@@ -560,7 +573,7 @@ static gj_status scratch_alloc(const gj_op *op, int layers, gj_setup_scratch_imp
     if (op->prec == GJ_FP32_MIXED) table_geometry<float>(op, zw, axis, geom);
     else table_geometry<double>(op, zw, axis, geom);
     const size_t zsb = (size_t)layers * op->Ny * op->ncol * sizeof(double2);
-    if ((e = cudaMalloc(&sc->lat, plane * (op->nz + 1) * sizeof(double))) != cudaSuccess ||
+    if ((e = cudaMalloc(&sc->lat, plane * (lat_layers + 1) * sizeof(double))) != cudaSuccess ||
         (e = cudaMalloc(&sc->Zs, zsb)) != cudaSuccess || (e = cudaMemset(sc->Zs, 0, zsb)) != cudaSuccess ||
         (e = cudaMalloc(&sc->zw, zw.size() * sizeof(double))) != cudaSuccess ||
         (e = cudaMalloc(&sc->axis, axis.size())) != cudaSuccess ||
@@ -575,19 +588,20 @@ static gj_status scratch_alloc(const gj_op *op, int layers, gj_setup_scratch_imp
     return GJ_OK;
 }
 
-// The corner lattice of every depth plane (enqueues one launch).  A point is a chain of
-// FP64 logarithms and arctangents, so the points are spread one warp a block.
-static void build_lattice(const gj_op *op, const gj_setup_scratch_impl &sc, cudaStream_t st) {
+// The corner lattice of the depth planes of layers r0 .. r0 + lat_layers - 1 (enqueues one
+// launch).  A point is a chain of FP64 logarithms and arctangents, so the points are spread
+// one warp a block.
+static void build_lattice(const gj_op *op, const gj_setup_scratch_impl &sc, int r0, cudaStream_t st) {
     const LatticeWindow lw = lattice_window(op);
     Lattice L;
     L.b_max = lw.b_max;
     L.a_max = lw.a_max;
     L.nbx1 = lw.nbx1;
     L.nby1 = lw.nby1;
-    L.nz1 = op->nz + 1;
+    L.nz1 = sc.lat_layers + 1;
     L.dx = op->dx;
     L.dy = op->dy;
-    L.zw = sc.zw;
+    L.zw = sc.zw + r0;
     const size_t pts = (size_t)L.nbx1 * L.nby1 * L.nz1;
     launch_after(k_corner_lattice, dim3((unsigned)std::min<size_t>(4864, (pts + 31) / 32)), dim3(32), 0, st, L,
                  op->field == GJ_MAGNETIC, mag_coef(op), sc.lat);
@@ -596,13 +610,15 @@ static void build_lattice(const gj_op *op, const gj_setup_scratch_impl &sc, cuda
 // Tables of layers r0 .. r0 + count - 1 (count <= the scratch's layers), after
 // build_lattice, and their FP64 row transforms into the scratch's Zs (even_rows: the rows
 // 0 .. Ny/2 alone).  Enqueues only (no synchronisation).
+// The builds go through the layers in order, from layer 0.
 template <typename F>
 static void launch_table_rows(const gj_op *op, const gj_setup_scratch_impl &sc, int r0, int count,
                               const OpView<double> &v, cudaStream_t st) {
-    const bool after_lattice = r0 == 0;  // the builds go through the layers in order
+    const bool all = sc.lat_layers == op->nz;     // one lattice for the whole build
+    const bool after_lattice = r0 == 0 || !all;  // else it is older than the launch before this one
     const LatticeWindow lw = lattice_window(op);
     TableGeom<F> G;
-    G.lat = sc.lat; G.nbx1 = lw.nbx1; G.nby1 = lw.nby1; G.k0 = r0;
+    G.lat = sc.lat; G.nbx1 = lw.nbx1; G.nby1 = lw.nby1; G.k0 = all ? r0 : 0;
     G.Nx = op->Nx; G.Ny = op->Ny; G.sx = op->sx; G.sy = op->sy; G.nx = op->nx; G.ny = op->ny;
     G.off_x = op->off_x; G.off_y = op->off_y; G.a_max = lw.a_max; G.b_max = lw.b_max;
     offset_span(op->off_y, op->sy, op->ny, G.a0, G.na);
@@ -667,10 +683,10 @@ static gj_status build_spectra(gj_op *op, cudaStream_t st) {
     // as many layers at a time as fit a quarter of a gigabyte of row transforms
     const size_t per = (size_t)op->Ny * op->ncol * sizeof(double2);
     const int most = (int)std::max<size_t>(1, std::min<size_t>(op->nz, ((size_t)256 << 20) / per));
-    gj_status rc = scratch_alloc(op, most, &sc);
+    gj_status rc = scratch_alloc(op, most, op->nz, &sc);
     if (rc != GJ_OK) return rc;
     set_build_attributes();
-    build_lattice(op, *sc, st);
+    build_lattice(op, *sc, 0, st);
     for (int r = 0; r < op->nz; r += most)
         build_layers<Rout>(op, *sc, r, std::min(most, op->nz - r),
                            static_cast<cpx<Rout> *>(op->spec) + spec_offset(op, r), st);
@@ -681,9 +697,12 @@ static gj_status build_spectra(gj_op *op, cudaStream_t st) {
     return GJ_OK;
 }
 
-void recompute_begin(const gj_op *op, cudaStream_t st) { build_lattice(op, *op->scratch, st); }
+void recompute_begin(const gj_op *op, cudaStream_t st) {
+    if (op->scratch->lat_layers == op->nz) build_lattice(op, *op->scratch, 0, st);
+}
 
 void recompute_rows(const gj_op *op, int r, cudaStream_t st) {
+    if (op->scratch->lat_layers != op->nz) build_lattice(op, *op->scratch, r, st);
     build_rows(op, *op->scratch, r, 1, st);
 }
 const double2 *recompute_rows_out(const gj_op *op) { return op->scratch->Zs; }
@@ -788,7 +807,7 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
     }
     if (op->recompute) {
         // one layer's spectrum plus the build's work buffers for one layer, kept
-        if ((rc = scratch_alloc(op, 1, &op->scratch)) != GJ_OK) goto fail;
+        if ((rc = scratch_alloc(op, 1, kept_lattice_layers(op), &op->scratch)) != GJ_OK) goto fail;
         set_build_attributes();
     } else {
         rc = (prec == GJ_FP64) ? build_spectra<double>(op, st) : build_spectra<float>(op, st);

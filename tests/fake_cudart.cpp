@@ -1,8 +1,8 @@
 // A stand-in for the CUDA runtime with two devices and no kernels, linked with the library's
 // objects so that their host code runs without a GPU.  Device memory is host memory.  It keeps
 // which device is current, which devices have kernels or copies that nothing has waited for, and
-// which device owns each block of pool memory, and counts blocks given back while their device
-// was still at work (freeing pool memory does not wait).
+// which device owns each block of pool memory, counts blocks given back while their device
+// was still at work (freeing pool memory does not wait), and sums the bytes that cudaMalloc holds.
 #include <cuda_runtime_api.h>
 #include <stdlib.h>
 #include <string.h>
@@ -13,6 +13,7 @@ namespace {
 int current = 0, early_frees = 0, launches = 0;
 bool busy[2] = {false, false};
 std::map<void *, int> pool_blocks;
+std::map<void *, size_t> held;
 cudaError_t give(void **p, size_t bytes) {
     *p = calloc(1, bytes ? bytes : 1);
     return *p ? cudaSuccess : cudaErrorMemoryAllocation;
@@ -26,6 +27,11 @@ cudaError_t handle(void *out) {
 extern "C" {
 int fake_early_frees() { return early_frees; }
 int fake_launches() { return launches; }
+long long fake_held_bytes() {
+    long long n = 0;
+    for (auto &b : held) n += (long long)b.second;
+    return n;
+}
 int fake_pool_blocks() { return (int)pool_blocks.size(); }
 
 cudaError_t cudaGetDevice(int *d) { *d = current; return cudaSuccess; }
@@ -40,7 +46,11 @@ cudaError_t cudaGetLastError() { return cudaSuccess; }
 const char *cudaGetErrorName(cudaError_t) { return "fake"; }
 const char *cudaGetErrorString(cudaError_t) { return "fake"; }
 
-cudaError_t cudaMalloc(void **p, size_t n) { return give(p, n); }
+cudaError_t cudaMalloc(void **p, size_t n) {
+    cudaError_t e = give(p, n);
+    if (e == cudaSuccess) held[*p] = n;
+    return e;
+}
 cudaError_t cudaMallocAsync(void **p, size_t n, cudaStream_t) { return give(p, n); }
 cudaError_t cudaMallocFromPoolAsync(void **p, size_t n, cudaMemPool_t, cudaStream_t) {
     cudaError_t e = give(p, n);
@@ -53,6 +63,7 @@ cudaError_t cudaFree(void *p) {
         early_frees += busy[it->second];
         pool_blocks.erase(it);
     }
+    held.erase(p);
     free(p);
     return cudaSuccess;
 }

@@ -73,3 +73,29 @@ def test_a_solver_is_freed_after_its_own_device_is_done(lib, current):
     lib.cudaSetDevice(0)
     for op in ops:
         lib.gj_op_destroy(op)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("dz", [10.0, 400.0])
+def test_a_recomputing_operator_keeps_one_layer(lib, dz, prec):
+    """Beside its intermediates (workspace_bytes) and the one spectrum plane, an operator that
+    rebuilds its spectra holds the work buffers of one layer's build: more layers add a few depths,
+    also when layers forty times as thick as the cells are wide take the near field over the whole
+    grid (a depth plane of corner values is then larger than a layer's spectrum)."""
+    from paper_2112_15562_gb300 import _lib as L
+
+    lib.fake_held_bytes.restype = ct.c_longlong
+    lib.cudaSetDevice(0)
+    extra = []
+    for nz in (2, 60):
+        z = (ct.c_double * (nz + 1))(*[k * dz for k in range(nz + 1)])
+        g = L.Grid(200, 180, 200, 180, nz, 10.0, 10.0, ct.cast(z, ct.POINTER(ct.c_double)), 0.0, 0, 0)
+        before = lib.fake_held_bytes()
+        h, info = ct.c_void_p(), L.OpInfo()
+        assert lib.gj_bttb_setup_ex(ct.byref(g), 1, None, prec, 0, 0, L.GJ_SETUP_RECOMPUTE_SPECTRA, None, ct.byref(h)) == 0
+        assert lib.gj_op_info(h, ct.byref(info)) == 0
+        extra.append(lib.fake_held_bytes() - before - info.workspace_bytes - info.spectrum_bytes)
+        lib.gj_op_destroy(h)
+        assert lib.fake_held_bytes() == before
+    plane = 400 * 360 * 8  # corner values of one depth plane over the whole grid
+    assert extra[1] - extra[0] <= plane, extra
