@@ -146,7 +146,8 @@ __device__ __forceinline__ void far_cubature(F uc, F hu, F vc, F hv, F wc, F hw,
 }
 
 // Depth range of a layer (centre and half height below the stations), its squared
-// near-field radius, and the cubature's volume element times the scale of the spectra.
+// near-field radius, all in length_unit, and the cubature's volume element times the scale of
+// the spectra.
 template <typename F> struct LayerGeom {
     F wc, hw, near2;
     double vol;
@@ -163,7 +164,7 @@ template <typename F> struct TableGeom {
     double scale;
     const F *axis;              // prism centres -|c + off| cell: [nb] along x, then [na] along y
     const LayerGeom<F> *layer;  // of the launch's first layer
-    F hu, hv;                   // half cells
+    F hu, hv;                   // half cells (lengths in length_unit)
     FarCoef<F> k;
 };
 
@@ -517,6 +518,10 @@ static void offset_span(int off, int s, int n, int &lo, int &count) {
     count = std::max(std::abs(first), std::abs(last)) - lo + 1;
 }
 
+// The cubature's lengths are in units of about a cell, a power of two, so that nothing rounds:
+// in metres, a distance's fifth power left FP32 beyond 3e7 m (or below 3e-8).
+static double length_unit(const gj_op *op) { return std::ldexp(1.0, std::ilogb(std::max(op->dx, op->dy))); }
+
 // TableGeom's axis and layer arrays in precision F (as bytes)
 template <typename F>
 static void table_geometry(const gj_op *op, const std::vector<double> &zw, std::vector<char> &axis,
@@ -527,15 +532,18 @@ static void table_geometry(const gj_op *op, const std::vector<double> &zw, std::
     axis.resize((nb + na) * sizeof(F));
     geom.resize(op->nz * sizeof(LayerGeom<F>));
     F *ax = reinterpret_cast<F *>(axis.data());
-    for (int i = 0; i < nb; ++i) ax[i] = (F)(-(double)(b0 + i) * op->dx);
-    for (int i = 0; i < na; ++i) ax[nb + i] = (F)(-(double)(a0 + i) * op->dy);
+    const double to = 1.0 / length_unit(op);
+    for (int i = 0; i < nb; ++i) ax[i] = (F)(-(double)(b0 + i) * op->dx * to);
+    for (int i = 0; i < na; ++i) ax[nb + i] = (F)(-(double)(a0 + i) * op->dy * to);
+    // of w / R^3 (gravity) and 1 / R^3 (magnetic) per unit of volume
+    const double per = op->field == GJ_MAGNETIC ? to * to * to : to * to;
     LayerGeom<F> *lg = reinterpret_cast<LayerGeom<F> *>(geom.data());
     for (int k = 0; k < op->nz; ++k) {
         const double size = std::max(std::max(op->dx, op->dy), zw[k + 1] - zw[k]);
-        lg[k].wc = (F)(0.5 * (zw[k] + zw[k + 1]));
-        lg[k].hw = (F)(0.5 * (zw[k + 1] - zw[k]));
-        lg[k].near2 = (F)(kFar * kFar * size * size);
-        lg[k].vol = 0.125 * op->dx * op->dy * (zw[k + 1] - zw[k]) * table_scale(op);
+        lg[k].wc = (F)(0.5 * (zw[k] + zw[k + 1]) * to);
+        lg[k].hw = (F)(0.5 * (zw[k + 1] - zw[k]) * to);
+        lg[k].near2 = (F)(kFar * kFar * (size * to) * (size * to));
+        lg[k].vol = 0.125 * op->dx * op->dy * (zw[k + 1] - zw[k]) * per * table_scale(op);
     }
 }
 
@@ -626,8 +634,8 @@ static void launch_table_rows(const gj_op *op, const gj_setup_scratch_impl &sc, 
     G.scale = table_scale(op);
     G.axis = static_cast<const F *>(sc.axis);
     G.layer = static_cast<const LayerGeom<F> *>(sc.layer) + r0;
-    G.hu = (F)(0.5 * op->dx);
-    G.hv = (F)(0.5 * op->dy);
+    G.hu = (F)(0.5 * op->dx / length_unit(op));
+    G.hv = (F)(0.5 * op->dy / length_unit(op));
     const MagCoef mc = mag_coef(op);
     const double tr = mc.c[0] + mc.c[1] + mc.c[2];
     G.k = FarCoef<F>{(F)(3 * mc.c[0] - tr), (F)(3 * mc.c[1] - tr), (F)(3 * mc.c[2] - tr),
