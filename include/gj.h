@@ -245,7 +245,8 @@ gj_status gj_g_adjoint_pair(const gj_op *const ops[2], const void *const r[2], v
  * S = (m1,m1)(m2,m2) - (m1,m2)^2 written to the device double *S, and the
  * ascent directions l1 = (m2,m2) m1 - (m1,m2) m2, l2 = (m1,m1) m2 - (m1,m2) m1
  * (half the gradient of S).  l1 / l2 may be NULL to skip them.  Vectors of
- * length n in the given precision; inner products accumulate in FP64.
+ * length n in the given precision; inner products accumulate in FP64.  l1 and l2
+ * may be m1 and m2 themselves, in either order.
  */
 gj_status gj_gramian_value_grad(int64_t n, gj_precision precision,
                                 const void *m1, const void *m2, double *S,

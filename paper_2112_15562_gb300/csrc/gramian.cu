@@ -23,12 +23,12 @@ template <typename R> struct Vec16;
 template <> struct Vec16<float> { using T = float4; static constexpr int N = 4; };
 template <> struct Vec16<double> { using T = double2; static constexpr int N = 2; };
 
-// Calls f(k, x, y) for the elements of this thread's chunks, k < kGramChunk a compile-time
-// position in the chunk, and chunk_done() after each chunk.  VEC: 16-byte loads (aligned
-// vectors), else one element a load.  get(i, x, y) when they are one element, else in vectors.
+// Calls each(i, x, y) for this thread's elements i, a vector of them (VEC: 16-byte loads, for
+// aligned vectors) or one at a time, and done() after each chunk of at most kGramChunk.  The
+// directions may be written over the vectors (a thread reads an element before it writes it, and
+// no other thread does either), so nothing here promises that they do not overlap.
 template <typename R, bool VEC, class Each, class Done>
-__device__ __forceinline__ void gram_chunks(int64_t n, const R *__restrict__ m1, const R *__restrict__ m2, Each each,
-                                            Done done) {
+__device__ __forceinline__ void gram_chunks(int64_t n, const R *m1, const R *m2, Each each, Done done) {
     const int64_t thread = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, threads = (int64_t)gridDim.x * blockDim.x;
     if constexpr (VEC) {
         using V = typename Vec16<R>::T;
