@@ -93,7 +93,8 @@ typedef struct {
                                 Nx = 1024 with at most 512 prisms and stations along x,
                                 and the general row kernels otherwise; 0: the
                                 general kernels */
-    int P_row, C_col, L_grp; /* launch shapes of the general kernels (gj_op_tune) */
+    int P_row, C_col, L_grp; /* launch shapes of the general kernels (gj_op_tune); of a launch
+                                that serves both fields while they are the library's choice */
     int radix_order;         /* radix plan of the general kernels' transforms (gj_op_tune) */
     int recompute;           /* 1: spectra rebuilt per layer (GJ_SETUP_RECOMPUTE_SPECTRA) */
 } gj_op_info_t;
@@ -161,10 +162,14 @@ gj_status gj_op_info(const gj_op *op, gj_op_info_t *info);
  * transforms (0: the cheapest stages of radix 2 to 17; 1: the same stages reversed;
  * 2: radix 4 for the power-of-two part, then the odd primes).  L_grp is raised where the
  * layer groups would outnumber the operator's partial-sum slots.  A value <= 0 (or < 0 for
- * radix_order) keeps the current choice.  Any choice gives the same products up
- * to rounding.  Synchronous, host-side only; GJ_ERR_ARG if a tile does not fit
- * in shared memory.  Not for operators in use on another stream.
+ * radix_order) keeps the current choice, except GJ_TUNE_AUTO, which gives it back to the
+ * library: until a shape is set, every launch takes its own for its pass, number of fields
+ * and sizes (gj_op_info then reports the row and forward column shapes of a launch that
+ * serves both fields).  Any choice gives the same products up to rounding.  Synchronous,
+ * host-side only; GJ_ERR_ARG if a tile does not fit in shared memory.  Not for operators in
+ * use on another stream.
  */
+enum { GJ_TUNE_AUTO = -2 }; /* for P_row, C_col and L_grp; radix_order: 0 */
 gj_status gj_op_tune(gj_op *op, int P_row, int C_col, int L_grp, int radix_order);
 
 /* Frees an operator (waits for the device to finish using it).  NULL is a no-op. */

@@ -15,6 +15,7 @@ GJ_GRAVITY, GJ_MAGNETIC = 1, 2
 GJ_FP64, GJ_FP32_MIXED = 0, 1
 GJ_SCALARS_AUTO, GJ_SCALARS_JOINT, GJ_SCALARS_PER_FIELD = 0, 1, 2
 GJ_SETUP_RECOMPUTE_SPECTRA = 1
+GJ_TUNE_AUTO = -2
 
 
 class GJError(RuntimeError):

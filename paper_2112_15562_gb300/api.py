@@ -53,7 +53,8 @@ class Op:
         return g_adjoint(self, r, g, stream)
 
     def tune(self, P_row: int = 0, C_col: int = 0, L_grp: int = 0, radix_order: int = -1):
-        """gj_op_tune: launch shapes and radix plan of the general product kernels."""
+        """gj_op_tune: launch shapes and radix plan of the general product kernels (0, and -1 for
+        radix_order, keep the current choice; GJ_TUNE_AUTO gives a shape back to the library)."""
         check(load().gj_op_tune(self._h, int(P_row), int(C_col), int(L_grp), int(radix_order)))
         check(load().gj_op_info(self._h, ct.byref(self.info)))
 

@@ -88,15 +88,16 @@ KNOBS = {"P_row": (1, 2, 4, 8, 16), "C_col": (1, 2, 4, 8, 16), "L_grp": (1, 2, 4
 
 def _refine(ops, reps, base_ms):
     """One pass of coordinate search over KNOBS on the general kernels; returns the
-    settings that differ from the library's defaults and the tuned time."""
-    from ._lib import GJError
+    settings to make (the others stay the library's own choice, which may differ from
+    pass to pass) and the time measured with exactly those."""
+    from ._lib import GJ_TUNE_AUTO, GJError
 
-    default = ops[0].tiles()
-    cur_set = dict(default)
+    chosen: Dict[str, int] = {}
     cur = base_ms
     for knob, values in KNOBS.items():
+        untuned = 0 if knob == "radix_order" else GJ_TUNE_AUTO
         for v in values:
-            if v == cur_set[knob]:
+            if v == untuned:
                 continue
             try:
                 for op in ops:
@@ -105,10 +106,10 @@ def _refine(ops, reps, base_ms):
                 continue
             t = _time_ops(ops, reps)
             if t < cur * 0.98:
-                cur, cur_set[knob] = t, v
+                cur, chosen[knob] = t, v
         for op in ops:  # leave the knob at its best value for the next one
-            op.tune(**{knob: cur_set[knob]})
-    return {k: v for k, v in cur_set.items() if v != default[k]}, cur
+            op.tune(**{knob: chosen.get(knob, untuned)})
+    return chosen, cur
 
 
 def tune_full(grid, mag, precision: str = "fp32", cache: Optional[str] = None, reps: int = 5):

@@ -680,6 +680,23 @@ static void set_build_attributes() {
     allow_max_smem(k_col_spec<double>);
 }
 
+// The library's choice of the launch shapes, as reported: those of both fields' launches (others
+// pick their own until tuned).
+static void auto_shapes(gj_op *op, bool rows, bool cols, bool layers) {
+    const size_t cs = 2 * elem_bytes(op->prec);
+    if (rows) {
+        op->rows_tuned = false;
+        op->P_row = pick_row_pairs(op->px, (long long)op->nz * op->ny, cs);
+        if (op->fast1024) {  // transposed intermediates: runs of P lines
+            op->P_row = 16;
+            while (op->P_row > 1 && row_smem(op->Nx, odd_pitch(op->P_row), cs) > kGenSmem) op->P_row >>= 1;
+        }
+    }
+    const ColPick both = pick_cols(op->py, op->ncol, op->recompute ? 1 : op->nz, 2, cs, false);
+    if (cols) { op->cols_tuned = false; op->C_col = both.C; }
+    if (layers) { op->layers_tuned = false; op->L_grp = both.L; }
+}
+
 // where layer r's spectrum starts, in complex values (the even real spectra: two values each)
 static size_t spec_offset(const gj_op *op, int r) {
     return op->real_spec ? (size_t)r * op->ncol * even_spec_len(op->Ny) / 2 : (size_t)r * op->Ny * op->ncol;
@@ -790,16 +807,8 @@ extern "C" gj_status gj_bttb_setup_ex(const gj_grid *grid, gj_field field, const
         op->slots = std::max(fast_slots(1, op->ncol, G.nz, warps), fast_slots(2, op->ncol, G.nz, warps));
         op->real_spec = op->even_table;
     }
-    // the shapes of both fields' launches (single-field ones pick their own until tuned)
     const int layers = op->recompute ? 1 : G.nz;
-    op->P_row = pick_row_pairs(op->px, (long long)G.nz * G.ny, cs);
-    if (op->fast1024) {  // transposed intermediates: runs of P lines
-        op->P_row = 16;
-        while (op->P_row > 1 && row_smem(Nx, odd_pitch(op->P_row), cs) > kGenSmem) op->P_row >>= 1;
-    }
-    const ColPick both = pick_cols(op->py, op->ncol, layers, 2, cs, false);
-    op->C_col = both.C;
-    op->L_grp = both.L;
+    auto_shapes(op, true, true, true);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     gj_status rc;
     cudaError_t e;
@@ -902,12 +911,14 @@ extern "C" gj_status gj_op_tune(gj_op *op, int P_row, int C_col, int L_grp, int 
     if (radix_order >= 0 && (!plan_size(op->Nx, px, radix_order) || !plan_size(op->Ny, py, radix_order))) {
         set_error("gj_op_tune: radix_order must be 0, 1 or 2"); return GJ_ERR_ARG;
     }
-    if (P_row > 0) { op->P_row = P_row; op->rows_tuned = true; }
-    if (C_col > 0) { op->C_col = C_col; op->cols_tuned = true; }
-    if (L_grp > 0) { op->L_grp = L_grp; op->layers_tuned = true; }
     if (radix_order >= 0) op->radix_order = radix_order;
     op->px = px;
     op->py = py;
+    auto_shapes(op, !op->rows_tuned || P_row == GJ_TUNE_AUTO, !op->cols_tuned || C_col == GJ_TUNE_AUTO,
+                !op->layers_tuned || L_grp == GJ_TUNE_AUTO);
+    if (P_row > 0) { op->P_row = P_row; op->rows_tuned = true; }
+    if (C_col > 0) { op->C_col = C_col; op->cols_tuned = true; }
+    if (L_grp > 0) { op->L_grp = L_grp; op->layers_tuned = true; }
     return GJ_OK;
 }
 

@@ -48,3 +48,29 @@ def test_largest_row_tiles(prec, npad_x, pairs):
         assert rel(x, y) <= TOL[prec]  # the same transforms, whatever the tile
     for op in ops:
         op.close()
+
+
+@pytest.mark.parametrize("prec,npad", [("fp64", (45, 66)), ("fp32", (45, 66)), ("fp32", (1024, 66))])
+def test_shapes_given_back_to_the_library(prec, npad):
+    """After GJ_TUNE_AUTO an operator is what it was before any setting, bit for bit."""
+    gj = lib()
+    from paper_2112_15562_gb300._lib import GJ_TUNE_AUTO
+
+    g = synth.uniform_grid(30, 22, 30, 22, 12, 40.0)
+    ops = [gj.bttb_setup(g, "gravity", precision=prec, npad=npad), gj.bttb_setup(g, "magnetic", MAG, precision=prec, npad=npad)]
+    rng = np.random.default_rng(4)
+    m = [to_dev(x, prec) for x in rng.standard_normal((2, g.n))]
+    r = [to_dev(x, prec) for x in rng.standard_normal((2, g.s))]
+    products = lambda: [*gj.g_forward_pair(ops, m), *gj.g_adjoint_pair(ops, r), ops[1].forward(m[1]), ops[0].adjoint(r[0])]
+    tiles, want = ops[0].tiles(), products()
+    for op in ops:
+        op.tune(P_row=3, C_col=1, L_grp=2, radix_order=2)
+    assert ops[0].tiles() == {"P_row": 3, "C_col": 1, "L_grp": 2, "radix_order": 2}
+    products()
+    for op in ops:
+        op.tune(P_row=GJ_TUNE_AUTO, C_col=GJ_TUNE_AUTO, L_grp=GJ_TUNE_AUTO, radix_order=0)
+    assert ops[0].tiles() == tiles
+    for x, y in zip(products(), want):
+        assert (x == y).all()
+    for op in ops:
+        op.close()
