@@ -35,7 +35,7 @@ constexpr unsigned long long kWaitLimitNs = 200ull * 1000ull * 1000ull;
 
 template <typename R> struct K16;
 template <> struct K16<float> {
-    static __device__ __forceinline__ float c1() { return 0.92387953251128675613f; }
+    static __device__ __forceinline__ float c1() { return root_part<float>(0.92387953251128675613); }
     static __device__ __forceinline__ float s1() { return 0.38268343236508977173f; }
     static __device__ __forceinline__ float r2() { return 0.70710678118654752440f; }
 };
@@ -106,7 +106,7 @@ template <typename R>
 __device__ __forceinline__ cpx<R> w32c(int j) {  // W32^j for 0 <= j < 16 (j known at compile time)
     const double c = j <= 8 ? cos_pi16(j) : -cos_pi16(16 - j);
     const double sn = j <= 8 ? cos_pi16(8 - j) : cos_pi16(j - 8);
-    return mk<cpx<R>>((R)c, (R)(-sn));
+    return mk<cpx<R>>(root_part<R>(c), root_part<R>(-sn));
 }
 
 // Per-lane twiddles, l = lane & 15.  Inverse form (load_inv): W256^(l k) =

@@ -106,7 +106,7 @@ __device__ __forceinline__ cpx<R> rot(cpx<R> a) {
         // a (c + i d) with |c| = |d| = h: (c a.x - d a.y, d a.x + c a.y)
         return mk<C>(re ? h * x : -h * x, im ? h * y : -h * y);
     } else {
-        constexpr R wr = (R)Root<k, N>::c, wi = (R)(INV ? Root<k, N>::s : -Root<k, N>::s);
+        constexpr R wr = root_part<R>(Root<k, N>::c), wi = root_part<R>(INV ? Root<k, N>::s : -Root<k, N>::s);
         return mk<C>(a.x * wr - a.y * wi, a.x * wi + a.y * wr);
     }
 }
