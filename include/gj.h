@@ -23,7 +23,12 @@
  *  - Errors: argument checks run synchronously and return a negative
  *    gj_status without enqueuing work; gj_last_error() then returns a message
  *    (per thread).  CUDA launch failures return GJ_ERR_CUDA.
- *  - Kernel attributes (shared-memory limits) are set once per kernel and device
+ *  - Solvers, the host-buffer solve, the Gramian and gj_pearson take their device
+ *    memory from a stream-ordered pool of the library's own, one per device, made on
+ *    first use and kept for the life of the process.  It holds on to at most 128 MB
+ *    between uses (for the next use; other allocators cannot have it) and gives the
+ *    rest back.  Safe from any thread and stream.
+ *  - Kernel attributes (shared-memory limits) and the pool are set up once per device
  *    and kept for the life of the process; a caller that resets a device
  *    (cudaDeviceReset) must not use the library on it afterwards.
  */
@@ -236,8 +241,9 @@ gj_status gj_g_adjoint(const gj_op *op, const void *r, void *g, gj_stream_t stre
  * with the same grid, padded size and launch shapes (the gravity and magnetic operators
  * of one joint problem), each pass is one launch over both fields, which fills the GPU
  * better than two single-field calls; a transform never mixes the fields, so that
- * the results round as the single-field products do.  Otherwise the call runs the
- * two products one after the other.  The two operators must differ
+ * each transform rounds as in a single-field product (the general kernels may add the
+ * layers in another order in a launch for both fields, so that the last bits of the
+ * results can differ).  Otherwise the call runs the two products one after the other.  The two operators must differ
  * (each owns its workspace); failures as for the single products.
  */
 gj_status gj_g_forward_pair(const gj_op *const ops[2], const void *const m[2], void *const d[2],
@@ -250,8 +256,9 @@ gj_status gj_g_adjoint_pair(const gj_op *const ops[2], const void *const r[2], v
  * S = (m1,m1)(m2,m2) - (m1,m2)^2 written to the device double *S, and the
  * ascent directions l1 = (m2,m2) m1 - (m1,m2) m2, l2 = (m1,m1) m2 - (m1,m2) m1
  * (half the gradient of S).  l1 / l2 may be NULL to skip them.  Vectors of
- * length n in the given precision; inner products accumulate in FP64.  l1 and l2
- * may be m1 and m2 themselves, in either order.
+ * length n in the given precision; inner products accumulate in FP64 (sums of at most
+ * 16 products a thread in the given precision).  l1 and l2 may be m1 and m2 themselves,
+ * in either order.  Asynchronous on `stream`; scratch as in gj_pearson.
  */
 gj_status gj_gramian_value_grad(int64_t n, gj_precision precision,
                                 const void *m1, const void *m2, double *S,
@@ -288,7 +295,8 @@ gj_status gj_gramian_value_grad_noalloc(int64_t n, gj_precision precision,
  * centred sums in FP64 (0 when either vector has no spread).  The measure of
  * "correlated models" in the lambda selection of Secs. 3.1.3 and 5, whose
  * figures judge it from density-susceptibility cross-plots.  Asynchronous on
- * `stream`; allocates its reduction scratch with cudaMallocAsync.
+ * `stream`; takes its reduction scratch from the library's pool (under stream capture
+ * from the device's default pool: an allocation node of the graph).
  */
 gj_status gj_pearson(int64_t n, gj_precision precision, const void *a, const void *b, double *r,
                      gj_stream_t stream);
@@ -346,7 +354,8 @@ typedef struct {
  * or NULL (identity); m_apr[i]: n values or NULL (zero).  m[i]: n values, the
  * starting model on entry, the result on return.  hist: device array of
  * kmax + 1 records or NULL.  *rep (host) is filled on return; the call
- * synchronises `stream`.  Non-convergence by kmax is not an error
+ * synchronises `stream`, which must not be capturing (GJ_ERR_CUDA, and the capture
+ * goes on).  Non-convergence by kmax is not an error
  * (rep->converged = 0).
  */
 gj_status gj_rrcg_joint_solve(const gj_op *const ops[2], const gj_rrcg_params *params,
@@ -359,7 +368,7 @@ gj_status gj_rrcg_joint_solve(const gj_op *const ops[2], const gj_rrcg_params *p
  * gj_rrcg_joint_solve_host - the same solve with HOST buffers: dobs, sigma,
  * w_depth, m_apr, w_hard and m are host pointers (m: the starting models on
  * entry, the result on return); everything else is as in gj_rrcg_joint_solve
- * (no history).  The call allocates one device block for the copies, copies
+ * (no history).  The call takes one device block for the copies from the pool, copies
  * the inputs in with cudaMemcpyAsync on `stream` (page-locked host memory lets
  * the copies run asynchronously), solves, copies both models back, frees the
  * block and synchronises `stream`.  On GJ_ERR_NONFINITE the models are still
@@ -379,6 +388,9 @@ gj_status gj_rrcg_joint_solve_host(const gj_op *const ops[2], const gj_rrcg_para
  * they are ordered (one stream, or explicit events). */
 typedef struct gj_rrcg gj_rrcg;
 
+/* Makes a solver on the current device and enqueues the first residual; ready for any
+ * stream on return.  `stream` must not be capturing: its memory would be a node of the
+ * graph (GJ_ERR_CUDA, and the capture goes on). */
 gj_status gj_rrcg_create(const gj_op *const ops[2], const gj_rrcg_params *params,
                          const void *const dobs[2], const void *const sigma[2],
                          const void *const m_apr[2], const void *const w_depth[2],
@@ -404,6 +416,7 @@ int gj_rrcg_done(gj_rrcg *solver, gj_stream_t stream);
  * previous read (for graph replays: the launches of the last replay). */
 gj_status gj_rrcg_profile(gj_rrcg *solver, int enable);
 gj_status gj_rrcg_profile_read(gj_rrcg *solver, int *launches, double *total_ms);
+/* Waits for the solver's device and frees it, whatever device is current.  NULL is a no-op. */
 void gj_rrcg_destroy(gj_rrcg *solver);
 
 /*

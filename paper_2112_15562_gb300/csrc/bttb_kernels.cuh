@@ -6,11 +6,11 @@
 // Z[k] and Z[N-k].  Only ncol = Nx/2 + 1 columns are kept.  Zero padding is never
 // stored: the first stage of each transform skips the inputs beyond the data.
 //
-// Forward product of one field:  rows (m -> Z) -> columns with the layer spectra
-// multiplied and summed over layers (Z -> Y) -> inverse columns (Y -> W) ->
-// inverse rows cropped to the stations (W -> d).  Adjoint: rows (r -> W) ->
-// columns (W -> Y = V^) -> per layer conj(T^_r) V^ and inverse columns (Y -> Z)
-// -> inverse rows cropped to the prisms (Z -> g).
+// Forward product, one launch a pass: rows (m -> Z) -> columns, multiplied by the layer
+// spectra and summed over layers on chip (between layer groups through Y), and inverse
+// columns of the sum (Z -> W) -> inverse rows cropped to the stations (W -> d).  Adjoint:
+// rows (r -> W) -> columns kept on chip (V^), and per layer the inverse columns of
+// conj(T^_r) V^ (W -> Z) -> inverse rows cropped to the prisms (Z -> g).
 #pragma once
 #include <utility>
 

@@ -207,12 +207,11 @@ __global__ void __launch_bounds__(CWF * 32, 1) k_col_fwd1024(View2<R> V, const i
 #pragma unroll
     for (int k = 0; k < 32; ++k) acc[k] = czero<C>();
     bool ok = __all_sync(0xffffffffu, f512::mbar_wait(&tabbar, 0, V.err));
-    int t_fail = ok ? t1 : t0;
     int seg_start = t0;
     for (int t = t0; t < t1 && ok; ++t, cu.next(nz, V.nfield)) {
         const int s = (t - t0) & 1;
         ok = __all_sync(0xffffffffu, f512::mbar_wait(&zbar[warp][s], (uint32_t)((t - t0) >> 1) & 1, V.err));
-        if (!ok) { t_fail = t; break; }
+        if (!ok) break;
         C v[32];
 #pragma unroll
         for (int j = 0; j < 16; ++j) v[j] = zs[s * H + lane + 32 * j];
@@ -220,7 +219,7 @@ __global__ void __launch_bounds__(CWF * 32, 1) k_col_fwd1024(View2<R> V, const i
         if (lane == 0 && tz < t1) issue_z();  // item t + 2, into the stage just read
         fwd1024<R>(v, xbuf, tab);
         ok = __all_sync(0xffffffffu, f512::mbar_wait(&tbar[warp], (uint32_t)(t - t0) & 1, V.err));
-        if (!ok) { t_fail = t; break; }
+        if (!ok) break;
         if (V.op[cu.fld].real_spec) {
             const R *tr = reinterpret_cast<const R *>(ts);
 #pragma unroll
