@@ -177,7 +177,8 @@ gj_status gj_op_info(const gj_op *op, gj_op_info_t *info);
 enum { GJ_TUNE_AUTO = -2 }; /* for P_row, C_col and L_grp; radix_order: 0 */
 gj_status gj_op_tune(gj_op *op, int P_row, int C_col, int L_grp, int radix_order);
 
-/* Frees an operator (waits for the device to finish using it).  NULL is a no-op. */
+/* Frees an operator (synchronises the current device, which must not be capturing except
+ * for the library's own graphs).  NULL is a no-op. */
 void gj_op_destroy(gj_op *op);
 
 /*
@@ -416,7 +417,10 @@ int gj_rrcg_done(gj_rrcg *solver, gj_stream_t stream);
  * previous read (for graph replays: the launches of the last replay). */
 gj_status gj_rrcg_profile(gj_rrcg *solver, int enable);
 gj_status gj_rrcg_profile_read(gj_rrcg *solver, int *launches, double *total_ms);
-/* Waits for the solver's device and frees it, whatever device is current.  NULL is a no-op. */
+/* Waits for the work enqueued on the solver and frees it, whatever device is current and
+ * whatever other threads capture.  (Iterations that were captured into a caller's graph are
+ * waited for by synchronising the solver's device, which must not be capturing then.)  NULL
+ * is a no-op. */
 void gj_rrcg_destroy(gj_rrcg *solver);
 
 /*

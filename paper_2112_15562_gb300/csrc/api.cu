@@ -19,6 +19,17 @@ gj_status cuda_fail(cudaError_t e, const char *what) {
     return e == cudaErrorMemoryAllocation ? GJ_ERR_OOM : GJ_ERR_CUDA;
 }
 
+std::mutex &capture_mutex() {
+    static std::mutex mu;
+    return mu;
+}
+cudaError_t sync_device() {
+    std::lock_guard<std::mutex> lock(capture_mutex());
+    cudaError_t e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
 constexpr uint64_t kPoolKeep = 128 << 20;  // (a pool reserves memory in pieces of 32 MB)
 static cudaMemPool_t own_pool(int dev) {
     static std::mutex mu;

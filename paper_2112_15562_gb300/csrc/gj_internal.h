@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -69,6 +70,13 @@ void make_twiddles(int N, std::vector<double> &re, std::vector<double> &im);
 // Any stream or thread may call; free with cudaFreeAsync in the stream, or with cudaFree once
 // the kernels on it are done: unlike cudaMalloc's memory, it is given back without waiting.
 cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t st);
+
+// Held while the library captures a graph, and by sync_device: synchronising a device fails, and
+// breaks the capture, while a stream of it is being captured, from whichever thread.
+std::mutex &capture_mutex();
+// Waits for the current device (an error, for instance of a capture by somebody else, is
+// returned and not left behind for the next check).
+cudaError_t sync_device();
 
 // Makes `dev` the current device until the end of the scope.
 class DeviceScope {

@@ -182,6 +182,8 @@ struct gj_rrcg {
     const gj_op *op[2];
     gj_precision prec;
     int dev = 0;              // the device that the solver was made on
+    cudaEvent_t used = nullptr;  // behind the last work enqueued on it
+    bool in_a_graph = false;     // some of it into a caller's capture, to run whenever that is launched
     SolverDev *S = nullptr;   // device
     void *vhat = nullptr;     // spectra of the residual's rows, both fields (vhat_values)
     void *buf = nullptr;      // p, l (2 fields each, n), v (2 x s), wd (2 x s)
@@ -206,6 +208,19 @@ struct gj_rrcg {
 };
 
 namespace gj {
+
+// Notes that work of the solver was enqueued on `st`: its destruction waits for that alone.
+// (Calls on one solver are ordered, so the last event stands for all of them.  Waiting for the
+// whole device instead fails, and breaks the capture, while any other thread captures a graph;
+// the solver's pool memory then went back with its kernels still running.)
+static cudaError_t mark_used(gj_rrcg *sv, cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e != cudaSuccess) return e;
+    if (cap == cudaStreamCaptureStatusNone) return cudaEventRecord(sv->used, st);
+    sv->in_a_graph = true;
+    return cudaSuccess;
+}
 
 static ProfilePair take_pair(gj_rrcg *sv) {
     ProfilePair p;
@@ -579,7 +594,9 @@ static gj_status rrcg_create(const gj_op *const ops[2], const gj_rrcg_params *P,
     const size_t nbuf = 4 * n + 4 * s + 2 * (size_t)o->nz + (sv->prev_anchor ? 2 * n : 0);
     constexpr size_t kStateBytes = (sizeof(SolverDev) + 255) / 256 * 256;
     void *blk = nullptr;
-    if ((e = pool_alloc(&blk, kStateBytes + vhat_bytes + nbuf * es, st)) != cudaSuccess) {
+    if ((e = cudaEventCreateWithFlags(&sv->used, cudaEventDisableTiming)) != cudaSuccess ||
+        (e = pool_alloc(&blk, kStateBytes + vhat_bytes + nbuf * es, st)) != cudaSuccess) {
+        if (sv->used) cudaEventDestroy(sv->used);
         delete sv;
         return cuda_fail(e, "solver state and vectors");
     }
@@ -607,10 +624,12 @@ static gj_status rrcg_create(const gj_op *const ops[2], const gj_rrcg_params *P,
     else launch_reciprocals(static_cast<float *>(sv->buf), n, s, o->nz, sigma, w_depth, st);
     if (o->prec == GJ_FP64) run_head<double>(sv, st); else run_head<float>(sv, st);
     e = cudaGetLastError();
+    if (e == cudaSuccess) e = mark_used(sv, st);
     if (e == cudaSuccess && wait) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         cudaStreamSynchronize(st);  // (freeing pool memory does not wait for its kernels)
         cudaFree(sv->S);
+        cudaEventDestroy(sv->used);
         delete sv;
         return cuda_fail(e, "gj_rrcg_create");
     }
@@ -626,14 +645,13 @@ extern "C" gj_status gj_rrcg_create(const gj_op *const ops[2], const gj_rrcg_par
     return rrcg_create(ops, P, dobs, sigma, m_apr, w_depth, w_hard, m, hist, stream, true, out);
 }
 
-extern "C" gj_status gj_rrcg_iterate(gj_rrcg *sv, int iters, int use_graph, gj_stream_t stream) {
-    if (!sv || iters < 0) { set_error("gj_rrcg_iterate: bad argument"); return GJ_ERR_ARG; }
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+static gj_status iterate_on(gj_rrcg *sv, int iters, int use_graph, cudaStream_t st) {
     if (use_graph && sv->profile && sv->prec == GJ_FP32_MIXED && sv->op[0]->fast) {
         // segments [.. | col | .. | col | ..] with stream events around the column launches
         if (sv->seg_exec.empty()) {
             cudaStream_t cap;
             GJ_CUDA(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
+            std::unique_lock<std::mutex> lock(capture_mutex());
             sv->capturing = true;
             sv->cap_err = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
             if (sv->cap_err == cudaSuccess) {
@@ -644,6 +662,7 @@ extern "C" gj_status gj_rrcg_iterate(gj_rrcg *sv, int iters, int use_graph, gj_s
                 else if (sv->cap_err == cudaSuccess) sv->cap_err = e;
             }
             sv->capturing = false;
+            lock.unlock();
             cudaStreamDestroy(cap);
             if (sv->cap_err != cudaSuccess || sv->seg_graph.size() != 5) {
                 for (auto g : sv->seg_graph) cudaGraphDestroy(g);
@@ -676,6 +695,7 @@ extern "C" gj_status gj_rrcg_iterate(gj_rrcg *sv, int iters, int use_graph, gj_s
         if (!sv->exec) {
             cudaStream_t cap;
             GJ_CUDA(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
+            std::unique_lock<std::mutex> lock(capture_mutex());
             sv->capturing = true;
             cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
             if (e == cudaSuccess) {
@@ -683,6 +703,7 @@ extern "C" gj_status gj_rrcg_iterate(gj_rrcg *sv, int iters, int use_graph, gj_s
                 e = cudaStreamEndCapture(cap, &sv->graph);
             }
             sv->capturing = false;
+            lock.unlock();
             cudaStreamDestroy(cap);
             if (e != cudaSuccess) return cuda_fail(e, "rrcg graph capture");
             GJ_CUDA(cudaGraphInstantiate(&sv->exec, sv->graph, 0));
@@ -695,6 +716,14 @@ extern "C" gj_status gj_rrcg_iterate(gj_rrcg *sv, int iters, int use_graph, gj_s
         GJ_CUDA(cudaGetLastError());
     }
     return GJ_OK;
+}
+
+extern "C" gj_status gj_rrcg_iterate(gj_rrcg *sv, int iters, int use_graph, gj_stream_t stream) {
+    if (!sv || iters < 0) { set_error("gj_rrcg_iterate: bad argument"); return GJ_ERR_ARG; }
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    gj_status rc = iterate_on(sv, iters, use_graph, st);
+    cudaError_t e = mark_used(sv, st);  // (a call that failed may have enqueued some of its work)
+    return rc == GJ_OK && e != cudaSuccess ? cuda_fail(e, "gj_rrcg_iterate") : rc;
 }
 
 extern "C" gj_status gj_rrcg_report_get(gj_rrcg *sv, gj_rrcg_report *rep, gj_stream_t stream) {
@@ -726,6 +755,7 @@ extern "C" gj_status gj_rrcg_report_device(gj_rrcg *sv, gj_rrcg_report *rep, gj_
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     k_report<<<1, 1, 0, st>>>(sv->S, sv->op[0]->err, rep);
     GJ_CUDA(cudaGetLastError());
+    GJ_CUDA(mark_used(sv, st));
     return GJ_OK;
 }
 
@@ -746,7 +776,7 @@ extern "C" gj_status gj_rrcg_profile(gj_rrcg *sv, int enable) {
 
 extern "C" gj_status gj_rrcg_profile_read(gj_rrcg *sv, int *launches, double *total_ms) {
     if (!sv || !launches || !total_ms) { set_error("gj_rrcg_profile_read: NULL argument"); return GJ_ERR_ARG; }
-    GJ_CUDA(cudaDeviceSynchronize());
+    GJ_CUDA(sync_device());
     double tot = 0.0;
     int cnt = 0;
     auto acc = [&](const std::vector<ProfilePair> &v) -> gj_status {
@@ -771,14 +801,18 @@ extern "C" gj_status gj_rrcg_profile_read(gj_rrcg *sv, int *launches, double *to
 extern "C" void gj_rrcg_destroy(gj_rrcg *sv) {
     if (!sv) return;
     DeviceScope scope(sv->dev);  // whatever device is current: its kernels are the ones to wait for
-    cudaDeviceSynchronize();
+    const cudaError_t e = sv->in_a_graph ? sync_device() : cudaEventSynchronize(sv->used);
     if (sv->exec) cudaGraphExecDestroy(sv->exec);
     if (sv->graph) cudaGraphDestroy(sv->graph);
     for (auto x : sv->seg_exec) cudaGraphExecDestroy(x);
     for (auto g : sv->seg_graph) cudaGraphDestroy(g);
     for (auto *v : {&sv->eager_pairs, &sv->graph_pairs, &sv->free_pairs})
         for (auto &p : *v) { cudaEventDestroy(p.a); cudaEventDestroy(p.b); }
-    cudaFree(sv->S);  // (the vectors are in the same block)
+    cudaEventDestroy(sv->used);
+    // The state and the vectors, one block.  Memory whose work could not be waited for (in a
+    // caller's graph, while somebody else captures) is not given back.
+    if (e == cudaSuccess) cudaFree(sv->S);
+    else cudaGetLastError();
     delete sv;
 }
 
@@ -855,6 +889,7 @@ struct gj_rrcg_batch {
     std::vector<gj_rrcg *> sv;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+    cudaEvent_t used = nullptr;  // behind the last step
 };
 
 extern "C" gj_status gj_rrcg_batch_create(gj_rrcg *const *solvers, int count, gj_stream_t stream,
@@ -910,11 +945,13 @@ extern "C" gj_status gj_rrcg_batch_create(gj_rrcg *const *solvers, int count, gj
     std::vector<cudaEvent_t> join(count, nullptr);
     cudaEvent_t fork = nullptr;
     cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->used, cudaEventDisableTiming);
     for (int i = 0; i < count && e == cudaSuccess; ++i) {
         e = cudaStreamCreateWithFlags(&br[i], cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[i], cudaEventDisableTiming);
     }
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+    std::unique_lock<std::mutex> lock(capture_mutex());
     if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         cudaError_t ce = cudaEventRecord(fork, cap);
@@ -931,6 +968,7 @@ extern "C" gj_status gj_rrcg_batch_create(gj_rrcg *const *solvers, int count, gj
         cudaError_t ee = cudaStreamEndCapture(cap, &b->graph);
         e = ce != cudaSuccess ? ce : ee;
     }
+    lock.unlock();
     if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
     for (gj_rrcg *sv : b->sv) sv->grid = 0;  // stepwise calls outside the batch use the full grid
     for (int i = 0; i < count; ++i) {
@@ -941,6 +979,7 @@ extern "C" gj_status gj_rrcg_batch_create(gj_rrcg *const *solvers, int count, gj
     if (cap) cudaStreamDestroy(cap);
     if (e != cudaSuccess) {
         if (b->graph) cudaGraphDestroy(b->graph);
+        if (b->used) cudaEventDestroy(b->used);
         delete b;
         return cuda_fail(e, "gj_rrcg_batch_create");
     }
@@ -951,15 +990,21 @@ extern "C" gj_status gj_rrcg_batch_create(gj_rrcg *const *solvers, int count, gj
 extern "C" gj_status gj_rrcg_batch_step(gj_rrcg_batch *b, int iters, gj_stream_t stream) {
     if (!b || iters < 0) { set_error("gj_rrcg_batch_step: bad argument"); return GJ_ERR_ARG; }
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    for (int it = 0; it < iters; ++it) GJ_CUDA(cudaGraphLaunch(b->exec, st));
-    return GJ_OK;
+    cudaError_t e = cudaSuccess;
+    for (int it = 0; it < iters && e == cudaSuccess; ++it) e = cudaGraphLaunch(b->exec, st);
+    cudaError_t e2 = cudaEventRecord(b->used, st);
+    for (gj_rrcg *sv : b->sv)
+        if (e2 == cudaSuccess) e2 = mark_used(sv, st);
+    if (e == cudaSuccess) e = e2;
+    return e == cudaSuccess ? GJ_OK : cuda_fail(e, "gj_rrcg_batch_step");
 }
 
 extern "C" void gj_rrcg_batch_destroy(gj_rrcg_batch *b) {
     if (!b) return;
-    cudaDeviceSynchronize();
+    cudaEventSynchronize(b->used);
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
+    cudaEventDestroy(b->used);
     delete b;
 }
 

@@ -938,7 +938,7 @@ extern "C" gj_status gj_op_info(const gj_op *op, gj_op_info_t *info) {
 
 extern "C" void gj_op_destroy(gj_op *op) {
     if (!op) return;
-    cudaDeviceSynchronize();
+    sync_device();
     free_op_memory(op);
     delete op;
 }

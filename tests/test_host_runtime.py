@@ -4,6 +4,8 @@ import ctypes as ct
 import glob
 import os
 import subprocess
+import threading
+import time
 
 import pytest
 
@@ -99,3 +101,55 @@ def test_a_recomputing_operator_keeps_one_layer(lib, dz, prec):
         assert lib.fake_held_bytes() == before
     plane = 400 * 360 * 8  # corner values of one depth plane over the whole grid
     assert extra[1] - extra[0] <= plane, extra
+
+
+@pytest.mark.parametrize("batch", [False, True])
+@pytest.mark.parametrize("graph", [0, 1])
+def test_a_solver_is_destroyed_while_another_thread_captures(lib, graph, batch):
+    """Synchronising the device then fails and breaks that capture, so the solver waits for its own
+    work alone; its block is not given back before."""
+    lib.cudaSetDevice(0)
+    h, ops, keep = solver(lib)
+    early, broken = lib.fake_early_frees(), lib.fake_broken_captures()
+    assert lib.gj_rrcg_iterate(h, 2, graph, None) == 0
+    if batch:
+        b = ct.c_void_p()
+        assert lib.gj_rrcg_batch_create((ct.c_void_p * 1)(h.value), 1, None, ct.byref(b)) == 0
+        assert lib.gj_rrcg_batch_step(b, 3, None) == 0
+    lib.fake_capture_elsewhere(1)
+    try:
+        if batch:
+            lib.gj_rrcg_batch_destroy(b)
+        lib.gj_rrcg_destroy(h)
+        assert lib.fake_broken_captures() == broken
+        assert lib.fake_early_frees() == early
+    finally:
+        lib.fake_capture_elsewhere(0)
+    for op in ops:
+        lib.gj_op_destroy(op)
+
+
+def test_one_thread_captures_while_another_destroys(lib):
+    """A solve's graph is captured (drawn out here to 0.2 s) while another thread takes its solver and
+    its operators down, which waits for the device: not during the capture."""
+    lib.cudaSetDevice(0)
+    (h, ops, keep), (h2, ops2, keep2) = solver(lib), solver(lib)
+    broken = lib.fake_broken_captures()
+    lib.fake_capture_lasts(200)
+    try:
+        status = []
+        t = threading.Thread(target=lambda: status.append(lib.gj_rrcg_iterate(h, 1, 1, None)))
+        t.start()
+        while lib.fake_captures() == 0 and t.is_alive():
+            time.sleep(0.001)
+        lib.gj_rrcg_destroy(h2)
+        for op in ops2:
+            lib.gj_op_destroy(op)
+        t.join()
+    finally:
+        lib.fake_capture_lasts(0)
+    assert status == [0]
+    assert lib.fake_broken_captures() == broken
+    lib.gj_rrcg_destroy(h)
+    for op in ops:
+        lib.gj_op_destroy(op)
