@@ -16,6 +16,7 @@ void set_error(const std::string &msg) { g_last_error = msg; }
 gj_status cuda_fail(cudaError_t e, const char *what) {
     std::string m = std::string(what) + ": " + cudaGetErrorName(e) + " (" + cudaGetErrorString(e) + ")";
     set_error(m);
+    cudaGetLastError();  // reported here: the next call's launches do not find it again
     return e == cudaErrorMemoryAllocation ? GJ_ERR_OOM : GJ_ERR_CUDA;
 }
 

@@ -24,9 +24,10 @@ struct Event { int dev; long at; };
 void wait_to(int dev, long at) {
     if (waited[dev] < at) waited[dev] = at;
 }
-cudaError_t give(void **p, size_t bytes) {
-    *p = calloc(1, bytes ? bytes : 1);
-    return *p ? cudaSuccess : cudaErrorMemoryAllocation;
+thread_local cudaError_t last = cudaSuccess;  // kept until it is read, as the runtime does
+cudaError_t give(void **p, size_t bytes) {  // (a device of 256 GB)
+    *p = bytes < (size_t)1 << 38 ? calloc(1, bytes ? bytes : 1) : nullptr;
+    return *p ? cudaSuccess : (last = cudaErrorMemoryAllocation);
 }
 cudaError_t handle(void *out) {
     *static_cast<void **>(out) = malloc(1);
@@ -54,7 +55,7 @@ cudaError_t cudaSetDevice(int d) { current = d; return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() {
     if (captures > 0) {
         ++broken_captures;
-        return cudaErrorStreamCaptureUnsupported;
+        return last = cudaErrorStreamCaptureUnsupported;
     }
     wait_to(current, enqueued[current]);
     return cudaSuccess;
@@ -64,7 +65,11 @@ cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr a, int) {
     *v = a == cudaDevAttrMultiProcessorCount ? 4 : a == cudaDevAttrMaxSharedMemoryPerBlockOptin ? 227 * 1024 : 0;
     return cudaSuccess;
 }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError() {
+    const cudaError_t e = last;
+    last = cudaSuccess;
+    return e;
+}
 const char *cudaGetErrorName(cudaError_t) { return "fake"; }
 const char *cudaGetErrorString(cudaError_t) { return "fake"; }
 

@@ -153,3 +153,22 @@ def test_one_thread_captures_while_another_destroys(lib):
     lib.gj_rrcg_destroy(h)
     for op in ops:
         lib.gj_op_destroy(op)
+
+
+def test_an_error_is_reported_once(lib):
+    """An operator that does not fit the device is refused with GJ_ERR_OOM, and the next call on
+    another operator is not told so again."""
+    from paper_2112_15562_gb300 import _lib as L
+
+    lib.cudaSetDevice(0)
+    h, ops, keep = solver(lib)
+    nz = 20000
+    z = (ct.c_double * (nz + 1))(*range(nz + 1))
+    g = L.Grid(1000, 1000, 1000, 1000, nz, 10.0, 10.0, ct.cast(z, ct.POINTER(ct.c_double)), 0.0, 0, 0)
+    big = ct.c_void_p()
+    assert lib.gj_bttb_setup(ct.byref(g), 1, None, 0, 2048, 2048, None, ct.byref(big)) == -2 and not big.value
+    m, d = (ct.c_double * 32)(), (ct.c_double * 16)()
+    assert lib.gj_g_forward(ops[0], ct.addressof(m), ct.addressof(d), None) == 0, lib.gj_last_error()
+    lib.gj_rrcg_destroy(h)
+    for op in ops:
+        lib.gj_op_destroy(op)
